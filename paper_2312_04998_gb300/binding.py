@@ -506,9 +506,8 @@ def probe_fma(device: int, fp64: bool) -> float:
     return v.value
 
 
-PHASE_NAMES = ["zero + dR + weights", "Jacobian gather + M", "sparse head (A11, L21, U12)",
-               "head Schur complement", "head packing", "panel loads", "panel LU", "U block load",
-               "U block solve", "trailing update", "epilogue"]
+PHASE_NAMES = ["state load / store", "predict", "reaction rates", "S R gather", "residual + substitution + update",
+               "finish", "dR/dx + Jacobian gather", "head program", "panel assembly", "panel updates", "panel LU"]
 
 
 def use_phase_build():

@@ -97,6 +97,7 @@ void release_all(sm_net* net) {
   lu.d_flev.release();
   lu.d_blev_ptr.release();
   lu.d_blev.release();
+  net->cell.blob.release();
   net->d_jt_slot.release();
   net->d_jdesc.release();
   net->d_jlong.release();

@@ -30,128 +30,13 @@
 #include <cstring>
 #include <vector>
 
+#include "cell.h"
+#include "integ.h"
 #include "internal.h"
 
+using namespace integ;
+
 namespace {
-
-constexpr int QMAX = 5;  // highest BDF order; the history keeps QMAX + 1 points
-// counters[] entries of the compaction (0..3 belong to the attempt loop and
-// the adjoint)
-constexpr int kCAct = 8;     // slots holding the running cells: [0, counters[kCAct])
-constexpr int kCHoles = 9;   // finished cells below the new boundary
-constexpr int kCRun = 10;    // running cells above it
-constexpr int kCLive = 11;   // running cells counted for the compaction
-constexpr int kCounters = 16;
-constexpr int kCkpt = SM_CHECKPOINT_EVERY;
-enum : int {
-  F_NEED_J = 1, F_REJECTED = 2, F_HAS_EPREV = 4, F_NEWTON = 8, F_CONV = 16,
-  F_FINAL = 32, F_REFRESH = 64, F_FAILED = 128, F_ATTEMPT = 256
-};
-
-struct Dev {
-  int n, n_r, nnz_j, mixed, tf32, head;
-  int64_t C, ld;
-  double rtol, atol, gamma_tol, newton_tol, eta_max, eta_keep, t_end;
-  int q_max, max_steps, j_age_max, newton_max, max_conv_fails;
-  // per-cell scalars [ld] (tn, alpha: [QMAX+1][ld])
-  double *t, *h, *gam, *gam_J, *crate, *dprev, *tn, *alpha;
-  int *q, *nh, *n_at_q, *j_age, *flags, *crej, *ccf, *status, *m_it;
-  int *steps, *rejects, *conv_fails, *newton_iters, *jac_evals;
-  // per-cell vectors [n][ld]; Y is [QMAX+1][n][ld]
-  double *Y, *ypred, *y, *psi, *f, *f0, *eprev, *w, *wf;
-  int *list, *counters;  // counters[0] = refresh list length, [1] = running cells
-  // compaction of the running cells (states that record no steps): cell
-  // slots are permuted so that running cells occupy slots [0, counters[kCAct])
-  int* slot_cell;        // [ld] slot -> cell of the caller's arrays (and of the packed factors)
-  int compact;           // 1: compaction on
-  double* kslot;         // [n_r][ld] rate coefficients in slot order (compaction on), else null
-  int *holes, *runners;  // [ld] each: the slot pairs of one compaction
-  // recording (record > 0): per accepted step m (1-based) at [m-1][ld]; the
-  // step history after every kCkpt-th accepted step at checkpoint m / kCkpt
-  int record;
-  double *log_t, *log_h;
-  int* log_q;
-  double *ck_Y, *ck_t;   // [K][QMAX+1][n][ld], [K][QMAX+1][ld]
-  int* ck_nh;            // [K][ld]
-  void* lu;
-  int64_t lu_stride;
-  int ldm;
-  // packed factors read by the substitution (see LUSymbolic): per cell
-  // lup_stride values from lup; null when the state keeps dense factors only
-  void* lup;
-  int64_t lup_stride;
-  int lu_cta;   // 1: lu holds one dense working matrix per refresh CTA (not per cell)
-  int p_l11, p_u11, p_dinv, p_l21, p_u12, p_d, ldd, n_flev, n_blev;
-  const int *u11ptr, *flev_ptr, *flev, *blev_ptr, *blev;
-  const int *hop_ptr, *hop_piv;     // head program (see LUSymbolic)
-  const int4* hop;
-  const int2* hterm;
-  int n_hlev;
-  const int *perm, *iperm, *lptr, *lidx, *uptr, *uidx, *lrptr, *lridx, *ucptr, *ucidx, *jp_ptr, *jt_ptr,
-      *jpos, *jrc, *uoff, *lrhead, *lrhoff, *u12off, *lrhk, *srow;
-  int n_srow;
-  const int2 *jt_word, *jt_slot, *reac;
-  const int* sc_ptr;
-  const uint32_t* sc_ent;
-  const int4* jdesc;     // per Jacobian entry {t0, t1, jrc, row << 16 | col}
-  const int* jlong;      // entries with more than kJLong terms
-  int n_jlong;
-  // coupled temperature (therm = 1, see sm_net_set_thermal): row t_idx of
-  // every state vector holds T; k' of the T-dependent reactions is
-  // recomputed from it (into kslot) before every right-hand side
-  int therm, t_idx, n_cool, bpad;
-  double th_heat, th_lam, th_Td, th_zeta;
-  const RatePar* rpar;
-  const double *th_L, *th_E, *th_dn;   // [n] cooling coefficients, [n] excitation temperatures, [n_r] net particle change
-  const int* th_cool;                  // [n_cool] the coolant species
-  const double *c_nH, *c_Av, *c_chi;   // [ld] cell conditions, cell order
-  double *bz, *bgv, *bs;               // per cell (cell order): z, gamma_J v ([ld][bpad]) and the Schur complement ([ld])
-};
-
-__device__ __forceinline__ double& V(double* a, const Dev& d, int s, int64_t c) {
-  return a[(int64_t)s * d.ld + c];
-}
-__device__ __forceinline__ double* Yh(const Dev& d, int i) { return d.Y + (int64_t)i * d.n * d.ld; }
-
-// Weights of the polynomial through (T[i], .), i < m, evaluated at t.
-__device__ void lagrange(const double* T, int m, double t, double* wts) {
-  for (int i = 0; i < m; ++i) {
-    double num = 1.0, den = 1.0;
-    for (int j = 0; j < m; ++j)
-      if (j != i) {
-        num *= t - T[j];
-        den *= T[i] - T[j];
-      }
-    wts[i] = num / den;
-  }
-}
-
-// alpha_i = h l_i'(tau_0) on nodes tau_0 = tnew, tau_i = T[i-1] (i = 1..q).
-__device__ void bdf_alphas(double tnew, const double* T, int q, double h, double* al) {
-  double tau[QMAX + 1];
-  tau[0] = tnew;
-  for (int i = 1; i <= q; ++i) tau[i] = T[i - 1];
-  double s = 0.0;
-  for (int i = 1; i <= q; ++i) s += 1.0 / (tau[0] - tau[i]);
-  al[0] = h * s;
-  for (int i = 1; i <= q; ++i) {
-    double num = 1.0, den = 1.0;
-    for (int m = 1; m <= q; ++m)
-      if (m != i) num *= tau[0] - tau[m];
-    for (int m = 0; m <= q; ++m)
-      if (m != i) den *= tau[i] - tau[m];
-    al[i] = h * num / den;
-  }
-}
-
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ float warp_sum(float v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // ---------------------------------------------------------------------------
 // init: copy y0 into the history, validate inputs; then (after f0 = f(y0))
@@ -352,28 +237,6 @@ __global__ void __launch_bounds__(32 * kCoopWarps) predict_kernel(Dev d) {
 //     update is a register-tiled GEMM.
 // Inverse pivots replace the diagonal.
 // ---------------------------------------------------------------------------
-// Optional per-phase cycle counters of the refresh kernel (build option
-// SM_PHASE_CLOCKS, see build.py): thread 0 of every CTA adds the clock64()
-// cycles between consecutive phase marks (taken right after the CTA-wide
-// barriers that end the phases) to g_phase_cycles[phase]; slot 15 counts the
-// refreshed cells.  Compiled out otherwise.
-constexpr int kPhaseSlots = 16;
-#ifdef SM_PHASE_CLOCKS
-__device__ unsigned long long g_phase_cycles[kPhaseSlots];
-#define PHASE_START() long long ph_t = clock64()
-#define PHASE_MARK(k)                                                                         \
-  do {                                                                                        \
-    if (threadIdx.x == 0) {                                                                   \
-      const long long ph_now = clock64();                                                     \
-      atomicAdd(&g_phase_cycles[(k)], (unsigned long long)(ph_now - ph_t));                   \
-      ph_t = ph_now;                                                                          \
-    }                                                                                         \
-  } while (0)
-#else
-#define PHASE_START() do {} while (0)
-#define PHASE_MARK(k) do {} while (0)
-#endif
-
 constexpr int kRefreshThreads = 256;
 constexpr int kNB = 32;
 constexpr int kTM = 4, kTN = 4;
@@ -525,7 +388,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
     T* A = static_cast<T*>(d.lu) + (d.lu_cta ? (int64_t)blockIdx.x : c) * d.lu_stride;
     T* P = d.lup ? static_cast<T*>(d.lup) + (int64_t)d.slot_cell[c] * d.lup_stride : nullptr;
     T* D = P ? P + d.p_d : nullptr;   // packed tail block, column-major
-    PHASE_START();
     const double gamma = d.gam[c];
     // zero the dense trailing block and the head's pattern entries
     for (int r = warp; r < nt; r += nwarps) {
@@ -555,7 +417,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         wif[s] = (float)(1.0 / wv);
       }
     __syncthreads();
-    PHASE_MARK(0);   // zero the working matrix, dR/dx, weights
     // M_ij = delta_ij - gamma sum_terms coef dR, stored in elimination order
     // (W M W^-1 with this step's error weights, scaled in FP32, when mixed)
     auto store_m = [&](const int4 ds, double acc) {
@@ -607,7 +468,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
       if (lb) store_m(db, ab);
     }
     __syncthreads();
-    PHASE_MARK(1);   // Jacobian gather, M = I - gamma J
     // ---- phase B: sparse head.  The head program (see LUSymbolic) computes
     // every head factor entry in the packed layout, in shared memory: level
     // by level, first the level's pivots (stored inverted), then the U rows
@@ -641,7 +501,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           __syncthreads();
         }
       }
-      PHASE_MARK(2);   // head program
       // ---- phase S: A22 -= L21 U12, one 32-column panel at a time.  U12's
       // panel columns are expanded into a dense h x 32 tile (in front of H);
       // each tail row with head entries is one warp's: lanes are the panel's
@@ -725,7 +584,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         __syncthreads();
       }
     }
-    PHASE_MARK(3);   // head Schur complement (or the pivot-by-pivot head)
     // the head's factors are final.  Packed output: copy them out (from H, or
     // from the dense matrix after the pivot-by-pivot head); dense output: put
     // H's values back at their dense positions
@@ -758,7 +616,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         for (int q = lane; q < cnt; q += 32) P[d.p_l21 + o + q] = Ai[__ldg(d.lridx + p0 + q)];
       }
     }
-    PHASE_MARK(4);   // packed head factors
     // ---- phase C: dense trailing block, blocked right-looking LU
     for (int pb = 0; pb * kNB < nt; ++pb) {
       const int p0 = h + pb * kNB;
@@ -769,7 +626,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
       for (int a = m + tid; a < pitch; a += nthr)
         for (int b = 0; b < w; ++b) Pt[b * pitch + a] = T(0);
       __syncthreads();
-      PHASE_MARK(5);   // panel loads
       if (sizeof(T) == 4 && w == kNB) {
         // full FP32 panel.  (1) warp 0 factors the kNB x kNB diagonal block in
         // registers (lane = row, pivot rows broadcast by shuffles); (2) every
@@ -827,7 +683,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         }
         __syncthreads();
       }
-      PHASE_MARK(6);   // panel LU
       if (D) {
         // the panel's columns (diagonal block and L below it) are final
         for (int b = warp; b < w; b += nwarps)
@@ -842,7 +697,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           for (int b = lane; b < rp; b += 32)
             U[a * upitch + b] = b < r ? A[(int64_t)(p0 + a) * ldm + p0 + w + b] : T(0);
         __syncthreads();
-        PHASE_MARK(7);   // panel stored, U block loaded
         // U12 = L11^-1 A12, one thread per column
         if (w == kNB) {
           for (int b = tid; b < r; b += nthr) {
@@ -864,7 +718,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
             }
         }
         __syncthreads();
-        PHASE_MARK(8);   // U block solved
         if (D) {
           // the panel's U rows are final: column b of the block, rows p0..p0+w
           for (int e = tid; e < r * 32; e += nthr) {
@@ -928,7 +781,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         }
       }
       __syncthreads();
-      PHASE_MARK(9);   // trailing update
     }
     if (tid == 0) {
       d.gam_J[c] = gamma;
@@ -938,10 +790,6 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
       d.jac_evals[c] += 1;
     }
     __syncthreads();
-#ifdef SM_PHASE_CLOCKS
-    if (tid == 0) atomicAdd(&g_phase_cycles[kPhaseSlots - 1], 1ull);
-#endif
-    PHASE_MARK(10);  // epilogue
   }
 }
 
@@ -1673,13 +1521,20 @@ __global__ void __launch_bounds__(32 * kCoopWarps) finish_kernel(Dev d) {
   d.flags[c] = fl;
 }
 
+// The solution and statistics to the caller's arrays: lanes = slots, the
+// species rows split over blockIdx.y.
+constexpr int kReadRows = 32;
 __global__ void read_kernel(Dev d, double* __restrict__ yout, int64_t ldu, sm_cell_stats* __restrict__ st) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.C) return;
   const int64_t oc = d.slot_cell[c];   // the caller's cell held in slot c
-  if (yout)
-    for (int s = 0; s < d.n; ++s) yout[(int64_t)s * ldu + oc] = Yh(d, 0)[(int64_t)s * d.ld + c];
-  if (st) {
+  if (yout) {
+    const int s1 = min(d.n, (int)(blockIdx.y + 1) * kReadRows);
+#pragma unroll 8
+    for (int s = blockIdx.y * kReadRows; s < s1; ++s)
+      yout[(int64_t)s * ldu + oc] = Yh(d, 0)[(int64_t)s * d.ld + c];
+  }
+  if (st && blockIdx.y == 0) {
     sm_cell_stats r;
     r.status = d.status[c];
     r.steps = d.steps[c];
@@ -2159,6 +2014,10 @@ struct sm_state {
   double graph_t_end = 0.0;   // the captured kernels hold Dev by value, t_end included
   int refresh_ctas = 0;
   RefreshPlan plan{};
+  // fused per-cell integrator (cell.cu): on when its shared-memory plan fits
+  bool fused = false;
+  CellLaunch cell{};
+  DevArray cell_scratch, ring, cell_time;
   // instrumentation
   int64_t launches = 0, timed = 0;
   double timed_ms = 0.0;
@@ -2235,6 +2094,9 @@ void free_state(sm_state* st) {
   st->adj_d.release();
   st->adj_i.release();
   st->adj_lu.release();
+  st->cell_scratch.release();
+  st->ring.release();
+  st->cell_time.release();
   if (st->h_counters) cudaFreeHost(st->h_counters);
   if (st->ev_in) cudaEventDestroy(st->ev_in);
   if (st->ev_out) cudaEventDestroy(st->ev_out);
@@ -2382,9 +2244,26 @@ sm_status enqueue_group(sm_state* st, const double* k, int64_t ldk, int attempts
   return SM_OK;
 }
 
+// Attempts of every cell in one launch of the fused integrator: a launch over
+// many cells stays within a few seconds, one over few cells covers most of an
+// integration.
+int fused_attempts(int64_t C) { return (int)std::min<int64_t>(512, std::max<int64_t>(16, (1LL << 20) / C)); }
+
+sm_status run_fused(sm_state* st, const double* k, int64_t ldk, int attempts) {
+  for (int done = 0; done < attempts;) {
+    const int a = std::min(attempts - done, fused_attempts(st->d.C));
+    sm_status r = launch_cell_attempts(st->net, st->d, st->cell, k, ldk, a, st->s);
+    if (r != SM_OK) return r;
+    st->launches += 2;
+    done += a;
+  }
+  return SM_OK;
+}
+
 // Runs `attempts` attempts on the state's stream, through a cached CUDA graph
 // when enabled (captured once per (k, ldk, C, t_end)).
 sm_status run_attempts(sm_state* st, const double* k, int64_t ldk, int attempts) {
+  if (st->fused) return run_fused(st, k, ldk, attempts);
   if (!st->opts.use_graph) {
     sm_status r = enqueue_group(st, k, ldk, attempts, st->s);
     if (r == SM_OK && st->opts.timing_kind != SM_TIME_NONE) {
@@ -2452,6 +2331,8 @@ sm_status running_count(sm_state* st, int64_t* out, int64_t* failed = nullptr) {
   if (failed) *failed = st->h_counters[2];
   return SM_OK;
 }
+
+dim3 read_grid(const sm_state* st) { return dim3(blocks(st->C, 64), (unsigned)((st->d.n + kReadRows - 1) / kReadRows)); }
 
 sm_status join_in(sm_state* st, void* stream) {
   SM_TRY_CUDA(cudaEventRecord(st->ev_in, (cudaStream_t)stream));
@@ -2745,18 +2626,43 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   if ((r = st->lup.ensure(esz * (size_t)d.lup_stride * C)) != SM_OK) return fail(r);
   if ((r = st->list.ensure(sizeof(int) * ld)) != SM_OK) return fail(r);
   if ((r = st->counters.ensure(sizeof(int) * kCounters)) != SM_OK) return fail(r);
+  int smem_max = 0;
+  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device);
+  st->cell.plan = cell_plan(net, esz, net->th_t >= 0, (size_t)std::max(0, smem_max - 1024));
+  if (st->cell.plan.ok) {
+    if ((r = cell_resident(d, st->cell.plan, o.refresh_ctas_per_sm, &st->cell.ctas)) != SM_OK) return fail(r);
+    st->fused = st->cell.ctas > 0;
+  }
+  if (st->fused) {
+    CellLaunch& cl = st->cell;
+    const int64_t ring = 2 + std::max<int64_t>(C, 16 * std::min<int64_t>(C, 8LL * cl.ctas));
+    const int64_t nc = std::min<int64_t>(C, cl.ctas);
+    if ((r = st->cell_scratch.ensure(sizeof(double) * (size_t)(cl.plan.scratch * nc))) != SM_OK) return fail(r);
+    if ((r = st->ring.ensure(sizeof(int) * (size_t)(ring + ld))) != SM_OK) return fail(r);
+    cl.scratch = st->cell_scratch.as<double>();
+    cl.ring = st->ring.as<int>();
+    cl.done = cl.ring + ring;
+    cl.timing_kind = o.timing_kind;
+    if (o.timing_kind != SM_TIME_NONE) {
+      if ((r = st->cell_time.ensure(2 * sizeof(double))) != SM_OK) return fail(r);
+      SM_TRY_CUDA(cudaMemset(st->cell_time.p, 0, 2 * sizeof(double)));
+      cl.timing = st->cell_time.as<double>();
+    }
+  }
   // compaction of running cells in states that record no steps (the
-  // adjoint's records are indexed by cell)
-  d.compact = o.record_steps > 0 ? 0 : 1;
+  // adjoint's records are indexed by cell); the fused integrator needs none
+  d.compact = o.record_steps > 0 || st->fused ? 0 : 1;
   // slot-ordered rate coefficients: with compaction, and always with a
   // coupled temperature (its k'(T) is rewritten before every right-hand side)
-  if (d.compact || net->th_t >= 0) {
+  if (d.compact || (net->th_t >= 0 && !st->fused)) {
     if ((r = st->kslot.ensure(sizeof(double) * (size_t)net->n_r * ld)) != SM_OK) return fail(r);
   }
   if (d.compact) {
     if ((r = st->cpt.ensure(sizeof(int) * 2 * (size_t)ld)) != SM_OK) return fail(r);
   }
-  if ((r = st->scratch.ensure(sizeof(double) * (size_t)net->n_r * ld)) != SM_OK) return fail(r);
+  if ((!st->fused || o.record_steps > 0) &&
+      (r = st->scratch.ensure(sizeof(double) * (size_t)net->n_r * ld)) != SM_OK)
+    return fail(r);
   double* ds = st->scal_d.as<double>();
   d.t = ds; d.h = ds + ld; d.gam = ds + 2 * ld; d.gam_J = ds + 3 * ld; d.crate = ds + 4 * ld;
   d.dprev = ds + 5 * ld; d.tn = ds + 6 * ld; d.alpha = ds + (6 + QMAX + 1) * ld;
@@ -2824,8 +2730,6 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   if (cudaMallocHost(&st->h_counters, kCounters * sizeof(int)) != cudaSuccess) return fail(SM_ENOMEM);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, net->device);
-  int smem_max = 0;
-  cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device);
   {
     // shared memory of the refresh kernel: the largest of its three phases
     RefreshPlan& pl = st->plan;
@@ -2855,7 +2759,9 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   }
   const size_t rsm = st->plan.bytes;
 
-  if ((int64_t)rsm > smem_max) return fail(SM_ENOTSUP);
+  // (a fused state without recorded steps never launches it)
+  const bool classes = !st->fused || d.record;
+  if (classes && (int64_t)rsm > smem_max) return fail(SM_ENOTSUP);
   // the attribute is a per-kernel cap shared by every state: set it to the
   // device limit so that a later state with a smaller plan cannot lower it
   // below what an earlier state launches with
@@ -2875,7 +2781,8 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   // dense working matrices of the refresh: one per refresh CTA, except in
   // recording states, whose replays keep dense factors per cell
   d.lu_cta = d.record ? 0 : 1;
-  if ((r = st->lu.ensure(esz * (size_t)d.lu_stride * (d.lu_cta ? st->refresh_ctas : C))) != SM_OK) return fail(r);
+  if (classes && (r = st->lu.ensure(esz * (size_t)d.lu_stride * (d.lu_cta ? st->refresh_ctas : C))) != SM_OK)
+    return fail(r);
   d.lu = st->lu.p;
   // coupled temperature: a copy of the network's setting
   d.therm = 0;
@@ -2947,7 +2854,7 @@ sm_status sm_state_bytes(const sm_state* st, size_t* bytes) {
            st->scal_d.bytes + st->scal_i.bytes + st->vec.bytes + st->lu.bytes + st->lup.bytes + st->kslot.bytes +
            st->cpt.bytes + st->list.bytes +
            st->counters.bytes + st->scratch.bytes + st->rec_d.bytes + st->rec_i.bytes + st->adj_d.bytes + st->adj_i.bytes +
-           st->adj_lu.bytes;
+           st->adj_lu.bytes + st->cell_scratch.bytes + st->ring.bytes + st->cell_time.bytes;
   return SM_OK;
 }
 
@@ -2966,6 +2873,11 @@ sm_status sm_state_init(sm_state* st, int64_t C, const double* d_k, const double
   d.C = C;
   d.t_end = t_end;
   if (therm) d_k = nullptr;
+  if (st->fused) {
+    if ((r = launch_cell_init(st->net, d, st->cell, d_y, ld, d_k, ld, st->s)) != SM_OK) return r;
+    st->launches += 1;
+    return join_out(st, stream);
+  }
   init_copy_kernel<<<blocks(C, 128), 128, 0, st->s>>>(d, d_y, ld, d_k, ld);
   SM_TRY_CUDA(cudaGetLastError());
   st->kslot_src = d_k;
@@ -3018,7 +2930,7 @@ sm_status sm_state_read(sm_state* st, double* d_y, int64_t ld, sm_cell_stats* d_
   sm_status r;
   if ((r = join_in(st, stream)) != SM_OK) return r;
   if (d_y || d_stats) {
-    read_kernel<<<blocks(st->C, 128), 128, 0, st->s>>>(st->d, d_y, ld, d_stats);
+    read_kernel<<<read_grid(st), 64, 0, st->s>>>(st->d, d_y, ld, d_stats);
     SM_TRY_CUDA(cudaGetLastError());
     st->launches += 1;
   }
@@ -3048,7 +2960,7 @@ sm_status sm_integrate(sm_state* st, int64_t C, const double* d_k, double* d_y, 
   Scope scope(st->net->device);
   if (!scope.ok) return SM_ECUDA;
   if ((r = join_in(st, stream)) != SM_OK) return r;
-  const int per = st->opts.attempts_per_sync;
+  const int per = st->fused ? fused_attempts(C) : st->opts.attempts_per_sync;
   // every attempt either accepts a step, shrinks h or counts a failure, so
   // this cap is never the binding limit for a well-posed problem
   const int64_t max_attempts = 20LL * st->opts.max_steps + 1000;
@@ -3057,7 +2969,7 @@ sm_status sm_integrate(sm_state* st, int64_t C, const double* d_k, double* d_y, 
     if ((r = run_attempts(st, d_k, ld, per)) != SM_OK) return r;
     if ((r = running_count(st, &running)) != SM_OK) return r;
   }
-  read_kernel<<<blocks(C, 128), 128, 0, st->s>>>(st->d, d_y, ld, d_stats);
+  read_kernel<<<read_grid(st), 64, 0, st->s>>>(st->d, d_y, ld, d_stats);
   SM_TRY_CUDA(cudaGetLastError());
   st->launches += 1;
   int64_t failed = 0;
@@ -3267,7 +3179,7 @@ extern "C" sm_status sm_state_load(sm_state* st, const void* host, size_t bytes,
   st->d.C = im.C;
   st->d.t_end = im.t_end;
   st->kslot_src = nullptr;   // regathered from the next sm_step_bdf's d_k
-  set_active_kernel<<<1, 32, 0, st->s>>>(st->d);
+  set_active_kernel<<<1, 32, 0, st->s>>>(st->d);   // (read by the class kernels only)
   SM_TRY_CUDA(cudaGetLastError());
   st->launches += 1;
   if (!im.with_factors) {
@@ -3282,9 +3194,25 @@ extern "C" sm_status sm_state_load(sm_state* st, const void* host, size_t bytes,
 
 extern "C" sm_status sm_state_timing(const sm_state* st, int64_t* launches, double* ms, int64_t* timed) {
   if (!st) return SM_EINVAL;
+  double t = st->timed_ms;
+  int64_t n = st->timed;
+  if (st->cell.timing) {
+    // the fused integrator counts clock cycles per CTA: their mean over the
+    // CTAs at the device's clock rate
+    Scope scope(st->net->device);
+    if (!scope.ok) return SM_ECUDA;
+    double v[2];
+    int khz = 0;
+    SM_TRY_CUDA(cudaMemcpyAsync(v, st->cell.timing, sizeof v, cudaMemcpyDeviceToHost, st->s));
+    SM_TRY_CUDA(cudaStreamSynchronize(st->s));
+    SM_TRY_CUDA(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, st->net->device));
+    const double ctas = (double)std::min<int64_t>(std::max<int64_t>(st->C, 1), st->cell.ctas);
+    t += v[0] / (khz > 0 ? khz : 1) / ctas;
+    n += (int64_t)v[1];
+  }
   if (launches) *launches = st->launches;
-  if (ms) *ms = st->timed_ms;
-  if (timed) *timed = st->timed;
+  if (ms) *ms = t;
+  if (timed) *timed = n;
   return SM_OK;
 }
 
@@ -3293,26 +3221,10 @@ extern "C" sm_status sm_state_timing_reset(sm_state* st) {
   st->launches = 0;
   st->timed = 0;
   st->timed_ms = 0.0;
-  return SM_OK;
-}
-
-extern "C" sm_status sm_phase_cycles(int32_t device, double* h_out, int32_t reset) {
-#ifdef SM_PHASE_CLOCKS
-  if (!h_out || device < 0) return SM_EINVAL;
-  Scope scope(device);
-  if (!scope.ok) return SM_ECUDA;
-  unsigned long long v[kPhaseSlots];
-  SM_TRY_CUDA(cudaMemcpyFromSymbol(v, g_phase_cycles, sizeof(v)));
-  for (int i = 0; i < kPhaseSlots; ++i) h_out[i] = (double)v[i];
-  if (reset) {
-    const unsigned long long z[kPhaseSlots] = {0};
-    SM_TRY_CUDA(cudaMemcpyToSymbol(g_phase_cycles, z, sizeof(z)));
+  if (st->cell.timing) {
+    Scope scope(st->net->device);
+    if (!scope.ok) return SM_ECUDA;
+    SM_TRY_CUDA(cudaMemsetAsync(st->cell.timing, 0, 2 * sizeof(double), st->s));
   }
   return SM_OK;
-#else
-  (void)device;
-  (void)h_out;
-  (void)reset;
-  return SM_ENOTSUP;
-#endif
 }

@@ -114,6 +114,43 @@ struct LUSymbolic {
       d_jrc, d_uoff, d_lrhead, d_lrhoff, d_u12off, d_lrhk, d_srow;
 };
 
+// Index programs of one network, packed into one device blob of 32-bit words
+// (offsets below in words).  "Sliced" lists hold work items in slices of 32
+// (one item per lane), items sorted by length inside a group and padded to
+// the slice's longest, entry e of lane l of slice s at 32 * (off[s] + e) + l,
+// so that a warp reads its index words in 128-byte lines.
+struct CellProg {
+  bool ok = false;               // false: the network is outside the programs' index ranges
+  int32_t nb = 0;                // 32-wide blocks of the dense tail
+  int32_t pitch = 0;             // rows of one tail column in shared memory (odd)
+  // right-hand side: rows of S in pieces; entry = reaction | sign << 31
+  // (coefficients of magnitude m appear m times, pads read slot n_r = 0)
+  int32_t n_rsl = 0, n_part = 0, n_rlong = 0;
+  int32_t rp_off = 0, rp_ent = 0, rp_dst = 0, row_ptr = 0, row_long = 0;
+  // Jacobian: entries by destination group (0 = head, 1 + J = 32-column panel
+  // J of the tail); entry word = derivative slot (2 * reaction + reactant
+  // slot) | sign << 31, pads read slot 2 n_r = 0.  Entries with more than
+  // kJLong words are gathered by a warp each.
+  int32_t n_jsl = 0, n_jl = 0;
+  int32_t jg_off = 0, jg_ent = 0, jg_rc = 0, jg_dst = 0, jg_grp = 0;
+  int32_t jl_ptr = 0, jl_ent = 0, jl_rc = 0, jl_dst = 0, jl_grp = 0;
+  // head program (see LUSymbolic): per op {dst | pivot << 16, first term};
+  // term = x | y << 16
+  int32_t hop = 0, hterm = 0, hop_ptr = 0;
+  // head's Schur complement on the tail: targets by panel; term = L21 index |
+  // U12 index << 16, pads read slot p_d = 0
+  int32_t n_tsl = 0;
+  int32_t tg_grp = 0, tg_off = 0, tg_ent = 0, tg_pos = 0;
+  // substitution: levels of the head rows, tail column of each U12 entry
+  int32_t lev_f = 0, lev_b = 0, u12c = 0;
+  // column sums of dn_j dR_j/dx_l (coupled temperature): reactant incidences
+  // in pieces like the right-hand side
+  int32_t n_vsl = 0, n_vpart = 0, n_vlong = 0;
+  int32_t vp_off = 0, vp_ent = 0, vp_dst = 0, vrow_ptr = 0, vrow_long = 0;
+  std::vector<int32_t> h;
+  DevArray blob;
+};
+
 struct sm_net {
   int device = 0;
   int32_t n_s = 0, n_r = 0, n_elem = 0;
@@ -138,6 +175,7 @@ struct sm_net {
   std::vector<int32_t> jp_ptr, jp_col, jt_ptr, jt_rx, jt_partner;
   std::vector<int8_t> jt_coef;
   LUSymbolic lu;
+  CellProg cell;
   // Device copies used by the kernels.
   DevArray d_reac;        // int2 per reaction: reactant indices (-1 = none)
   DevArray d_rate;        // RatePar per reaction: (log alpha | alpha, beta, gamma, class)

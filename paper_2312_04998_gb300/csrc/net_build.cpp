@@ -7,6 +7,7 @@
 #include <cmath>
 #include <numeric>
 
+#include "cell.h"
 #include "internal.h"
 
 namespace {
@@ -216,10 +217,9 @@ void build_lu_symbolic(sm_net& net) {
       if (g[v][u]) {
         g[v][u] = g[u][v] = 0;
       }
-    for (int32_t i = 0; i < n; ++i) {
-      if (!alive[i]) continue;
+    for (int32_t i : nb) {   // only v's neighbours change degree (dead nodes keep no edges)
       int32_t d = 0;
-      for (int32_t l = 0; l < n; ++l) d += alive[l] && g[i][l];
+      for (int32_t l = 0; l < n; ++l) d += g[i][l];
       degree[i] = d;
     }
   }
@@ -818,6 +818,8 @@ sm_status net_upload(sm_net* net) {
   if (!lu.blev.empty() && (st = lu.d_blev.upload(lu.blev.data(), lu.blev.size() * 4)) != SM_OK) return st;
   if ((st = lu.d_perm.upload(lu.perm.data(), lu.perm.size() * 4)) != SM_OK) return st;
   if ((st = lu.d_iperm.upload(lu.iperm.data(), lu.iperm.size() * 4)) != SM_OK) return st;
+  build_cell_prog(net, &net->cell);
+  if (net->cell.ok && (st = net->cell.blob.upload(net->cell.h.data(), net->cell.h.size() * 4)) != SM_OK) return st;
   int32_t zero = 0;
   if ((st = net->d_status.upload(&zero, 4)) != SM_OK) return st;
   return integ_format(net, SM_ORDER_NONE);
