@@ -26,6 +26,7 @@
 //                 while the diagonal block's 32-step chain runs
 #include "cell.h"
 #include <algorithm>
+#include <type_traits>
 
 #include "integ.h"
 
@@ -33,31 +34,36 @@ using namespace integ;
 
 namespace {
 
-constexpr int XP = 40;         // row pitch of the 32 x 32 exchange blocks (words): 16-byte rows, few conflicts
+constexpr int XP = 36;         // row pitch of the 32 x 32 exchange blocks (words): 16-byte rows, few conflicts
 constexpr unsigned kFull = 0xffffffffu;
 
 // A cell's scalars while a CTA works on it.
 struct CellS {
-  double t, h, gam, gam_J, crate, dprev, tnew, err, eta[3];
-  double tn[QMAX + 1], alpha[QMAX + 1], wts[QMAX + 1];
+  double t, h, gam, gam_J, crate, dprev, tnew, err, eta, inv_a0, scale;
+  double tn[QMAX + 1], alpha[QMAX + 1], wts[QMAX + 1], wlo[QMAX + 1];
   int q, nh, n_at_q, j_age, flags, crej, ccf, status, m_it, steps, rejects, conv_fails, newton_iters, jac_evals;
   int base;      // history point i is scratch slot (base + i) % (QMAX + 1)
-  int state, c, best_q;
-  int lo, hi;
+  int state, best_q;
+  int hn;                         // stride of a history point in scratch
+  long long c, oc;                // slot and cell
+  double *kc, *hist, *eprev, *pbuf;   // this CTA's global scratch: k', history ring, last error vector, piece sums
+  void *mbuf, *P;                 // Jacobian values in program order (scratch); the cell's packed factors
+  double nH, Av, chi;             // conditions (coupled temperature)
+  long long t0, ph_t;             // clocks of the timed class and the last phase mark
 };
-static_assert(sizeof(CellS) <= 512, "shared-memory plan");
+static_assert(sizeof(CellS) <= kCellScalars, "shared-memory plan");
 
 struct Args {
   Dev d;
   CellPlan p;
   const int* w;            // index programs (CellProg blob)
-  int nb, pitch;
-  int n_rsl, n_part, n_rlong, rp_off, rp_ent, rp_dst, row_ptr, row_long;
-  int n_jsl, n_jl, jg_off, jg_ent, jg_rc, jg_dst, jg_grp, jl_ptr, jl_ent, jl_rc, jl_dst, jl_grp;
+  int nb, pitch, n_slot, rx, iperm;
+  int n_rsl, rp_off, rp_ent, rp_dst, row, row_more;
+  int n_jsl, n_jl, jg_off, jg_ent, jg_rc, jg_dst, jg_grp, n_jp, n_jw, jp_ent, jl_ptr, jl_rc, jd_grp, jd_ent;
   int n_hlev, hop, hterm, hop_ptr;
-  int tg_grp, tg_off, tg_ent, tg_pos;
-  int lev_f, lev_b, u12c, n_l21, n_u12;
-  int n_vsl, n_vpart, n_vlong, vp_off, vp_ent, vp_dst, vrow_ptr, vrow_long;
+  int tg_grp, tg_ent;
+  int lev_f, lev_b, hx;
+  int n_vsl, vp_off, vp_ent, vp_dst, vrow, vrow_more;
   const double* k;
   int64_t ldk;
   double* scratch;
@@ -67,25 +73,32 @@ struct Args {
   int timing_kind;
 };
 
+static_assert(sizeof(Args) <= kCellArgs, "shared-memory plan");
+
+// The launch's arguments are copied to the front of the CTA's shared memory;
+// the phases are separate functions that take them and the vectors from there.
+// As one inlined body the kernel kept so many addresses alive that its inner
+// loops spilled, each spill a trip to L2 next to 230 KB of shared memory.
+extern __shared__ __align__(16) unsigned char sm[];
+__device__ __forceinline__ const Args& args() { return *reinterpret_cast<const Args*>(sm); }
+__device__ __forceinline__ CellS& scalars() { return *reinterpret_cast<CellS*>(sm + kCellArgs); }
+template <class V> __device__ __forceinline__ V* at(int offset) { return reinterpret_cast<V*>(sm + offset); }
+
 // optional cycle counters of the phases (build option SM_PHASE_CLOCKS)
 constexpr int kPhaseSlots = 16;
 enum { PH_LOAD, PH_PREDICT, PH_RATES, PH_GATHER, PH_SOLVE, PH_FINISH, PH_JAC, PH_HEAD, PH_ASSEMBLE, PH_UPDATE, PH_PANEL };
 #ifdef SM_PHASE_CLOCKS
 __device__ unsigned long long g_phase_cycles[kPhaseSlots];
-#define PHASE_MARK(k)                                                          \
-  do {                                                                         \
-    if (threadIdx.x == 0) {                                                    \
-      const long long ph_now = clock64();                                      \
-      atomicAdd(&g_phase_cycles[(k)], (unsigned long long)(ph_now - ph_t));    \
-      ph_t = ph_now;                                                           \
-    }                                                                          \
+#define PHASE_MARK(k)                                                                 \
+  do {                                                                                \
+    if (threadIdx.x == 0) {                                                           \
+      const long long ph_now = clock64();                                             \
+      atomicAdd(&g_phase_cycles[(k)], (unsigned long long)(ph_now - scalars().ph_t)); \
+      scalars().ph_t = ph_now;                                                        \
+    }                                                                                 \
   } while (0)
-#define PHASE_ARG , long long& ph_t
-#define PHASE_PASS , ph_t
 #else
 #define PHASE_MARK(k) do {} while (0)
-#define PHASE_ARG
-#define PHASE_PASS
 #endif
 
 // ---- packed FP32 arithmetic: two FMAs an instruction -----------------------
@@ -121,119 +134,168 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ void cp16(void* smem, const void* g) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(g) : "memory");
 }
+// The CTA's barrier, for code whose warps reach it from different places.
+__device__ __forceinline__ void cta_bar() { asm volatile("bar.sync 0;" ::: "memory"); }
+// A plain load that stays where it is written: left to itself the compiler
+// forms the addresses of a whole block of strided loads first, and spills.
+__device__ __forceinline__ float ld_here(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_here(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ __forceinline__ double flip(double v, int word) {   // v, negated when bit 31 of word is set
   return __hiloint2double(__double2hiint(v) ^ (word & 0x80000000), __double2loint(v));
 }
 
-// Sums of the rows cut into pieces: partial sums of the table's entries
-// (a piece per lane, two chains), then the pieces of each row in order (rows
-// of more than 4 pieces: a warp).  tab[pad slot] must be 0.  All threads.
-__device__ __forceinline__ void row_sums(const int* __restrict__ w, int n_sl, int off, int ent, int dst, int row_ptr,
-                                         int n_long, int row_long, const double* tab, double* part, double* out,
-                                         int n) {
+// Sums of rows cut into chains (see Chains in cell_prog.cpp): a chain per lane,
+// a slice of 32 chains per warp, longest first, so that the warps of each
+// scheduler keep its FP64 unit (a warp's FMA holds it for 64 cycles) busy.
+// tab[pad slot] must be 0.  All threads.
+__device__ __forceinline__ void row_sums(const int* __restrict__ w, int n_sl, int off, int ent, int dst, int row,
+                                         int more, const double* tab, double* part, double* out, int n) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int2* meta = reinterpret_cast<const int2*>(w + off);
+  int rw = (int)threadIdx.x < n ? __ldg(w + row + threadIdx.x) : 0;
+  int2 mt = warp < n_sl ? __ldg(meta + warp) : make_int2(0, 0);
   for (int s = warp; s < n_sl; s += nw) {
-    const int e0 = __ldg(w + off + s), e1 = __ldg(w + off + s + 1);
-    const int* q = w + ent + 32 * e0 + lane;
-    const int m = e1 - e0;
-    double a0 = 0.0, a1 = 0.0;
-    int e = 0;
-    for (; e + 4 <= m; e += 4) {
-      const int w0 = __ldg(q + 32 * e), w1 = __ldg(q + 32 * e + 32), w2 = __ldg(q + 32 * e + 64), w3 = __ldg(q + 32 * e + 96);
-      const double v0 = tab[w0 & 0x7FFFFFFF], v1 = tab[w1 & 0x7FFFFFFF], v2 = tab[w2 & 0x7FFFFFFF],
-                   v3 = tab[w3 & 0x7FFFFFFF];
-      a0 += flip(v0, w0);
-      a1 += flip(v1, w1);
-      a0 += flip(v2, w2);
-      a1 += flip(v3, w3);
+    const int* q = w + ent + 32 * mt.x + lane;
+    const int m = mt.y, to = __ldg(w + dst + 32 * s + lane);
+    int t[4], nx[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) t[u] = u < m ? __ldg(q + 32 * u) : 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) nx[u] = 4 + u < m ? __ldg(q + 32 * (4 + u)) : 0;
+    if (s + nw < n_sl) mt = __ldg(meta + s + nw);
+    double a = 0.0;
+    for (int e = 0; e < m; e += 4) {
+      int n2[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) n2[u] = e + 8 + u < m ? __ldg(q + 32 * (e + 8 + u)) : 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (e + u < m) a = fma(__hiloint2double(t[u] & 0xFFFF0000, 0), tab[t[u] & 0xFFFF], a);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        t[u] = nx[u];
+        nx[u] = n2[u];
+      }
     }
-    for (; e < m; ++e) {
-      const int w0 = __ldg(q + 32 * e);
-      a0 += flip(tab[w0 & 0x7FFFFFFF], w0);
-    }
-    part[__ldg(w + dst + 32 * s + lane)] = a0 + a1;
+    part[to] = a;
   }
   __syncthreads();
+  auto of = [&](int word) {
+    const double* p = part + (word & 0xFFFF);
+    return word < 0 ? (p[0] + p[1]) + (p[2] + p[3]) : p[0];
+  };
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int p0 = __ldg(w + row_ptr + i), p1 = __ldg(w + row_ptr + i + 1);
-    if (p1 - p0 > 4) continue;
-    double v = 0.0;
-    for (int p = p0; p < p1; ++p) v += part[p];
+    if (i >= (int)blockDim.x) rw = __ldg(w + row + i);
+    double v = of(rw);
+    const int x = (rw & 0x7FFFFFFF) >> 16;
+    if (x)
+      for (int q = x - 1;; ++q) {
+        const int word = __ldg(w + more + q);
+        v += of(word);
+        if (word & (1 << 30)) break;
+      }
     out[i] = v;
   }
-  for (int q = nw - 1 - warp; q < n_long; q += nw) {
-    const int i = __ldg(w + row_long + q);
-    const int p1 = __ldg(w + row_ptr + i + 1);
-    double v = 0.0;
-    for (int p = __ldg(w + row_ptr + i) + lane; p < p1; p += 32) v += part[p];
-    v = warp_sum(v);
-    if (lane == 0) out[i] = v;
+}
+
+// Sums over the CTA are formed as by 512 threads whatever the CTA's size, so
+// that a cell's result does not depend on the batch that it is part of: the
+// term of index i belongs to virtual thread i mod 512, each warp of those is
+// summed by shuffles, the warps in order.
+constexpr int kVirt = 512, RS = kVirt / 32;
+
+// Partial sums of f(i), i < n, into reduction slot `slot`; all threads.
+template <class F>
+__device__ __forceinline__ void sum_parts(int slot, int n, F f) {
+  double* red = at<double>(kCellRed) + RS * slot;
+  const int top = min(kVirt, (n + 31) / 32 * 32);
+  for (int v = threadIdx.x; v < top; v += blockDim.x) {
+    double a = 0.0;
+    for (int i = v; i < n; i += kVirt) a += f(i);
+    a = warp_sum(a);
+    if ((v & 31) == 0) red[v >> 5] = a;
   }
 }
-
-// Sum over the CTA, valid in warp 0 (all threads must call; one barrier
-// inside; `slot` 0..3 keeps independent sums apart).
-__device__ __forceinline__ double cta_sum(double v, double* red, int slot) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  v = warp_sum(v);
-  if (lane == 0) red[32 * slot + warp] = v;
-  __syncthreads();
-  if (warp == 0) v = warp_sum(lane < nw ? red[32 * slot + lane] : 0.0);
-  return v;
+// Their sum, by one warp after a barrier; the result in every lane.
+__device__ __forceinline__ double sum_total(int slot, int n) {
+  const int lane = threadIdx.x & 31, parts = min(RS, (n + 31) / 32);
+  return warp_sum(lane < parts ? at<double>(kCellRed)[RS * slot + lane] : 0.0);
 }
 
-// R_j = k'_j prod y into tab (slot n_r = 0), then fs = S R.  Ends with a barrier.
-__device__ void cell_rhs(const Args& A, const double* kc, const double* y, double* tab, double* part, double* fs PHASE_ARG) {
+// R_j = k'_j prod y (slot n_r of the table = 0), then fs = S R at state y.
+// Ends with a barrier.
+__device__ __forceinline__ void cell_rhs() {
+  const Args& A = args();
   const int n_r = A.d.n_r;
+  const int2* rx = reinterpret_cast<const int2*>(A.w + A.rx);
+  const double* kc = scalars().kc;
+  const double* y = at<double>(A.p.o_ys);
+  double* tab = at<double>(A.p.o_r);
+#pragma unroll 4
   for (int j = threadIdx.x; j < n_r; j += blockDim.x) {
-    const int2 rc = __ldg(A.d.reac + j);
-    double v = kc[j] * y[rc.x];
-    if (rc.y >= 0) v *= y[rc.y];
+    const int ab = __ldg(rx + j).x;
+    double v = kc[j] * y[ab & 0xFFFF];
+    const int b = (uint32_t)ab >> 16;
+    if (b != 0xFFFF) v *= y[b];
     tab[j] = v;
   }
   if (threadIdx.x == 0) tab[n_r] = 0.0;
   __syncthreads();
   PHASE_MARK(PH_RATES);
-  row_sums(A.w, A.n_rsl, A.rp_off, A.rp_ent, A.rp_dst, A.row_ptr, A.n_rlong, A.row_long, tab, part, fs, A.d.n);
+  row_sums(A.w, A.n_rsl, A.rp_off, A.rp_ent, A.rp_dst, A.row, A.row_more, tab, at<double>(A.p.o_part),
+           at<double>(A.p.o_fs), A.d.n);
   __syncthreads();
   PHASE_MARK(PH_GATHER);
 }
 
 // ---- coupled temperature ----------------------------------------------------
 // k' of the T-dependent reactions (all reactions when init) at temperature T.
-__device__ void cell_th_rates(const Args& A, double* kc, double T, double nH, double Av, double chi, bool init) {
-  const double lt = log(T * (1.0 / 300.0)), it = 1.0 / T;
+__device__ __forceinline__ void cell_th_rates(double T, bool init) {
+  const Args& A = args();
+  const CellS& S = scalars();
+  double* kc = S.kc;
+  const double nH = S.nH, lt = log(T * (1.0 / 300.0)), it = 1.0 / T;
+  const RatePar* par = A.d.rpar;
   for (int j = threadIdx.x; j < A.d.n_r; j += blockDim.x) {
-    const RatePar p = A.d.rpar[j];
+    const RatePar p = par[j];
     const int cls = (int)p.w;
     if (cls == SM_TWO_BODY || cls == SM_DISS_RECOMB) kc[j] = exp(fma(p.y, lt, p.x) - p.z * it) * nH;
-    else if (init) kc[j] = cls == SM_COSMIC_RAY ? p.x * A.d.th_zeta : chi * p.x * exp(-p.z * Av);
+    else if (init) kc[j] = cls == SM_COSMIC_RAY ? p.x * A.d.th_zeta : S.chi * p.x * exp(-p.z * S.Av);
   }
   __syncthreads();
 }
 
 // Temperature row of fs from y and the chemical rows.  Ends with a barrier.
-__device__ void cell_energy(const Args& A, const double* y, double* fs, double nH, double* red) {
+__device__ __forceinline__ void cell_energy() {
+  const Args& A = args();
   const Dev& d = A.d;
+  const double* y = at<double>(A.p.o_ys);
+  double* fs = at<double>(A.p.o_fs);
   const int t = d.t_idx;
-  const double T = y[t];
-  double xt = 0.0, F = 0.0, line = 0.0;
-  for (int s = threadIdx.x; s < d.n; s += blockDim.x) {
-    if (s == t) continue;
-    xt += y[s];
-    F += fs[s];
-  }
-  for (int q = threadIdx.x; q < d.n_cool; q += blockDim.x) {
+  const double T = y[t], nH = scalars().nH;
+  const int n = d.n;
+  sum_parts(0, n, [&](int i) { return i == t ? 0.0 : y[i]; });
+  sum_parts(1, n, [&](int i) { return i == t ? 0.0 : fs[i]; });
+  sum_parts(2, d.n_cool, [&](int q) {
     const int i = __ldg(d.th_cool + q);
-    line = fma(y[i], d.th_L[i] * exp(-d.th_E[i] / T), line);
+    return y[i] * (d.th_L[i] * exp(-d.th_E[i] / T));
+  });
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double xt = sum_total(0, n), F = sum_total(1, n), line = sum_total(2, d.n_cool);
+    if (threadIdx.x == 0)
+      fs[t] = (d.th_heat - nH * line - d.th_lam * nH * (T - d.th_Td) - 1.5 * T * F) / (1.5 * xt);
   }
-  xt = cta_sum(xt, red, 0);
-  F = cta_sum(F, red, 1);
-  line = cta_sum(line, red, 2);
-  if (threadIdx.x == 0)
-    fs[t] = (d.th_heat - nH * line - d.th_lam * nH * (T - d.th_Td) - 1.5 * T * F) / (1.5 * xt);
   __syncthreads();
 }
 
@@ -246,202 +308,207 @@ __device__ __forceinline__ void load4(const double* p, double (&v)[4]) {
   const double2 q = *reinterpret_cast<const double2*>(p), r = *reinterpret_cast<const double2*>(p + 2);
   v[0] = q.x; v[1] = q.y; v[2] = r.x; v[3] = r.y;
 }
+__device__ __forceinline__ void store4(float* p, const float (&v)[4]) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store4(double* p, const double (&v)[4]) {
+  *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+  *reinterpret_cast<double2*>(p + 2) = make_double2(v[2], v[3]);
+}
 
-// x := M^-1 x with a cell's packed factors P; x in elimination order, head
-// part xh[h], tail part xt (16-byte aligned, 32 nb entries).  tmp holds the
-// products of the L21 / U12 entries, which all threads form at once (their
-// rows have up to a hundred entries, a chain no single thread should walk).
+// Before a substitution, asynchronously into shared memory: the head's packed
+// factors (hd) and the tail's diagonal blocks (dg: [nb][32 columns][32 rows]),
+// which the dependent chains read.
+template <class T>
+__device__ __forceinline__ void solve_prefetch() {
+  constexpr int PER = 16 / sizeof(T), CPC = 32 / PER;
+  const Args& A = args();
+  const Dev& d = A.d;
+  const T* P = static_cast<const T*>(scalars().P);
+  T* hd = at<T>(A.p.o_hd);
+  T* dg = at<T>(A.p.o_dg);
+  const int nt = d.n - d.head, p_d = d.p_d, nthr = blockDim.x;
+  const int64_t ldd = d.ldd;
+  for (int e = threadIdx.x * PER; e < p_d; e += nthr * PER) cp16(hd + e, P + e);
+  for (int q = threadIdx.x; q < nt * CPC; q += nthr) {   // q: (column, chunk of its block's rows)
+    const int c = q / CPC, i = q % CPC * PER;
+    cp16(dg + c * 32 + i, P + p_d + c * ldd + (c & ~31) + i);
+  }
+}
+
+// Diagonal blocks (a row per lane), column by column: one shuffle and one FMA
+// a step, the factors' loads ahead of the chain.
+template <class T>
+__device__ __forceinline__ T diag_forward(T xi, const T* dg, int lane, int w) {
+#pragma unroll 8
+  for (int k = 0; k < 32; ++k) {
+    const T l = lane > k ? dg[k * 32 + lane] : T(0);
+    const T xk = __shfl_sync(kFull, xi, k);
+    if (k < w) xi -= l * xk;   // (past w: padding)
+  }
+  return xi;
+}
+template <class T>
+__device__ __forceinline__ T diag_backward(T xi, const T* dg, int lane, int w) {
+#pragma unroll 8
+  for (int k = 31; k >= 0; --k) {
+    const T u = lane <= k ? dg[k * 32 + lane] : T(0);
+    const T t = xi * u;   // the solved entry in lane k (inverse pivots)
+    const T xk = __shfl_sync(kFull, t, k);
+    if (k < w) xi = lane == k ? t : (lane < k ? xi - u * xk : xi);   // (past w: padding)
+  }
+  return xi;
+}
+
+// One row block of the tail in a warp's registers: its entry per lane and the
+// 32 columns in flight.
+template <class T>
+struct RowBlock {
+  T x, ln[32];
+  // From the first of w columns at p; with fewer than 32 the last one again,
+  // for entries of x that are 0.  (Rows past the tail's end are padding: their
+  // lanes compute on it and are not read.)
+  __device__ __forceinline__ void load(const T* p, int64_t ldd, int w) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      ln[k] = ld_here(p);
+      if (k + 1 < w) p += ldd;
+    }
+  }
+  __device__ __forceinline__ void apply(const T* xk) {
+    T a = T(0);
+#pragma unroll
+    for (int k = 0; k < 32; k += 4) {
+      T v[4];
+      load4(xk + k, v);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a += ln[k + u] * v[u];
+    }
+    x -= a;
+  }
+};
+
+// x := M^-1 x with the cell's packed factors; x in elimination order, head part
+// xh[h], tail part xt (16-byte aligned, 32 nb entries), after solve_prefetch.
+// In the tail warp i carries row block i,
+// its next 32 columns in flight; as soon as a block's columns are applied its
+// warp solves the next diagonal block.  (Row blocks past the CTA's warps are
+// worked on in place, by warp i mod nw, without loads ahead.)
 // Begins and ends with a barrier.
 template <class T>
-__device__ void cell_solve(const Args& A, const T* P, T* xh, T* xt, T* tmp) {
-  constexpr int CH = sizeof(T) == 4 ? 32 : 16;   // columns of a block in registers at a time
+__device__ __forceinline__ void cell_solve() {
+  const Args& A = args();
   const Dev& d = A.d;
-  const int n = d.n, h = d.head, nt = n - h, ldd = d.ldd, nb = A.nb;
-  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, rb = tid >> 5;
-  const T* D = P + d.p_d;
-  const int row = 32 * rb + lane;
+  T* xh = at<T>(A.p.o_xh);
+  T* xt = at<T>(A.p.o_xt);
+  T* hd = at<T>(A.p.o_hd);
+  const T* dg = at<T>(A.p.o_dg);
+  const int n = d.n, h = d.head, nt = n - h, nb = A.nb;
+  const int64_t ldd = d.ldd;
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, nw = nthr >> 5;
+  const int ra = tid >> 5;   // this warp's row block
+  const T* D = static_cast<const T*>(scalars().P) + d.p_d;
+  const bool ina = 32 * ra + lane < nt;
+  RowBlock<T> a;
+  if (ra > 0 && ra < nb) a.load(D + 32 * ra + lane, ldd, 32);
+  cp_wait();
   __syncthreads();
-  // head, forward: a row per thread, level by level, its entries loaded ahead
-  constexpr int HE = 4;
+  // a row of head factors against x: entries [e0, e1) of the packed head, hx
+  // their index in x
+  const uint16_t* hx = at<uint16_t>(A.p.o_hx);
+  auto row_dot = [&](int e0, int e1, const T* x) {
+    T v = T(0);
+#pragma unroll 4
+    for (int e = e0; e < e1; ++e) v += hd[e] * x[hx[e]];
+    return v;
+  };
+  // head, forward: a row per thread, level by level
   for (int i0 = 0; i0 < h; i0 += nthr) {   // one pass unless the head outgrows the CTA (rows of a pass come first)
     const int i = i0 + tid;
-    const bool in = i < h;
-    const int p0 = in ? __ldg(d.lrptr + i) : 0, cnt = in ? __ldg(d.lrptr + i + 1) - p0 : 0;
-    const int lev = in ? __ldg(A.w + A.lev_f + i) : -1;
-    T pv[HE];
-    int pi[HE];
-#pragma unroll
-    for (int e = 0; e < HE; ++e) {
-      pv[e] = e < cnt ? P[d.p_l11 + p0 + e] : T(0);
-      pi[e] = e < cnt ? __ldg(d.lridx + p0 + e) : 0;
-    }
+    const bool inh = i < h;
+    const int p0 = inh ? __ldg(d.lrptr + i) : 0, p1 = inh ? __ldg(d.lrptr + i + 1) : 0;
+    const int lev = inh ? __ldg(A.w + A.lev_f + i) : -1;
     for (int l = i0 == 0 ? 1 : 0; l < d.n_flev; ++l) {
-      if (lev == l) {
-        T s = T(0);
-#pragma unroll
-        for (int e = 0; e < HE; ++e) s += pv[e] * xh[pi[e]];
-        for (int e = HE; e < cnt; ++e) s += P[d.p_l11 + p0 + e] * xh[__ldg(d.lridx + p0 + e)];
-        xh[i] -= s;
-      }
+      if (lev == l) xh[i] -= row_dot(d.p_l11 + p0, d.p_l11 + p1, xh);
       __syncthreads();
     }
   }
-  // L21
-#pragma unroll 4
-  for (int e = tid; e < A.n_l21; e += nthr) tmp[e] = P[d.p_l21 + e] * xh[__ldg(d.lrhk + e)];
-  __syncthreads();
-  T xi = T(0);
-  if (row < nt) {
-    const int e1 = __ldg(d.lrhoff + row + 1);
-    T s0 = T(0), s1 = T(0);
-    int e = __ldg(d.lrhoff + row);
-    for (; e + 4 <= e1; e += 4) {
-      s0 += tmp[e];
-      s1 += tmp[e + 1];
-      s0 += tmp[e + 2];
-      s1 += tmp[e + 3];
-    }
-    for (; e < e1; ++e) s0 += tmp[e];
-    xi = xt[row] - (s0 + s1);
-  }
+  if (h == 0) __syncthreads();
+  auto l21_row = [&](int row) {
+    return xt[row] - row_dot(d.p_l21 + __ldg(d.lrhoff + row), d.p_l21 + __ldg(d.lrhoff + row + 1), xh);
+  };
+  a.x = ina ? l21_row(32 * ra + lane) : T(0);
+  for (int r = ra + nw; r < nb; r += nw)
+    if (32 * r + lane < nt) xt[32 * r + lane] = l21_row(32 * r + lane);
+  // block column K applied to row block r in place
+  auto far = [&](int r, int K, int w) {
+    const T* p = D + (32 * K) * ldd + 32 * r + lane;
+    T v = T(0);
+#pragma unroll 8
+    for (int k = 0; k < w; ++k) v += p[k * ldd] * xt[32 * K + k];
+    if (32 * r + lane < nt) xt[32 * r + lane] -= v;
+  };
+  auto far_solve = [&](int r, bool forward) {
+    const int w = min(32, nt - 32 * r);
+    const T v = xt[32 * r + lane];
+    const T x = forward ? diag_forward(v, dg + r * 1024, lane, w) : diag_backward(v, dg + r * 1024, lane, w);
+    xt[32 * r + lane] = lane < w ? x : T(0);
+  };
   // tail, forward (unit lower triangle)
-  for (int K = 0; K < nb; ++K) {
-    const int w = min(32, nt - 32 * K);
-    const T* col = D + (int64_t)(32 * K) * ldd + row;
-    T l[CH];
-    const bool use = rb >= K && row < nt;
-#pragma unroll
-    for (int k = 0; k < CH; ++k) l[k] = use && k < w && (rb > K || k < lane) ? col[(int64_t)k * ldd] : T(0);
-    if (rb == K) {
-#pragma unroll
-      for (int k0 = 0; k0 < 32; k0 += CH) {
-        if (k0) {
-#pragma unroll
-          for (int k = 0; k < CH; ++k) l[k] = use && k0 + k < w && k0 + k < lane ? col[(int64_t)(k0 + k) * ldd] : T(0);
-        }
-#pragma unroll
-        for (int k = 0; k < CH; ++k) {
-          const T xk = __shfl_sync(kFull, xi, k0 + k);
-          xi -= l[k] * xk;   // l is 0 on and above the diagonal
-        }
+  for (int K = -1; K < nb - 1; ++K) {
+    if (K >= 0) {
+      __syncthreads();
+      if (K < ra && ra < nb) {
+        a.apply(xt + 32 * K);
+        if (K + 1 < ra) a.load(D + (32 * (K + 1)) * ldd + 32 * ra + lane, ldd, 32);
       }
-      xt[row] = row < nt ? xi : T(0);
+      for (int r = ra + nw; r < nb; r += nw)
+        if (r > K) far(r, K, 32);
     }
-    __syncthreads();
-    if (rb > K && rb < nb) {
-#pragma unroll
-      for (int k0 = 0; k0 < 32; k0 += CH) {
-        if (k0) {
-#pragma unroll
-          for (int k = 0; k < CH; ++k) l[k] = use ? col[(int64_t)(k0 + k) * ldd] : T(0);
-        }
-        T a0 = T(0), a1 = T(0);
-#pragma unroll
-        for (int k = 0; k < CH; k += 4) {
-          T xv[4];
-          load4(xt + 32 * K + k0 + k, xv);
-          a0 += l[k] * xv[0];
-          a1 += l[k + 1] * xv[1];
-          a0 += l[k + 2] * xv[2];
-          a1 += l[k + 3] * xv[3];
-        }
-        xi -= a0 + a1;
-      }
+    if (K + 1 == ra) {
+      a.x = diag_forward(a.x, dg + ra * 1024, lane, min(32, nt - 32 * ra));
+      xt[32 * ra + lane] = ina ? a.x : T(0);
+    } else if (K + 1 >= nw && (K + 1) % nw == ra) {
+      __syncwarp();
+      far_solve(K + 1, true);
     }
   }
-  // tail, backward (inverse pivots on the diagonal)
-  for (int K = nb - 1; K >= 0; --K) {
-    const int w = min(32, nt - 32 * K);
-    const T* col = D + (int64_t)(32 * K) * ldd + row;
-    T l[CH];
-    const bool use = rb <= K && row < nt;
-    constexpr int kTop = 32 - CH;
-#pragma unroll
-    for (int k = 0; k < CH; ++k)
-      l[k] = use && kTop + k < w && (rb < K || kTop + k >= lane) ? col[(int64_t)(kTop + k) * ldd] : T(0);
-    if (rb == K) {
-#pragma unroll
-      for (int k0 = kTop; k0 >= 0; k0 -= CH) {
-        if (k0 != kTop) {
-#pragma unroll
-          for (int k = 0; k < CH; ++k) l[k] = use && k0 + k < w && k0 + k >= lane ? col[(int64_t)(k0 + k) * ldd] : T(0);
-        }
-#pragma unroll
-        for (int k = CH - 1; k >= 0; --k) {
-          if (lane == k0 + k) xi *= l[k];
-          const T xk = __shfl_sync(kFull, xi, k0 + k);
-          if (lane < k0 + k) xi -= l[k] * xk;
-        }
-      }
-      xt[row] = row < nt ? xi : T(0);
-    }
-    __syncthreads();
-    if (rb < K) {
-#pragma unroll
-      for (int k0 = kTop; k0 >= 0; k0 -= CH) {
-        if (k0 != kTop) {
-#pragma unroll
-          for (int k = 0; k < CH; ++k) l[k] = use && k0 + k < w ? col[(int64_t)(k0 + k) * ldd] : T(0);
-        }
-        T a0 = T(0), a1 = T(0);
-#pragma unroll
-        for (int k = 0; k < CH; k += 4) {
-          T xv[4];
-          load4(xt + 32 * K + k0 + k, xv);
-          a0 += l[k] * xv[0];
-          a1 += l[k + 1] * xv[1];
-          a0 += l[k + 2] * xv[2];
-          a1 += l[k + 3] * xv[3];
-        }
-        xi -= a0 + a1;
-      }
-    }
-  }
-  // U12, then the head backward
-#pragma unroll 4
-  for (int e = tid; e < A.n_u12; e += nthr) tmp[e] = P[d.p_u12 + e] * xt[__ldg(A.w + A.u12c + e)];
   __syncthreads();
+  // tail, backward (inverse pivots on the diagonal)
+  auto col = [&](int K) { return D + (32 * K) * ldd + 32 * ra + lane; };
+  if (ra < nb - 1) a.load(col(nb - 1), ldd, nt - 32 * (nb - 1));
+  for (int K = nb; K > 0; --K) {
+    if (K < nb) {
+      __syncthreads();
+      if (K > ra) {
+        a.apply(xt + 32 * K);
+        if (K - 1 > ra) a.load(col(K - 1), ldd, 32);
+      }
+      for (int r = ra + nw; r < K; r += nw) far(r, K, min(32, nt - 32 * K));
+    }
+    if (K - 1 == ra) {
+      a.x = diag_backward(a.x, dg + ra * 1024, lane, min(32, nt - 32 * ra));
+      xt[32 * ra + lane] = ina ? a.x : T(0);
+    } else if (K - 1 >= nw && (K - 1) % nw == ra) {
+      __syncwarp();
+      far_solve(K - 1, false);
+    }
+  }
+  __syncthreads();
+  // U12, then the head backward
   for (int i0 = h > 0 ? (h - 1) / nthr * nthr : -1; i0 >= 0; i0 -= nthr) {
     const int i = i0 + tid;
-    const bool in = i < h;
+    const bool inh = i < h;
     T xv = T(0);
-    int p0 = 0, cnt = 0, u0 = 0, lev = -1;
-    T pv[HE], dinv = T(0);
-    int pi[HE];
-    if (in) {
-      p0 = __ldg(d.u11ptr + i);
-      cnt = __ldg(d.u11ptr + i + 1) - p0;
-      u0 = __ldg(d.uptr + i);
+    int e0 = 0, e1 = 0, lev = -1;
+    if (inh) {
+      e0 = d.p_u11 + __ldg(d.u11ptr + i);
+      e1 = d.p_u11 + __ldg(d.u11ptr + i + 1);
       lev = __ldg(A.w + A.lev_b + i);
-      dinv = P[d.p_dinv + i];
-    }
-#pragma unroll
-    for (int e = 0; e < HE; ++e) {
-      pv[e] = e < cnt ? P[d.p_u11 + p0 + e] : T(0);
-      pi[e] = e < cnt ? __ldg(d.uidx + u0 + e) : 0;
-    }
-    if (in) {
-      const int e1 = __ldg(d.u12off + i + 1);
-      T s0 = T(0), s1 = T(0);
-      int e = __ldg(d.u12off + i);
-      for (; e + 4 <= e1; e += 4) {
-        s0 += tmp[e];
-        s1 += tmp[e + 1];
-        s0 += tmp[e + 2];
-        s1 += tmp[e + 3];
-      }
-      for (; e < e1; ++e) s0 += tmp[e];
-      xv = xh[i] - (s0 + s1);
+      xv = xh[i] - row_dot(d.p_u12 + __ldg(d.u12off + i), d.p_u12 + __ldg(d.u12off + i + 1), xt);
     }
     for (int l = 0; l < d.n_blev; ++l) {
-      if (lev == l) {
-        T s = T(0);
-#pragma unroll
-        for (int e = 0; e < HE; ++e)
-          if (e < cnt) s += pv[e] * xh[pi[e]];
-        for (int e = HE; e < cnt; ++e) s += P[d.p_u11 + p0 + e] * xh[__ldg(d.uidx + u0 + e)];
-        xh[i] = (xv - s) * dinv;
-      }
+      if (lev == l) xh[i] = (xv - row_dot(e0, e1, xh)) * hd[d.p_dinv + i];
       __syncthreads();
     }
   }
@@ -449,573 +516,695 @@ __device__ void cell_solve(const Args& A, const T* P, T* xh, T* xt, T* tmp) {
 }
 
 // ---- factorisation ----------------------------------------------------------
-// Triangular solve of a 32-column block row of the panel: the 32 x 32 block X
-// (rows in xk, pitch XP) becomes L_KK^-1 X, L_KK unit lower in ld[k][i].
-// One lane per column; pairs of rows share one packed FMA.
-__device__ __forceinline__ void trsm_block(float* xk, const float* ld, int lane) {
-  f2 x[16];
+// The triangular kernels of 32 x 32 blocks hold one row (or column) of 32
+// entries per lane and run eight of them at a time in rolled loops, the
+// remaining ones rotated to the front of the register array: unrolled over all
+// 32 each would be straight-line code executed once per panel.  `more(g)`
+// says whether the entries 8 g .. 8 g + 7 past the current eight exist.
+
+// LU of the diagonal block in uj (by rows, pitch XP), a row per lane, pivot rows
+// by shuffles: U and the inverse pivots back to uj, L by columns into
+// lj[k][i]; the first w columns to D (dst: this lane's row).
+template <class T>
+__device__ __forceinline__ void lu_block(T* uj, T* lj, T* dst, int64_t ldd, int w, int lane) {
+  T c[32];   // row `lane` of the block (in uj); the identity past w
 #pragma unroll
-  for (int p = 0; p < 16; ++p) x[p] = pack2(xk[(2 * p) * XP + lane], xk[(2 * p + 1) * XP + lane]);
+  for (int j = 0; j < 32; ++j) c[j] = j == lane ? T(1) : T(0);
+  if (lane < w) {
 #pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    float a, b;
-    unpack2(x[k / 2], a, b);
-    const float v = -((k & 1) ? b : a);
-    if (!(k & 1)) {
-      b = fmaf(ld[k * 32 + k + 1], v, b);
-      x[k / 2] = pack2(a, b);
+    for (int j = 0; j < 32; ++j)
+      if (j < w) c[j] = uj[lane * XP + j];
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int b0 = 0; b0 < 32; b0 += 8) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const T inv = T(1) / __shfl_sync(kFull, c[k], b0 + k);
+      const T l = lane > b0 + k ? c[k] * inv : T(0);
+#pragma unroll
+      for (int j = k + 1; j < 8; ++j) c[j] -= l * __shfl_sync(kFull, c[j], b0 + k);
+#pragma unroll
+      for (int g = 8; g < 32; g += 8)
+        if (b0 + g < 32) {
+#pragma unroll
+          for (int j = g; j < g + 8; ++j) c[j] -= l * __shfl_sync(kFull, c[j], b0 + k);
+        }
+      if (lane > b0 + k) c[k] = l;
+      if (lane == b0 + k) c[k] = inv;
     }
-    const f2 vv = pack2(v, v);
 #pragma unroll
-    for (int p = k / 2 + 1; p < 16; ++p) {
-      const f2 l = *reinterpret_cast<const f2*>(ld + k * 32 + 2 * p);
-      x[p] = fma2(l, vv, x[p]);
+    for (int k = 0; k < 8; ++k) {
+      uj[lane * XP + b0 + k] = c[k];
+      lj[(b0 + k) * 32 + lane] = c[k];
+      if (lane < w && b0 + k < w) dst[(b0 + k) * ldd] = c[k];
     }
+#pragma unroll
+    for (int j = 0; j < 24; ++j) c[j] = c[j + 8];
   }
-#pragma unroll
-  for (int p = 0; p < 16; ++p) {
-    float a, b;
-    unpack2(x[p], a, b);
-    xk[(2 * p) * XP + lane] = a;
-    xk[(2 * p + 1) * XP + lane] = b;
-  }
-}
-// FP64: 16 columns (c0 ..); lanes 0-15 carry rows 0-15 of a column, lanes
-// 16-31 rows 16-31, so every FP64 instruction works for all 32 lanes.
-__device__ __forceinline__ void trsm_block16(double* xk, const double* ld, int c0, int lane) {
-  const int half = lane >> 4, c = c0 + (lane & 15);
-  double x[16];
-#pragma unroll
-  for (int r = 0; r < 16; ++r) x[r] = xk[(16 * half + r) * XP + c];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const double v = __shfl_sync(kFull, x[k], lane & 15);
-#pragma unroll
-    for (int r = 0; r < 16; ++r)
-      if (half || r > k) x[r] = fma(-ld[k * 32 + 16 * half + r], v, x[r]);
-  }
-  if (half) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k)
-#pragma unroll
-      for (int r = k + 1; r < 16; ++r) x[r] = fma(-ld[(16 + k) * 32 + 16 + r], x[k], x[r]);
-  }
-#pragma unroll
-  for (int r = 0; r < 16; ++r) xk[(16 * half + r) * XP + c] = x[r];
 }
 
-// The head's factors in shared memory (Hv), by dependency levels.
+// c := c U^-1 for a row c (U by rows at tri, inverse pivots on its diagonal),
+// or c := L^-1 c for a column c (UNIT; L by columns at tri); pitch TP.  out(i,
+// v): entry i's eight results from i on.
+template <class T, bool UNIT, int TP, class Out>
+__device__ __forceinline__ void tri_solve(T (&c)[32], const T* tri, Out out) {
+#pragma unroll 1
+  for (int b0 = 0; b0 < 32; b0 += 8) {
+    const T* t = tri + b0 * TP + b0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      T r[8];
+#pragma unroll
+      for (int g = 0; g < 8; g += 4) {
+        T q[4];
+        load4(t + k * TP + g, q);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) r[g + u] = q[u];
+      }
+      if (!UNIT) c[k] *= r[k];
+#pragma unroll
+      for (int j = k + 1; j < 8; ++j) c[j] -= c[k] * r[j];
+#pragma unroll
+      for (int g = 8; g < 32; g += 4)
+        if (b0 + g < 32) {
+          T q[4];
+          load4(t + k * TP + g, q);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) c[g + u] -= c[k] * q[u];
+        }
+    }
+    out(b0, c);
+#pragma unroll
+    for (int j = 0; j < 24; ++j) c[j] = c[j + 8];
+  }
+}
+
+// 32 x 32 blocks of the trailing update in a warp's registers as 4 x 8 tiles:
+// lane (ty, tx) = (lane / 4, lane % 4) has rows 4 ty .. 4 ty + 3 and columns
+// 8 tx .. 8 tx + 7.  A column of the left operand and a row of the right one
+// then cost three 16-byte shared-memory reads per 32 FP32 FMAs (a row per lane
+// needs eight, which bound the update at half the FMA rate); FP32 FMAs in
+// pairs.  mul: C -= L X with L [k][LP] and X [k][UP].
+template <class T, bool TF> struct Tile;
+
+template <> struct Tile<float, false> {
+  static constexpr int LP = 32, UP = 32, CW = 32;   // pitches, columns
+  f2 x[4][4];
+  __device__ __forceinline__ void load(const float* D, int64_t ldd, int cols, int lane) {   // D: the block's corner
+    const float* p = D + (8 * (lane & 3)) * ldd + 4 * (lane >> 2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float a[4] = {0.f, 0.f, 0.f, 0.f}, b[4] = {0.f, 0.f, 0.f, 0.f};
+      if (8 * (lane & 3) + 2 * q < cols) load4(p + (2 * q) * ldd, a);
+      if (8 * (lane & 3) + 2 * q + 1 < cols) load4(p + (2 * q + 1) * ldd, b);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i][q] = pack2(a[i], b[i]);
+    }
+  }
+  __device__ __forceinline__ void store(float* D, int64_t ldd, int cols, int lane) const {
+    float* p = D + (8 * (lane & 3)) * ldd + 4 * (lane >> 2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) unpack2(x[i][q], a[i], b[i]);
+      if (8 * (lane & 3) + 2 * q < cols) store4(p + (2 * q) * ldd, a);
+      if (8 * (lane & 3) + 2 * q + 1 < cols) store4(p + (2 * q + 1) * ldd, b);
+    }
+  }
+  __device__ __forceinline__ void to_rows(float* X, int lane) const {   // row-major, pitch XP
+    float* p = X + 4 * (lane >> 2) * XP + 8 * (lane & 3);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      *reinterpret_cast<ulonglong2*>(p + i * XP) = make_ulonglong2(x[i][0], x[i][1]);
+      *reinterpret_cast<ulonglong2*>(p + i * XP + 4) = make_ulonglong2(x[i][2], x[i][3]);
+    }
+  }
+  __device__ __forceinline__ void mul(const float* L, const float* X, int lane) {
+    const float* lp = L + 4 * (lane >> 2);
+    const float* xp = X + 8 * (lane & 3);
+#pragma unroll 4
+    for (int k = 0; k < 32; ++k) {
+      float l[4];
+      load4(lp + LP * k, l);
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(xp + UP * k);
+      const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(xp + UP * k + 4);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const f2 a = pack2(-l[i], -l[i]);
+        x[i][0] = fma2(a, v.x, x[i][0]);
+        x[i][1] = fma2(a, v.y, x[i][1]);
+        x[i][2] = fma2(a, u.x, x[i][2]);
+        x[i][3] = fma2(a, u.y, x[i][3]);
+      }
+    }
+  }
+};
+
+// FP64: half a block, 32 x 16, as 4 x 4 tiles.
+template <> struct Tile<double, false> {
+  static constexpr int LP = 32, UP = 32, CW = 16;
+  double x[4][4];
+  __device__ __forceinline__ void load(const double* D, int64_t ldd, int cols, int lane) {
+    const double* p = D + (4 * (lane & 3)) * ldd + 4 * (lane >> 2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+      if (4 * (lane & 3) + q < cols) load4(p + q * ldd, a);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i][q] = a[i];
+    }
+  }
+  __device__ __forceinline__ void store(double* D, int64_t ldd, int cols, int lane) const {
+    double* p = D + (4 * (lane & 3)) * ldd + 4 * (lane >> 2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double a[4] = {x[0][q], x[1][q], x[2][q], x[3][q]};
+      if (4 * (lane & 3) + q < cols) store4(p + q * ldd, a);
+    }
+  }
+  __device__ __forceinline__ void to_rows(double* X, int lane) const {
+    double* p = X + 4 * (lane >> 2) * XP + 4 * (lane & 3);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) store4(p + i * XP, x[i]);
+  }
+  __device__ __forceinline__ void mul(const double* L, const double* X, int lane) {
+    const double* lp = L + 4 * (lane >> 2);
+    const double* xp = X + 4 * (lane & 3);
+#pragma unroll 4
+    for (int k = 0; k < 32; ++k) {
+      double l[4], v[4];
+      load4(lp + LP * k, l);
+      load4(xp + UP * k, v);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[i][q] = fma(-l[i], v[q], x[i][q]);
+    }
+  }
+};
+
+// The same block as mma.m16n8k8 fragments: each operand x = hi + lo with hi =
+// tf32(x), lo = tf32(x - hi), products hi hi + hi lo + lo hi, FP32 sums.
+template <> struct Tile<float, true> {
+  static constexpr int LP = 36, UP = 36, CW = 32;   // (fragment reads of four rows at a time)
+  float c[2][4][4];
+  template <class F> __device__ __forceinline__ void each(int lane, F f) {
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) f(mt * 16 + (lane >> 2) + (e >> 1) * 8, q * 8 + 2 * (lane & 3) + (e & 1), c[mt][q][e]);
+  }
+  __device__ __forceinline__ void load(const float* D, int64_t ldd, int cols, int lane) {
+    each(lane, [&](int i, int j, float& v) { v = j < cols ? D[j * ldd + i] : 0.f; });
+  }
+  __device__ __forceinline__ void store(float* D, int64_t ldd, int cols, int lane) {
+    each(lane, [&](int i, int j, float& v) {
+      if (j < cols) D[j * ldd + i] = v;
+    });
+  }
+  __device__ __forceinline__ void to_rows(float* X, int lane) {
+    each(lane, [&](int i, int j, float& v) { X[i * XP + j] = v; });
+  }
+  __device__ __forceinline__ void mul(const float* L, const float* X, int lane) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll 1
+    for (int k0 = 0; k0 < 32; k0 += 8) {
+      uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          split_tf32(-L[(k0 + t + (e >> 1) * 4) * LP + mt * 16 + g + (e & 1) * 8], ah[mt][e], al[mt][e]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) split_tf32(X[(k0 + t + 4 * e) * UP + q * 8 + g], bh[q][e], bl[q][e]);
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          mma_tf32(c[mt][q], al[mt], bh[q]);
+          mma_tf32(c[mt][q], ah[mt], bl[q]);
+          mma_tf32(c[mt][q], ah[mt], bh[q]);
+        }
+    }
+  }
+};
+
+// The head's factors in shared memory (Hv), by dependency levels; each
+// thread's first op of the next level is loaded ahead of the barrier.
 template <class T>
-__device__ __forceinline__ void head_program(const Args& A, T* Hv) {
+__device__ __forceinline__ void head_program() {
+  const Args& A = args();
+  T* Hv = at<T>(A.p.o_hv);
   const int* w = A.w;
-  for (int l = 0; l < 2 * A.n_hlev; ++l) {
-    const int o1 = __ldg(w + A.hop_ptr + l + 1);
-    for (int o = __ldg(w + A.hop_ptr + l) + threadIdx.x; o < o1; o += blockDim.x) {
-      const int2 op = __ldg(reinterpret_cast<const int2*>(w + A.hop) + o);
-      const int t1 = __ldg(w + A.hop + 2 * o + 3);
+  const int4* ops = reinterpret_cast<const int4*>(w + A.hop);
+  const int tid = threadIdx.x, nthr = blockDim.x, parts = 2 * A.n_hlev;
+  int o0 = 0, o1 = parts > 0 ? __ldg(w + A.hop_ptr + 1) : 0;
+  int4 first = tid < o1 ? __ldg(ops + tid) : make_int4(0, 0, 0, 0);
+  for (int l = 0; l < parts; ++l) {
+    const int o2 = l + 1 < parts ? __ldg(w + A.hop_ptr + l + 2) : o1;
+    auto run = [&](const int4& op) {
       const int dst = op.x & 0xFFFF, piv = (uint32_t)op.x >> 16;
       T v = Hv[dst];
-      for (int t = op.y; t < t1; ++t) {
-        const uint32_t tm = (uint32_t)__ldg(w + A.hterm + t);
-        v -= Hv[tm & 0xFFFF] * Hv[tm >> 16];
+      for (int t = op.y; t < op.z; t += 4) {
+        uint32_t tm[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) tm[u] = t + u < op.z ? (uint32_t)__ldg(w + A.hterm + t + u) : 0u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (t + u < op.z) v -= Hv[tm[u] & 0xFFFF] * Hv[tm[u] >> 16];
       }
       if (!(l & 1)) v = T(1) / v;
       else if (piv != 0xFFFF) v *= Hv[piv];
       Hv[dst] = v;
+    };
+    int o = o0 + tid;
+    if (o < o1) run(first);
+    for (o += nthr; o < o1; o += 4 * nthr) {
+      int4 op[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (o + u * nthr < o1) op[u] = __ldg(ops + o + u * nthr);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (o + u * nthr < o1) run(op[u]);
     }
+    o0 = o1;
+    o1 = o2;
+    if (o0 + tid < o1) first = __ldg(ops + o0 + tid);
     __syncthreads();
   }
 }
 
-// Panel J of the tail before elimination, in X (column-major, pitch rows):
-// its Jacobian entries and the head's Schur complement.  Ends with a barrier.
+// The tail before elimination (Jacobian entries and the head's Schur
+// complement) into its place in the packed factors.  A warp forms kGroup
+// columns at a time in its own shared tile, so that the warps' loads overlap
+// and no barrier separates the steps.
 template <class T>
-__device__ __forceinline__ void assemble_panel(const Args& A, int J, T* X, const T* Hv, const T* mbuf) {
+__device__ __forceinline__ void assemble_tail() {
+  const Args& A = args();
   const int* w = A.w;
-  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
-  for (int e = tid; e < 32 * A.pitch; e += nthr) X[e] = T(0);
-  __syncthreads();
-  {
-    const int s1 = __ldg(w + A.jg_grp + J + 2);
-    for (int e = 32 * __ldg(w + A.jg_grp + J + 1) + tid; e < 32 * s1; e += nthr) {
-      const int p = __ldg(w + A.jg_dst + e);
-      if (p >= 0) X[p] = mbuf[e];
-    }
-    const int q1 = __ldg(w + A.jl_grp + J + 2);
-    for (int q = __ldg(w + A.jl_grp + J + 1) + tid; q < q1; q += nthr)
-      X[__ldg(w + A.jl_dst + q)] = mbuf[32 * A.n_jsl + q];
-  }
-  __syncthreads();
-  const int s1 = __ldg(w + A.tg_grp + J + 1);
-  for (int s = __ldg(w + A.tg_grp + J) + warp; s < s1; s += nw) {
-    const int e0 = __ldg(w + A.tg_off + s), m = __ldg(w + A.tg_off + s + 1) - e0;
-    const int* q = w + A.tg_ent + 32 * e0 + lane;
-    const int pos = __ldg(w + A.tg_pos + 32 * s + lane);
-    T a = T(0);
-    int e = 0;
-    for (; e + 4 <= m; e += 4) {
-      uint32_t t[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) t[u] = (uint32_t)__ldg(q + 32 * (e + u));
-#pragma unroll
-      for (int u = 0; u < 4; ++u) a += Hv[t[u] & 0xFFFF] * Hv[t[u] >> 16];
-    }
-    for (; e < m; ++e) {
-      const uint32_t t = (uint32_t)__ldg(q + 32 * e);
-      a += Hv[t & 0xFFFF] * Hv[t >> 16];
-    }
-    if (pos >= 0) X[pos] -= a;
-  }
-  __syncthreads();
-}
-
-// L_KK's columns into ld[k][i] (one warp, 16-byte asynchronous copies).
-template <class T>
-__device__ __forceinline__ void fetch_diag(const T* D, int ldd, int K, T* ld, int lane) {
-  constexpr int PER = 16 / sizeof(T), CPC = 32 / PER;   // chunks per column
-#pragma unroll
-  for (int u = 0; u < CPC; ++u) {
-    const int id = 32 * u + lane, k = id / CPC, i = id % CPC * PER;
-    cp16(ld + k * 32 + i, D + (int64_t)(32 * K + k) * ldd + 32 * K + i);
-  }
-}
-
-// FP32 tail factorisation; TF: the updates on the tensor cores (3xTF32).
-template <bool TF>
-__device__ void factor_tail(const Args& A, float* D, float* X, float* Xk, float* Ld, const float* Hv, const float* mbuf PHASE_ARG) {
-  const int n = A.d.n, nt = n - A.d.head, ldd = A.d.ldd, nb = A.nb, pitch = A.pitch;
-  const int lane = threadIdx.x & 31, rb = threadIdx.x >> 5;
-  const int row = 32 * rb + lane;
-  const bool in = row < nt;
-  const int g = lane >> 2, tq = lane & 3;   // fragment coordinates
-  for (int J = 0; J < nb; ++J) {
-    assemble_panel(A, J, X, Hv, mbuf);
-    PHASE_MARK(PH_ASSEMBLE);
-    const int w = min(32, nt - 32 * J);
-    f2 x[16];             // row `row`, columns in pairs
-    float acc[2][4][4];   // TF: the warp's 32 x 32 block as m16n8 fragments
-    if (rb < nb) {
-      if constexpr (TF) {
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-          for (int nt8 = 0; nt8 < 4; ++nt8)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int r = 32 * rb + mt * 16 + g + (e >> 1) * 8, c = nt8 * 8 + 2 * tq + (e & 1);
-              acc[mt][nt8][e] = r < nt ? X[c * pitch + r] : 0.f;
-            }
-      } else {
-#pragma unroll
-        for (int p = 0; p < 16; ++p)
-          x[p] = in ? pack2(X[2 * p * pitch + row], X[(2 * p + 1) * pitch + row]) : pack2(0.f, 0.f);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pitch = A.pitch;
+  const int nt = A.d.n - A.d.head, groups = (nt + kGroup - 1) / kGroup, nwa = A.p.asm_warps;
+  const int64_t ldd = A.d.ldd;
+  T* X = at<T>(A.p.o_x) + warp * A.p.asm_tile;
+  const T* Hv = at<T>(A.p.o_hv);
+  const T* mbuf = static_cast<const T*>(scalars().mbuf);
+  T* D = static_cast<T*>(scalars().P) + A.d.p_d;
+  if (warp >= nwa) return;
+  for (int G = warp; G < groups; G += nwa) {
+    for (int e = lane * (16 / (int)sizeof(T)); e < A.p.asm_tile; e += 32 * (16 / (int)sizeof(T)))
+      *reinterpret_cast<float4*>(X + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncwarp();
+    {
+      const int* gp = w + A.jg_grp + G + 1;
+      const int e1 = 32 * __ldg(gp + 1), l0 = __ldg(w + A.jd_grp + G + 1), l1 = __ldg(w + A.jd_grp + G + 2);
+#pragma unroll 4
+      for (int e = 32 * __ldg(gp) + lane; e < e1; e += 32) {
+        const int p = __ldg(w + A.jg_dst + e);
+        const T v = mbuf[e];
+        if (p >= 0) X[p] = v;
+      }
+      for (int q = l0 + lane; q < l1; q += 32) {   // long entries: {position, index}
+        const int2 t = __ldg(reinterpret_cast<const int2*>(w + A.jd_ent) + q);
+        X[t.x] = mbuf[32 * A.n_jsl + t.y];
       }
     }
-    if (J > 0 && rb == 0) fetch_diag(D, ldd, 0, Ld, lane);
-    for (int K = 0; K < J; ++K) {
-      float* xk = Xk + (K & 1) * 32 * XP;
-      float* ld = Ld + (K & 1) * 32 * 32;
-      if (rb == K) {
-        // this warp's rows are block K: finish their U
-        if constexpr (TF) {
+    __syncwarp();
+    // the group's targets: a stream of rows of words, per slice {position |
+    // terms << 16}, then the terms; kRows rows in flight ahead of their use
+    {
+      constexpr int kRows = 12;
+      const int r1 = __ldg(w + A.tg_grp + G + 1);
+      int r = __ldg(w + A.tg_grp + G);
+      const int* q = w + A.tg_ent + lane;
+      uint32_t t[kRows];
 #pragma unroll
-          for (int mt = 0; mt < 2; ++mt)
+      for (int u = 0; u < kRows; ++u) t[u] = r + u < r1 ? (uint32_t)__ldg(q + 32 * (r + u)) : 0xFFFFu;
+      T a = T(0);
+      uint32_t pos = 0xFFFFu;
+      int left = 0;
+      for (; r < r1 + 1; r += kRows) {   // (one row more: the last slice's result)
+        uint32_t nx[kRows];
 #pragma unroll
-            for (int nt8 = 0; nt8 < 4; ++nt8)
+        for (int u = 0; u < kRows; ++u) nx[u] = r + kRows + u < r1 ? (uint32_t)__ldg(q + 32 * (r + kRows + u)) : 0xFFFFu;
 #pragma unroll
-              for (int e = 0; e < 4; ++e)
-                xk[(mt * 16 + g + (e >> 1) * 8) * XP + nt8 * 8 + 2 * tq + (e & 1)] = acc[mt][nt8][e];
-        } else {
-#pragma unroll
-          for (int p = 0; p < 16; ++p) *reinterpret_cast<f2*>(xk + lane * XP + 2 * p) = x[p];
-        }
-        cp_wait();
-        __syncwarp();
-        trsm_block(xk, ld, lane);
-        __syncwarp();
-        if (lane < w) {   // column `lane` of the block, 32 consecutive rows
-          float* dst = D + (int64_t)(32 * J + lane) * ldd + 32 * K;
-#pragma unroll
-          for (int r = 0; r < 32; r += 4)
-            *reinterpret_cast<float4*>(dst + r) = make_float4(xk[r * XP + lane], xk[(r + 1) * XP + lane],
-                                                               xk[(r + 2) * XP + lane], xk[(r + 3) * XP + lane]);
-        }
-      }
-      __syncthreads();
-      if (rb == K + 1 && K + 1 < J) fetch_diag(D, ldd, K + 1, Ld + ((K + 1) & 1) * 32 * 32, lane);
-      if (rb > K && rb < nb) {
-        if constexpr (TF) {
-          const float* lcol = D + (int64_t)(32 * K) * ldd + 32 * rb;
-#pragma unroll
-          for (int k0 = 0; k0 < 32; k0 += 8) {
-            uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const int r = mt * 16 + g + (e & 1) * 8, kk = k0 + tq + (e >> 1) * 4;
-                const float v = 32 * rb + r < nt ? -lcol[(int64_t)kk * ldd + r] : 0.f;
-                split_tf32(v, ah[mt][e], al[mt][e]);
-              }
-#pragma unroll
-            for (int nt8 = 0; nt8 < 4; ++nt8)
-#pragma unroll
-              for (int e = 0; e < 2; ++e) split_tf32(xk[(k0 + tq + 4 * e) * XP + nt8 * 8 + g], bh[nt8][e], bl[nt8][e]);
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-              for (int nt8 = 0; nt8 < 4; ++nt8) {
-                mma_tf32(acc[mt][nt8], al[mt], bh[nt8]);
-                mma_tf32(acc[mt][nt8], ah[mt], bl[nt8]);
-                mma_tf32(acc[mt][nt8], ah[mt], bh[nt8]);
-              }
-          }
-        } else {
-          const float* lcol = D + (int64_t)(32 * K) * ldd + row;
-#pragma unroll
-          for (int k0 = 0; k0 < 32; k0 += 16) {
-            float l[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) l[k] = in ? -lcol[(int64_t)(k0 + k) * ldd] : 0.f;
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              const f2 ll = pack2(l[k], l[k]);
-              const ulonglong2* xr = reinterpret_cast<const ulonglong2*>(xk + (k0 + k) * XP);
-#pragma unroll
-              for (int c = 0; c < 8; ++c) {
-                const ulonglong2 v = xr[c];
-                x[2 * c] = fma2(ll, v.x, x[2 * c]);
-                x[2 * c + 1] = fma2(ll, v.y, x[2 * c + 1]);
-              }
-            }
+        for (int u = 0; u < kRows; ++u) {
+          if (left > 0) {
+            a += Hv[t[u] & 0xFFFF] * Hv[t[u] >> 16];
+            --left;
+          } else {
+            if (pos != 0xFFFFu) X[pos] -= a;
+            pos = t[u] & 0xFFFF;
+            left = (int)(t[u] >> 16);
+            a = T(0);
           }
         }
+#pragma unroll
+        for (int u = 0; u < kRows; ++u) t[u] = nx[u];
       }
+      if (pos != 0xFFFFu && left == 0) X[pos] -= a;
     }
-    PHASE_MARK(PH_UPDATE);
-    // block J: LU of the diagonal block, then L of the rows below
-    float* uj = Xk + (J & 1) * 32 * XP;
-    float rv[32];
-    if (rb >= J && rb < nb) {
-      if constexpr (TF) {
+    __syncwarp();
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-          for (int nt8 = 0; nt8 < 4; ++nt8)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int r = 32 * rb + mt * 16 + g + (e >> 1) * 8, c = nt8 * 8 + 2 * tq + (e & 1);
-              if (r < nt) X[c * pitch + r] = acc[mt][nt8][e];
-            }
-        __syncwarp();
-#pragma unroll
-        for (int b = 0; b < 32; ++b) rv[b] = in ? X[b * pitch + row] : 0.f;
-      } else {
-#pragma unroll
-        for (int p = 0; p < 16; ++p) unpack2(x[p], rv[2 * p], rv[2 * p + 1]);
+    for (int c = 0; c < kGroup; ++c)
+      if (kGroup * G + c < nt) {
+        T* col = D + (kGroup * G + c) * ldd;
+#pragma unroll 4
+        for (int r = lane; r < nt; r += 32) col[r] = X[c * pitch + r];
       }
-    }
-    if (rb == J) {
-      if (lane >= w) {   // rows and columns past the last block's edge: the identity
-#pragma unroll
-        for (int b = 0; b < 32; ++b) rv[b] = b == lane ? 1.f : 0.f;
-      }
-#pragma unroll
-      for (int kk = 0; kk < 32; ++kk) {
-        const float inv = 1.f / __shfl_sync(kFull, rv[kk], kk);
-        const float l = rv[kk] * inv;
-        const bool below = lane > kk;
-        if (below) rv[kk] = l;
-#pragma unroll
-        for (int b = kk + 1; b < 32; ++b) {
-          const float pb = __shfl_sync(kFull, rv[b], kk);
-          if (below) rv[b] -= l * pb;
-        }
-        if (lane == kk) rv[kk] = inv;
-      }
-#pragma unroll
-      for (int b = 0; b < 32; ++b) uj[lane * XP + b] = rv[b];
-      float* dst = D + (int64_t)(32 * J) * ldd + row;
-#pragma unroll
-      for (int b = 0; b < 32; ++b)
-        if (in && b < w) dst[(int64_t)b * ldd] = rv[b];
-    }
-    __syncthreads();
-    if (rb > J && rb < nb) {   // then w == 32
-#pragma unroll
-      for (int kk = 0; kk < 32; ++kk) {
-        const float l = rv[kk] * uj[kk * XP + kk];   // inverse pivot
-        rv[kk] = l;
-#pragma unroll
-        for (int b = kk + 1; b < 32; ++b) rv[b] -= l * uj[kk * XP + b];
-      }
-      float* dst = D + (int64_t)(32 * J) * ldd + row;
-#pragma unroll
-      for (int b = 0; b < 32; ++b)
-        if (in) dst[(int64_t)b * ldd] = rv[b];
-    }
-    __syncthreads();
-    PHASE_MARK(PH_PANEL);
+    __syncwarp();
   }
 }
 
-// FP64 tail factorisation: two warps per 32 rows, 16 columns each, so that
-// the four FP64 pipes of the SM get even shares.
-__device__ void factor_tail(const Args& A, double* D, double* X, double* Xk, double* Ld, const double* Hv, const double* mbuf PHASE_ARG) {
-  const int n = A.d.n, nt = n - A.d.head, ldd = A.d.ldd, nb = A.nb, pitch = A.pitch;
-  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  const int cs = wi >= nb, rb = wi < 2 * nb ? wi - cs * nb : nb, c0 = 16 * cs;
-  const int row = 32 * rb + lane;
-  const bool in = row < nt;
-  for (int J = 0; J < nb; ++J) {
-    assemble_panel(A, J, X, Hv, mbuf);
-    PHASE_MARK(PH_ASSEMBLE);
-    const int w = min(32, nt - 32 * J);
-    double rv[16];
-#pragma unroll
-    for (int b = 0; b < 16; ++b) rv[b] = in ? X[(c0 + b) * pitch + row] : 0.0;
-    if (J > 0 && rb == 0) fetch_diag(D, ldd, 0, Ld, lane);
-    for (int K = 0; K < J; ++K) {
-      double* xk = Xk + (K & 1) * 32 * XP;
-      double* ld = Ld + (K & 1) * 32 * 32;
-      if (rb == K) {
-#pragma unroll
-        for (int b = 0; b < 16; ++b) xk[lane * XP + c0 + b] = rv[b];
-        cp_wait();
-        __syncwarp();
-        trsm_block16(xk, ld, c0, lane);
-        __syncwarp();
-#pragma unroll
-        for (int b = 0; b < 16; ++b)
-          if (c0 + b < w) D[(int64_t)(32 * J + c0 + b) * ldd + row] = xk[lane * XP + c0 + b];
-      }
-      __syncthreads();
-      if (rb == K + 1 && K + 1 < J) fetch_diag(D, ldd, K + 1, Ld + ((K + 1) & 1) * 32 * 32, lane);
-      if (rb > K && rb < nb) {
-        const double* lcol = D + (int64_t)(32 * K) * ldd + row;
-#pragma unroll
-        for (int k0 = 0; k0 < 32; k0 += 8) {
-          double l[8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k) l[k] = in ? -lcol[(int64_t)(k0 + k) * ldd] : 0.0;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const double2* xr = reinterpret_cast<const double2*>(xk + (k0 + k) * XP + c0);
-#pragma unroll
-            for (int b = 0; b < 8; ++b) {
-              const double2 v = xr[b];
-              rv[2 * b] = fma(l[k], v.x, rv[2 * b]);
-              rv[2 * b + 1] = fma(l[k], v.y, rv[2 * b + 1]);
-            }
-          }
-        }
-      }
-    }
-    PHASE_MARK(PH_UPDATE);
-    // block J in four stages: LU of its first 16 columns; L of the rows below
-    // there and U12 / LU of the second 16 columns; L of the rows below
-    double* uj = Xk + (J & 1) * 32 * XP;
-    if (rb == J && lane >= w) {
-#pragma unroll
-      for (int b = 0; b < 16; ++b) rv[b] = c0 + b == lane ? 1.0 : 0.0;
-    }
-    auto lu16 = [&](int r0) {   // pivots in lanes r0 .. r0 + 15
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) {
-        const double inv = 1.0 / __shfl_sync(kFull, rv[kk], r0 + kk);
-        const double l = rv[kk] * inv;
-        const bool below = lane > r0 + kk;
-        if (below) rv[kk] = l;
-#pragma unroll
-        for (int b = kk + 1; b < 16; ++b) {
-          const double pb = __shfl_sync(kFull, rv[b], r0 + kk);
-          if (below) rv[b] -= l * pb;
-        }
-        if (lane == r0 + kk) rv[kk] = inv;
-      }
-    };
-    auto lrow16 = [&](int r0) {   // l U = a for this thread's row, U at uj rows and columns r0 ..
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) {
-        const double l = rv[kk] * uj[(r0 + kk) * XP + r0 + kk];
-        rv[kk] = l;
-#pragma unroll
-        for (int b = kk + 1; b < 16; ++b) rv[b] -= l * uj[(r0 + kk) * XP + r0 + b];
-      }
-    };
-    auto store = [&]() {
-#pragma unroll
-      for (int b = 0; b < 16; ++b)
-        if (in && c0 + b < w) D[(int64_t)(32 * J + c0 + b) * ldd + row] = rv[b];
-    };
-    if (rb == J && cs == 0) {
-      lu16(0);
-#pragma unroll
-      for (int b = 0; b < 16; ++b) uj[lane * XP + b] = rv[b];
-      store();
-    }
-    __syncthreads();
-    if (cs == 0 && rb > J && rb < nb) {
-      lrow16(0);
-#pragma unroll
-      for (int b = 0; b < 16; ++b)
-        if (in) X[b * pitch + row] = rv[b];
-      store();
-    }
-    if (rb == J && cs == 1) {
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) {
-        const double l = lane > kk ? uj[lane * XP + kk] : 0.0;
-#pragma unroll
-        for (int b = 0; b < 16; ++b) rv[b] -= l * __shfl_sync(kFull, rv[b], kk);
-      }
-      lu16(16);
-#pragma unroll
-      for (int b = 0; b < 16; ++b) uj[lane * XP + 16 + b] = rv[b];
-      store();
-    }
-    __syncthreads();
-    if (cs == 1 && rb > J && rb < nb) {
-#pragma unroll
-      for (int kk = 0; kk < 16; ++kk) {
-        const double l = in ? X[kk * pitch + row] : 0.0;
-#pragma unroll
-        for (int b = 0; b < 16; ++b) rv[b] -= l * uj[kk * XP + 16 + b];
-      }
-      lrow16(16);
-      store();
-    }
-    __syncthreads();
-    PHASE_MARK(PH_PANEL);
+// LU of the tail, right-looking by 32-column panels on the packed factors (in
+// L2): per panel the rows below the diagonal block and the block row right of
+// it are solved block by block, every warp a block at a time, and kept in
+// shared memory for the trailing update, whose blocks the warps take in turn.
+// The block that holds the next panel's diagonal comes first and is factorised
+// at once by the warp that updated it, while the others go on.  Against a
+// left-looking form (a chain of a product and a triangular solve per pair of
+// blocks: 55 links for 11 block columns against 11 here) this reads and writes
+// the trailing blocks, 3 MB of L2 traffic per 349-column tail.
+struct TailView {
+  int nt, nb, lane, warp, nw;
+  int64_t ldd;
+  __device__ __forceinline__ TailView() {
+    const Args& A = args();
+    nt = A.d.n - A.d.head;
+    nb = A.nb;
+    ldd = A.d.ldd;
+    lane = threadIdx.x & 31;
+    warp = threadIdx.x >> 5;
+    nw = blockDim.x >> 5;
   }
-}
-
-template <bool TF>
-__device__ __forceinline__ void factor(const Args& A, float* D, float* X, float* Xk, float* Ld, const float* Hv, const float* mbuf PHASE_ARG) {
-  factor_tail<TF>(A, D, X, Xk, Ld, Hv, mbuf PHASE_PASS);
-}
-template <bool TF>
-__device__ __forceinline__ void factor(const Args& A, double* D, double* X, double* Xk, double* Ld, const double* Hv, const double* mbuf PHASE_ARG) {
-  factor_tail(A, D, X, Xk, Ld, Hv, mbuf PHASE_PASS);
-}
-
-// The cell being worked on: its shared vectors and global buffers.
-template <class T>
-struct Cell {
-  CellS* S;
-  double *red, *yp, *ps, *ws, *wf, *ys, *fs, *tab, *part;
-  T *xh, *xt, *tmp;
-  double *kc, *hist, *eprev;   // this CTA's global scratch
-  T* mbuf;
-  T* P;                        // packed factors
-  int64_t c, oc;               // slot and cell
-  int hn;                      // stride of a history point in scratch
-  double nH, Av, chi;
+  template <class T> __device__ __forceinline__ T* block(int r, int j) const {
+    return static_cast<T*>(scalars().P) + args().d.p_d + (32 * j) * ldd + 32 * r;
+  }
+  __device__ __forceinline__ int width(int j) const { return min(32, nt - 32 * j); }
 };
+
+// L of the blocks below the diagonal block J and U of the blocks right of it.
+template <class T, bool TF>
+__device__ __forceinline__ void solve_panel(int J) {
+  constexpr int LP = Tile<T, TF>::LP, UP = Tile<T, TF>::UP;
+  const Args& A = args();
+  const TailView v;
+  const int64_t ldd = v.ldd;
+  const int lane = v.lane, m = v.nb - 1 - J;   // block rows below, block columns to the right
+  for (int q = v.warp; q < 2 * m; q += v.nw) {
+    T c[32];
+    if (q < m) {   // rows of block (J + 1 + q, J), a row per lane
+      const int r = J + 1 + q;
+      T* p = v.block<T>(r, J) + lane;
+      {   // (rows past the tail's end are padding)
+        const T* s = p;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          c[j] = ld_here(s);
+          s += ldd;
+        }
+      }
+      T* o = at<T>(A.p.o_lp) + (r - 1) * 32 * LP + lane;
+      tri_solve<T, false, XP>(c, at<T>(A.p.o_uj), [&](int, const T(&x)[32]) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          *o = x[k];
+          *p = x[k];
+          o += LP;
+          p += ldd;
+        }
+      });
+    } else {   // columns of block (J, j), a column per lane
+      const int j = J + 1 + q - m;
+      const bool in = lane < v.width(j);
+      T* p = v.block<T>(J, j) + (in ? lane : 0) * ldd;   // (lanes past the last column: not stored)
+#pragma unroll
+      for (int i = 0; i < 32; i += 4) {
+        T x[4];
+        load4(p + i, x);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[i + u] = x[u];
+      }
+      T* o = at<T>(A.p.o_up) + (j - 1) * 32 * UP + lane;
+      tri_solve<T, true, 32>(c, at<T>(A.p.o_lj), [&](int b0, const T(&x)[32]) {
+        const T lo[4] = {x[0], x[1], x[2], x[3]}, hi[4] = {x[4], x[5], x[6], x[7]};
+        if (in) {
+          store4(p + b0, lo);
+          store4(p + b0 + 4, hi);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o[(b0 + k) * UP] = x[k];
+      });
+    }
+  }
+}
+
+template <class T, bool TF>
+__device__ __forceinline__ void factor_tail() {
+  using Tl = Tile<T, TF>;
+  constexpr int LP = Tl::LP, UP = Tl::UP, CW = Tl::CW, HB = 32 / CW;
+  const Args& A = args();
+  const TailView v;
+  const int lane = v.lane, nb = v.nb;
+  int* next = at<int>(A.p.o_next);
+  auto take = [&]() {
+    int t = 0;
+    if (lane == 0) t = atomicAdd(next, 1);
+    return __shfl_sync(kFull, t, 0);
+  };
+  for (int J = -1; J + 1 < nb; ++J) {
+    const int m = nb - 1 - J;
+    const T* Lp = at<T>(A.p.o_lp) + J * 32 * LP;   // of block row J + 1
+    const T* Up = at<T>(A.p.o_up) + J * 32 * UP;
+    if (J >= 0) {
+      __syncthreads();
+      if (threadIdx.x == 0) *next = HB;   // (the first block is warp 0's)
+      solve_panel<T, TF>(J);
+      __syncthreads();
+      PHASE_MARK(PH_PANEL);
+    }
+    if (v.warp == 0) {
+      // the next diagonal block: updated, and factorised at once
+      T *uj = at<T>(A.p.o_uj), *D = v.block<T>(J + 1, J + 1);
+      const int w = v.width(J + 1);
+#pragma unroll 1
+      for (int h = 0; h < HB; ++h) {
+        Tl x;
+        x.load(D + (CW * h) * v.ldd, v.ldd, w - CW * h, lane);
+        if (J >= 0) x.mul(Lp, Up + CW * h, lane);
+        x.to_rows(uj + CW * h, lane);
+      }
+      __syncwarp();
+      lu_block(uj, at<T>(A.p.o_lj), D + lane, v.ldd, w, lane);
+    }
+    if (J < 0) continue;
+    // the other trailing blocks in turn, by columns
+    const int mm = m * m * HB;
+    auto corner = [&](int t) { return v.block<T>(J + 1 + t / HB % m, J + 1 + t / HB / m) + (CW * (t % HB)) * v.ldd; };
+    auto cols = [&](int t) { return v.width(J + 1 + t / HB / m) - CW * (t % HB); };
+    int t = take();
+    Tl x;
+    if (t < mm) x.load(corner(t), v.ldd, cols(t), lane);
+    while (t < mm) {
+      const T *lp = Lp + (t / HB % m) * 32 * LP, *up = Up + (t / HB / m) * 32 * UP + CW * (t % HB);
+      if constexpr (sizeof(T) == 4) {
+        const int u = take();
+        Tl y;   // the next block is on its way while this one is worked on
+        if (u < mm) y.load(corner(u), v.ldd, cols(u), lane);
+        x.mul(lp, up, lane);
+        x.store(corner(t), v.ldd, cols(t), lane);
+        x = y;
+        t = u;
+      } else {   // (a block's FP64 products take a hundred times its loads)
+        x.mul(lp, up, lane);
+        x.store(corner(t), v.ldd, cols(t), lane);
+        t = take();
+        if (t < mm) x.load(corner(t), v.ldd, cols(t), lane);
+      }
+    }
+    PHASE_MARK(PH_UPDATE);
+  }
+  __syncthreads();
+}
 
 // Jacobian at the predicted state, M = I - gamma J and its packed factors.
 // y (= predicted state) is restored at the end.
-template <class T, bool TF>
-__device__ void cell_refresh(const Args& A, Cell<T>& q, unsigned char* sm PHASE_ARG) {
+
+// First the Jacobian: -gamma dR_j/dx in a shared table, then M's entries in
+// program order into mbuf (global scratch).
+template <class T>
+__device__ __forceinline__ void cell_jacobian() {
+  const Args& A = args();
   const Dev& d = A.d;
+  const CellS& S = scalars();
   const int n = d.n, n_r = d.n_r, tid = threadIdx.x, nthr = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
   const int* w = A.w;
-  double* dR = reinterpret_cast<double*>(sm + A.p.o_dr);
-  float* wsf = reinterpret_cast<float*>(sm + A.p.o_wsf);
-  float* wif = reinterpret_cast<float*>(sm + A.p.o_wif);
-  const double gamma = q.S->gam;
-  // -gamma dR_j/dx for both reactant slots
+  double* dR = at<double>(A.p.o_dr);
+  float* wsf = at<float>(A.p.o_wsf);
+  float* wif = at<float>(A.p.o_wif);
+  const double* yp = at<double>(A.p.o_yp);
+  const double* kc = S.kc;
+  T* mbuf = static_cast<T*>(S.mbuf);
+  const double gamma = S.gam;
+  // -gamma dR_j/dx for every reactant
+  const int2* rx = reinterpret_cast<const int2*>(w + A.rx);
+#pragma unroll 4
   for (int j = tid; j < n_r; j += nthr) {
-    const int2 rc = __ldg(d.reac + j);
-    const double kv = -gamma * q.kc[j];
-    dR[2 * j] = rc.y >= 0 ? kv * q.yp[rc.y] : kv;
-    dR[2 * j + 1] = rc.y >= 0 ? kv * q.yp[rc.x] : 0.0;
+    const int2 r = __ldg(rx + j);
+    const double kv = -gamma * kc[j];
+    const int b = (uint32_t)r.x >> 16;
+    dR[r.y] = b != 0xFFFF ? kv * yp[b] : kv;
+    if (b != 0xFFFF) dR[r.y + 1] = kv * yp[r.x & 0xFFFF];
   }
-  if (tid == 0) dR[2 * n_r] = 0.0;
-  for (int s = tid; s < n; s += nthr) {
-    const double wv = q.ws[s];
-    q.wf[s] = wv;
-    if (d.mixed) {
+  if (tid == 0) dR[A.n_slot] = 0.0;
+  if constexpr (sizeof(T) == 4) {
+    const double* ws = at<double>(A.p.o_ws);
+    double *wf = at<double>(A.p.o_wf), *wi = at<double>(A.p.o_wi);
+    for (int s = tid; s < n; s += nthr) {
+      const double wv = ws[s], iv = 1.0 / wv;
+      wf[s] = wv;
+      wi[s] = iv;
       wsf[s] = (float)wv;
-      wif[s] = (float)(1.0 / wv);
+      wif[s] = (float)iv;
     }
   }
   __syncthreads();
   auto m_value = [&](int rc, double acc) {   // M (W M W^-1 in FP32) at (row species, column species)
     const int i = rc & 0xFFFF, l = (uint32_t)rc >> 16;
     if (i == l) acc += 1.0;
-    return sizeof(T) == 4 ? T((float)acc * (wsf[i] * wif[l])) : T(acc);
+    if constexpr (sizeof(T) == 4) return T((float)acc * (wsf[i] * wif[l]));
+    else return T(acc);
   };
-  for (int s = warp; s < A.n_jsl; s += nw) {
-    const int e0 = __ldg(w + A.jg_off + s), m = __ldg(w + A.jg_off + s + 1) - e0;
-    const int* p = w + A.jg_ent + 32 * e0 + lane;
-    const int rc = __ldg(w + A.jg_rc + 32 * s + lane);
-    double a = 0.0;
-    if (m > 0) {
-      const int w0 = __ldg(p);
-      a = flip(dR[w0 & 0x7FFFFFFF], w0);
+  // entries of at most kJShort words, four slices at a time, all their index
+  // words in flight at once
+  {
+    const int4* off = reinterpret_cast<const int4*>(w + A.jg_off);
+    const int* p = w + A.jg_ent + lane;
+    int s = 4 * warp;
+    int4 m0 = make_int4(0, 0, 0, 0), m1 = m0;
+    if (s < A.n_jsl) {
+      m0 = __ldg(off + s / 2);
+      m1 = __ldg(off + s / 2 + 1);
     }
-    int e = 1;
-    for (; e + 4 <= m; e += 4) {
-      int t[4];
+    for (; s < A.n_jsl; s += 4 * nw) {
+      const int of[4] = {m0.x, m0.z, m1.x, m1.z}, len[4] = {m0.y, m0.w, m1.y, m1.w};
+      int rc[4], t[kJShort][4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) t[u] = __ldg(p + 32 * (e + u));
+      for (int u = 0; u < 4; ++u) {
+        rc[u] = __ldg(w + A.jg_rc + 32 * (s + u) + lane);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) a += flip(dR[t[u] & 0x7FFFFFFF], t[u]);
+        for (int e = 0; e < kJShort; ++e) t[e][u] = e < len[u] ? __ldg(p + 32 * (of[u] + e)) : A.n_slot;
+      }
+      if (s + 4 * nw < A.n_jsl) {
+        m0 = __ldg(off + (s + 4 * nw) / 2);
+        m1 = __ldg(off + (s + 4 * nw) / 2 + 1);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        double a = flip(dR[t[0][u] & 0x7FFFFFFF], t[0][u]);
+#pragma unroll
+        for (int e = 1; e < kJShort; ++e)
+          if (e < len[u]) a += flip(dR[t[e][u] & 0x7FFFFFFF], t[e][u]);
+        if (len[u] > 0) mbuf[32 * (s + u) + lane] = m_value(rc[u], a);
+      }
     }
-    for (; e < m; ++e) {
-      const int w0 = __ldg(p + 32 * e);
-      a += flip(dR[w0 & 0x7FFFFFFF], w0);
-    }
-    q.mbuf[32 * s + lane] = m_value(rc, a);
   }
-  for (int s = nw - 1 - warp; s < A.n_jl; s += nw) {   // long entries
-    const int e1 = __ldg(w + A.jl_ptr + s + 1);
-    double a = 0.0;
-    for (int e = __ldg(w + A.jl_ptr + s) + lane; e < e1; e += 32) {
-      const int w0 = __ldg(w + A.jl_ent + e);
-      a += flip(dR[w0 & 0x7FFFFFFF], w0);
+  // the entries of more words, in pieces of at most kJPiece
+  for (int s = nw - 1 - warp; s < A.n_jp; s += nw) {
+    int t[kJPiece];
+#pragma unroll
+    for (int e = 0; e < kJPiece; ++e) t[e] = __ldg(w + A.jp_ent + 32 * (kJPiece * s + e) + lane);
+    double a = flip(dR[t[0] & 0x7FFFFFFF], t[0]), b = flip(dR[t[1] & 0x7FFFFFFF], t[1]);
+#pragma unroll
+    for (int e = 2; e < kJPiece; e += 2) {
+      a += flip(dR[t[e] & 0x7FFFFFFF], t[e]);
+      b += flip(dR[t[e + 1] & 0x7FFFFFFF], t[e + 1]);
     }
+    S.pbuf[32 * s + lane] = a + b;
+  }
+  __syncthreads();
+  // and their pieces (rows of pieces: longest first; more than 8 a warp each)
+  for (int q = warp; q < A.n_jw; q += nw) {
+    const int p1 = __ldg(w + A.jl_ptr + q + 1);
+    double a = 0.0;
+    for (int p = __ldg(w + A.jl_ptr + q) + lane; p < p1; p += 32) a += S.pbuf[p];
     a = warp_sum(a);
-    if (lane == 0) q.mbuf[32 * A.n_jsl + s] = m_value(__ldg(w + A.jl_rc + s), a);
+    if (lane == 0) mbuf[32 * A.n_jsl + q] = m_value(__ldg(w + A.jl_rc + q), a);
+  }
+  for (int q = A.n_jw + tid; q < A.n_jl; q += nthr) {
+    const int p0 = __ldg(w + A.jl_ptr + q), p1 = __ldg(w + A.jl_ptr + q + 1);
+    double a = 0.0;
+    for (int p = p0; p < p1; ++p) a += S.pbuf[p];
+    mbuf[32 * A.n_jsl + q] = m_value(__ldg(w + A.jl_rc + q), a);
   }
   if (d.therm) {
     // gamma_J sum_j dn_j dR_j/dx_l per species, kept in the border's row
     __syncthreads();
     for (int j = tid; j < n_r; j += nthr) {
       const double dn = -__ldg(d.th_dn + j);
-      dR[2 * j] *= dn;
-      dR[2 * j + 1] *= dn;
+      const int2 r = __ldg(rx + j);
+      dR[r.y] *= dn;
+      if ((uint32_t)r.x >> 16 != 0xFFFF) dR[r.y + 1] *= dn;
     }
     __syncthreads();
-    row_sums(w, A.n_vsl, A.vp_off, A.vp_ent, A.vp_dst, A.vrow_ptr, A.n_vlong, A.vrow_long, dR,
-             reinterpret_cast<double*>(sm + A.p.o_vp), d.bgv + q.oc * d.bpad, n);
+    row_sums(w, A.n_vsl, A.vp_off, A.vp_ent, A.vp_dst, A.vrow, A.vrow_more, dR, at<double>(A.p.o_vp),
+             d.bgv + S.oc * d.bpad, n);
   }
   __syncthreads();
   PHASE_MARK(PH_JAC);
-  T* Hv = reinterpret_cast<T*>(sm + A.p.o_hv);
-  for (int e = tid; e <= d.p_d; e += nthr) Hv[e] = T(0);
+}
+
+// The head's entries of M into shared memory, their factors, and those out.
+template <class T>
+__device__ __forceinline__ void cell_head() {
+  const Args& A = args();
+  const int tid = threadIdx.x, nthr = blockDim.x, p_d = A.d.p_d;
+  const int* w = A.w;
+  T* Hv = at<T>(A.p.o_hv);
+  const T* mbuf = static_cast<const T*>(scalars().mbuf);
+  for (int e = tid; e <= p_d; e += nthr) Hv[e] = T(0);
   __syncthreads();
   {
     const int s1 = __ldg(w + A.jg_grp + 1);
+#pragma unroll 4
     for (int e = tid; e < 32 * s1; e += nthr) {
       const int p = __ldg(w + A.jg_dst + e);
-      if (p >= 0) Hv[p] = q.mbuf[e];
+      const T v = mbuf[e];
+      if (p >= 0) Hv[p] = v;
     }
-    const int q1 = __ldg(w + A.jl_grp + 1);
-    for (int e = tid; e < q1; e += nthr) Hv[__ldg(w + A.jl_dst + e)] = q.mbuf[32 * A.n_jsl + e];
+    const int q1 = __ldg(w + A.jd_grp + 1);
+    for (int e = tid; e < q1; e += nthr) {
+      const int2 t = __ldg(reinterpret_cast<const int2*>(w + A.jd_ent) + e);
+      Hv[t.x] = mbuf[32 * A.n_jsl + t.y];
+    }
   }
   __syncthreads();
-  head_program(A, Hv);
-  for (int e = tid; e < d.p_d; e += nthr) q.P[e] = Hv[e];
+  head_program<T>();
+  T* P = static_cast<T*>(scalars().P);
+  for (int e = tid; e < p_d; e += nthr) P[e] = Hv[e];
   PHASE_MARK(PH_HEAD);
-  factor<TF>(A, q.P + d.p_d, reinterpret_cast<T*>(sm + A.p.o_x), reinterpret_cast<T*>(sm + A.p.o_xk),
-             reinterpret_cast<T*>(sm + A.p.o_ld), Hv, q.mbuf PHASE_PASS);
-  for (int s = tid; s < n; s += nthr) q.ys[s] = q.yp[s];
-  if (tid == 0) {
-    CellS& S = *q.S;
-    S.gam_J = gamma;
+}
+
+template <class T, bool TF>
+__device__ __forceinline__ void cell_refresh() {
+  cell_jacobian<T>();
+  cell_head<T>();
+  assemble_tail<T>();
+  __syncthreads();
+  PHASE_MARK(PH_ASSEMBLE);
+  factor_tail<T, TF>();
+  const Args& A = args();
+  for (int s = threadIdx.x; s < A.d.n; s += blockDim.x) at<double>(A.p.o_ys)[s] = at<double>(A.p.o_yp)[s];
+  if (threadIdx.x == 0) {
+    CellS& S = scalars();
+    S.gam_J = S.gam;
     S.j_age = 0;
     S.crate = 1.0;
     S.flags &= ~F_NEED_J;
@@ -1024,19 +1213,26 @@ __device__ void cell_refresh(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
   __syncthreads();
 }
 
-// x := M^-1 b with b given by species in bs (scaled by wf when mixed); the
-// solution by species through get(s).
+// The substitution's vector by species: x_put scales the right-hand side by
+// the factorisation's weights (FP32), x_get undoes it.
 template <class T>
-__device__ __forceinline__ T x_get(const Args& A, const Cell<T>& q, int s) {
-  const int p = __ldg(A.d.iperm + s);
-  return p < A.d.head ? q.xh[p] : q.xt[p - A.d.head];
+__device__ __forceinline__ double x_get(const Args& A, int s) {
+  const int p = at<uint16_t>(A.p.o_ip)[s];
+  const double v = (double)(p < A.d.head ? at<T>(A.p.o_xh)[p] : at<T>(A.p.o_xt)[p - A.d.head]);
+  if constexpr (sizeof(T) == 4) {
+    // v / w: from the rounded reciprocal, corrected by the quotient's residual
+    const double w = at<double>(A.p.o_wf)[s], iw = at<double>(A.p.o_wi)[s], q = v * iw;
+    return fma(fma(-q, w, v), iw, q);
+  } else {
+    return v;
+  }
 }
 template <class T>
-__device__ __forceinline__ void x_put(const Args& A, const Cell<T>& q, int s, double b) {
-  if (A.d.mixed) b *= q.wf[s];
-  const int p = __ldg(A.d.iperm + s);
-  if (p < A.d.head) q.xh[p] = T(b);
-  else q.xt[p - A.d.head] = T(b);
+__device__ __forceinline__ void x_put(const Args& A, int s, double b) {
+  if constexpr (sizeof(T) == 4) b *= at<double>(A.p.o_wf)[s];
+  const int p = at<uint16_t>(A.p.o_ip)[s];
+  if (p < A.d.head) at<T>(A.p.o_xh)[p] = T(b);
+  else at<T>(A.p.o_xt)[p - A.d.head] = T(b);
 }
 
 // Temperature border of a refreshed Newton matrix (T eliminated last): with
@@ -1044,92 +1240,99 @@ __device__ __forceinline__ void x_put(const Args& A, const Cell<T>& q, int s, do
 // z = M^-1 (-gJ u) and s = 1 - gJ w + gJ v.z; a residual (r, r_T) then has the
 // correction (a0 - z b, b), a0 = M^-1 r, b = (r_T + gJ v.a0) / s.
 template <class T>
-__device__ void cell_border(const Args& A, Cell<T>& q) {
+__device__ __forceinline__ void cell_border() {
+  const Args& A = args();
   const Dev& d = A.d;
+  const CellS& S = scalars();
+  const double* yp = at<double>(A.p.o_yp);
+  const double* fs = at<double>(A.p.o_fs);
+  double* tab = at<double>(A.p.o_r);
+  double* red = at<double>(kCellRed);
+  const double nH = S.nH;
   const int n = d.n, n_r = d.n_r, t = d.t_idx, tid = threadIdx.x, nthr = blockDim.x;
-  const double Tc = q.yp[t], it = 1.0 / Tc;
-  double F = 0.0, U = 0.0;
+  const double Tc = yp[t], it = 1.0 / Tc;
+  // R_j, and R_j d ln k'_j/dT into the table
+  auto rate = [&](int j) {
+    const int ab = __ldg(A.w + A.rx + 2 * j);
+    double R = S.kc[j] * yp[ab & 0xFFFF];
+    if ((uint32_t)ab >> 16 != 0xFFFF) R *= yp[(uint32_t)ab >> 16];
+    return R;
+  };
   for (int j = tid; j < n_r; j += nthr) {
-    const int2 rc = __ldg(d.reac + j);
-    double R = q.kc[j] * q.yp[rc.x];
-    if (rc.y >= 0) R *= q.yp[rc.y];
     const RatePar p = d.rpar[j];
     const int cls = (int)p.w;
-    const double g = (cls == SM_TWO_BODY || cls == SM_DISS_RECOMB) ? (p.y + p.z * it) * it : 0.0;   // d ln k'/dT
-    const double dn = __ldg(d.th_dn + j), Rg = R * g;
-    F = fma(dn, R, F);
-    U = fma(dn, Rg, U);
-    q.tab[j] = Rg;
+    tab[j] = cls == SM_TWO_BODY || cls == SM_DISS_RECOMB ? rate(j) * ((p.y + p.z * it) * it) : 0.0;
   }
-  if (tid == 0) q.tab[n_r] = 0.0;
+  if (tid == 0) tab[n_r] = 0.0;
   __syncthreads();
-  row_sums(A.w, A.n_rsl, A.rp_off, A.rp_ent, A.rp_dst, A.row_ptr, A.n_rlong, A.row_long, q.tab, q.part, q.fs, n);
-  F = cta_sum(F, q.red, 0);
-  U = cta_sum(U, q.red, 1);
-  double xt = 0.0, line = 0.0, dline = 0.0;
-  for (int s = tid; s < n; s += nthr)
-    if (s != t) xt += q.yp[s];
-  for (int e = tid; e < d.n_cool; e += nthr) {
-    const int i = __ldg(d.th_cool + e);
-    const double cl = d.th_L[i] * exp(-d.th_E[i] * it);
-    line = fma(q.yp[i], cl, line);
-    dline = fma(q.yp[i] * cl, d.th_E[i] * it * it, dline);
-  }
-  xt = cta_sum(xt, q.red, 2);
-  line = cta_sum(line, q.red, 3);
+  row_sums(A.w, A.n_rsl, A.rp_off, A.rp_ent, A.rp_dst, A.row, A.row_more, tab, at<double>(A.p.o_part),
+           at<double>(A.p.o_fs), n);
+  sum_parts(0, n_r, [&](int j) { return __ldg(d.th_dn + j) * rate(j); });
+  sum_parts(1, n_r, [&](int j) { return __ldg(d.th_dn + j) * tab[j]; });
+  sum_parts(2, n, [&](int i) { return i == t ? 0.0 : yp[i]; });
+  sum_parts(3, d.n_cool, [&](int q) {
+    const int i = __ldg(d.th_cool + q);
+    return yp[i] * (d.th_L[i] * exp(-d.th_E[i] * it));
+  });
+  sum_parts(4, d.n_cool, [&](int q) {
+    const int i = __ldg(d.th_cool + q);
+    return yp[i] * (d.th_L[i] * exp(-d.th_E[i] * it)) * (d.th_E[i] * it * it);
+  });
   __syncthreads();
-  dline = cta_sum(dline, q.red, 0);
-  const double gJ = q.S->gam_J;
-  if (tid == 0) {
+  const double gJ = S.gam_J;
+  if (tid < 32) {
+    const double F = sum_total(0, n_r), U = sum_total(1, n_r), xt = sum_total(2, n), line = sum_total(3, d.n_cool),
+                 dline = sum_total(4, d.n_cool);
     const double i15x = 1.0 / (1.5 * xt);
-    const double fT = (d.th_heat - q.nH * line - d.th_lam * q.nH * (Tc - d.th_Td) - 1.5 * Tc * F) * i15x;
-    const double w = (-q.nH * dline - d.th_lam * q.nH - 1.5 * F - 1.5 * Tc * U) * i15x;
-    q.red[96] = i15x;
-    q.red[97] = fT / xt;
-    q.red[98] = w;
+    const double fT = (d.th_heat - nH * line - d.th_lam * nH * (Tc - d.th_Td) - 1.5 * Tc * F) * i15x;
+    const double w = (-nH * dline - d.th_lam * nH - 1.5 * F - 1.5 * Tc * U) * i15x;
+    red[kRedX] = i15x;
+    red[kRedX + 1] = fT / xt;
+    red[kRedX + 2] = w;
   }
-  for (int s = tid; s < n; s += nthr) x_put(A, q, s, s == t ? 0.0 : -gJ * q.fs[s]);
-  cell_solve<T>(A, q.P, q.xh, q.xt, q.tmp);
-  const double i15x = q.red[96], fTx = q.red[97], w = q.red[98];
-  double* bz = d.bz + q.oc * d.bpad;
-  double* bgv = d.bgv + q.oc * d.bpad;
-  double vz = 0.0;
-  for (int s = tid; s < n; s += nthr) {
+  solve_prefetch<T>();
+  for (int s = tid; s < n; s += nthr) x_put<T>(A, s, s == t ? 0.0 : -gJ * fs[s]);
+  cell_solve<T>();
+  const double i15x = red[kRedX], fTx = red[kRedX + 1], w = red[kRedX + 2];
+  double* bz = d.bz + S.oc * d.bpad;
+  double* bgv = d.bgv + S.oc * d.bpad;
+  sum_parts(0, n, [&](int s) {
     double z = 0.0, gv = 0.0;
     if (s != t) {
-      z = (double)x_get(A, q, s);
-      if (d.mixed) z /= q.wf[s];
+      z = x_get<T>(A, s);
       const double cl = d.th_L[s] > 0.0 ? d.th_L[s] * exp(-d.th_E[s] * it) : 0.0;
-      gv = (gJ * (-q.nH * cl) - 1.5 * Tc * bgv[s]) * i15x - gJ * fTx;
+      gv = (gJ * (-nH * cl) - 1.5 * Tc * bgv[s]) * i15x - gJ * fTx;
     }
     bz[s] = z;
     bgv[s] = gv;
-    vz = fma(gv, z, vz);
+    return gv * z;
+  });
+  __syncthreads();
+  if (tid < 32) {
+    const double vz = sum_total(0, n);
+    if (tid == 0) d.bs[S.oc] = 1.0 - gJ * w + vz;
   }
-  vz = cta_sum(vz, q.red, 1);
-  if (tid == 0) d.bs[q.oc] = 1.0 - gJ * w + vz;
-  for (int s = tid; s < n; s += nthr) q.ys[s] = q.yp[s];
+  for (int s = tid; s < n; s += nthr) at<double>(A.p.o_ys)[s] = yp[s];
   __syncthreads();
 }
 
 // One BDF attempt of the cell; returns false when the cell stopped before it.
-template <class T, bool TF>
-__device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_ARG) {
+__device__ __forceinline__ void class_begin(int kind) {
+  if (args().timing_kind == kind && threadIdx.x == 0) scalars().t0 = clock64();
+}
+__device__ __forceinline__ void class_end(int kind) {
+  if (args().timing_kind == kind && threadIdx.x == 0) {
+    atomicAdd(args().timing, (double)(clock64() - scalars().t0));
+    atomicAdd(args().timing + 1, 1.0);
+  }
+}
+
+__device__ __forceinline__ void cell_predict() {
+  const Args& A = args();
   const Dev& d = A.d;
-  CellS& S = *q.S;
+  CellS& S = scalars();
   const int n = d.n, tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  long long t0 = 0;
-  auto class_begin = [&](int kind) {
-    if (A.timing_kind == kind && tid == 0) t0 = clock64();
-  };
-  auto class_end = [&](int kind) {
-    if (A.timing_kind == kind && tid == 0) {
-      atomicAdd(A.timing, (double)(clock64() - t0));
-      atomicAdd(A.timing + 1, 1.0);
-    }
-  };
   __syncthreads();   // every thread has taken the last attempt's outcome from S
-  // ---- predict
   class_begin(SM_TIME_PREDICT);
   if (warp < 2) {
     // both warps derive the step from the same scalars; warp 0 forms the
@@ -1144,15 +1347,18 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
     if (S.steps >= d.max_steps) state = 1;
     else if (tnew == t || !(h > 0.0)) state = 2;
     if (warp == 0) {
-      if (state == 3 && nh > 1 && lane <= qq) {
+      // lanes 0..q: the predictor on q + 1 points; lanes 16..: the order
+      // q - 1 predictor on q points, which the error test may rate
+      const int i = lane & 15, np = lane < 16 ? qq + 1 : qq;
+      if (state == 3 && nh > 1 && i < np) {
         double num = 1.0, den = 1.0;
-        const double ti = S.tn[lane];
-        for (int j = 0; j <= qq; ++j)
-          if (j != lane) {
+        const double ti = S.tn[i];
+        for (int j = 0; j < np; ++j)
+          if (j != i) {
             num *= tnew - S.tn[j];
             den *= ti - S.tn[j];
           }
-        S.wts[lane] = num / den;
+        (lane < 16 ? S.wts : S.wlo)[i] = num / den;
       }
     } else {
       double al = 0.0;
@@ -1195,10 +1401,9 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
     }
   }
   __syncthreads();
-  if (S.state != 3) return false;
-  const double h = S.err, tnew = S.tnew;
+  if (S.state != 3) return;
+  const double h = S.err;
   const int qo = S.q, nh = S.nh;
-  const bool refresh = (S.flags & F_REFRESH) != 0;
   {
     double wt[QMAX + 1], al[QMAX + 1];
     const double* Yp[QMAX + 1];
@@ -1209,11 +1414,11 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
       al[i] = S.alpha[i];
       int slot = S.base + i;
       if (slot > QMAX) slot -= QMAX + 1;
-      Yp[i] = q.hist + (int64_t)slot * q.hn;
+      Yp[i] = S.hist + (int64_t)slot * S.hn;
     }
     for (int s = tid; s < n; s += nthr) {
       const double y0 = Yp[0][s];
-      double yp = euler ? y0 + h * d.f0[(int64_t)s * d.ld + q.c] : wt[0] * y0, pv = 0.0;
+      double yp = euler ? y0 + h * d.f0[(int64_t)s * d.ld + S.c] : wt[0] * y0, pv = 0.0;
 #pragma unroll
       for (int i = 1; i <= QMAX; ++i) {
         if (i > qo) break;
@@ -1225,181 +1430,187 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
         if (i > qo) break;
         pv += al[i] * (i == 1 ? y0 : Yp[i - 1][s]);
       }
-      q.yp[s] = yp;
-      q.ys[s] = yp;
-      q.ps[s] = pv;
-      q.ws[s] = 1.0 / (d.rtol * fabs(y0) + d.atol);
+      at<double>(A.p.o_yp)[s] = yp;
+      at<double>(A.p.o_ys)[s] = yp;
+      at<double>(A.p.o_ps)[s] = pv;
+      at<double>(A.p.o_ws)[s] = 1.0 / (d.rtol * fabs(y0) + d.atol);
     }
   }
   if (tid == 0) S.h = h;
   __syncthreads();
   class_end(SM_TIME_PREDICT);
   PHASE_MARK(PH_PREDICT);
-  if (d.therm) cell_th_rates(A, q.kc, q.yp[d.t_idx], q.nH, q.Av, q.chi, false);
-  // ---- Jacobian and factors
-  if (refresh) {
-    class_begin(SM_TIME_REFRESH);
-    cell_refresh<T, TF>(A, q, sm PHASE_PASS);
-    if (d.therm) cell_border<T>(A, q);
-    class_end(SM_TIME_REFRESH);
+}
+
+// One Newton round after the right-hand side: FP64 residual, substitution,
+// update, convergence test.
+template <class T>
+__device__ __forceinline__ void cell_newton() {
+  const Args& A = args();
+  const Dev& d = A.d;
+  CellS& S = scalars();
+  const int n = d.n, tid = threadIdx.x, nthr = blockDim.x;
+  double* ys = at<double>(A.p.o_ys);
+  double* red = at<double>(kCellRed);
+  class_begin(SM_TIME_SOLVE);
+  solve_prefetch<T>();   // in place of the rates, which are done with
+  {
+    const double* ps = at<double>(A.p.o_ps);
+    const double* fs = at<double>(A.p.o_fs);
+    const double a0 = S.alpha[0], inv_a0 = S.inv_a0, h = S.h;
+    for (int s = tid; s < n; s += nthr) {
+      const double b = -(a0 * ys[s] + ps[s] - h * fs[s]) * inv_a0;
+      if (s == d.t_idx) red[kRedX + 3] = b;
+      x_put<T>(A, s, b);
+    }
   }
-  // ---- Newton rounds
-  const double a0 = S.alpha[0], inv_a0 = 1.0 / a0;
-  const double gam = S.gam, gJ = S.gam_J;
-  const double scale = gam != gJ ? 2.0 / (1.0 + gam / gJ) : 1.0;
-  for (int m = 0; m < d.newton_max; ++m) {
-    class_begin(SM_TIME_RHS);
-    if (d.therm && m > 0) cell_th_rates(A, q.kc, q.ys[d.t_idx], q.nH, q.Av, q.chi, false);
-    cell_rhs(A, q.kc, q.ys, q.tab, q.part, q.fs PHASE_PASS);
-    if (d.therm) cell_energy(A, q.ys, q.fs, q.nH, q.red);
-    class_end(SM_TIME_RHS);
-    class_begin(SM_TIME_SOLVE);
-    for (int s = tid; s < n; s += nthr) {
-      const double b = -(a0 * q.ys[s] + q.ps[s] - h * q.fs[s]) * inv_a0;
-      if (s == d.t_idx) q.red[99] = b;
-      x_put(A, q, s, b);
-    }
-    cell_solve<T>(A, q.P, q.xh, q.xt, q.tmp);
-    double bT = 0.0;
-    const double* bz = nullptr;
-    if (d.therm) {
-      const double* bgv = d.bgv + q.oc * d.bpad;
-      bz = d.bz + q.oc * d.bpad;
-      double dot = 0.0;
-      for (int s = tid; s < n; s += nthr) {
-        if (s == d.t_idx) continue;
-        double a = (double)x_get(A, q, s);
-        if (d.mixed) a /= q.wf[s];
-        dot = fma(bgv[s], a, dot);
-      }
-      dot = cta_sum(dot, q.red, 0);
-      if (tid == 0) q.red[100] = (q.red[99] + dot) / d.bs[q.oc];
-      __syncthreads();
-      bT = q.red[100];
-    }
-    double acc = 0.0;
-    for (int s = tid; s < n; s += nthr) {
-      double del = (double)x_get(A, q, s);
-      if (d.mixed) del /= q.wf[s];
-      if (bz) del = s == d.t_idx ? bT : fma(-bz[s], bT, del);
-      del *= scale;
-      q.ys[s] += del;
-      const double v = del * q.ws[s];
-      acc += v * v;
-    }
-    acc = cta_sum(acc, q.red, 1);
-    if (tid == 0) {
-      const double dn = sqrt(acc / n);
-      const int mi = S.m_it;
-      double crate = S.crate;
-      const double dp = S.dprev;
-      bool conv = false, fail = false;
-      if (!isfinite(dn)) {
-        fail = true;
-      } else {
-        if (mi > 0) crate = fmax(0.3 * crate, dn / dp);
-        if (dn * fmin(1.0, crate) <= d.newton_tol) conv = true;
-        else if (mi > 0 && dn > 2.0 * dp) fail = true;
-        else if (mi + 1 >= d.newton_max) fail = true;
-      }
-      S.crate = crate;
-      S.dprev = dn;
-      S.m_it = mi + 1;
-      S.newton_iters += 1;
-      if (conv || fail) S.flags = (S.flags & ~F_NEWTON) | (conv ? F_CONV : F_FAILED);
+  cell_solve<T>();
+  double bT = 0.0;
+  const double* bz = nullptr;
+  if (d.therm) {
+    const double* bgv = d.bgv + S.oc * d.bpad;
+    bz = d.bz + S.oc * d.bpad;
+    sum_parts(0, n, [&](int s) { return s == d.t_idx ? 0.0 : bgv[s] * x_get<T>(A, s); });
+    __syncthreads();
+    if (tid < 32) {
+      const double dot = sum_total(0, n);
+      if (tid == 0) red[kRedX + 4] = (red[kRedX + 3] + dot) / d.bs[S.oc];
     }
     __syncthreads();
-    class_end(SM_TIME_SOLVE);
-    PHASE_MARK(PH_SOLVE);
-    if (!(S.flags & F_NEWTON)) break;
+    bT = red[kRedX + 4];
   }
-  // ---- finish: error test, step / order selection, history
-  class_begin(SM_TIME_FINISH);
-  const bool work = !(S.flags & F_FAILED);
+  const double scale = S.scale;
+  const double* ws = at<double>(A.p.o_ws);
+  sum_parts(1, n, [&](int s) {
+    double del = x_get<T>(A, s);
+    if (bz) del = s == d.t_idx ? bT : fma(-bz[s], bT, del);
+    del *= scale;
+    ys[s] += del;
+    const double v = del * ws[s];
+    return v * v;
+  });
+  __syncthreads();
   double acc = 0.0;
-  if (work)
-    for (int s = tid; s < n; s += nthr) {
-      const double v = (q.ys[s] - q.yp[s]) * q.ws[s];
-      acc += v * v;
+  if (tid < 32) acc = sum_total(1, n);
+  if (tid == 0) {
+    const double dn = sqrt(acc / n);
+    const int mi = S.m_it;
+    double crate = S.crate;
+    const double dp = S.dprev;
+    bool conv = false, fail = false;
+    if (!isfinite(dn)) {
+      fail = true;
+    } else {
+      if (mi > 0) crate = fmax(0.3 * crate, dn / dp);
+      if (dn * fmin(1.0, crate) <= d.newton_tol) conv = true;
+      else if (mi > 0 && dn > 2.0 * dp) fail = true;
+      else if (mi + 1 >= d.newton_max) fail = true;
     }
-  acc = cta_sum(acc, q.red, 0);
-  if (warp == 0) {
-    const double err = work ? (nh >= qo + 1 ? h / (tnew - S.tn[qo]) : 1.0 / (qo + 1)) * sqrt(acc / n) : 0.0;
-    const bool accepted = work && isfinite(err) && err <= 1.0;
-    const int naq = accepted ? S.n_at_q + 1 : 0;
-    const bool lo = accepted && naq >= qo + 1 && qo > 1;
-    const bool hi = accepted && naq >= qo + 1 && qo < d.q_max && (S.flags & F_HAS_EPREV) && nh + 1 >= qo + 2;
-    if (lo && lane < qo) {   // weights of the order q - 1 predictor, a point per lane
-      double num = 1.0, den = 1.0;
-      const double ti = S.tn[lane];
-      for (int j = 0; j < qo; ++j)
-        if (j != lane) {
-          num *= tnew - S.tn[j];
-          den *= ti - S.tn[j];
-        }
-      S.wts[lane] = num / den;
-    }
-    if (lane == 0) {
-      S.err = err;
-      S.state = accepted;
-      S.lo = lo;
-      S.hi = hi;
-    }
+    S.crate = crate;
+    S.dprev = dn;
+    S.m_it = mi + 1;
+    S.newton_iters += 1;
+    if (conv || fail) S.flags = (S.flags & ~F_NEWTON) | (conv ? F_CONV : F_FAILED);
   }
   __syncthreads();
-  const bool accepted = S.state != 0, lo = S.lo != 0, hi = S.hi != 0;
-  double acc_lo = 0.0, acc_hi = 0.0;
-  if (lo || hi) {
+  class_end(SM_TIME_SOLVE);
+  PHASE_MARK(PH_SOLVE);
+}
+
+// Error test, step / order selection, history.
+__device__ __forceinline__ void cell_finish() {
+  const Args& A = args();
+  const Dev& d = A.d;
+  CellS& S = scalars();
+  const int n = d.n, tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const double* ys = at<double>(A.p.o_ys);
+  const double* yp = at<double>(A.p.o_yp);
+  const double* ws = at<double>(A.p.o_ws);
+  const double h = S.h, tnew = S.tnew;
+  const int qo = S.q, nh = S.nh;
+  class_begin(SM_TIME_FINISH);
+  // the error and the neighbouring orders' estimates in one pass (the latter
+  // count only if the step is accepted); one pow call serves the three step
+  // factors, an order per lane
+  const bool work = !(S.flags & F_FAILED);
+  const bool due = work && S.n_at_q + 1 >= qo + 1;
+  const bool lo = due && qo > 1;
+  const bool hi = due && qo < d.q_max && (S.flags & F_HAS_EPREV) && nh + 1 >= qo + 2;
+  double* nv = at<double>(A.p.o_nv);
+  const int N = A.p.nv;
+  if (work)
     for (int s = tid; s < n; s += nthr) {
-      const double yv = q.ys[s], wv = q.ws[s];
+      const double y = ys[s], dy = y - yp[s], wv = ws[s];
+      nv[s] = dy * wv;
       if (lo) {
         double p = 0.0;
         for (int i = 0; i < qo; ++i) {
           int slot = S.base + i;
           if (slot > QMAX) slot -= QMAX + 1;
-          p += S.wts[i] * q.hist[(int64_t)slot * q.hn + s];
+          p += S.wlo[i] * S.hist[(int64_t)slot * S.hn + s];
         }
-        const double v = (yv - p) * wv;
-        acc_lo += v * v;
+        nv[N + s] = (y - p) * wv;
       }
-      if (hi) {
-        const double v = ((yv - q.yp[s]) - q.eprev[s]) * wv;
-        acc_hi += v * v;
-      }
+      if (hi) nv[2 * N + s] = (dy - S.eprev[s]) * wv;
     }
-    acc_lo = cta_sum(acc_lo, q.red, 1);
-    acc_hi = cta_sum(acc_hi, q.red, 2);
-  }
-  if (warp == 0 && accepted) {
-    // step factors of the three candidate orders, one per lane
+  __syncthreads();
+  if (warp == 0) {
+    // eight lanes a norm, each every eighth term, then the eight in order: the
+    // order of the class-by-class finish kernel (the step that follows depends
+    // on the last bit)
+    const int g = lane >> 3;
+    double sq = 0.0;
+    if (g == 0 ? work : g == 1 ? lo : g == 2 ? hi : false) {
+      const double* p = nv + g * N;
+#pragma unroll 8
+      for (int s = lane & 7; s < n; s += 8) sq = fma(p[s], p[s], sq);
+    }
+    double tot = __shfl_sync(kFull, sq, 8 * g);
+#pragma unroll
+    for (int i = 1; i < 8; ++i) tot += __shfl_sync(kFull, sq, 8 * g + i);
+    const double acc = __shfl_sync(kFull, tot, 0), acc_lo = __shfl_sync(kFull, tot, 8), acc_hi = __shfl_sync(kFull, tot, 16);
+    const double err = work ? (nh >= qo + 1 ? h / (tnew - S.tn[qo]) : 1.0 / (qo + 1)) * sqrt(acc / n) : 0.0;
+    const bool accepted = work && isfinite(err) && err <= 1.0;
+    double base = err, ord = qo + 1, fac = 0.9;
+    if (lane == 1 && lo) {
+      base = h / (tnew - S.tn[qo - 1]) * sqrt(acc_lo / n);
+      ord = qo;
+      fac = 0.8;
+    }
+    if (lane == 2 && hi) {
+      base = sqrt(acc_hi / n) / (qo + 2);
+      ord = qo + 2;
+      fac = 0.7;
+    }
+    // accepted: bounded below (a zero error must not stop the step's growth)
     double eta = 0.0;
-    if (lane == 0) eta = 0.9 * pow(fmax(S.err, 1e-10), -1.0 / (qo + 1));
-    if (lane == 1 && lo) eta = 0.8 * pow(fmax(h / (tnew - S.tn[qo - 1]) * sqrt(acc_lo / n), 1e-10), -1.0 / qo);
-    if (lane == 2 && hi) eta = 0.7 * pow(fmax(sqrt(acc_hi / n) / (qo + 2), 1e-10), -1.0 / (qo + 2));
+    if (work && isfinite(err)) eta = fac * pow(accepted ? fmax(base, 1e-10) : base, -1.0 / ord);
     const double e1 = __shfl_sync(kFull, eta, 1), e2 = __shfl_sync(kFull, eta, 2);
     if (lane == 0) {
       int bq = qo;
-      if (lo && e1 > eta) {
+      if (accepted && lo && e1 > eta) {
         eta = e1;
         bq = qo - 1;
       }
-      if (hi && e2 > eta) {
+      if (accepted && hi && e2 > eta) {
         eta = e2;
         bq = qo + 1;
       }
-      S.eta[0] = eta;
+      S.eta = eta;
       S.best_q = bq;
+      S.err = err;
+      S.state = accepted;
     }
   }
   __syncthreads();
-  const bool keep_e = S.best_q == qo;
+  const bool accepted = S.state != 0, keep_e = S.best_q == qo;
   if (accepted) {
     // the newest point takes the slot in front of the ring
     const int slot = S.base == 0 ? QMAX : S.base - 1;
-    double* Y0 = q.hist + (int64_t)slot * q.hn;
+    double* Y0 = S.hist + (int64_t)slot * S.hn;
     for (int s = tid; s < n; s += nthr) {
-      const double yv = q.ys[s];
-      if (keep_e) q.eprev[s] = yv - q.yp[s];
+      const double yv = ys[s];
+      if (keep_e) S.eprev[s] = yv - yp[s];
       Y0[s] = yv;
     }
   }
@@ -1420,7 +1631,7 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
     } else if (!accepted) {
       S.rejects += 1;
       S.crej += 1;
-      const double eta = fmax(0.2, 0.9 * pow(S.err, -1.0 / (qo + 1)));
+      const double eta = fmax(0.2, S.eta);
       if (S.crej >= 3 && qo > 1) {
         S.q = 1;
         S.n_at_q = 0;
@@ -1437,7 +1648,7 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
       S.t = tnew;
       S.steps += 1;
       if (d.record && S.steps <= d.record) {
-        const int64_t o = (int64_t)(S.steps - 1) * d.ld + q.c;
+        const int64_t o = (int64_t)(S.steps - 1) * d.ld + S.c;
         d.log_t[o] = tnew;
         d.log_h[o] = h;
         d.log_q[o] = qo;
@@ -1453,7 +1664,7 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
         S.n_at_q += 1;
         fl |= F_HAS_EPREV;
       }
-      double eta = fmin(S.eta[0], (fl & F_REJECTED) ? 1.0 : d.eta_max);
+      double eta = fmin(S.eta, (fl & F_REJECTED) ? 1.0 : d.eta_max);
       eta = fmax(eta, 0.2);
       if (eta >= 1.0 && eta < d.eta_keep) eta = 1.0;
       S.h = h * eta;
@@ -1471,68 +1682,109 @@ __device__ bool cell_attempt(const Args& A, Cell<T>& q, unsigned char* sm PHASE_
     for (int i = 0; i < nhc; ++i) {
       int slot = S.base + i;
       if (slot > QMAX) slot -= QMAX + 1;
-      for (int s = tid; s < n; s += nthr) dst[i * vs + (int64_t)s * d.ld + q.c] = q.hist[(int64_t)slot * q.hn + s];
-      if (tid == 0) d.ck_t[((int64_t)kk * (QMAX + 1) + i) * d.ld + q.c] = S.tn[i];
+      for (int s = tid; s < n; s += nthr) dst[i * vs + (int64_t)s * d.ld + S.c] = S.hist[(int64_t)slot * S.hn + s];
+      if (tid == 0) d.ck_t[((int64_t)kk * (QMAX + 1) + i) * d.ld + S.c] = S.tn[i];
     }
-    if (tid == 0) d.ck_nh[(int64_t)kk * d.ld + q.c] = nhc;
+    if (tid == 0) d.ck_nh[(int64_t)kk * d.ld + S.c] = nhc;
   }
   class_end(SM_TIME_FINISH);
   PHASE_MARK(PH_FINISH);
+}
+
+// One BDF attempt of the cell; returns false when the cell stopped before or
+// in it.
+template <class T, bool TF>
+__device__ __forceinline__ bool cell_attempt() {
+  const Args& A = args();
+  const Dev& d = A.d;
+  CellS& S = scalars();
+  cell_predict();
+  if (S.state != 3) return false;
+  if (d.therm) cell_th_rates(at<double>(A.p.o_yp)[d.t_idx], false);
+  if (S.flags & F_REFRESH) {
+    class_begin(SM_TIME_REFRESH);
+    cell_refresh<T, TF>();
+    if (d.therm) cell_border<T>();
+    class_end(SM_TIME_REFRESH);
+  }
+  if (threadIdx.x == 0) {
+    const double gam = S.gam, gJ = S.gam_J;
+    S.inv_a0 = 1.0 / S.alpha[0];
+    S.scale = gam != gJ ? 2.0 / (1.0 + gam / gJ) : 1.0;
+  }
+  for (int m = 0; m < d.newton_max; ++m) {
+    class_begin(SM_TIME_RHS);
+    if (d.therm && m > 0) cell_th_rates(at<double>(A.p.o_ys)[d.t_idx], false);
+    cell_rhs();
+    if (d.therm) cell_energy();
+    class_end(SM_TIME_RHS);
+    cell_newton<T>();
+    if (!(S.flags & F_NEWTON)) break;
+  }
+  cell_finish();
   return S.status == SM_CELL_RUNNING;
 }
 
-// Shared-memory views and this CTA's global scratch.
+// Copies the launch's arguments to shared memory and sets up this CTA's global
+// scratch.  Ends with a barrier.
 template <class T>
-__device__ __forceinline__ void cell_views(const Args& A, unsigned char* sm, Cell<T>& q) {
-  const CellPlan& p = A.p;
-  q.S = reinterpret_cast<CellS*>(sm + p.o_s);
-  q.red = reinterpret_cast<double*>(sm + p.o_red);
-  q.yp = reinterpret_cast<double*>(sm + p.o_yp);
-  q.ps = reinterpret_cast<double*>(sm + p.o_ps);
-  q.ws = reinterpret_cast<double*>(sm + p.o_ws);
-  q.wf = reinterpret_cast<double*>(sm + p.o_wf);
-  q.ys = reinterpret_cast<double*>(sm + p.o_ys);
-  q.fs = reinterpret_cast<double*>(sm + p.o_fs);
-  q.tab = reinterpret_cast<double*>(sm + p.o_r);
-  q.part = reinterpret_cast<double*>(sm + p.o_part);
-  q.xh = reinterpret_cast<T*>(sm + p.o_xh);
-  q.xt = reinterpret_cast<T*>(sm + p.o_xt);
-  q.tmp = reinterpret_cast<T*>(sm + p.o_tmp);
-  q.hn = (A.d.n + 31) / 32 * 32;
-  q.kc = A.scratch + (int64_t)blockIdx.x * p.scratch;
-  q.hist = q.kc + (A.d.n_r + 31) / 32 * 32;
-  q.eprev = q.hist + (int64_t)(QMAX + 1) * q.hn;
-  q.mbuf = reinterpret_cast<T*>(q.eprev + q.hn);
+__device__ __forceinline__ void cell_begin(const Args& from) {
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(&from);
+  for (int i = threadIdx.x; i < (int)(sizeof(Args) / 4); i += blockDim.x) reinterpret_cast<uint32_t*>(sm)[i] = src[i];
+  __syncthreads();
+  const Args& A = args();
+  uint16_t* ip = at<uint16_t>(A.p.o_ip);
+  for (int s = threadIdx.x; s < A.d.n; s += blockDim.x) ip[s] = (uint16_t)__ldg(A.w + A.iperm + s);
+  uint16_t* hx = at<uint16_t>(A.p.o_hx);
+  for (int e = threadIdx.x; e < A.d.p_d; e += blockDim.x) hx[e] = (uint16_t)__ldg(A.w + A.hx + e);
+  if (threadIdx.x == 0) {
+    CellS& S = scalars();
+    S.hn = (A.d.n + 31) / 32 * 32;
+    S.kc = A.scratch + (int64_t)blockIdx.x * A.p.scratch;
+    S.hist = S.kc + (A.d.n_r + 31) / 32 * 32;
+    S.eprev = S.hist + (int64_t)(QMAX + 1) * S.hn;
+    S.pbuf = S.eprev + S.hn;
+    S.mbuf = S.pbuf + 32 * A.n_jp;
+#ifdef SM_PHASE_CLOCKS
+    S.ph_t = clock64();
+#endif
+  }
+  __syncthreads();
 }
 
-// Rate coefficients of the cell into this CTA's scratch (cell-major).
-template <class T>
-__device__ __forceinline__ void cell_conditions(const Args& A, Cell<T>& q) {
+// Rate coefficients of cell oc into this CTA's scratch (cell-major), or the
+// cell's conditions with a coupled temperature (to S, by thread 0).
+__device__ __forceinline__ void cell_conditions(int64_t oc) {
+  const Args& A = args();
   const Dev& d = A.d;
+  CellS& S = scalars();
   if (d.therm) {
-    q.nH = d.c_nH[q.oc];
-    q.Av = d.c_Av[q.oc];
-    q.chi = d.c_chi[q.oc];
+    if (threadIdx.x == 0) {
+      S.nH = d.c_nH[oc];
+      S.Av = d.c_Av[oc];
+      S.chi = d.c_chi[oc];
+    }
   } else {
-    for (int j = threadIdx.x; j < d.n_r; j += blockDim.x) q.kc[j] = A.k[(int64_t)j * A.ldk + q.oc];
+    double* kc = S.kc;
+    const double* k = A.k + oc;
+    const int64_t ldk = A.ldk;
+#pragma unroll 8
+    for (int j = threadIdx.x; j < d.n_r; j += blockDim.x) kc[j] = k[(int64_t)j * ldk];
   }
 }
 
-// The 704-thread bound caps a thread at 88 registers, so that two FP32 CTAs of
-// 352 threads (470 species: 11 row blocks) or one FP64 CTA of 704 fill the
-// register file of an SM.
+// 512 threads leave a thread 128 registers: one CTA of 16 warps fills the
+// register file of an SM, or two of 8 warps, whose two cells are in different
+// phases and fill each other's gaps; FP64 (its shared memory holds one CTA per
+// SM) always takes 16 warps.
 template <class T, bool TF>
-__global__ void __launch_bounds__(704, 1) cell_kernel(const __grid_constant__ Args A) {
-  extern __shared__ __align__(16) unsigned char sm[];
+__global__ void __launch_bounds__(kMaxCellThreads, 1) cell_kernel(const __grid_constant__ Args from) {
   __shared__ int sh_c;
+  cell_begin<T>(from);
+  const Args& A = args();
   const Dev& d = A.d;
   const int tid = threadIdx.x, nthr = blockDim.x, n = d.n;
-  Cell<T> q;
-  cell_views<T>(A, sm, q);
-  CellS& S = *q.S;
-#ifdef SM_PHASE_CLOCKS
-  long long ph_t = clock64();
-#endif
+  CellS& S = scalars();
   // per-cell scalars: the double rows t .. alpha and the int rows q ..
   // slot_cell of the state are contiguous with stride ld
   constexpr int kD = 6 + 2 * (QMAX + 1);
@@ -1561,9 +1813,7 @@ __global__ void __launch_bounds__(704, 1) cell_kernel(const __grid_constant__ Ar
     if (c < 0) break;
     if (d.status[c] != SM_CELL_RUNNING) continue;
     __threadfence();
-    q.c = c;
-    q.oc = d.slot_cell[c];
-    q.P = static_cast<T*>(d.lup) + q.oc * d.lup_stride;
+    const int64_t oc = d.slot_cell[c];
     if (tid < kD) {
       const double v = d.t[(int64_t)tid * d.ld + c];
       if (tid == 0) S.t = v;
@@ -1576,6 +1826,9 @@ __global__ void __launch_bounds__(704, 1) cell_kernel(const __grid_constant__ Ar
       else S.alpha[tid - 6 - (QMAX + 1)] = v;
     }
     if (tid == 0) {
+      S.c = c;
+      S.oc = oc;
+      S.P = static_cast<T*>(d.lup) + oc * d.lup_stride;
       S.q = d.q[c];
       S.nh = d.nh[c];
       S.n_at_q = d.n_at_q[c];
@@ -1593,26 +1846,30 @@ __global__ void __launch_bounds__(704, 1) cell_kernel(const __grid_constant__ Ar
       S.base = 0;
       S.best_q = 0;
     }
-    cell_conditions<T>(A, q);
+    cell_conditions(oc);
     const int nh0 = d.nh[c];
     for (int s = tid; s < n; s += nthr) {
       const int64_t o = (int64_t)s * d.ld + c;
-      for (int i = 0; i < nh0; ++i) q.hist[(int64_t)i * q.hn + s] = Yh(d, i)[o];
-      q.eprev[s] = d.eprev[o];
-      q.wf[s] = d.wf[o];
+      for (int i = 0; i < nh0; ++i) S.hist[(int64_t)i * S.hn + s] = Yh(d, i)[o];
+      S.eprev[s] = d.eprev[o];
+      if constexpr (sizeof(T) == 4) {
+        const double wv = d.wf[o];
+        at<double>(A.p.o_wf)[s] = wv;
+        at<double>(A.p.o_wi)[s] = 1.0 / wv;   // (meaningless, and unused, before the first factorisation)
+      }
     }
     __syncthreads();
     if (d.therm) {
       // every coefficient from the current T; the attempt's own passes refresh
       // the T-dependent ones
-      cell_th_rates(A, q.kc, q.hist[d.t_idx], q.nH, q.Av, q.chi, true);
+      cell_th_rates(S.hist[d.t_idx], true);
     }
     PHASE_MARK(PH_LOAD);
     const int before = A.done[c], todo = min(A.slice, A.attempts - before);
     int made = 0;
     bool run = true;
     while (run && made < todo) {
-      run = cell_attempt<T, TF>(A, q, sm PHASE_PASS);
+      run = cell_attempt<T, TF>();
       ++made;
     }
     __syncthreads();
@@ -1634,10 +1891,10 @@ __global__ void __launch_bounds__(704, 1) cell_kernel(const __grid_constant__ Ar
       for (int i = 0; i < S.nh; ++i) {
         int slot = S.base + i;
         if (slot > QMAX) slot -= QMAX + 1;
-        Yh(d, i)[o] = q.hist[(int64_t)slot * q.hn + s];
+        Yh(d, i)[o] = S.hist[(int64_t)slot * S.hn + s];
       }
-      d.eprev[o] = q.eprev[s];
-      d.wf[o] = q.wf[s];
+      d.eprev[o] = S.eprev[s];
+      if constexpr (sizeof(T) == 4) d.wf[o] = at<double>(A.p.o_wf)[s];
     }
     if (tid == 0) {
       d.q[c] = S.q;
@@ -1682,45 +1939,45 @@ __global__ void ring_kernel(int64_t C, int* ring, int* done, int64_t total) {
 // Start of an integration: validates the inputs of each cell, f0 = f(y0) and
 // h0 = min(0.01 / |f0|_wrms, t_end).
 template <class T>
-__global__ void __launch_bounds__(704, 1) cell_init_kernel(const __grid_constant__ Args A, const double* __restrict__ y,
+__global__ void __launch_bounds__(kMaxCellThreads, 1) cell_init_kernel(const __grid_constant__ Args from, const double* __restrict__ y,
                                                            int64_t ldu) {
-  extern __shared__ __align__(16) unsigned char sm[];
+  cell_begin<T>(from);
+  const Args& A = args();
   const Dev& d = A.d;
+  const CellS& S = scalars();
   const int tid = threadIdx.x, nthr = blockDim.x, n = d.n;
-  Cell<T> q;
-  cell_views<T>(A, sm, q);
-#ifdef SM_PHASE_CLOCKS
-  long long ph_t = clock64();
-#endif
+  double* ys = at<double>(A.p.o_ys);
+  const double* fs = at<double>(A.p.o_fs);
   for (int64_t c = blockIdx.x; c < d.C; c += gridDim.x) {
-    q.c = q.oc = c;
     bool ok = true;
     for (int s = tid; s < n; s += nthr) {
       const double v = y[(int64_t)s * ldu + c];
-      q.ys[s] = v;
+      ys[s] = v;
       Yh(d, 0)[(int64_t)s * d.ld + c] = v;
       ok = ok && isfinite(v);
     }
-    cell_conditions<T>(A, q);
+    cell_conditions(c);
     if (!d.therm)
-      for (int j = tid; j < d.n_r; j += nthr) ok = ok && isfinite(q.kc[j]);
+      for (int j = tid; j < d.n_r; j += nthr) ok = ok && isfinite(S.kc[j]);
     __syncthreads();
-    if (d.therm)
-      ok = ok && q.ys[d.t_idx] > 0.0 && isfinite(q.nH) && q.nH > 0.0 && isfinite(q.Av) && isfinite(q.chi);
+    if (d.therm) ok = ok && ys[d.t_idx] > 0.0 && isfinite(S.nH) && S.nH > 0.0 && isfinite(S.Av) && isfinite(S.chi);
     ok = __syncthreads_and(ok);
     if (ok) {
-      if (d.therm) cell_th_rates(A, q.kc, q.ys[d.t_idx], q.nH, q.Av, q.chi, true);
-      cell_rhs(A, q.kc, q.ys, q.tab, q.part, q.fs PHASE_PASS);
-      if (d.therm) cell_energy(A, q.ys, q.fs, q.nH, q.red);
+      if (d.therm) cell_th_rates(ys[d.t_idx], true);
+      cell_rhs();
+      if (d.therm) cell_energy();
     }
-    double acc = 0.0;
+    double* nv = at<double>(A.p.o_nv);
     if (ok)
       for (int s = tid; s < n; s += nthr) {
-        d.f0[(int64_t)s * d.ld + c] = q.fs[s];
-        const double v = q.fs[s] / (d.rtol * fabs(q.ys[s]) + d.atol);
-        acc += v * v;
+        d.f0[(int64_t)s * d.ld + c] = fs[s];
+        nv[s] = fs[s] / (d.rtol * fabs(ys[s]) + d.atol);
       }
-    acc = cta_sum(acc, q.red, 3);
+    __syncthreads();
+    double acc = 0.0;
+    if (ok && tid == 0)   // in order, as the class-by-class path
+#pragma unroll 8
+      for (int s = 0; s < n; ++s) acc = fma(nv[s], nv[s], acc);
     if (tid == 0) {
       d.slot_cell[c] = (int)c;
       d.status[c] = ok ? SM_CELL_RUNNING : SM_CELL_NAN;
@@ -1745,29 +2002,31 @@ __global__ void __launch_bounds__(704, 1) cell_init_kernel(const __grid_constant
       }
     }
     if (d.record && ok)
-      for (int s = tid; s < n; s += nthr) d.ck_Y[(int64_t)s * d.ld + c] = q.ys[s];
+      for (int s = tid; s < n; s += nthr) d.ck_Y[(int64_t)s * d.ld + c] = ys[s];
     __syncthreads();
   }
 }
+
+// The CTA shape of a batch: wide CTAs (one per SM) where every cell gets an SM
+// of its own, narrow ones (two and more per SM) for more cells.
+const CellShape& shape(const CellLaunch& L, int64_t C) { return C > L.sms && L.narrow.ctas > 0 ? L.narrow : L.wide; }
 
 Args make_args(const sm_net* net, const Dev& d, const CellLaunch& L, const double* k, int64_t ldk) {
   const CellProg& p = net->cell;
   Args a{};
   a.d = d;
-  a.p = L.plan;
+  a.p = shape(L, d.C).plan;
   a.w = p.blob.as<int>();
-  a.nb = p.nb; a.pitch = p.pitch;
-  a.n_rsl = p.n_rsl; a.n_part = p.n_part; a.n_rlong = p.n_rlong;
-  a.rp_off = p.rp_off; a.rp_ent = p.rp_ent; a.rp_dst = p.rp_dst; a.row_ptr = p.row_ptr; a.row_long = p.row_long;
+  a.nb = p.nb; a.pitch = p.pitch; a.n_slot = p.n_slot; a.rx = p.rx; a.iperm = p.iperm;
+  a.n_rsl = p.n_rsl; a.rp_off = p.rp_off; a.rp_ent = p.rp_ent; a.rp_dst = p.rp_dst; a.row = p.row; a.row_more = p.row_more;
   a.n_jsl = p.n_jsl; a.n_jl = p.n_jl;
   a.jg_off = p.jg_off; a.jg_ent = p.jg_ent; a.jg_rc = p.jg_rc; a.jg_dst = p.jg_dst; a.jg_grp = p.jg_grp;
-  a.jl_ptr = p.jl_ptr; a.jl_ent = p.jl_ent; a.jl_rc = p.jl_rc; a.jl_dst = p.jl_dst; a.jl_grp = p.jl_grp;
+  a.n_jp = p.n_jp; a.n_jw = p.n_jw; a.jp_ent = p.jp_ent;
+  a.jl_ptr = p.jl_ptr; a.jl_rc = p.jl_rc; a.jd_grp = p.jd_grp; a.jd_ent = p.jd_ent;
   a.n_hlev = net->lu.n_hlev; a.hop = p.hop; a.hterm = p.hterm; a.hop_ptr = p.hop_ptr;
-  a.tg_grp = p.tg_grp; a.tg_off = p.tg_off; a.tg_ent = p.tg_ent; a.tg_pos = p.tg_pos;
-  a.lev_f = p.lev_f; a.lev_b = p.lev_b; a.u12c = p.u12c;
-  a.n_l21 = net->lu.lrhoff.back(); a.n_u12 = net->lu.u12off.back();
-  a.n_vsl = p.n_vsl; a.n_vpart = p.n_vpart; a.n_vlong = p.n_vlong;
-  a.vp_off = p.vp_off; a.vp_ent = p.vp_ent; a.vp_dst = p.vp_dst; a.vrow_ptr = p.vrow_ptr; a.vrow_long = p.vrow_long;
+  a.tg_grp = p.tg_grp; a.tg_ent = p.tg_ent;
+  a.lev_f = p.lev_f; a.lev_b = p.lev_b; a.hx = p.hx;
+  a.n_vsl = p.n_vsl; a.vp_off = p.vp_off; a.vp_ent = p.vp_ent; a.vp_dst = p.vp_dst; a.vrow = p.vrow; a.vrow_more = p.vrow_more;
   a.k = k;
   a.ldk = ldk;
   a.scratch = L.scratch;
@@ -1794,33 +2053,47 @@ const void* kernel_of(const Dev& d) {
 
 }  // namespace
 
-sm_status cell_resident(const Dev& d, const CellPlan& plan, int per_sm_cap, int* ctas) {
-  *ctas = 0;
-  int dev = 0, sms = 0, smem = 0, per = 0;
-  SM_TRY_CUDA(cudaGetDevice(&dev));
-  SM_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  SM_TRY_CUDA(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+sm_status cell_shapes(const sm_net* net, const Dev& d, bool thermal, int per_sm_cap, CellLaunch* L) {
+  L->wide = L->narrow = CellShape{};
+  int smem = 0;
+  SM_TRY_CUDA(cudaDeviceGetAttribute(&L->sms, cudaDevAttrMultiProcessorCount, net->device));
+  SM_TRY_CUDA(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device));
   const void* init = d.mixed ? (const void*)cell_init_kernel<float> : (const void*)cell_init_kernel<double>;
+  const size_t esz = d.mixed ? 4 : 8;
   // per-kernel caps are shared by every state: always the device's limit
-  SM_TRY_CUDA(cudaFuncSetAttribute(kernel_of(d), cudaFuncAttributeMaxDynamicSharedMemorySize, smem - 1024));
-  SM_TRY_CUDA(cudaFuncSetAttribute(init, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  SM_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of(d), 32 * plan.warps, plan.bytes));
-  if (per_sm_cap > 0) per = std::min(per, per_sm_cap);
-  *ctas = sms * per;
+  // (less the kernel's own static shared memory)
+  const int top = smem - 1024;
+  SM_TRY_CUDA(cudaFuncSetAttribute(kernel_of(d), cudaFuncAttributeMaxDynamicSharedMemorySize, top));
+  SM_TRY_CUDA(cudaFuncSetAttribute(init, cudaFuncAttributeMaxDynamicSharedMemorySize, top));
+  auto resident = [&](int warps, CellShape* s) -> sm_status {
+    s->plan = cell_plan(net, esz, d.tf32 != 0, thermal, warps, (size_t)std::max(top, 0));
+    if (!s->plan.ok) return SM_OK;
+    int per = 0;
+    SM_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel_of(d), 32 * warps, s->plan.bytes));
+    if (per_sm_cap > 0) per = std::min(per, per_sm_cap);
+    s->ctas = L->sms * per;
+    return SM_OK;
+  };
+  sm_status r = resident(kMaxCellThreads / 32, &L->wide);
+  if (r != SM_OK) return r;
+  // a tail of few blocks has no work for more than four warps
+  if (net->cell.nb <= 4 && (r = resident(4, &L->narrow)) != SM_OK) return r;
+  if (L->narrow.ctas < 2 * L->sms) L->narrow.ctas = 0;   // alone on an SM the wide one is faster
   return SM_OK;
 }
 
-int64_t cell_ring_ints(int64_t C, int ctas, int attempts) {
-  const int tn = turn(C, ctas, attempts);
+int64_t cell_ring_ints(const CellLaunch& L, int64_t C, int attempts) {
+  const int tn = turn(C, shape(L, C).ctas, attempts);
   return 2 + C * ((attempts + tn - 1) / tn);
 }
 
 sm_status launch_cell_init(const sm_net* net, const Dev& d, const CellLaunch& L, const double* y, int64_t ldu,
                            const double* k, int64_t ldk, cudaStream_t s) {
   const Args a = make_args(net, d, L, k, ldk);
-  const unsigned grid = (unsigned)std::min<int64_t>(d.C, L.ctas);
-  if (d.mixed) cell_init_kernel<float><<<grid, 32 * L.plan.warps, L.plan.bytes, s>>>(a, y, ldu);
-  else cell_init_kernel<double><<<grid, 32 * L.plan.warps, L.plan.bytes, s>>>(a, y, ldu);
+  const CellShape& q = shape(L, d.C);
+  const unsigned grid = (unsigned)std::min<int64_t>(d.C, q.ctas);
+  if (d.mixed) cell_init_kernel<float><<<grid, 32 * q.plan.warps, q.plan.bytes, s>>>(a, y, ldu);
+  else cell_init_kernel<double><<<grid, 32 * q.plan.warps, q.plan.bytes, s>>>(a, y, ldu);
   SM_TRY_CUDA(cudaGetLastError());
   return SM_OK;
 }
@@ -1829,15 +2102,16 @@ sm_status launch_cell_attempts(const sm_net* net, const Dev& d, const CellLaunch
                                int attempts, cudaStream_t s) {
   Args a = make_args(net, d, L, k, ldk);
   a.attempts = attempts;
-  a.slice = turn(d.C, L.ctas, attempts);
-  const int64_t total = cell_ring_ints(d.C, L.ctas, attempts) - 2;
+  const CellShape& q = shape(L, d.C);
+  a.slice = turn(d.C, q.ctas, attempts);
+  const int64_t total = cell_ring_ints(L, d.C, attempts) - 2;
   ring_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(d.C, L.ring, L.done, total);
   SM_TRY_CUDA(cudaGetLastError());
-  const unsigned grid = (unsigned)std::min<int64_t>(d.C, L.ctas);
-  const int threads = 32 * L.plan.warps;
-  if (!d.mixed) cell_kernel<double, false><<<grid, threads, L.plan.bytes, s>>>(a);
-  else if (d.tf32) cell_kernel<float, true><<<grid, threads, L.plan.bytes, s>>>(a);
-  else cell_kernel<float, false><<<grid, threads, L.plan.bytes, s>>>(a);
+  const unsigned grid = (unsigned)std::min<int64_t>(d.C, q.ctas);
+  const int threads = 32 * q.plan.warps;
+  if (!d.mixed) cell_kernel<double, false><<<grid, threads, q.plan.bytes, s>>>(a);
+  else if (d.tf32) cell_kernel<float, true><<<grid, threads, q.plan.bytes, s>>>(a);
+  else cell_kernel<float, false><<<grid, threads, q.plan.bytes, s>>>(a);
   SM_TRY_CUDA(cudaGetLastError());
   return SM_OK;
 }

@@ -1,6 +1,7 @@
 // Index programs of the fused per-cell integrator (see cell.h), built once per
 // network on the host.
 #include <algorithm>
+#include <cstring>
 #include <numeric>
 
 #include "cell.h"
@@ -8,22 +9,31 @@
 namespace {
 
 struct Sliced {
-  std::vector<int32_t> off, ent;   // off in rows of 32 words
-  int32_t slices() const { return (int32_t)off.size() - 1; }
-  Sliced() : off(1, 0) {}
+  std::vector<int32_t> off, ent;   // off: {first row, rows} per slice, rows of 32 words
+  int32_t slices() const { return (int32_t)off.size() / 2; }
 };
 
-// Appends the items (lists of words) named by `order` as slices of 32 lanes.
+// Appends the items (lists of words) named by `order` as slices of 32 lanes,
+// their lengths rounded up to a multiple of `mult`.
 void add_slices(const std::vector<std::vector<int32_t>>& items, const std::vector<int32_t>& order, int32_t pad,
-                Sliced* s) {
+                size_t mult, Sliced* s) {
   for (size_t b = 0; b < order.size(); b += 32) {
     size_t len = 0;
     for (size_t l = b; l < std::min(order.size(), b + 32); ++l) len = std::max(len, items[order[l]].size());
+    len = (len + mult - 1) / mult * mult;
     const size_t base = s->ent.size();
     s->ent.resize(base + 32 * len, pad);
     for (size_t l = b; l < std::min(order.size(), b + 32); ++l)
       for (size_t e = 0; e < items[order[l]].size(); ++e) s->ent[base + 32 * e + (l - b)] = items[order[l]][e];
-    s->off.push_back(s->off.back() + (int32_t)len);
+    s->off.push_back((int32_t)(base / 32));
+    s->off.push_back((int32_t)len);
+  }
+}
+// Empty slices up to a multiple of 4.
+void fill_slices(Sliced* s) {
+  while (s->slices() % 4) {
+    s->off.push_back((int32_t)(s->ent.size() / 32));
+    s->off.push_back(0);
   }
 }
 
@@ -34,36 +44,61 @@ std::vector<int32_t> by_length(const std::vector<std::vector<int32_t>>& items, i
   return o;
 }
 
-// Rows of words cut into pieces; piece results land row-contiguously.
-struct Pieces {
+// Rows of words cut into chains.  A row is summed as the CRS gather sums it:
+// the nonzeros of the matrix in kChunks equal chunks; of a row's part in a
+// chunk the entries 0, 4, 8 .., 1, 5, .. and so on are four sums (what is left
+// past the last four goes to the first), added as (0 + 1) + (2 + 3); then the
+// parts in order.  So a cell's results do not depend on whether its right-hand
+// side comes from here or from the gather, to the last bit, and a longest chain
+// is an eighth of a hub row.
+struct Chains {
   Sliced s;
-  std::vector<int32_t> dst, row_ptr, lng;
-  int32_t n_part = 0;
+  // row: first chain | four chains << 31 | (first further part + 1) << 16;
+  // more: the further parts, a word each (the last one's bit 30 set)
+  std::vector<int32_t> dst, row, more;
+  int32_t n_chain = 0;
+  bool ok = true;
 };
-constexpr int kLongRow = 4;   // rows of more pieces are summed by a warp
+constexpr size_t kChunks = 32;
 
-Pieces cut_rows(const std::vector<std::vector<int32_t>>& rows, int32_t pad) {
-  size_t words = 0;
+Chains cut_rows(const std::vector<std::vector<int32_t>>& rows, int32_t pad) {
+  size_t words = 0, z = 0, ch = 0;
   for (auto& r : rows) words += r.size();
-  // about 24 slices of pieces where the rows are long enough, so that every
-  // warp of a CTA has one or two; pieces of 4 to 32 entries
-  const size_t len = std::min<size_t>(32, std::max<size_t>(4, (words + 767) / 768));
-  Pieces p;
+  Chains p;
   std::vector<std::vector<int32_t>> items;
-  p.row_ptr.push_back(0);
-  for (size_t i = 0; i < rows.size(); ++i) {
-    const size_t n = rows[i].size(), np = (n + len - 1) / len;
-    for (size_t q = 0; q < np; ++q)
-      items.emplace_back(rows[i].begin() + n * q / np, rows[i].begin() + n * (q + 1) / np);
-    p.row_ptr.push_back((int32_t)items.size());
-    if (np > kLongRow) p.lng.push_back((int32_t)i);
+  for (const auto& r : rows) {
+    std::vector<int32_t> parts;
+    for (size_t b = 0; b < r.size() || parts.empty();) {
+      while (ch + 1 < kChunks && z + b >= words * (ch + 1) / kChunks) ++ch;   // the chunk that holds entry z + b
+      const size_t e = ch + 1 < kChunks ? std::min(r.size(), words * (ch + 1) / kChunks - z) : r.size();
+      const size_t m = (e - b) / 4 * 4, first = items.size();
+      items.resize(first + (m > 0 ? 4 : 1));
+      for (size_t q = b; q < e; ++q) items[first + (q - b < m ? (q - b) % 4 : 0)].push_back(r[q]);
+      parts.push_back((int32_t)first | (m > 0 ? (int32_t)0x80000000 : 0));
+      b = std::max(e, b + 1);
+    }
+    z += r.size();
+    if (parts.size() > 1) parts[0] |= (int32_t)(p.more.size() + 1) << 16;
+    p.row.push_back(parts[0]);
+    p.more.insert(p.more.end(), parts.begin() + 1, parts.end());
+    if (parts.size() > 1) p.more.back() |= 1 << 30;
   }
-  p.n_part = (int32_t)items.size();
-  const std::vector<int32_t> order = by_length(items, 0, p.n_part);
-  add_slices(items, order, pad, &p.s);
+  p.n_chain = (int32_t)items.size();
+  p.ok = items.size() < 65535 && p.more.size() < 16383;
+  const std::vector<int32_t> order = by_length(items, 0, p.n_chain);
+  add_slices(items, order, pad, 1, &p.s);
   p.dst = order;
-  p.dst.resize((size_t)p.s.slices() * 32, p.n_part);   // pad lanes write one slot past the pieces
+  p.dst.resize((size_t)p.s.slices() * 32, p.n_chain);   // pad lanes write one slot past the chains
   return p;
+}
+
+// An entry's word: table slot | the upper half of the double c << 16 (c of at
+// most five significant bits).
+int32_t entry(int32_t slot, int c) {
+  const double v = c;
+  uint64_t u;
+  std::memcpy(&u, &v, sizeof u);
+  return (int32_t)((uint32_t)slot | (uint32_t)(u >> 48) << 16);
 }
 
 }  // namespace
@@ -74,7 +109,7 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
   const int32_t n = net->n_s, n_r = net->n_r, h = lu.head, nt = n - h;
   p.nb = (nt + 31) / 32;
   p.pitch = nt | 1;
-  if (n >= 65535 || lu.p_d >= 65535 || (int64_t)32 * p.pitch >= 65536) {
+  if (n >= 65535 || n_r >= 32000 || lu.p_d >= 65535 || (int64_t)kGroup * p.pitch >= 65535 || h >= 32768) {
     *out = std::move(p);
     return;
   }
@@ -85,40 +120,57 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     return o;
   };
   const int32_t kSign = (int32_t)0x80000000;
+  bool fits = true;
+  std::vector<int32_t> slot(n_r);   // first derivative slot of each reaction
+  {
+    std::vector<int32_t> rx;
+    for (int32_t j = 0; j < n_r; ++j) {
+      const int32_t a = net->reac[2 * j], b = net->reac[2 * j + 1];
+      slot[j] = p.n_slot;
+      p.n_slot += b >= 0 ? 2 : 1;
+      rx.push_back((int32_t)((uint32_t)a | (uint32_t)(b >= 0 ? b : 0xFFFF) << 16));
+      rx.push_back(slot[j]);
+    }
+    p.rx = put(rx);
+    p.iperm = put(lu.iperm);
+  }
   // right-hand side
   {
     std::vector<std::vector<int32_t>> rows(n);
     for (int32_t j = 0; j < n_r; ++j)
       for (int32_t q = net->s_colptr[j]; q < net->s_colptr[j + 1]; ++q)
-        for (int c = std::abs((int)net->s_coef[q]); c > 0; --c)
-          rows[net->s_row[q]].push_back(j | (net->s_coef[q] < 0 ? kSign : 0));
-    const Pieces r = cut_rows(rows, n_r);
+        for (int c = net->s_coef[q]; c != 0;) {   // (beyond +-31 in parts of five bits)
+          const int part = std::abs(c) <= 31 ? c : c / 32 * 32;
+          rows[net->s_row[q]].push_back(entry(j, part));
+          c -= part;
+        }
+    const Chains r = cut_rows(rows, entry(n_r, 1));
     p.n_rsl = r.s.slices();
-    p.n_part = r.n_part;
-    p.n_rlong = (int32_t)r.lng.size();
+    p.n_chain = r.n_chain;
     p.rp_off = put(r.s.off);
     p.rp_ent = put(r.s.ent);
     p.rp_dst = put(r.dst);
-    p.row_ptr = put(r.row_ptr);
-    p.row_long = put(r.lng);
+    p.row = put(r.row);
+    p.row_more = put(r.more);
+    fits = fits && r.ok;
   }
   // reactant incidences
   {
     std::vector<std::vector<int32_t>> rows(n);
     for (int32_t j = 0; j < n_r; ++j) {
       const int32_t a = net->reac[2 * j], b = net->reac[2 * j + 1];
-      rows[a].push_back(2 * j);
-      if (b >= 0) rows[b].push_back(2 * j + 1);
+      rows[a].push_back(entry(slot[j], 1));
+      if (b >= 0) rows[b].push_back(entry(slot[j] + 1, 1));
     }
-    const Pieces r = cut_rows(rows, 2 * n_r);
+    const Chains r = cut_rows(rows, entry(p.n_slot, 1));
     p.n_vsl = r.s.slices();
-    p.n_vpart = r.n_part;
-    p.n_vlong = (int32_t)r.lng.size();
+    p.n_vchain = r.n_chain;
     p.vp_off = put(r.s.off);
     p.vp_ent = put(r.s.ent);
     p.vp_dst = put(r.dst);
-    p.vrow_ptr = put(r.row_ptr);
-    p.vrow_long = put(r.lng);
+    p.vrow = put(r.row);
+    p.vrow_more = put(r.more);
+    fits = fits && r.ok;
   }
   // packed index of the head's factors (as in the head program of LUSymbolic)
   std::vector<int32_t> hpos((size_t)n * n, -1);   // (row, column) in elimination order -> packed head index
@@ -139,10 +191,10 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
       }
     }
   }
-  auto tail_pos = [&](int32_t i, int32_t j) { return ((j - h) % 32) * p.pitch + (i - h); };
+  auto tail_pos = [&](int32_t i, int32_t j) { return ((j - h) % kGroup) * p.pitch + (i - h); };
   // Jacobian entries by destination group
   {
-    const int32_t ng = 1 + p.nb;
+    const int32_t ng = 1 + (nt + kGroup - 1) / kGroup;
     std::vector<std::vector<int32_t>> items(net->jp_col.size());
     std::vector<int32_t> rc(items.size()), dst(items.size()), grp(items.size());
     for (int32_t i = 0; i < n; ++i)
@@ -150,23 +202,25 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
         const int32_t l = net->jp_col[e], pi = lu.iperm[i], pl = lu.iperm[l];
         for (int32_t t = net->jt_ptr[e]; t < net->jt_ptr[e + 1]; ++t) {
           const int32_t j = net->jt_rx[t], cf = net->jt_coef[t];
-          const int32_t w = 2 * j + (net->reac[2 * j] == l ? 0 : 1);
+          const int32_t w = slot[j] + (net->reac[2 * j] == l ? 0 : 1);
           for (int c = std::abs(cf); c > 0; --c) items[e].push_back(w | (cf < 0 ? kSign : 0));
         }
         rc[e] = i | (l << 16);
         const bool tail = pi >= h && pl >= h;
-        grp[e] = tail ? 1 + (pl - h) / 32 : 0;
+        grp[e] = tail ? 1 + (pl - h) / kGroup : 0;
         dst[e] = tail ? tail_pos(pi, pl) : hpos[(size_t)pi * n + pl];
       }
-    std::vector<std::vector<int32_t>> in(ng), lng(ng);
+    std::vector<std::vector<int32_t>> in(ng);
+    std::vector<int32_t> lng;
     for (size_t e = 0; e < items.size(); ++e)
-      (items[e].size() > (size_t)kJLong ? lng : in)[grp[e]].push_back((int32_t)e);
+      if (items[e].size() > (size_t)kJShort) lng.push_back((int32_t)e);
+      else in[grp[e]].push_back((int32_t)e);
     Sliced s;
-    std::vector<int32_t> g(1, 0), src, sd, sr, lp(1, 0), le, lr, ld, lg(1, 0);
+    std::vector<int32_t> g(1, 0), sd, sr;
     for (int32_t q = 0; q < ng; ++q) {
       std::stable_sort(in[q].begin(), in[q].end(),
                        [&](int32_t a, int32_t b) { return items[a].size() > items[b].size(); });
-      add_slices(items, in[q], 2 * n_r, &s);
+      add_slices(items, in[q], p.n_slot, 1, &s);
       for (int32_t e : in[q]) {
         sr.push_back(rc[e]);
         sd.push_back(dst[e]);
@@ -174,26 +228,48 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
       sr.resize((size_t)s.slices() * 32, 0);
       sd.resize((size_t)s.slices() * 32, -1);
       g.push_back(s.slices());
-      for (int32_t e : lng[q]) {
-        le.insert(le.end(), items[e].begin(), items[e].end());
-        lp.push_back((int32_t)le.size());
-        lr.push_back(rc[e]);
-        ld.push_back(dst[e]);
+    }
+    fill_slices(&s);
+    sr.resize((size_t)s.slices() * 32, 0);
+    sd.resize((size_t)s.slices() * 32, -1);
+    // long entries, longest first
+    std::stable_sort(lng.begin(), lng.end(), [&](int32_t a, int32_t b) { return items[a].size() > items[b].size(); });
+    std::vector<int32_t> lp(1, 0), lr, pe, dg(1, 0), de;
+    int32_t np = 0;
+    for (int32_t e : lng) {
+      const size_t n_w = items[e].size();
+      const int32_t n_p = (int32_t)((n_w + kJPiece - 1) / kJPiece);
+      pe.resize((size_t)((np + n_p + 31) / 32) * 32 * kJPiece, p.n_slot);
+      for (size_t t = 0; t < n_w; ++t) {
+        const int32_t q = np + (int32_t)(t / kJPiece);
+        pe[(size_t)32 * (kJPiece * (q / 32) + t % kJPiece) + q % 32] = items[e][t];
       }
-      lg.push_back((int32_t)ld.size());
+      np += n_p;
+      lp.push_back(np);
+      lr.push_back(rc[e]);
+      if (n_p > 8) ++p.n_jw;
+    }
+    for (int32_t q = 0; q < ng; ++q) {
+      for (size_t t = 0; t < lng.size(); ++t)
+        if (grp[lng[t]] == q) {
+          de.push_back(dst[lng[t]]);
+          de.push_back((int32_t)t);
+        }
+      dg.push_back((int32_t)de.size() / 2);
     }
     p.n_jsl = s.slices();
-    p.n_jl = (int32_t)ld.size();
+    p.n_jl = (int32_t)lng.size();
+    p.n_jp = (np + 31) / 32;
     p.jg_off = put(s.off);
     p.jg_ent = put(s.ent);
     p.jg_rc = put(sr);
     p.jg_dst = put(sd);
     p.jg_grp = put(g);
+    p.jp_ent = put(pe);
     p.jl_ptr = put(lp);
-    p.jl_ent = put(le);
     p.jl_rc = put(lr);
-    p.jl_dst = put(ld);
-    p.jl_grp = put(lg);
+    p.jd_grp = put(dg);
+    p.jd_ent = put(de);
   }
   // head program, terms packed
   {
@@ -202,9 +278,9 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     for (size_t o = 0; o < nops; ++o) {
       op.push_back(lu.hop[4 * o] | (lu.hop_piv[o] >= 0 ? lu.hop_piv[o] << 16 : (int32_t)0xFFFF0000));
       op.push_back(lu.hop[4 * o + 2]);
+      op.push_back(lu.hop[4 * o + 3]);
+      op.push_back(0);
     }
-    op.push_back(0);
-    op.push_back((int32_t)lu.hterm.size() / 2);
     for (size_t t = 0; t < lu.hterm.size(); t += 2) tm.push_back(lu.hterm[t] | (lu.hterm[t + 1] << 16));
     p.hop = put(op);
     p.hterm = put(tm);
@@ -223,64 +299,74 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
             tgt[(size_t)(j - h) * nt + (i - h)].push_back(hpos[(size_t)i * n + k] | (hpos[(size_t)k * n + j] << 16));
         }
       }
-    Sliced s;
-    std::vector<int32_t> g(1, 0), pos;
-    for (int32_t J = 0; J < p.nb; ++J) {
-      const int32_t lo = 32 * J * nt, hi = std::min(32 * (J + 1), nt) * nt;
+    std::vector<int32_t> g(1, 0), ent;
+    const int32_t pad = lu.p_d | (lu.p_d << 16);
+    for (int32_t J = 0; J * kGroup < nt; ++J) {
+      const int32_t lo = kGroup * J * nt, hi = std::min(kGroup * (J + 1), nt) * nt;
       std::vector<int32_t> o = by_length(tgt, lo, hi);
       while (!o.empty() && tgt[o.back()].empty()) o.pop_back();
-      add_slices(tgt, o, lu.p_d | (lu.p_d << 16), &s);
-      for (int32_t q : o) pos.push_back(tail_pos(h + q % nt, h + q / nt));
-      pos.resize((size_t)s.slices() * 32, -1);
-      g.push_back(s.slices());
+      for (size_t b = 0; b < o.size(); b += 32) {
+        const size_t len = tgt[o[b]].size(), base = ent.size();
+        ent.resize(base + 32 * (len + 1), pad);
+        for (size_t l = 0; l < 32; ++l) {
+          const bool in = b + l < o.size();
+          const int32_t q = in ? o[b + l] : 0;
+          ent[base + l] = (in ? tail_pos(h + q % nt, h + q / nt) : 0xFFFF) | (int32_t)(len << 16);
+          if (in)
+            for (size_t e = 0; e < tgt[q].size(); ++e) ent[base + 32 * (e + 1) + l] = tgt[q][e];
+        }
+      }
+      g.push_back((int32_t)(ent.size() / 32));
     }
-    p.n_tsl = s.slices();
     p.tg_grp = put(g);
-    p.tg_off = put(s.off);
-    p.tg_ent = put(s.ent);
-    p.tg_pos = put(pos);
+    p.tg_ent = put(ent);
   }
   // levels of the head rows and columns of U12
   {
-    std::vector<int32_t> lf(h, 0), lb(h, 0), uc;
+    std::vector<int32_t> lf(h, 0), lb(h, 0), hx(lu.p_d, 0);
     for (size_t l = 0; l + 1 < lu.flev_ptr.size(); ++l)
       for (int32_t q = lu.flev_ptr[l]; q < lu.flev_ptr[l + 1]; ++q) lf[lu.flev[q]] = (int32_t)l;
     for (size_t l = 0; l + 1 < lu.blev_ptr.size(); ++l)
       for (int32_t q = lu.blev_ptr[l]; q < lu.blev_ptr[l + 1]; ++q) lb[lu.blev[q]] = (int32_t)l;
-    for (int32_t k = 0; k < h; ++k)
-      for (int32_t q = lu.uoff[(size_t)k * (p.nb + 1)]; q < lu.uptr[k + 1]; ++q) uc.push_back(lu.uidx[q] - h);
+    for (int32_t i = 0; i < h; ++i)
+      for (int32_t q = lu.lrptr[i]; q < lu.lrptr[i + 1]; ++q) hx[lu.p_l11 + q] = lu.lridx[q];
+    for (size_t q = 0; q < lu.lrhk.size(); ++q) hx[lu.p_l21 + q] = lu.lrhk[q];
+    for (int32_t k = 0; k < h; ++k) {
+      const int32_t u0 = lu.uptr[k], q12 = lu.uoff[(size_t)k * (p.nb + 1)];
+      for (int32_t q = u0; q < q12; ++q) hx[lu.p_u11 + lu.u11ptr[k] + (q - u0)] = lu.uidx[q];
+      for (int32_t q = q12; q < lu.uptr[k + 1]; ++q) hx[lu.p_u12 + lu.u12off[k] + (q - q12)] = lu.uidx[q] - h;
+    }
     p.lev_f = put(lf);
     p.lev_b = put(lb);
-    p.u12c = put(uc);
+    p.hx = put(hx);
   }
-  p.ok = true;
+  p.ok = fits;
   *out = std::move(p);
 }
 
-CellPlan cell_plan(const sm_net* net, size_t esz, bool thermal, size_t smem_max) {
+CellPlan cell_plan(const sm_net* net, size_t esz, bool tf, bool thermal, int warps, size_t smem_max) {
   CellPlan c;
   const CellProg& p = net->cell;
   const LUSymbolic& lu = net->lu;
   const int n = net->n_s, n_r = net->n_r, h = lu.head;
-  // FP64 blocks of 32 rows are shared by two warps (16 columns each)
-  const int lw = p.nb * (esz == 8 ? 2 : 1);
-  c.warps = std::max(8, lw);
-  if (!p.ok || c.warps > 22) return c;   // 22 warps x 88 registers a thread fill the register file
+  c.warps = warps;
+  if (!p.ok) return c;
   auto up = [](size_t v) { return (int)((v + 15) / 16 * 16); };
   c.nv = (n + 1) / 2 * 2;
-  size_t o = 0;
+  size_t o = kCellFixed;
   auto take = [&](size_t bytes) {
     const int at = (int)o;
     o = up(o + bytes);
     return at;
   };
   const size_t vec = sizeof(double) * c.nv;
-  c.o_red = take(sizeof(double) * 4 * 32);
-  c.o_s = take(512);
+  c.o_ip = take(sizeof(uint16_t) * n);
+  c.o_hx = take(sizeof(uint16_t) * lu.p_d);
   c.o_yp = take(vec);
   c.o_ps = take(vec);
   c.o_ws = take(vec);
-  c.o_wf = take(vec);
+  c.o_wf = take(esz == 4 ? vec : 0);
+  c.o_wi = take(esz == 4 ? vec : 0);
   c.o_u = (int)o;
   size_t top = o;
   auto phase = [&]() { top = std::max(top, o); o = c.o_u; };
@@ -290,27 +376,42 @@ CellPlan cell_plan(const sm_net* net, size_t esz, bool thermal, size_t smem_max)
   c.o_fs = take(vec);
   const size_t o_b = o;
   c.o_r = take(sizeof(double) * (n_r + 1));
-  c.o_part = take(sizeof(double) * (std::max(p.n_part, thermal ? p.n_vpart : 0) + 1));
+  c.o_part = take(sizeof(double) * (std::max(p.n_chain, thermal ? p.n_vchain : 0) + 1));
   top = std::max(top, o);
   o = o_b;
   c.o_xh = take(esz * std::max(h, 1));
   c.o_xt = take(esz * 32 * p.nb);
-  c.o_tmp = take(esz * std::max<size_t>(1, std::max(lu.lrhoff.back(), lu.u12off.back())));
+  c.o_hd = take(esz * std::max(lu.p_d, 1));
+  c.o_dg = take(esz * 1024 * p.nb);
+  top = std::max(top, o);
+  o = o_b;
+  c.o_nv = take(3 * vec);   // the error test's terms
   phase();
   // Jacobian gather (vpart of the coupled temperature follows the table)
-  c.o_dr = take(sizeof(double) * (2 * (size_t)n_r + 1));
-  c.o_wsf = take(sizeof(float) * n);
-  c.o_wif = take(sizeof(float) * n);
-  c.o_vp = take(thermal ? sizeof(double) * (p.n_vpart + 1) : 0);
+  c.o_dr = take(sizeof(double) * ((size_t)p.n_slot + 1));
+  c.o_wsf = take(esz == 4 ? sizeof(float) * n : 0);
+  c.o_wif = take(esz == 4 ? sizeof(float) * n : 0);
+  c.o_vp = take(thermal ? sizeof(double) * (p.n_vchain + 1) : 0);
   phase();
   c.o_hv = take(esz * (lu.p_d + 1));
-  c.o_x = take(esz * 32 * p.pitch);
-  c.o_xk = take(esz * 2 * 32 * 40);
-  c.o_ld = take(esz * 2 * 32 * 32);
+  {
+    // assembly tiles: one per warp as far as they fit
+    c.asm_tile = (int)(up(esz * kGroup * p.pitch) / esz);
+    const size_t left = smem_max > o ? smem_max - o : 0;
+    c.asm_warps = std::min<int>(warps, (int)(left / (esz * c.asm_tile)));
+    // (FP32 with 8 warps: two CTAs are to fit an SM)
+    c.o_x = take(esz * c.asm_tile * std::max(c.asm_warps, 1));
+  }
+  phase();
+  c.o_lp = take(esz * 32 * (tf ? 36 : 32) * std::max(p.nb - 1, 1));
+  c.o_up = take(esz * 32 * (tf ? 36 : 32) * std::max(p.nb - 1, 1));
+  c.o_uj = take(esz * (32 * 36 + 32));   // (reads past the last row's end stay inside)
+  c.o_lj = take(esz * (32 * 32 + 32));
+  c.o_next = take(16);
   phase();
   c.bytes = top;
-  c.ok = top <= smem_max;
-  const size_t mb = esz * ((size_t)p.n_jsl * 32 + p.n_jl);
+  c.ok = top <= smem_max && c.asm_warps > 0;
+  const size_t mb = esz * ((size_t)p.n_jsl * 32 + p.n_jl) + sizeof(double) * 32 * (size_t)p.n_jp;
   c.scratch = (int64_t)((n_r + 31) / 32 * 32 + (QMAX_HIST + 1) * (int64_t)((n + 31) / 32 * 32) + (mb + 7) / 8 + 32) / 32 * 32;
   return c;
 }

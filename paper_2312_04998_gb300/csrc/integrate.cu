@@ -2628,16 +2628,13 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   if ((r = st->counters.ensure(sizeof(int) * kCounters)) != SM_OK) return fail(r);
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device);
-  st->cell.plan = cell_plan(net, esz, net->th_t >= 0, (size_t)std::max(0, smem_max - 1024));
-  if (st->cell.plan.ok) {
-    if ((r = cell_resident(d, st->cell.plan, o.refresh_ctas_per_sm, &st->cell.ctas)) != SM_OK) return fail(r);
-    st->fused = st->cell.ctas > 0;
-  }
+  if ((r = cell_shapes(net, d, net->th_t >= 0, o.refresh_ctas_per_sm, &st->cell)) != SM_OK) return fail(r);
+  st->fused = st->cell.wide.ctas > 0;
   if (st->fused) {
     CellLaunch& cl = st->cell;
-    const int64_t ring = 2 + std::max<int64_t>(C, 16 * std::min<int64_t>(C, 8LL * cl.ctas));
-    const int64_t nc = std::min<int64_t>(C, cl.ctas);
-    if ((r = st->cell_scratch.ensure(sizeof(double) * (size_t)(cl.plan.scratch * nc))) != SM_OK) return fail(r);
+    const int64_t ring = 2 + std::max<int64_t>(C, 16 * std::min<int64_t>(C, 8LL * cl.max_ctas()));
+    const int64_t nc = std::min<int64_t>(C, cl.max_ctas());
+    if ((r = st->cell_scratch.ensure(sizeof(double) * (size_t)(cl.wide.plan.scratch * nc))) != SM_OK) return fail(r);
     if ((r = st->ring.ensure(sizeof(int) * (size_t)(ring + ld))) != SM_OK) return fail(r);
     cl.scratch = st->cell_scratch.as<double>();
     cl.ring = st->ring.as<int>();
@@ -3206,7 +3203,9 @@ extern "C" sm_status sm_state_timing(const sm_state* st, int64_t* launches, doub
     SM_TRY_CUDA(cudaMemcpyAsync(v, st->cell.timing, sizeof v, cudaMemcpyDeviceToHost, st->s));
     SM_TRY_CUDA(cudaStreamSynchronize(st->s));
     SM_TRY_CUDA(cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, st->net->device));
-    const double ctas = (double)std::min<int64_t>(std::max<int64_t>(st->C, 1), st->cell.ctas);
+    const CellLaunch& cl = st->cell;
+    const int64_t c = std::max<int64_t>(st->C, 1);
+    const double ctas = (double)std::min<int64_t>(c, c > cl.sms && cl.narrow.ctas > 0 ? cl.narrow.ctas : cl.wide.ctas);
     t += v[0] / (khz > 0 ? khz : 1) / ctas;
     n += (int64_t)v[1];
   }

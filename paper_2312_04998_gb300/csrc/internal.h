@@ -114,39 +114,49 @@ struct LUSymbolic {
       d_jrc, d_uoff, d_lrhead, d_lrhoff, d_u12off, d_lrhk, d_srow;
 };
 
-// Index programs of one network, packed into one device blob of 32-bit words
-// (offsets below in words).  "Sliced" lists hold work items in slices of 32
-// (one item per lane), items sorted by length inside a group and padded to
-// the slice's longest, entry e of lane l of slice s at 32 * (off[s] + e) + l,
-// so that a warp reads its index words in 128-byte lines.
+constexpr int kJShort = 4, kJPiece = 8;   // piece lengths (see CellProg)
+
+// Index programs of one network for the fused integrator (cell.cu), packed
+// into one device blob of 32-bit words (offsets below in words).  "Sliced"
+// lists hold work items in slices of 32 (one item per lane), sorted by length
+// inside a group and padded to the slice's longest; slice s has the pair
+// {first row, rows} at off + 2 s, and entry e of lane l lies at
+// 32 * (first row + e) + l, so a warp reads its index words in 128-byte lines.
 struct CellProg {
   bool ok = false;               // false: the network is outside the programs' index ranges
   int32_t nb = 0;                // 32-wide blocks of the dense tail
   int32_t pitch = 0;             // rows of one tail column in shared memory (odd)
-  // right-hand side: rows of S in pieces; entry = reaction | sign << 31
-  // (coefficients of magnitude m appear m times, pads read slot n_r = 0)
-  int32_t n_rsl = 0, n_part = 0, n_rlong = 0;
-  int32_t rp_off = 0, rp_ent = 0, rp_dst = 0, row_ptr = 0, row_long = 0;
-  // Jacobian: entries by destination group (0 = head, 1 + J = 32-column panel
-  // J of the tail); entry word = derivative slot (2 * reaction + reactant
-  // slot) | sign << 31, pads read slot 2 n_r = 0.  Entries with more than
-  // kJLong words are gathered by a warp each.
-  int32_t n_jsl = 0, n_jl = 0;
+  int32_t n_slot = 0;            // derivative slots: one per reactant
+  int32_t rx = 0;                // per reaction {reactants a | b << 16 (0xFFFF: none), first derivative slot}
+  int32_t iperm = 0;             // per species: position in elimination order
+  // right-hand side: rows of S in chains (see cell_prog.cpp); entry = reaction |
+  // upper half of the double coefficient << 16 (pads read slot n_r = 0)
+  int32_t n_rsl = 0, n_chain = 0;
+  int32_t rp_off = 0, rp_ent = 0, rp_dst = 0, row = 0, row_more = 0;
+  // Jacobian: entries of at most kJShort words in slices by destination group
+  // (0 = head, 1 + G = the tail's columns kGroup G .. of the assembly); entry
+  // word = derivative slot | sign << 31, pads read slot n_slot = 0.  The other
+  // entries ("long") are cut into pieces of at most kJPiece words (slices of
+  // exactly that length), an entry's pieces contiguous: jl_ptr; the first n_jw
+  // have more than 8 pieces.  jd: by group {destination, long entry}.
+  int32_t n_jsl = 0, n_jl = 0, n_jp = 0, n_jw = 0;
   int32_t jg_off = 0, jg_ent = 0, jg_rc = 0, jg_dst = 0, jg_grp = 0;
-  int32_t jl_ptr = 0, jl_ent = 0, jl_rc = 0, jl_dst = 0, jl_grp = 0;
-  // head program (see LUSymbolic): per op {dst | pivot << 16, first term};
-  // term = x | y << 16
+  int32_t jp_ent = 0, jl_ptr = 0, jl_rc = 0, jd_grp = 0, jd_ent = 0;
+  // head program (see LUSymbolic): per op {dst | pivot << 16, first term, end
+  // of terms, 0}; term = x | y << 16
   int32_t hop = 0, hterm = 0, hop_ptr = 0;
-  // head's Schur complement on the tail: targets by panel; term = L21 index |
-  // U12 index << 16, pads read slot p_d = 0
-  int32_t n_tsl = 0;
-  int32_t tg_grp = 0, tg_off = 0, tg_ent = 0, tg_pos = 0;
-  // substitution: levels of the head rows, tail column of each U12 entry
-  int32_t lev_f = 0, lev_b = 0, u12c = 0;
-  // column sums of dn_j dR_j/dx_l (coupled temperature): reactant incidences
-  // in pieces like the right-hand side
-  int32_t n_vsl = 0, n_vpart = 0, n_vlong = 0;
-  int32_t vp_off = 0, vp_ent = 0, vp_dst = 0, vrow_ptr = 0, vrow_long = 0;
+  // head's Schur complement on the tail: targets by column group, in slices of
+  // 32 sorted by length: a row of {position | terms << 16} (0xFFFF: no target),
+  // then the rows of terms (L21 index | U12 index << 16, pads read slot p_d =
+  // 0), in pivot order; tg_grp: first row of each group
+  int32_t tg_grp = 0, tg_ent = 0;
+  // substitution: levels of the head rows; per packed head entry the index in x
+  // (L11, U11, L21: head part, U12: tail part) that it multiplies
+  int32_t lev_f = 0, lev_b = 0, hx = 0;
+  // column sums of dn_j dR_j/dx_l (coupled temperature): derivative slots of
+  // each species in chains like the right-hand side
+  int32_t n_vsl = 0, n_vchain = 0;
+  int32_t vp_off = 0, vp_ent = 0, vp_dst = 0, vrow = 0, vrow_more = 0;
   std::vector<int32_t> h;
   DevArray blob;
 };
