@@ -46,7 +46,7 @@ struct CellS {
   int state, best_q;
   int hn;                         // stride of a history point in scratch
   long long c, oc;                // slot and cell
-  double *kc, *hist, *eprev, *pbuf;   // this CTA's global scratch: k', history ring, last error vector, piece sums
+  double *kc, *hist, *eprev;      // this CTA's global scratch: k', history ring, last error vector
   void *mbuf, *P;                 // Jacobian values in program order (scratch); the cell's packed factors
   double nH, Av, chi;             // conditions (coupled temperature)
   long long t0, ph_t;             // clocks of the timed class and the last phase mark
@@ -59,7 +59,7 @@ struct Args {
   const int* w;            // index programs (CellProg blob)
   int nb, pitch, n_slot, rx, iperm;
   int n_rsl, rp_off, rp_ent, rp_dst, row, row_more;
-  int n_jsl, n_jl, jg_off, jg_ent, jg_rc, jg_dst, jg_grp, n_jp, n_jw, jp_ent, jl_ptr, jl_rc, jd_grp, jd_ent;
+  int n_jsl, n_jl, n_jw, jg_off, jg_ent, jg_rc, jg_dst, jg_grp, jl_off, jl_ent, jl_rc, jd_grp, jd_ent;
   int n_hlev, hop, hterm, hop_ptr;
   int tg_grp, tg_ent;
   int lev_f, lev_b, hx;
@@ -134,8 +134,6 @@ __device__ __forceinline__ void mma_tf32(float (&c)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ void cp16(void* smem, const void* g) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(g) : "memory");
 }
-// The CTA's barrier, for code whose warps reach it from different places.
-__device__ __forceinline__ void cta_bar() { asm volatile("bar.sync 0;" ::: "memory"); }
 // A plain load that stays where it is written: left to itself the compiler
 // forms the addresses of a whole block of strided loads first, and spills.
 __device__ __forceinline__ float ld_here(const float* p) {
@@ -149,10 +147,6 @@ __device__ __forceinline__ double ld_here(const double* p) {
   return v;
 }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-__device__ __forceinline__ double flip(double v, int word) {   // v, negated when bit 31 of word is set
-  return __hiloint2double(__double2hiint(v) ^ (word & 0x80000000), __double2loint(v));
-}
 
 // Sums of rows cut into chains (see Chains in cell_prog.cpp): a chain per lane,
 // a slice of 32 chains per warp, longest first, so that the warps of each
@@ -286,13 +280,19 @@ __device__ __forceinline__ void cell_energy() {
   const int n = d.n;
   sum_parts(0, n, [&](int i) { return i == t ? 0.0 : y[i]; });
   sum_parts(1, n, [&](int i) { return i == t ? 0.0 : fs[i]; });
-  sum_parts(2, d.n_cool, [&](int q) {
-    const int i = __ldg(d.th_cool + q);
-    return y[i] * (d.th_L[i] * exp(-d.th_E[i] / T));
-  });
   __syncthreads();
   if (threadIdx.x < 32) {
-    const double xt = sum_total(0, n), F = sum_total(1, n), line = sum_total(2, d.n_cool);
+    const double xt = sum_total(0, n), F = sum_total(1, n);
+    double line = 0.0;   // in order
+    for (int q0 = 0; q0 < d.n_cool; q0 += 32) {
+      double v = 0.0, yv = 0.0;
+      if (q0 + (int)threadIdx.x < d.n_cool) {
+        const int i = __ldg(d.th_cool + q0 + threadIdx.x);
+        v = d.th_L[i] * exp(-d.th_E[i] / T);
+        yv = y[i];
+      }
+      for (int q = 0; q < min(32, d.n_cool - q0); ++q) line = fma(__shfl_sync(kFull, yv, q), __shfl_sync(kFull, v, q), line);
+    }
     if (threadIdx.x == 0)
       fs[t] = (d.th_heat - nH * line - d.th_lam * nH * (T - d.th_Td) - 1.5 * T * F) / (1.5 * xt);
   }
@@ -1053,12 +1053,12 @@ __device__ __forceinline__ void cell_jacobian() {
   const double* kc = S.kc;
   T* mbuf = static_cast<T*>(S.mbuf);
   const double gamma = S.gam;
-  // -gamma dR_j/dx for every reactant
+  // dR_j/dx for every reactant
   const int2* rx = reinterpret_cast<const int2*>(w + A.rx);
 #pragma unroll 4
   for (int j = tid; j < n_r; j += nthr) {
     const int2 r = __ldg(rx + j);
-    const double kv = -gamma * kc[j];
+    const double kv = kc[j];
     const int b = (uint32_t)r.x >> 16;
     dR[r.y] = b != 0xFFFF ? kv * yp[b] : kv;
     if (b != 0xFFFF) dR[r.y + 1] = kv * yp[r.x & 0xFFFF];
@@ -1078,9 +1078,9 @@ __device__ __forceinline__ void cell_jacobian() {
   __syncthreads();
   auto m_value = [&](int rc, double acc) {   // M (W M W^-1 in FP32) at (row species, column species)
     const int i = rc & 0xFFFF, l = (uint32_t)rc >> 16;
-    if (i == l) acc += 1.0;
-    if constexpr (sizeof(T) == 4) return T((float)acc * (wsf[i] * wif[l]));
-    else return T(acc);
+    const double m = fma(-gamma, acc, i == l ? 1.0 : 0.0);
+    if constexpr (sizeof(T) == 4) return T((float)m * (wsf[i] * wif[l]));
+    else return T(m);
   };
   // entries of at most kJShort words, four slices at a time, all their index
   // words in flight at once
@@ -1108,47 +1108,45 @@ __device__ __forceinline__ void cell_jacobian() {
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        double a = flip(dR[t[0][u] & 0x7FFFFFFF], t[0][u]);
+        double a = 0.0;
 #pragma unroll
-        for (int e = 1; e < kJShort; ++e)
-          if (e < len[u]) a += flip(dR[t[e][u] & 0x7FFFFFFF], t[e][u]);
+        for (int e = 0; e < kJShort; ++e)
+          if (e < len[u]) a = fma(__hiloint2double(t[e][u] & 0xFFFF0000, 0), dR[t[e][u] & 0xFFFF], a);
         if (len[u] > 0) mbuf[32 * (s + u) + lane] = m_value(rc[u], a);
       }
     }
   }
-  // the entries of more words, in pieces of at most kJPiece
-  for (int s = nw - 1 - warp; s < A.n_jp; s += nw) {
-    int t[kJPiece];
+  // the entries of more words: a chain per lane, of up to kJLong words of an
+  // entry or of every 32nd word of a longer one
+  {
+    const int2* off = reinterpret_cast<const int2*>(w + A.jl_off);
+    for (int s = nw - 1 - warp; s < A.n_jl; s += nw) {
+      const int2 mt = __ldg(off + s);
+      const int* q = w + A.jl_ent + 32 * mt.x + lane;
+      const int m = mt.y, rc = __ldg(w + A.jl_rc + 32 * s + lane);
+      int t[4];
 #pragma unroll
-    for (int e = 0; e < kJPiece; ++e) t[e] = __ldg(w + A.jp_ent + 32 * (kJPiece * s + e) + lane);
-    double a = flip(dR[t[0] & 0x7FFFFFFF], t[0]), b = flip(dR[t[1] & 0x7FFFFFFF], t[1]);
+      for (int u = 0; u < 4; ++u) t[u] = u < m ? __ldg(q + 32 * u) : 0;
+      double a = 0.0;
+      for (int e = 0; e < m; e += 4) {
+        int nx[4];
 #pragma unroll
-    for (int e = 2; e < kJPiece; e += 2) {
-      a += flip(dR[t[e] & 0x7FFFFFFF], t[e]);
-      b += flip(dR[t[e + 1] & 0x7FFFFFFF], t[e + 1]);
+        for (int u = 0; u < 4; ++u) nx[u] = e + 4 + u < m ? __ldg(q + 32 * (e + 4 + u)) : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (e + u < m) a = fma(__hiloint2double(t[u] & 0xFFFF0000, 0), dR[t[u] & 0xFFFF], a);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t[u] = nx[u];
+      }
+      if (s < A.n_jw) a = warp_sum(a);
+      mbuf[32 * (A.n_jsl + s) + lane] = m_value(rc, a);
     }
-    S.pbuf[32 * s + lane] = a + b;
-  }
-  __syncthreads();
-  // and their pieces (rows of pieces: longest first; more than 8 a warp each)
-  for (int q = warp; q < A.n_jw; q += nw) {
-    const int p1 = __ldg(w + A.jl_ptr + q + 1);
-    double a = 0.0;
-    for (int p = __ldg(w + A.jl_ptr + q) + lane; p < p1; p += 32) a += S.pbuf[p];
-    a = warp_sum(a);
-    if (lane == 0) mbuf[32 * A.n_jsl + q] = m_value(__ldg(w + A.jl_rc + q), a);
-  }
-  for (int q = A.n_jw + tid; q < A.n_jl; q += nthr) {
-    const int p0 = __ldg(w + A.jl_ptr + q), p1 = __ldg(w + A.jl_ptr + q + 1);
-    double a = 0.0;
-    for (int p = p0; p < p1; ++p) a += S.pbuf[p];
-    mbuf[32 * A.n_jsl + q] = m_value(__ldg(w + A.jl_rc + q), a);
   }
   if (d.therm) {
-    // gamma_J sum_j dn_j dR_j/dx_l per species, kept in the border's row
+    // sum_j dn_j dR_j/dx_l per species, kept in the border's row
     __syncthreads();
     for (int j = tid; j < n_r; j += nthr) {
-      const double dn = -__ldg(d.th_dn + j);
+      const double dn = __ldg(d.th_dn + j);
       const int2 r = __ldg(rx + j);
       dR[r.y] *= dn;
       if ((uint32_t)r.x >> 16 != 0xFFFF) dR[r.y + 1] *= dn;
@@ -1301,16 +1299,16 @@ __device__ __forceinline__ void cell_border() {
     if (s != t) {
       z = x_get<T>(A, s);
       const double cl = d.th_L[s] > 0.0 ? d.th_L[s] * exp(-d.th_E[s] * it) : 0.0;
-      gv = (gJ * (-nH * cl) - 1.5 * Tc * bgv[s]) * i15x - gJ * fTx;
+      gv = (-nH * cl - 1.5 * Tc * bgv[s]) * i15x - fTx;
     }
     bz[s] = z;
-    bgv[s] = gv;
+    bgv[s] = gJ * gv;
     return gv * z;
   });
   __syncthreads();
   if (tid < 32) {
     const double vz = sum_total(0, n);
-    if (tid == 0) d.bs[S.oc] = 1.0 - gJ * w + vz;
+    if (tid == 0) d.bs[S.oc] = 1.0 - gJ * w + gJ * vz;
   }
   for (int s = tid; s < n; s += nthr) at<double>(A.p.o_ys)[s] = yp[s];
   __syncthreads();
@@ -1743,8 +1741,7 @@ __device__ __forceinline__ void cell_begin(const Args& from) {
     S.kc = A.scratch + (int64_t)blockIdx.x * A.p.scratch;
     S.hist = S.kc + (A.d.n_r + 31) / 32 * 32;
     S.eprev = S.hist + (int64_t)(QMAX + 1) * S.hn;
-    S.pbuf = S.eprev + S.hn;
-    S.mbuf = S.pbuf + 32 * A.n_jp;
+    S.mbuf = S.eprev + S.hn;
 #ifdef SM_PHASE_CLOCKS
     S.ph_t = clock64();
 #endif
@@ -2021,8 +2018,8 @@ Args make_args(const sm_net* net, const Dev& d, const CellLaunch& L, const doubl
   a.n_rsl = p.n_rsl; a.rp_off = p.rp_off; a.rp_ent = p.rp_ent; a.rp_dst = p.rp_dst; a.row = p.row; a.row_more = p.row_more;
   a.n_jsl = p.n_jsl; a.n_jl = p.n_jl;
   a.jg_off = p.jg_off; a.jg_ent = p.jg_ent; a.jg_rc = p.jg_rc; a.jg_dst = p.jg_dst; a.jg_grp = p.jg_grp;
-  a.n_jp = p.n_jp; a.n_jw = p.n_jw; a.jp_ent = p.jp_ent;
-  a.jl_ptr = p.jl_ptr; a.jl_rc = p.jl_rc; a.jd_grp = p.jd_grp; a.jd_ent = p.jd_ent;
+  a.n_jw = p.n_jw; a.jl_off = p.jl_off; a.jl_ent = p.jl_ent;
+  a.jl_rc = p.jl_rc; a.jd_grp = p.jd_grp; a.jd_ent = p.jd_ent;
   a.n_hlev = net->lu.n_hlev; a.hop = p.hop; a.hterm = p.hterm; a.hop_ptr = p.hop_ptr;
   a.tg_grp = p.tg_grp; a.tg_ent = p.tg_ent;
   a.lev_f = p.lev_f; a.lev_b = p.lev_b; a.hx = p.hx;

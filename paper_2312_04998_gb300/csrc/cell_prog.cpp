@@ -119,7 +119,6 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     p.h.resize((p.h.size() + 31) / 32 * 32, 0);   // every list starts on a 128-byte line
     return o;
   };
-  const int32_t kSign = (int32_t)0x80000000;
   bool fits = true;
   std::vector<int32_t> slot(n_r);   // first derivative slot of each reaction
   {
@@ -203,7 +202,11 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
         for (int32_t t = net->jt_ptr[e]; t < net->jt_ptr[e + 1]; ++t) {
           const int32_t j = net->jt_rx[t], cf = net->jt_coef[t];
           const int32_t w = slot[j] + (net->reac[2 * j] == l ? 0 : 1);
-          for (int c = std::abs(cf); c > 0; --c) items[e].push_back(w | (cf < 0 ? kSign : 0));
+          for (int v = cf; v != 0;) {
+            const int part = std::abs(v) <= 31 ? v : v / 32 * 32;
+            items[e].push_back(entry(w, part));
+            v -= part;
+          }
         }
         rc[e] = i | (l << 16);
         const bool tail = pi >= h && pl >= h;
@@ -220,7 +223,7 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     for (int32_t q = 0; q < ng; ++q) {
       std::stable_sort(in[q].begin(), in[q].end(),
                        [&](int32_t a, int32_t b) { return items[a].size() > items[b].size(); });
-      add_slices(items, in[q], p.n_slot, 1, &s);
+      add_slices(items, in[q], entry(p.n_slot, 1), 1, &s);
       for (int32_t e : in[q]) {
         sr.push_back(rc[e]);
         sd.push_back(dst[e]);
@@ -232,41 +235,51 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     fill_slices(&s);
     sr.resize((size_t)s.slices() * 32, 0);
     sd.resize((size_t)s.slices() * 32, -1);
-    // long entries, longest first
+    // long entries, longest first: a slice each while they have more than kJLong
+    // words (dealt to the lanes in turn), else a slice of 32
     std::stable_sort(lng.begin(), lng.end(), [&](int32_t a, int32_t b) { return items[a].size() > items[b].size(); });
-    std::vector<int32_t> lp(1, 0), lr, pe, dg(1, 0), de;
-    int32_t np = 0;
-    for (int32_t e : lng) {
-      const size_t n_w = items[e].size();
-      const int32_t n_p = (int32_t)((n_w + kJPiece - 1) / kJPiece);
-      pe.resize((size_t)((np + n_p + 31) / 32) * 32 * kJPiece, p.n_slot);
-      for (size_t t = 0; t < n_w; ++t) {
-        const int32_t q = np + (int32_t)(t / kJPiece);
-        pe[(size_t)32 * (kJPiece * (q / 32) + t % kJPiece) + q % 32] = items[e][t];
+    Sliced ls;
+    std::vector<int32_t> lr, at(lng.size()), dg(1, 0), de;
+    size_t t = 0;
+    for (; t < lng.size() && items[lng[t]].size() > (size_t)kJLong; ++t) {
+      const std::vector<int32_t>& it = items[lng[t]];
+      std::vector<std::vector<int32_t>> lanes(32);
+      std::vector<int32_t> all(32);
+      std::iota(all.begin(), all.end(), 0);
+      for (size_t e = 0; e < it.size(); ++e) lanes[e % 32].push_back(it[e]);
+      at[t] = 32 * ls.slices();
+      add_slices(lanes, all, entry(p.n_slot, 1), 1, &ls);
+      lr.resize((size_t)32 * ls.slices(), 0);
+      lr[at[t]] = rc[lng[t]];
+    }
+    p.n_jw = ls.slices();
+    for (; t < lng.size(); t += 32) {
+      const size_t m = std::min<size_t>(32, lng.size() - t);
+      const int32_t base = 32 * ls.slices();
+      add_slices(items, std::vector<int32_t>(lng.begin() + t, lng.begin() + t + m), entry(p.n_slot, 1), 1, &ls);
+      lr.resize((size_t)32 * ls.slices(), 0);
+      for (size_t l = 0; l < m; ++l) {
+        at[t + l] = base + (int32_t)l;
+        lr[base + l] = rc[lng[t + l]];
       }
-      np += n_p;
-      lp.push_back(np);
-      lr.push_back(rc[e]);
-      if (n_p > 8) ++p.n_jw;
     }
     for (int32_t q = 0; q < ng; ++q) {
-      for (size_t t = 0; t < lng.size(); ++t)
-        if (grp[lng[t]] == q) {
-          de.push_back(dst[lng[t]]);
-          de.push_back((int32_t)t);
+      for (size_t l = 0; l < lng.size(); ++l)
+        if (grp[lng[l]] == q) {
+          de.push_back(dst[lng[l]]);
+          de.push_back(at[l]);
         }
       dg.push_back((int32_t)de.size() / 2);
     }
     p.n_jsl = s.slices();
-    p.n_jl = (int32_t)lng.size();
-    p.n_jp = (np + 31) / 32;
+    p.n_jl = ls.slices();
     p.jg_off = put(s.off);
     p.jg_ent = put(s.ent);
     p.jg_rc = put(sr);
     p.jg_dst = put(sd);
     p.jg_grp = put(g);
-    p.jp_ent = put(pe);
-    p.jl_ptr = put(lp);
+    p.jl_off = put(ls.off);
+    p.jl_ent = put(ls.ent);
     p.jl_rc = put(lr);
     p.jd_grp = put(dg);
     p.jd_ent = put(de);
@@ -411,7 +424,7 @@ CellPlan cell_plan(const sm_net* net, size_t esz, bool tf, bool thermal, int war
   phase();
   c.bytes = top;
   c.ok = top <= smem_max && c.asm_warps > 0;
-  const size_t mb = esz * ((size_t)p.n_jsl * 32 + p.n_jl) + sizeof(double) * 32 * (size_t)p.n_jp;
+  const size_t mb = esz * 32 * ((size_t)p.n_jsl + p.n_jl);
   c.scratch = (int64_t)((n_r + 31) / 32 * 32 + (QMAX_HIST + 1) * (int64_t)((n + 31) / 32 * 32) + (mb + 7) / 8 + 32) / 32 * 32;
   return c;
 }

@@ -114,7 +114,7 @@ struct LUSymbolic {
       d_jrc, d_uoff, d_lrhead, d_lrhoff, d_u12off, d_lrhk, d_srow;
 };
 
-constexpr int kJShort = 4, kJPiece = 8;   // piece lengths (see CellProg)
+constexpr int kJShort = 4;   // (see CellProg)
 
 // Index programs of one network for the fused integrator (cell.cu), packed
 // into one device blob of 32-bit words (offsets below in words).  "Sliced"
@@ -135,13 +135,13 @@ struct CellProg {
   int32_t rp_off = 0, rp_ent = 0, rp_dst = 0, row = 0, row_more = 0;
   // Jacobian: entries of at most kJShort words in slices by destination group
   // (0 = head, 1 + G = the tail's columns kGroup G .. of the assembly); entry
-  // word = derivative slot | sign << 31, pads read slot n_slot = 0.  The other
-  // entries ("long") are cut into pieces of at most kJPiece words (slices of
-  // exactly that length), an entry's pieces contiguous: jl_ptr; the first n_jw
-  // have more than 8 pieces.  jd: by group {destination, long entry}.
-  int32_t n_jsl = 0, n_jl = 0, n_jp = 0, n_jw = 0;
+  // word = derivative slot | upper half of the double coefficient << 16, pads
+  // read slot n_slot = 0.  Of the other entries ("long") those of more than
+  // kJLong words have a slice each (the first n_jw, word e in lane e mod 32).
+  // jd: by group {destination, 32 x slice + lane of the long entry}.
+  int32_t n_jsl = 0, n_jl = 0, n_jw = 0;
   int32_t jg_off = 0, jg_ent = 0, jg_rc = 0, jg_dst = 0, jg_grp = 0;
-  int32_t jp_ent = 0, jl_ptr = 0, jl_rc = 0, jd_grp = 0, jd_ent = 0;
+  int32_t jl_off = 0, jl_ent = 0, jl_rc = 0, jd_grp = 0, jd_ent = 0;
   // head program (see LUSymbolic): per op {dst | pivot << 16, first term, end
   // of terms, 0}; term = x | y << 16
   int32_t hop = 0, hterm = 0, hop_ptr = 0;
