@@ -112,6 +112,8 @@ void release_all(sm_net* net) {
   lu.d_iperm.release();
   net->d_reac.release();
   net->d_rate.release();
+  net->d_ratefix.release();
+  net->d_ratetab.release();
   net->d_jp_ptr.release();
   net->d_jt_ptr.release();
   net->d_jt_word.release();

@@ -189,6 +189,7 @@ struct sm_net {
   // Device copies used by the kernels.
   DevArray d_reac;        // int2 per reaction: reactant indices (-1 = none)
   DevArray d_rate;        // RatePar per reaction: (log alpha | alpha, beta, gamma, class)
+  DevArray d_ratefix, d_ratetab;           // the same for the fixed-point exponential (see kern_rates.cu)
   DevArray d_jp_ptr, d_jt_ptr, d_jt_word;  // Jacobian gather lists
   DevArray d_jt_slot;                      // (reaction | coef << 24, reactant slot) per term
   std::vector<int32_t> jlong;              // Jacobian entries with more than kJLong terms
@@ -217,6 +218,14 @@ sm_status build_format(const sm_net* net, int32_t fmt, int32_t order, int32_t C,
 sm_status integ_format(sm_net* net, int32_t order);
 
 // Kernel launchers (one per .cu file).
+struct __align__(32) RateFix {   // a reaction's rate for the fixed-point exponential; OTHER: from its RatePar
+  enum { OTHER, TWO_BODY, PHOTO };
+  double beta = 0.0, gamma = 0.0;
+  long long la = 0;   // log2 alpha
+  long long kind = OTHER;
+};
+std::vector<double> rate_table();
+std::vector<RateFix> rate_fixed(const sm_net* net, const std::vector<double>& table);
 sm_status launch_rates(const sm_net* net, int64_t C, const double* T, const double* nH,
                        const double* Av, const double* chi, double zeta, double* k, int64_t ld, cudaStream_t s);
 sm_status launch_rhs(const sm_net* net, int64_t C, const double* k, const double* y,

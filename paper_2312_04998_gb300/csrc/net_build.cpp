@@ -724,6 +724,10 @@ sm_status net_upload(sm_net* net) {
   if ((st = rhs_prepare_device(net->device)) != SM_OK) return st;
   if ((st = net->d_reac.upload(reac2.data(), reac2.size() * 4)) != SM_OK) return st;
   if ((st = net->d_rate.upload(rate.data(), rate.size() * 8)) != SM_OK) return st;
+  static const std::vector<double> table = rate_table();
+  const std::vector<RateFix> fix = rate_fixed(net, table);
+  if ((st = net->d_ratefix.upload(fix.data(), fix.size() * sizeof(RateFix))) != SM_OK) return st;
+  if ((st = net->d_ratetab.upload(table.data(), table.size() * 8)) != SM_OK) return st;
   // Jacobian gather words: reaction (low 23 bits) | partner+1 ... packed as two
   // int32 per term: (reaction | coef << 24, partner)
   std::vector<int32_t> words(2 * net->jt_rx.size());
