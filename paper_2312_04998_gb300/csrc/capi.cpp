@@ -79,9 +79,6 @@ void release_all(sm_net* net) {
   LUSymbolic& lu = net->lu;
   lu.d_lrptr.release();
   lu.d_lridx.release();
-  lu.d_ucptr.release();
-  lu.d_ucidx.release();
-  lu.d_jrc.release();
   lu.d_uoff.release();
   lu.d_lrhead.release();
   lu.d_lrhoff.release();
@@ -107,17 +104,13 @@ void release_all(sm_net* net) {
   lu.d_lidx.release();
   lu.d_uptr.release();
   lu.d_uidx.release();
-  lu.d_jpos.release();
   lu.d_perm.release();
   lu.d_iperm.release();
   net->d_reac.release();
   net->d_rate.release();
   net->d_ratefix.release();
   net->d_ratetab.release();
-  net->d_jp_ptr.release();
-  net->d_jt_ptr.release();
-  net->d_jt_word.release();
-  net->d_jchunk.release();
+  net->jac.blob.release();
   net->d_status.release();
   net->d_scratch.release();
 }

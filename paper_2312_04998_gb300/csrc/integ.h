@@ -59,10 +59,9 @@ struct Dev {
   const int4* hop;
   const int2* hterm;
   int n_hlev;
-  const int *perm, *iperm, *lptr, *lidx, *uptr, *uidx, *lrptr, *lridx, *ucptr, *ucidx, *jp_ptr, *jt_ptr,
-      *jpos, *jrc, *uoff, *lrhead, *lrhoff, *u12off, *lrhk, *srow;
+  const int *perm, *iperm, *lptr, *lidx, *uptr, *uidx, *lrptr, *lridx, *uoff, *lrhead, *lrhoff, *u12off, *lrhk, *srow;
   int n_srow;
-  const int2 *jt_word, *jt_slot, *reac;
+  const int2 *jt_slot, *reac;
   const int* sc_ptr;
   const uint32_t* sc_ent;
   const int4* jdesc;     // per Jacobian entry {t0, t1, jrc, row << 16 | col}

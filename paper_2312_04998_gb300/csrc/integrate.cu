@@ -2690,8 +2690,7 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   d.lptr = lu.d_lptr.as<int>(); d.lidx = lu.d_lidx.as<int>();
   d.uptr = lu.d_uptr.as<int>(); d.uidx = lu.d_uidx.as<int>();
   d.lrptr = lu.d_lrptr.as<int>(); d.lridx = lu.d_lridx.as<int>();
-  d.ucptr = lu.d_ucptr.as<int>(); d.ucidx = lu.d_ucidx.as<int>();
-  d.jrc = lu.d_jrc.as<int>(); d.uoff = lu.d_uoff.as<int>(); d.lrhead = lu.d_lrhead.as<int>();
+  d.uoff = lu.d_uoff.as<int>(); d.lrhead = lu.d_lrhead.as<int>();
   d.lrhoff = lu.d_lrhoff.as<int>();
   d.u12off = lu.d_u12off.as<int>();
   d.lrhk = lu.d_lrhk.as<int>();
@@ -2700,8 +2699,6 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   d.jt_slot = net->d_jt_slot.as<int2>(); d.reac = net->d_reac.as<int2>();
   d.sc_ptr = net->d_sc_ptr.as<int>(); d.sc_ent = net->d_sc_ent.as<uint32_t>();
   d.jdesc = net->d_jdesc.as<int4>(); d.jlong = net->d_jlong.as<int>(); d.n_jlong = (int)net->jlong.size();
-  d.jp_ptr = net->d_jp_ptr.as<int>(); d.jt_ptr = net->d_jt_ptr.as<int>();
-  d.jt_word = net->d_jt_word.as<int2>(); d.jpos = lu.d_jpos.as<int>();
   d.record = o.record_steps > 0 ? o.record_steps : 0;
   if (d.record) {
     const int64_t R = d.record, K = R / kCkpt + 1;

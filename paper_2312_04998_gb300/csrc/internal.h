@@ -110,9 +110,25 @@ struct LUSymbolic {
   int32_t n_hlev = 0;
   int64_t nnz = 0, flops = 0;
   DevArray d_u11ptr, d_flev_ptr, d_flev, d_blev_ptr, d_blev, d_hop_ptr, d_hop, d_hop_piv, d_hterm;
-  DevArray d_lptr, d_lidx, d_uptr, d_uidx, d_lrptr, d_lridx, d_ucptr, d_ucidx, d_jpos, d_perm, d_iperm,
-      d_jrc, d_uoff, d_lrhead, d_lrhoff, d_u12off, d_lrhk, d_srow;
+  DevArray d_lptr, d_lidx, d_uptr, d_uidx, d_lrptr, d_lridx, d_perm, d_iperm, d_uoff, d_lrhead, d_lrhoff, d_u12off, d_lrhk, d_srow;
 };
+
+// Words of the index programs: table slot (16 bits) | the upper half of the
+// double c << 16, for c of at most five significant bits; any other c goes in
+// parts.
+inline int32_t coef_word(int32_t slot, int c) {
+  const double v = c;
+  uint64_t u;
+  std::memcpy(&u, &v, sizeof u);
+  return (int32_t)((uint32_t)slot | (uint32_t)(u >> 48) << 16);
+}
+template <class F> void for_coef_parts(int c, F f) {
+  while (c != 0) {
+    const int part = c >= -31 && c <= 31 ? c : c / 32 * 32;
+    f(part);
+    c -= part;
+  }
+}
 
 constexpr int kJShort = 4;   // (see CellProg)
 
@@ -161,6 +177,15 @@ struct CellProg {
   DevArray blob;
 };
 
+// Program of the Jacobian kernel (kern_jac.cu): per group (a CTA's columns) a
+// run of passes {slots, segments}; slot = product {reaction, partner or -1};
+// segment = an entry's terms in the pass's products (coef_word each).
+struct JacProg {
+  std::vector<int32_t> group, pass, slot, seg, term;
+  int32_t slots = 0;   // most products of a pass
+  DevArray blob;       // pass, seg, term, slot, group
+};
+
 struct sm_net {
   int device = 0;
   int32_t n_s = 0, n_r = 0, n_elem = 0;
@@ -190,13 +215,11 @@ struct sm_net {
   DevArray d_reac;        // int2 per reaction: reactant indices (-1 = none)
   DevArray d_rate;        // RatePar per reaction: (log alpha | alpha, beta, gamma, class)
   DevArray d_ratefix, d_ratetab;           // the same for the fixed-point exponential (see kern_rates.cu)
-  DevArray d_jp_ptr, d_jt_ptr, d_jt_word;  // Jacobian gather lists
   DevArray d_jt_slot;                      // (reaction | coef << 24, reactant slot) per term
   std::vector<int32_t> jlong;              // Jacobian entries with more than kJLong terms
   DevArray d_jdesc, d_jlong;               // per entry {t0, t1, jrc, row << 16 | col}; long entries
   DevArray d_sc_ptr, d_sc_ent;             // S by columns: pointers and (species | coef << 24)
-  std::vector<int32_t> jchunk;             // J entries per gather chunk (balanced by terms)
-  DevArray d_jchunk;
+  JacProg jac;
   DevArray d_status;      // int32 device status word
   DevArray d_scratch;     // reaction-rate scratch for rhs_eval
   sm_net_info info{};
@@ -239,6 +262,7 @@ sm_status launch_rhs_masked(const sm_net* net, int64_t C, const double* k, int64
 // Per-device set-up of the right-hand-side kernels (constant tables); called
 // when a network is uploaded.
 sm_status rhs_prepare_device(int device);
+JacProg build_jac_prog(const sm_net* net);
 sm_status launch_jac(const sm_net* net, int64_t C, const double* k, const double* y,
                      double* J, int64_t ld, cudaStream_t s);
 

@@ -728,22 +728,12 @@ sm_status net_upload(sm_net* net) {
   const std::vector<RateFix> fix = rate_fixed(net, table);
   if ((st = net->d_ratefix.upload(fix.data(), fix.size() * sizeof(RateFix))) != SM_OK) return st;
   if ((st = net->d_ratetab.upload(table.data(), table.size() * 8)) != SM_OK) return st;
-  // Jacobian gather words: reaction (low 23 bits) | partner+1 ... packed as two
-  // int32 per term: (reaction | coef << 24, partner)
-  std::vector<int32_t> words(2 * net->jt_rx.size());
-  for (size_t t = 0; t < net->jt_rx.size(); ++t) {
-    words[2 * t] = (int32_t)pack(net->jt_rx[t], net->jt_coef[t]);
-    words[2 * t + 1] = net->jt_partner[t];
-  }
   {
     std::vector<uint32_t> ent(net->s_row.size());
     for (size_t p = 0; p < ent.size(); ++p) ent[p] = pack(net->s_row[p], net->s_coef[p]);
     if ((st = net->d_sc_ptr.upload(net->s_colptr.data(), net->s_colptr.size() * 4)) != SM_OK) return st;
     if ((st = net->d_sc_ent.upload(ent.data(), ent.size() * 4)) != SM_OK) return st;
   }
-  if ((st = net->d_jp_ptr.upload(net->jp_ptr.data(), net->jp_ptr.size() * 4)) != SM_OK) return st;
-  if ((st = net->d_jt_ptr.upload(net->jt_ptr.data(), net->jt_ptr.size() * 4)) != SM_OK) return st;
-  if ((st = net->d_jt_word.upload(words.data(), words.size() * 4)) != SM_OK) return st;
   // the same terms with the reactant slot whose derivative they use: slot 0 =
   // d/d(first reactant) = k' x_second (or k'), slot 1 = d/d(second reactant)
   {
@@ -759,19 +749,12 @@ sm_status net_upload(sm_net* net) {
       }
     if ((st = net->d_jt_slot.upload(ws.data(), ws.size() * 4)) != SM_OK) return st;
   }
-  // gather chunks of about equal term count over the J pattern entries
   {
-    const int64_t n_e = (int64_t)net->jp_col.size(), n_t = (int64_t)net->jt_rx.size();
-    const int64_t n_ch = std::max<int64_t>(1, std::min<int64_t>(256, n_e));
-    net->jchunk.assign(1, 0);
-    int64_t e = 0;
-    for (int64_t c = 1; c < n_ch; ++c) {
-      const int64_t target = n_t * c / n_ch;
-      while (e < n_e && net->jt_ptr[e + 1] <= target) ++e;
-      net->jchunk.push_back((int32_t)std::max<int64_t>(e, net->jchunk.back()));
-    }
-    net->jchunk.push_back((int32_t)n_e);
-    if ((st = net->d_jchunk.upload(net->jchunk.data(), net->jchunk.size() * 4)) != SM_OK) return st;
+    net->jac = build_jac_prog(net);
+    const JacProg& p = net->jac;
+    std::vector<int32_t> all;
+    for (const std::vector<int32_t>* v : {&p.pass, &p.seg, &p.term, &p.slot, &p.group}) all.insert(all.end(), v->begin(), v->end());
+    if ((st = net->jac.blob.upload(all.data(), all.size() * 4)) != SM_OK) return st;
   }
   LUSymbolic& lu = net->lu;
   if ((st = lu.d_lptr.upload(lu.lptr.data(), lu.lptr.size() * 4)) != SM_OK) return st;
@@ -780,10 +763,6 @@ sm_status net_upload(sm_net* net) {
   if (!lu.uidx.empty() && (st = lu.d_uidx.upload(lu.uidx.data(), lu.uidx.size() * 4)) != SM_OK) return st;
   if ((st = lu.d_lrptr.upload(lu.lrptr.data(), lu.lrptr.size() * 4)) != SM_OK) return st;
   if (!lu.lridx.empty() && (st = lu.d_lridx.upload(lu.lridx.data(), lu.lridx.size() * 4)) != SM_OK) return st;
-  if ((st = lu.d_ucptr.upload(lu.ucptr.data(), lu.ucptr.size() * 4)) != SM_OK) return st;
-  if (!lu.ucidx.empty() && (st = lu.d_ucidx.upload(lu.ucidx.data(), lu.ucidx.size() * 4)) != SM_OK) return st;
-  if ((st = lu.d_jpos.upload(lu.jpos.data(), lu.jpos.size() * 4)) != SM_OK) return st;
-  if ((st = lu.d_jrc.upload(lu.jrc.data(), lu.jrc.size() * 4)) != SM_OK) return st;
   // one 16-byte descriptor per Jacobian entry for the refresh gather: term
   // range, (row, column) in elimination order, (row, column) species; and
   // the entries with more than kJLong terms, which a warp gathers
