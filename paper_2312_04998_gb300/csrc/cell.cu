@@ -148,6 +148,9 @@ __device__ __forceinline__ double ld_here(const double* p) {
 }
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// The coefficient of an index word.
+__device__ __forceinline__ double coef(int word) { return __hiloint2double(word & 0xFFFF0000, 0); }
+
 // Sums of rows cut into chains (see Chains in cell_prog.cpp): a chain per lane,
 // a slice of 32 chains per warp, longest first, so that the warps of each
 // scheduler keep its FP64 unit (a warp's FMA holds it for 64 cycles) busy.
@@ -168,18 +171,26 @@ __device__ __forceinline__ void row_sums(const int* __restrict__ w, int n_sl, in
     for (int u = 0; u < 4; ++u) nx[u] = 4 + u < m ? __ldg(q + 32 * (4 + u)) : 0;
     if (s + nw < n_sl) mt = __ldg(meta + s + nw);
     double a = 0.0;
-    for (int e = 0; e < m; e += 4) {
+    int e = 4;
+    for (; e <= m; e += 4) {
       int n2[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) n2[u] = e + 8 + u < m ? __ldg(q + 32 * (e + 8 + u)) : 0;
+      for (int u = 0; u < 4; ++u) n2[u] = e + 4 + u < m ? __ldg(q + 32 * (e + 4 + u)) : 0;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (e + u < m) a = fma(__hiloint2double(t[u] & 0xFFFF0000, 0), tab[t[u] & 0xFFFF], a);
+      for (int u = 0; u < 4; ++u) a = fma(coef(t[u]), tab[t[u] & 0xFFFF], a);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         t[u] = nx[u];
         nx[u] = n2[u];
       }
+    }
+    // (an FP64 instruction that is predicated off holds the unit all the same,
+    // and short branches become predicates: the rest as a loop)
+#pragma unroll 1
+    for (e -= 4; e < m; ++e) {
+      a = fma(coef(t[0]), tab[t[0] & 0xFFFF], a);
+      t[0] = t[1];
+      t[1] = t[2];
     }
     part[to] = a;
   }
@@ -1108,10 +1119,17 @@ __device__ __forceinline__ void cell_jacobian() {
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        double a = 0.0;
+        // the first word's coefficient is +-1; most slices end there
+        const double v = dR[t[0][u] & 0xFFFF];
+        double a = __hiloint2double(__double2hiint(v) ^ (t[0][u] & 0x80000000), __double2loint(v));
+        if (len[u] > 1) {
+          double x[kJShort];
 #pragma unroll
-        for (int e = 0; e < kJShort; ++e)
-          if (e < len[u]) a = fma(__hiloint2double(t[e][u] & 0xFFFF0000, 0), dR[t[e][u] & 0xFFFF], a);
+          for (int e = 1; e < kJShort; ++e) x[e] = dR[t[e][u] & 0xFFFF];
+#pragma unroll
+          for (int e = 1; e < kJShort; ++e)
+            asm volatile("fma.rn.f64 %0, %1, %2, %0;" : "+d"(a) : "d"(coef(t[e][u])), "d"(x[e]));   // (not ahead of the branch)
+        }
         if (len[u] > 0) mbuf[32 * (s + u) + lane] = m_value(rc[u], a);
       }
     }
@@ -1128,15 +1146,21 @@ __device__ __forceinline__ void cell_jacobian() {
 #pragma unroll
       for (int u = 0; u < 4; ++u) t[u] = u < m ? __ldg(q + 32 * u) : 0;
       double a = 0.0;
-      for (int e = 0; e < m; e += 4) {
+      int e = 4;
+      for (; e <= m; e += 4) {
         int nx[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) nx[u] = e + 4 + u < m ? __ldg(q + 32 * (e + 4 + u)) : 0;
+        for (int u = 0; u < 4; ++u) nx[u] = e + u < m ? __ldg(q + 32 * (e + u)) : 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (e + u < m) a = fma(__hiloint2double(t[u] & 0xFFFF0000, 0), dR[t[u] & 0xFFFF], a);
+        for (int u = 0; u < 4; ++u) a = fma(coef(t[u]), dR[t[u] & 0xFFFF], a);
 #pragma unroll
         for (int u = 0; u < 4; ++u) t[u] = nx[u];
+      }
+#pragma unroll 1
+      for (e -= 4; e < m; ++e) {
+        a = fma(coef(t[0]), dR[t[0] & 0xFFFF], a);
+        t[0] = t[1];
+        t[1] = t[2];
       }
       if (s < A.n_jw) a = warp_sum(a);
       mbuf[32 * (A.n_jsl + s) + lane] = m_value(rc, a);

@@ -1,7 +1,6 @@
 // Index programs of the fused per-cell integrator (see cell.h), built once per
 // network on the host.
 #include <algorithm>
-#include <cstring>
 #include <numeric>
 
 #include "cell.h"
@@ -92,15 +91,6 @@ Chains cut_rows(const std::vector<std::vector<int32_t>>& rows, int32_t pad) {
   return p;
 }
 
-// An entry's word: table slot | the upper half of the double c << 16 (c of at
-// most five significant bits).
-int32_t entry(int32_t slot, int c) {
-  const double v = c;
-  uint64_t u;
-  std::memcpy(&u, &v, sizeof u);
-  return (int32_t)((uint32_t)slot | (uint32_t)(u >> 48) << 16);
-}
-
 }  // namespace
 
 void build_cell_prog(const sm_net* net, CellProg* out) {
@@ -138,12 +128,8 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     std::vector<std::vector<int32_t>> rows(n);
     for (int32_t j = 0; j < n_r; ++j)
       for (int32_t q = net->s_colptr[j]; q < net->s_colptr[j + 1]; ++q)
-        for (int c = net->s_coef[q]; c != 0;) {   // (beyond +-31 in parts of five bits)
-          const int part = std::abs(c) <= 31 ? c : c / 32 * 32;
-          rows[net->s_row[q]].push_back(entry(j, part));
-          c -= part;
-        }
-    const Chains r = cut_rows(rows, entry(n_r, 1));
+        for_coef_parts(net->s_coef[q], [&](int c) { rows[net->s_row[q]].push_back(coef_word(j, c)); });
+    const Chains r = cut_rows(rows, coef_word(n_r, 1));
     p.n_rsl = r.s.slices();
     p.n_chain = r.n_chain;
     p.rp_off = put(r.s.off);
@@ -158,10 +144,10 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     std::vector<std::vector<int32_t>> rows(n);
     for (int32_t j = 0; j < n_r; ++j) {
       const int32_t a = net->reac[2 * j], b = net->reac[2 * j + 1];
-      rows[a].push_back(entry(slot[j], 1));
-      if (b >= 0) rows[b].push_back(entry(slot[j] + 1, 1));
+      rows[a].push_back(coef_word(slot[j], 1));
+      if (b >= 0) rows[b].push_back(coef_word(slot[j] + 1, 1));
     }
-    const Chains r = cut_rows(rows, entry(p.n_slot, 1));
+    const Chains r = cut_rows(rows, coef_word(p.n_slot, 1));
     p.n_vsl = r.s.slices();
     p.n_vchain = r.n_chain;
     p.vp_off = put(r.s.off);
@@ -202,12 +188,10 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
         for (int32_t t = net->jt_ptr[e]; t < net->jt_ptr[e + 1]; ++t) {
           const int32_t j = net->jt_rx[t], cf = net->jt_coef[t];
           const int32_t w = slot[j] + (net->reac[2 * j] == l ? 0 : 1);
-          for (int v = cf; v != 0;) {
-            const int part = std::abs(v) <= 31 ? v : v / 32 * 32;
-            items[e].push_back(entry(w, part));
-            v -= part;
-          }
+          if (items[e].empty() && cf != 1 && cf != -1) items[e].push_back(coef_word(p.n_slot, 1));   // (see cell_jacobian)
+          for_coef_parts(cf, [&](int c) { items[e].push_back(coef_word(w, c)); });
         }
+        if (items[e].empty()) items[e].push_back(coef_word(p.n_slot, 1));
         rc[e] = i | (l << 16);
         const bool tail = pi >= h && pl >= h;
         grp[e] = tail ? 1 + (pl - h) / kGroup : 0;
@@ -223,7 +207,7 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     for (int32_t q = 0; q < ng; ++q) {
       std::stable_sort(in[q].begin(), in[q].end(),
                        [&](int32_t a, int32_t b) { return items[a].size() > items[b].size(); });
-      add_slices(items, in[q], entry(p.n_slot, 1), 1, &s);
+      add_slices(items, in[q], coef_word(p.n_slot, 1), 1, &s);
       for (int32_t e : in[q]) {
         sr.push_back(rc[e]);
         sd.push_back(dst[e]);
@@ -248,7 +232,7 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
       std::iota(all.begin(), all.end(), 0);
       for (size_t e = 0; e < it.size(); ++e) lanes[e % 32].push_back(it[e]);
       at[t] = 32 * ls.slices();
-      add_slices(lanes, all, entry(p.n_slot, 1), 1, &ls);
+      add_slices(lanes, all, coef_word(p.n_slot, 1), 1, &ls);
       lr.resize((size_t)32 * ls.slices(), 0);
       lr[at[t]] = rc[lng[t]];
     }
@@ -256,7 +240,7 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
     for (; t < lng.size(); t += 32) {
       const size_t m = std::min<size_t>(32, lng.size() - t);
       const int32_t base = 32 * ls.slices();
-      add_slices(items, std::vector<int32_t>(lng.begin() + t, lng.begin() + t + m), entry(p.n_slot, 1), 1, &ls);
+      add_slices(items, std::vector<int32_t>(lng.begin() + t, lng.begin() + t + m), coef_word(p.n_slot, 1), 1, &ls);
       lr.resize((size_t)32 * ls.slices(), 0);
       for (size_t l = 0; l < m; ++l) {
         at[t + l] = base + (int32_t)l;
