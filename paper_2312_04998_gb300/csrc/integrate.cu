@@ -359,10 +359,28 @@ __device__ void tf32_trailing_update(float* C, int ldc, int r, const float* L, i
   }
 }
 
+// A cluster of S CTAs may share a cell (FP64 replays of few cells, dense
+// output): rank 0 forms M, its head and the panels; the rows of the head's Schur
+// complement and the columns (in tiles of kBN) of the U blocks and the trailing
+// updates are dealt over the ranks, with a cluster barrier where one reads what
+// another wrote.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+template <class T> __device__ __forceinline__ T from_rank0(const T* p) {   // rank 0's value at this shared address
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)));
+  T v;
+  if constexpr (sizeof(T) == 8) asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a));
+  else asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(a));
+  return v;
+}
+
 template <class T>
 __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, const double* __restrict__ k,
-                                                                 int64_t ldk, RefreshPlan plan) {
+                                                                 int64_t ldk, RefreshPlan plan, int S) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int rank = S > 1 ? blockIdx.x % S : 0;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
   const int n = d.n, n_r = d.n_r, ldm = d.ldm, h = d.head, nt = n - h, pitch = plan.pitch;
@@ -383,89 +401,91 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
   wsf = reinterpret_cast<float*>(coef + 256);
   wif = wsf + n;
   const int count = d.counters[0];
-  for (int e = blockIdx.x; e < count; e += gridDim.x) {
+  for (int e = blockIdx.x / S; e < count; e += gridDim.x / S) {
     const int64_t c = d.list[e];
     T* A = static_cast<T*>(d.lu) + (d.lu_cta ? (int64_t)blockIdx.x : c) * d.lu_stride;
     T* P = d.lup ? static_cast<T*>(d.lup) + (int64_t)d.slot_cell[c] * d.lup_stride : nullptr;
     T* D = P ? P + d.p_d : nullptr;   // packed tail block, column-major
     const double gamma = d.gam[c];
-    // zero the dense trailing block and the head's pattern entries
-    for (int r = warp; r < nt; r += nwarps) {
-      T* row = A + (int64_t)(h + r) * ldm + h;
-      for (int q = lane; q < nt; q += 32) row[q] = T(0);
-    }
-    for (int kp = warp; kp < h; kp += nwarps) {
-      for (int p = __ldg(d.lptr + kp) + lane; p < __ldg(d.lptr + kp + 1); p += 32)
-        A[(int64_t)__ldg(d.lidx + p) * ldm + kp] = T(0);
-      for (int p = __ldg(d.uptr + kp) + lane; p < __ldg(d.uptr + kp + 1); p += 32)
-        A[(int64_t)kp * ldm + __ldg(d.uidx + p)] = T(0);
-      if (lane == 0) A[(int64_t)kp * ldm + kp] = T(0);
-    }
-    // ---- phase A
-    for (int i = tid; i < 256; i += nthr) coef[i] = (double)(int8_t)i;
-    for (int j = tid; j < n_r; j += nthr) {
-      const int2 rc = __ldg(d.reac + j);
-      const double kv = k[(int64_t)j * ldk + c];
-      dR[2 * j] = rc.y >= 0 ? kv * d.ypred[(int64_t)rc.y * d.ld + c] : kv;
-      dR[2 * j + 1] = rc.y >= 0 ? kv * d.ypred[(int64_t)rc.x * d.ld + c] : 0.0;
-    }
-    if (d.mixed)
-      for (int s = tid; s < n; s += nthr) {
-        const double wv = V(d.w, d, s, c);
-        V(d.wf, d, s, c) = wv;
-        wsf[s] = (float)wv;
-        wif[s] = (float)(1.0 / wv);
+    if (rank == 0) {
+      // zero the dense trailing block and the head's pattern entries
+      for (int r = warp; r < nt; r += nwarps) {
+        T* row = A + (int64_t)(h + r) * ldm + h;
+        for (int q = lane; q < nt; q += 32) row[q] = T(0);
       }
-    __syncthreads();
-    // M_ij = delta_ij - gamma sum_terms coef dR, stored in elimination order
-    // (W M W^-1 with this step's error weights, scaled in FP32, when mixed)
-    auto store_m = [&](const int4 ds, double acc) {
-      const int pi = ds.z >> 16, pj = ds.z & 0xFFFF;
-      const double m = fma(-gamma, acc, pi == pj ? 1.0 : 0.0);
-      T* dst = A + (int64_t)pi * ldm + pj;
-      if (d.mixed) *dst = T((float)m * (wsf[ds.w >> 16] * wif[ds.w & 0xFFFF]));
-      else *dst = T(m);
-    };
-    auto term = [&](double acc, int t) {
-      const int2 w = __ldg(d.jt_slot + t);
-      return fma(coef[(uint32_t)w.x >> 24], dR[2 * (w.x & 0xFFFFFF) + w.y], acc);
-    };
-    // entries with more than kJLong terms (the hub species'): a warp each
-    for (int q = warp; q < d.n_jlong; q += nwarps) {
-      const int4 ds = __ldg(d.jdesc + __ldg(d.jlong + q));
-      double acc = 0.0;
-      for (int t = ds.x + lane; t < ds.y; t += 32) acc = term(acc, t);
-      acc = warp_sum(acc);
-      if (lane == 0) store_m(ds, acc);
-    }
-    // the others: a thread each, two entries at a time; the first kJPre term
-    // words of both entries are loaded before any is used, so that their
-    // loads overlap (most entries have at most kJPre terms)
-    constexpr int kJPre = 4;
-    for (int p = tid; p < d.nnz_j; p += 2 * nthr) {
-      const bool hb = p + nthr < d.nnz_j;
-      const int4 da = __ldg(d.jdesc + p);
-      const int4 db = hb ? __ldg(d.jdesc + p + nthr) : make_int4(0, 0, 0, 0);
-      const bool la = da.y - da.x <= kJLong, lb = hb && db.y - db.x <= kJLong;
-      double aa = 0.0, ab = 0.0;
-      const int na = la ? da.y - da.x : 0, nb = lb ? db.y - db.x : 0;
-      int2 wa[kJPre], wb[kJPre];
+      for (int kp = warp; kp < h; kp += nwarps) {
+        for (int p = __ldg(d.lptr + kp) + lane; p < __ldg(d.lptr + kp + 1); p += 32)
+          A[(int64_t)__ldg(d.lidx + p) * ldm + kp] = T(0);
+        for (int p = __ldg(d.uptr + kp) + lane; p < __ldg(d.uptr + kp + 1); p += 32)
+          A[(int64_t)kp * ldm + __ldg(d.uidx + p)] = T(0);
+        if (lane == 0) A[(int64_t)kp * ldm + kp] = T(0);
+      }
+      // ---- phase A
+      for (int i = tid; i < 256; i += nthr) coef[i] = (double)(int8_t)i;
+      for (int j = tid; j < n_r; j += nthr) {
+        const int2 rc = __ldg(d.reac + j);
+        const double kv = k[(int64_t)j * ldk + c];
+        dR[2 * j] = rc.y >= 0 ? kv * d.ypred[(int64_t)rc.y * d.ld + c] : kv;
+        dR[2 * j + 1] = rc.y >= 0 ? kv * d.ypred[(int64_t)rc.x * d.ld + c] : 0.0;
+      }
+      if (d.mixed)
+        for (int s = tid; s < n; s += nthr) {
+          const double wv = V(d.w, d, s, c);
+          V(d.wf, d, s, c) = wv;
+          wsf[s] = (float)wv;
+          wif[s] = (float)(1.0 / wv);
+        }
+      __syncthreads();
+      // M_ij = delta_ij - gamma sum_terms coef dR, stored in elimination order
+      // (W M W^-1 with this step's error weights, scaled in FP32, when mixed)
+      auto store_m = [&](const int4 ds, double acc) {
+        const int pi = ds.z >> 16, pj = ds.z & 0xFFFF;
+        const double m = fma(-gamma, acc, pi == pj ? 1.0 : 0.0);
+        T* dst = A + (int64_t)pi * ldm + pj;
+        if (d.mixed) *dst = T((float)m * (wsf[ds.w >> 16] * wif[ds.w & 0xFFFF]));
+        else *dst = T(m);
+      };
+      auto term = [&](double acc, int t) {
+        const int2 w = __ldg(d.jt_slot + t);
+        return fma(coef[(uint32_t)w.x >> 24], dR[2 * (w.x & 0xFFFFFF) + w.y], acc);
+      };
+      // entries with more than kJLong terms (the hub species'): a warp each
+      for (int q = warp; q < d.n_jlong; q += nwarps) {
+        const int4 ds = __ldg(d.jdesc + __ldg(d.jlong + q));
+        double acc = 0.0;
+        for (int t = ds.x + lane; t < ds.y; t += 32) acc = term(acc, t);
+        acc = warp_sum(acc);
+        if (lane == 0) store_m(ds, acc);
+      }
+      // the others: a thread each, two entries at a time; the first kJPre term
+      // words of both entries are loaded before any is used, so that their
+      // loads overlap (most entries have at most kJPre terms)
+      constexpr int kJPre = 4;
+      for (int p = tid; p < d.nnz_j; p += 2 * nthr) {
+        const bool hb = p + nthr < d.nnz_j;
+        const int4 da = __ldg(d.jdesc + p);
+        const int4 db = hb ? __ldg(d.jdesc + p + nthr) : make_int4(0, 0, 0, 0);
+        const bool la = da.y - da.x <= kJLong, lb = hb && db.y - db.x <= kJLong;
+        double aa = 0.0, ab = 0.0;
+        const int na = la ? da.y - da.x : 0, nb = lb ? db.y - db.x : 0;
+        int2 wa[kJPre], wb[kJPre];
 #pragma unroll
-      for (int u = 0; u < kJPre; ++u) {
-        wa[u] = u < na ? __ldg(d.jt_slot + da.x + u) : make_int2(0, 0);
-        wb[u] = u < nb ? __ldg(d.jt_slot + db.x + u) : make_int2(0, 0);
-      }
+        for (int u = 0; u < kJPre; ++u) {
+          wa[u] = u < na ? __ldg(d.jt_slot + da.x + u) : make_int2(0, 0);
+          wb[u] = u < nb ? __ldg(d.jt_slot + db.x + u) : make_int2(0, 0);
+        }
 #pragma unroll
-      for (int u = 0; u < kJPre; ++u) {
-        if (u < na) aa = fma(coef[(uint32_t)wa[u].x >> 24], dR[2 * (wa[u].x & 0xFFFFFF) + wa[u].y], aa);
-        if (u < nb) ab = fma(coef[(uint32_t)wb[u].x >> 24], dR[2 * (wb[u].x & 0xFFFFFF) + wb[u].y], ab);
+        for (int u = 0; u < kJPre; ++u) {
+          if (u < na) aa = fma(coef[(uint32_t)wa[u].x >> 24], dR[2 * (wa[u].x & 0xFFFFFF) + wa[u].y], aa);
+          if (u < nb) ab = fma(coef[(uint32_t)wb[u].x >> 24], dR[2 * (wb[u].x & 0xFFFFFF) + wb[u].y], ab);
+        }
+        for (int u = kJPre; u < max(na, nb); ++u) {
+          if (u < na) aa = term(aa, da.x + u);
+          if (u < nb) ab = term(ab, db.x + u);
+        }
+        if (la) store_m(da, aa);
+        if (lb) store_m(db, ab);
       }
-      for (int u = kJPre; u < max(na, nb); ++u) {
-        if (u < na) aa = term(aa, da.x + u);
-        if (u < nb) ab = term(ab, db.x + u);
-      }
-      if (la) store_m(da, aa);
-      if (lb) store_m(db, ab);
     }
     __syncthreads();
     // ---- phase B: sparse head.  The head program (see LUSymbolic) computes
@@ -480,7 +500,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         for (int q = lane; q < cnt; q += 32) sx_u12[o12 + q] = (unsigned short)(__ldg(d.uidx + base + q) - h);
         for (int b = lane; b < np1; b += 32) sx_off[kr * np1 + b] = o12 + __ldg(d.uoff + kr * np1 + b) - base;
       }
-      for (int l = 0; l < d.n_hlev; ++l) {
+      for (int l = 0; rank == 0 && l < d.n_hlev; ++l) {
         for (int part = 0; part < 2; ++part) {
           const int o1 = __ldg(d.hop_ptr + 2 * l + part + 1);
           for (int o = __ldg(d.hop_ptr + 2 * l + part) + tid; o < o1; o += nthr) {
@@ -500,6 +520,12 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           }
           __syncthreads();
         }
+      }
+      if (S > 1) {
+        cluster_sync();   // M and the head are complete
+        if (rank > 0)
+          for (int i = tid; i < d.p_d; i += nthr) Hv[i] = from_rank0(Hv + i);
+        __syncthreads();
       }
       // ---- phase S: A22 -= L21 U12, one 32-column panel at a time.  U12's
       // panel columns are expanded into a dense h x 32 tile (in front of H);
@@ -524,7 +550,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         // longest rows stay spread over the warps): their loads of A go out
         // together before any row's sums are formed
         constexpr int kSB = 8;
-        for (int t0 = 0; t0 < d.n_srow; t0 += kSB * nwarps) {
+        for (int t0 = rank * kSB * nwarps; t0 < d.n_srow; t0 += S * kSB * nwarps) {
           T cur[kSB][kPS];
           int ir[kSB], ro[kSB], rc[kSB];
 #pragma unroll
@@ -563,7 +589,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         }
         __syncthreads();
       }
-    } else {
+    } else if (rank == 0) {
       // pivot by pivot, Schur complement applied immediately
       for (int kp = 0; kp < h; ++kp) {
         const T inv = T(1) / A[(int64_t)kp * ldm + kp];
@@ -590,7 +616,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
     if (plan.head_smem) {
       if (P) {
         for (int i = tid; i < d.p_d; i += nthr) P[i] = Hv[i];
-      } else {
+      } else if (rank == 0) {
         const int o1 = __ldg(d.hop_ptr + 2 * d.n_hlev);
         for (int o = tid; o < o1; o += nthr) {
           const int4 op = __ldg(d.hop + o);
@@ -616,17 +642,23 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         for (int q = lane; q < cnt; q += 32) P[d.p_l21 + o + q] = Ai[__ldg(d.lridx + p0 + q)];
       }
     }
+    if (S > 1) cluster_sync();   // the Schur complement is complete, rank 0's head has been read
     // ---- phase C: dense trailing block, blocked right-looking LU
     for (int pb = 0; pb * kNB < nt; ++pb) {
       const int p0 = h + pb * kNB;
       const int w = min(kNB, n - p0), m = n - p0, r = m - w;
+      auto load_panel = [&]() {
 #pragma unroll 4
-      for (int a = warp; a < m; a += nwarps)
-        if (lane < w) Pt[lane * pitch + a] = A[(int64_t)(p0 + a) * ldm + p0 + lane];
+        for (int a = warp; a < m; a += nwarps)
+          if (lane < w) Pt[lane * pitch + a] = A[(int64_t)(p0 + a) * ldm + p0 + lane];
+      };
+      if (rank == 0) load_panel();
       for (int a = m + tid; a < pitch; a += nthr)
         for (int b = 0; b < w; ++b) Pt[b * pitch + a] = T(0);
       __syncthreads();
-      if (sizeof(T) == 4 && w == kNB) {
+      if (rank > 0) {
+        // (rank 0's)
+      } else if (sizeof(T) == 4 && w == kNB) {
         // full FP32 panel.  (1) warp 0 factors the kNB x kNB diagonal block in
         // registers (lane = row, pivot rows broadcast by shuffles); (2) every
         // row below solves l U11 = a on its own (thread per row, U11 read as
@@ -687,19 +719,25 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         // the panel's columns (diagonal block and L below it) are final
         for (int b = warp; b < w; b += nwarps)
           for (int a = lane; a < m; a += 32) D[(int64_t)(p0 - h + b) * d.ldd + (p0 - h + a)] = Pt[b * pitch + a];
-      } else {
+      } else if (rank == 0) {
         for (int a = warp; a < m; a += nwarps)
           if (lane < w) A[(int64_t)(p0 + a) * ldm + p0 + lane] = Pt[lane * pitch + a];
       }
+      if (S > 1 && r > 0) {
+        cluster_sync();   // the panel is final
+        if (rank > 0) load_panel();
+      }
+      const auto mine = [&](int b) { return S == 1 || b / kBN % S == rank; };   // columns of the trailing block
       if (r > 0) {
         const int rp = round_up(r, 4);
         for (int a = warp; a < w; a += nwarps)
           for (int b = lane; b < rp; b += 32)
-            U[a * upitch + b] = b < r ? A[(int64_t)(p0 + a) * ldm + p0 + w + b] : T(0);
+            if (mine(b)) U[a * upitch + b] = b < r ? A[(int64_t)(p0 + a) * ldm + p0 + w + b] : T(0);
         __syncthreads();
         // U12 = L11^-1 A12, one thread per column
         if (w == kNB) {
           for (int b = tid; b < r; b += nthr) {
+            if (!mine(b)) continue;
             T col[kNB];
 #pragma unroll
             for (int a = 0; a < kNB; ++a) col[a] = U[a * upitch + b];
@@ -712,7 +750,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           }
         } else {
           for (int b = tid; b < r; b += nthr)
-            for (int kk = 0; kk < w; ++kk) {
+            for (int kk = 0; mine(b) && kk < w; ++kk) {
               const T u = U[kk * upitch + b];
               for (int a = kk + 1; a < w; ++a) U[a * upitch + b] -= Pt[kk * pitch + a] * u;
             }
@@ -726,7 +764,8 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           }
         } else {
           for (int a = warp; a < w; a += nwarps)
-            for (int b = lane; b < r; b += 32) A[(int64_t)(p0 + a) * ldm + p0 + w + b] = U[a * upitch + b];
+            for (int b = lane; b < r; b += 32)
+              if (mine(b)) A[(int64_t)(p0 + a) * ldm + p0 + w + b] = U[a * upitch + b];
         }
         // A22 -= L21 U12; L21 column kk is Pt[kk * pitch + w + i]
         bool done = false;
@@ -741,10 +780,11 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         // thread; the next tile's values of A are loaded while this tile's
         // products are formed
         const int ty = tid / 16, tx = tid % 16;
-        const int nbu = (r + kBN - 1) / kBN, ntile = done ? 0 : ((r + kBM - 1) / kBM) * nbu;
+        // (nbu: this rank's columns of tiles)
+        const int nbu = max(0, ((r + kBN - 1) / kBN - rank + S - 1) / S), ntile = done ? 0 : ((r + kBM - 1) / kBM) * nbu;
         T nxt[kTM][kTN];
         auto load_c = [&](int tt) {
-          const int i0 = (tt / nbu) * kBM + ty * kTM, j0 = (tt % nbu) * kBN + tx * kTN;
+          const int i0 = (tt / nbu) * kBM + ty * kTM, j0 = (rank + S * (tt % nbu)) * kBN + tx * kTN;
 #pragma unroll
           for (int a = 0; a < kTM; ++a)
 #pragma unroll
@@ -759,7 +799,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
 #pragma unroll
             for (int b = 0; b < kTN; ++b) acc[a][b] = nxt[a][b];
           if (tt + 1 < ntile) load_c(tt + 1);
-          const int i0 = (tt / nbu) * kBM + ty * kTM, j0 = (tt % nbu) * kBN + tx * kTN;
+          const int i0 = (tt / nbu) * kBM + ty * kTM, j0 = (rank + S * (tt % nbu)) * kBN + tx * kTN;
           if (i0 >= r || j0 >= r) continue;
           const T* lp = Pt + w + i0;
           const T* up = U + j0;
@@ -781,8 +821,9 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         }
       }
       __syncthreads();
+      if (S > 1 && r > 0) cluster_sync();   // the trailing block is up to date
     }
-    if (tid == 0) {
+    if (tid == 0 && rank == 0) {
       d.gam_J[c] = gamma;
       d.j_age[c] = 0;
       d.crate[c] = 1.0;
@@ -1692,7 +1733,7 @@ __device__ __forceinline__ double* slot_lu(const Dev& d, const AdjDev& a, int j,
   return a.slots + ((int64_t)j * d.C + c) * d.lu_stride;
 }
 
-__global__ void adj_setup_kernel(Dev d, AdjDev a, const double* __restrict__ k, int64_t ldk) {
+__global__ void adj_setup_kernel(Dev d, AdjDev a) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.C) return;
   const int N = d.steps[c];
@@ -1703,8 +1744,6 @@ __global__ void adj_setup_kernel(Dev d, AdjDev a, const double* __restrict__ k, 
   a.astat[c] = ok ? 0 : 1;
   atomicMax(&d.counters[3], K);
   atomicMax(&d.counters[1], ok ? N : 0);
-  for (int j = 0; j < d.n_r; ++j) a.kc[c * d.n_r + j] = k[(int64_t)j * ldk + c];
-  for (int64_t i = 0; i < (int64_t)a.n_cot * d.n_r; ++i) a.g[c * a.n_cot * d.n_r + i] = 0.0;
   for (int i = 0; i < kRing; ++i) a.ring_q[(int64_t)i * a.lda + c] = 0;
 }
 
@@ -1736,12 +1775,13 @@ __device__ __forceinline__ int seg_step(const AdjDev& a, int64_t c, int j) {
 
 // Predictor, BDF coefficients and Newton set-up of frozen step m; with
 // `store` the step's h, q and alpha are kept for the backward pass.
-__global__ void rpredict_kernel(Dev d, AdjDev a, int j, int store) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32 * kCoopWarps) rpredict_kernel(Dev d, AdjDev a, int j, int store) {
+  const int64_t c = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  const int wi = threadIdx.x >> 5;
   if (c >= d.C) return;
   const int m = seg_step(a, c, j);
   if (!m) {
-    d.flags[c] = 0;
+    if (wi == 0) d.flags[c] = 0;
     return;
   }
   const double tnew = d.log_t[(int64_t)(m - 1) * d.ld + c];
@@ -1753,41 +1793,43 @@ __global__ void rpredict_kernel(Dev d, AdjDev a, int j, int store) {
   const bool lagr = nh > q;
   if (lagr) lagrange(T, q + 1, tnew, wts);
   bdf_alphas(tnew, T, q, h, al);
-  d.h[c] = h;
-  d.gam[c] = h / al[0];
-  for (int i = 0; i <= QMAX; ++i) {
-    const double v = i <= q ? al[i] : 0.0;
-    d.alpha[(int64_t)i * d.ld + c] = v;
-    if (store) a.seg_alpha[((int64_t)j * (QMAX + 1) + i) * a.lda + c] = v;
-  }
-  if (store) {
-    a.seg_h[(int64_t)j * a.lda + c] = h;
-    a.seg_q[(int64_t)j * a.lda + c] = q;
-  }
-  // the previous step's factors serve as Newton matrix unless gamma moved too
-  // far from theirs (the integrator's own refresh rule); every kCkpt-th step
-  // (each segment's first) starts from fresh factors at the predictor
-  const bool fresh = j % kCkpt == 0 || fabs(h / al[0] / d.gam_J[c] - 1.0) > d.gamma_tol;
-  d.flags[c] = F_NEWTON | (fresh ? F_REFRESH : 0);
-  d.m_it[c] = 0;
-  d.dprev[c] = 0.0;
-  d.crate[c] = 1.0;
-  for (int s = 0; s < d.n; ++s) {
-    const int64_t o = (int64_t)s * d.ld + c;
-    const double y0 = Yh(d, 0)[o];
-    double yp;
-    if (lagr) {
-      yp = 0.0;
-      for (int i = 0; i <= q; ++i) yp += wts[i] * Yh(d, i)[o];
-    } else {
-      yp = y0 + h * d.f0[o];
+  if (wi == 0) {   // (nothing above reads what warp 0 writes here)
+    d.h[c] = h;
+    d.gam[c] = h / al[0];
+    for (int i = 0; i <= QMAX; ++i) {
+      const double v = i <= q ? al[i] : 0.0;
+      d.alpha[(int64_t)i * d.ld + c] = v;
+      if (store) a.seg_alpha[((int64_t)j * (QMAX + 1) + i) * a.lda + c] = v;
     }
-    double ps = 0.0;
-    for (int i = 1; i <= q; ++i) ps += al[i] * Yh(d, i - 1)[o];
+    if (store) {
+      a.seg_h[(int64_t)j * a.lda + c] = h;
+      a.seg_q[(int64_t)j * a.lda + c] = q;
+    }
+    // the previous step's factors serve as Newton matrix unless gamma moved too
+    // far from theirs (the integrator's own refresh rule); every kCkpt-th step
+    // (each segment's first) starts from fresh factors at the predictor
+    const bool fresh = j % kCkpt == 0 || fabs(h / al[0] / d.gam_J[c] - 1.0) > d.gamma_tol;
+    d.flags[c] = F_NEWTON | (fresh ? F_REFRESH : 0);
+    d.m_it[c] = 0;
+    d.dprev[c] = 0.0;
+    d.crate[c] = 1.0;
+  }
+#pragma unroll 4
+  for (int s = wi; s < d.n; s += kCoopWarps) {
+    const int64_t o = (int64_t)s * d.ld + c;
+    double Yv[QMAX + 1];
+#pragma unroll
+    for (int i = 0; i <= QMAX; ++i) Yv[i] = i <= q && (i == 0 || i < nh) ? Yh(d, i)[o] : 0.0;
+    double yp = lagr ? 0.0 : Yv[0] + h * d.f0[o], ps = 0.0;
+#pragma unroll
+    for (int i = 0; i <= QMAX; ++i) {
+      if (lagr && i <= q) yp += wts[i] * Yv[i];
+      if (i >= 1 && i <= q) ps += al[i] * Yv[i - 1];
+    }
     d.ypred[o] = yp;
     d.y[o] = yp;
     d.psi[o] = ps;
-    d.w[o] = 1.0 / (d.rtol * fabs(y0) + d.atol);
+    d.w[o] = 1.0 / (d.rtol * fabs(Yv[0]) + d.atol);
   }
 }
 
@@ -1819,35 +1861,78 @@ __global__ void rretry_kernel(Dev d, AdjDev a, int j) {
 
 // Keeps the solved state for the backward pass and shifts the history; the
 // state also becomes the point at which the next refresh evaluates J.
-__global__ void rcommit_kernel(Dev d, AdjDev a, int j, int store) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d.C) return;
-  const int m = seg_step(a, c, j);
-  if (!m) return;
+__global__ void __launch_bounds__(32 * kCoopWarps) rcommit_kernel(Dev d, AdjDev a, int j, int store) {
+  const int64_t c = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+  const int wi = threadIdx.x >> 5;
+  const int m = c < d.C ? seg_step(a, c, j) : 0;
+  const int nh = m ? d.nh[c] : 0, nh_new = min(nh + 1, d.q_max + 1);
+  if (m) {
+#pragma unroll 4
+    for (int s = wi; s < d.n; s += kCoopWarps) {
+      const int64_t o = (int64_t)s * d.ld + c;
+      const double yv = d.y[o];
+      double Yv[QMAX];
+#pragma unroll
+      for (int i = 0; i < QMAX; ++i) Yv[i] = i < nh_new - 1 ? Yh(d, i)[o] : 0.0;
+      if (store) {
+        a.seg_y[((int64_t)j * d.n + s) * a.lda + c] = yv;
+        d.ypred[o] = yv;
+      }
+#pragma unroll
+      for (int i = 0; i < QMAX; ++i)
+        if (i < nh_new - 1) Yh(d, i + 1)[o] = Yv[i];
+      Yh(d, 0)[o] = yv;
+    }
+  }
+  __syncthreads();   // every warp has read nh
+  if (wi != 0 || !m) return;
   // iterations stopped short of the replay tolerance still count when the
   // last correction met the tolerance the recorded run was solved to
   if (!(d.flags[c] & F_CONV) && !(d.dprev[c] <= a.run_tol)) a.astat[c] = 2;
-  const int nh = d.nh[c], nh_new = min(nh + 1, d.q_max + 1);
-  for (int s = 0; s < d.n; ++s) {
-    const int64_t o = (int64_t)s * d.ld + c;
-    const double yv = d.y[o];
-    if (store) {
-      a.seg_y[((int64_t)j * d.n + s) * a.lda + c] = yv;
-      d.ypred[o] = yv;
-    }
-    for (int i = nh_new - 1; i >= 1; --i) Yh(d, i)[o] = Yh(d, i - 1)[o];
-    Yh(d, 0)[o] = yv;
-  }
   for (int i = nh_new - 1; i >= 1; --i) d.tn[(int64_t)i * d.ld + c] = d.tn[(int64_t)(i - 1) * d.ld + c];
   d.tn[c] = d.log_t[(int64_t)(m - 1) * d.ld + c];
   d.nh[c] = nh_new;
 }
 
-// One backward step at segment position j: block = one cell, one warp per
-// cotangent.  The slot holds the factors of M_m in elimination order (unit L,
-// U with inverse pivots on the diagonal), so M_m^T = U^T L^T is solved as a
+// One backward step at segment position j: gridDim.y blocks per cell, one warp
+// per cotangent.  The slot holds the factors of M_m in elimination order (unit
+// L, U with inverse pivots on the diagonal), so M_m^T = U^T L^T is solved as a
 // forward sweep over the rows of U followed by a backward sweep over the rows
-// of L, each row scattering its contribution.
+// of L, each row scattering its contribution.  The sweeps are a chain of 2 n
+// rows whose entries come from L2: they are read three rows ahead in stages
+// (row pointers, column indices, values), so that a row costs its arithmetic and
+// not three trips to memory.
+struct RowAhead {   // a row's first 32 kE entries, kE per lane
+  static constexpr int kE = 12;
+  int p0, p1, j[kE];
+  double v[kE];
+  __device__ __forceinline__ void pointers(const int* __restrict__ ptr, int row, bool in) {
+    p0 = in ? __ldg(ptr + row) : 0;
+    p1 = in ? __ldg(ptr + row + 1) : 0;
+  }
+  __device__ __forceinline__ void indices(const int* __restrict__ idx, int lane) {
+#pragma unroll
+    for (int e = 0; e < kE; ++e) j[e] = p0 + lane + 32 * e < p1 ? __ldg(idx + p0 + lane + 32 * e) : -1;
+  }
+  __device__ __forceinline__ void values(const double* __restrict__ A) {
+#pragma unroll
+    for (int e = 0; e < kE; ++e) v[e] = j[e] >= 0 ? A[j[e]] : 0.0;
+  }
+  // xs[j] -= v x; longer rows finish from memory
+  __device__ __forceinline__ void apply(double* xs, double x, const int* __restrict__ idx, const double* __restrict__ A,
+                                        int lane) const {
+#pragma unroll
+    for (int e = 0; e < kE; ++e) {
+      if (p0 + 32 * e >= p1) break;
+      if (j[e] >= 0) xs[j[e]] -= v[e] * x;
+    }
+    for (int p = p0 + 32 * kE + lane; p < p1; p += 32) {
+      const int jj = __ldg(idx + p);
+      xs[jj] -= A[jj] * x;
+    }
+  }
+};
+
 __global__ void adj_step_kernel(Dev d, AdjDev a, int j) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int64_t c = blockIdx.x;
@@ -1871,7 +1956,7 @@ __global__ void adj_step_kernel(Dev d, AdjDev a, int j) {
   const int N = a.N[c];
   const int slot = m % kRing;
   const double* A = slot_lu(d, a, j, c);
-  for (int v = warp; v < a.n_cot; v += nwarps) {
+  for (int v = blockIdx.y * nwarps + warp; v < a.n_cot; v += gridDim.y * nwarps) {
     for (int s = lane; s < n; s += 32) {
       double b = m == N ? a.cot[((int64_t)v * n + s) * a.ldu + c] : 0.0;
       for (int dd = 1; dd <= QMAX && m + dd <= N; ++dd) {
@@ -1884,29 +1969,42 @@ __global__ void adj_step_kernel(Dev d, AdjDev a, int j) {
     }
     __syncwarp();
     // U^T: u_k = x_k / u_kk, then x_j -= u_kj u_k over row k of U
-    for (int kk = 0; kk < n; ++kk) {
-      const double uk = xs[kk] * A[(int64_t)kk * ldm + kk];
-      __syncwarp();
-      if (lane == 0) xs[kk] = uk;
-      const double* Ak = A + (int64_t)kk * ldm;
-      const int p1 = __ldg(d.uptr + kk + 1);
-      for (int p = __ldg(d.uptr + kk) + lane; p < p1; p += 32) {
-        const int jj = __ldg(d.uidx + p);
-        xs[jj] -= Ak[jj] * uk;
-      }
-      __syncwarp();
-    }
     // L^T (unit): v_i is final once the rows below it are done; x_k -= l_ik v_i
-    for (int ii = n - 1; ii > 0; --ii) {
-      const double vi = xs[ii];
-      const double* Ai = A + (int64_t)ii * ldm;
-      const int p1 = __ldg(d.lrptr + ii + 1);
-      for (int p = __ldg(d.lrptr + ii) + lane; p < p1; p += 32) {
-        const int kk = __ldg(d.lridx + p);
-        xs[kk] -= Ai[kk] * vi;
+    auto sweep = [&](const int* ptr, const int* idx, bool up) {
+      auto row = [&](int t) { return up ? t : n - 1 - t; };
+      const int rows = up ? n : n - 1;
+      RowAhead w0, w1, w2, w3;   // rows t .. t + 3
+      auto diag = [&](int t) { return up && t < rows ? A[(int64_t)t * ldm + t] : 1.0; };
+      w0.pointers(ptr, row(0), rows > 0);
+      w1.pointers(ptr, row(1), rows > 1);
+      w2.pointers(ptr, row(2), rows > 2);
+      w0.indices(idx, lane);
+      w1.indices(idx, lane);
+      w0.values(A + (int64_t)row(0) * ldm);
+      double d0 = diag(0), d1 = diag(1);
+      for (int t = 0; t < rows; ++t) {
+        const int k = row(t);
+        const double d2 = diag(t + 2);
+        w3.pointers(ptr, row(t + 3), t + 3 < rows);
+        w2.indices(idx, lane);
+        w1.values(A + (int64_t)(t + 1 < rows ? row(t + 1) : 0) * ldm);
+        double x = xs[k];
+        if (up) {
+          x *= d0;
+          __syncwarp();
+          if (lane == 0) xs[k] = x;
+        }
+        w0.apply(xs, x, idx, A + (int64_t)k * ldm, lane);
+        __syncwarp();
+        w0 = w1;
+        w1 = w2;
+        w2 = w3;
+        d0 = d1;
+        d1 = d2;
       }
-      __syncwarp();
-    }
+    };
+    sweep(d.uptr, d.uidx, true);
+    sweep(d.lrptr, d.lridx, false);
     for (int s = lane; s < n; s += 32) {
       const double lv = xs[__ldg(d.iperm + s)];
       ls[s] = lv;
@@ -1914,32 +2012,69 @@ __global__ void adj_step_kernel(Dev d, AdjDev a, int j) {
     }
     __syncwarp();
     double* gv = a.g + (c * a.n_cot + v) * n_r;
-    for (int r = lane; r < n_r; r += 32) {
-      double w = 0.0;
-      const int p1 = __ldg(d.sc_ptr + r + 1);
-      for (int p = __ldg(d.sc_ptr + r); p < p1; ++p) {
-        const uint32_t e = __ldg(d.sc_ent + p);
-        w = fma((double)(int8_t)(e >> 24), ls[e & 0xFFFFFFu], w);
+    constexpr int kU = 4, kP = 4;   // reactions at a time, entries read ahead of each
+    for (int r0 = lane; r0 < n_r; r0 += 32 * kU) {
+      int p0[kU], p1[kU];
+      uint32_t e[kU][kP];
+      double g[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int r = r0 + 32 * u;
+        p0[u] = r < n_r ? __ldg(d.sc_ptr + r) : 0;
+        p1[u] = r < n_r ? __ldg(d.sc_ptr + r + 1) : 0;
+        g[u] = r < n_r ? gv[r] : 0.0;
       }
-      gv[r] = fma(h * Rs[r], w, gv[r]);
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+#pragma unroll
+        for (int q = 0; q < kP; ++q) e[u][q] = p0[u] + q < p1[u] ? __ldg(d.sc_ent + p0[u] + q) : 0;
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        if (r0 + 32 * u >= n_r) break;
+        double w = 0.0;
+#pragma unroll
+        for (int q = 0; q < kP; ++q)
+          if (p0[u] + q < p1[u]) w = fma((double)(int8_t)(e[u][q] >> 24), ls[e[u][q] & 0xFFFFFFu], w);
+        for (int p = p0[u] + kP; p < p1[u]; ++p) {
+          const uint32_t x = __ldg(d.sc_ent + p);
+          w = fma((double)(int8_t)(x >> 24), ls[x & 0xFFFFFFu], w);
+        }
+        gv[r0 + 32 * u] = fma(h * Rs[r0 + 32 * u], w, g[u]);
+      }
     }
     __syncwarp();
   }
   __syncthreads();
+  if (blockIdx.y > 0) return;
   if (tid == 0) a.ring_q[(int64_t)slot * a.lda + c] = a.seg_q[(int64_t)j * a.lda + c];
   if (tid <= QMAX)
     a.ring_alpha[((int64_t)slot * (QMAX + 1) + tid) * a.lda + c] =
         a.seg_alpha[((int64_t)j * (QMAX + 1) + tid) * a.lda + c];
 }
 
-// Gradient out as [n_cot][n_r][ldg] (cells fastest), per-cell status, and the
-// number of cells without a usable result in counters[2].
-__global__ void adj_out_kernel(Dev d, AdjDev a, double* __restrict__ out, int64_t ldg, int* __restrict__ astat_out) {
+// out[c][r] = in[r][c] over rows r < R, cells c < C (32 x 32 tiles).
+__global__ void __launch_bounds__(256) transpose_kernel(const double* __restrict__ in, int64_t ldi, double* __restrict__ out,
+                                                        int64_t ldo, int64_t R, int64_t C) {
+  __shared__ double t[32][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
+  for (int i = y; i < 32; i += 8)
+    if (r0 + i < R && c0 + x < C) t[i][x] = in[(r0 + i) * ldi + c0 + x];
+  __syncthreads();
+  for (int i = y; i < 32; i += 8)
+    if (c0 + i < C && r0 + x < R) out[(c0 + i) * ldo + r0 + x] = t[x][i];
+}
+void transpose(const double* in, int64_t ldi, double* out, int64_t ldo, int64_t R, int64_t C, cudaStream_t s) {
+  const dim3 grid((unsigned)((C + 31) / 32), (unsigned)((R + 31) / 32));
+  transpose_kernel<<<grid, 256, 0, s>>>(in, ldi, out, ldo, R, C);
+}
+
+// Per-cell status out, and the number of cells without a usable result in
+// counters[2].  (The gradient [n_cot][n_r][ldg], cells fastest, is a.g
+// transposed.)
+__global__ void adj_out_kernel(Dev d, AdjDev a, int* __restrict__ astat_out) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= d.C) return;
-  for (int v = 0; v < a.n_cot; ++v)
-    for (int r = 0; r < d.n_r; ++r)
-      out[((int64_t)v * d.n_r + r) * ldg + c] = a.g[(c * a.n_cot + v) * d.n_r + r];
   const int s = a.astat[c];
   if (astat_out) astat_out[c] = s;
   if (s) atomicAdd(&d.counters[2], 1);
@@ -1949,21 +2084,19 @@ __global__ void adj_out_kernel(Dev d, AdjDev a, double* __restrict__ out, int64_
 // q_{m'} >= m' (their lambdas are still in the ring once segment 0 is done),
 // as out[n_cot][n][ldg]; 0 for cells without a usable result.
 __global__ void adj_y0_kernel(Dev d, AdjDev a, double* __restrict__ out, int64_t ldg) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d.C) return;
+  const int64_t c = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);   // a warp per (species, target)
+  const int s = blockIdx.y * 8 + (threadIdx.x >> 5), v = blockIdx.z;
+  if (c >= d.C || s >= d.n) return;
   const bool ok = a.astat[c] == 0;
   const int N = a.N[c];
-  for (int v = 0; v < a.n_cot; ++v)
-    for (int s = 0; s < d.n; ++s) {
-      double g = 0.0;
-      for (int mp = 1; ok && mp <= QMAX && mp <= N; ++mp) {
-        const int sl = mp % kRing;
-        if (a.ring_q[(int64_t)sl * a.lda + c] >= mp)
-          g -= a.ring_alpha[((int64_t)sl * (QMAX + 1) + mp) * a.lda + c] *
-               a.lam[(((int64_t)sl * a.n_cot + v) * d.n + s) * a.lda + c];
-      }
-      out[((int64_t)v * d.n + s) * ldg + c] = g;
-    }
+  double g = 0.0;
+  for (int mp = 1; ok && mp <= QMAX && mp <= N; ++mp) {
+    const int sl = mp % kRing;
+    if (a.ring_q[(int64_t)sl * a.lda + c] >= mp)
+      g -= a.ring_alpha[((int64_t)sl * (QMAX + 1) + mp) * a.lda + c] *
+           a.lam[(((int64_t)sl * a.n_cot + v) * d.n + s) * a.lda + c];
+  }
+  out[((int64_t)v * d.n + s) * ldg + c] = g;
 }
 
 // Replay result: y_N of replayed cells, NaN for the others.
@@ -2170,7 +2303,7 @@ sm_status enqueue_attempt(sm_state* st, const double* k, int64_t ldk, cudaStream
     th_rates_kernel<<<th_grid, 128, 0, s>>>(d, d.ypred + (int64_t)d.t_idx * d.ld, 0);
     st->launches += 1;
   }
-  refresh_kernel<T><<<st->refresh_ctas, kRefreshThreads, st->plan.bytes, s>>>(d, k, ldk, st->plan);
+  refresh_kernel<T><<<st->refresh_ctas, kRefreshThreads, st->plan.bytes, s>>>(d, k, ldk, st->plan, 1);
   if (d.therm) {
     const unsigned nb = (unsigned)std::min<int64_t>(blocks(d.C, kBorderWarps), 152LL * 16);
     th_border_kernel<T><<<nb, 32 * kBorderWarps, st->border_smem, s>>>(d);
@@ -2397,11 +2530,13 @@ sm_status adj_prepare(sm_state* st, int64_t c0, int64_t Cp, int64_t lda, const d
   a.cot = cot ? cot + c0 : nullptr;
   a.ldu = ldk;
   SM_TRY_CUDA(cudaMemsetAsync(dd.counters, 0, 4 * sizeof(int), s));
-  adj_setup_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, k + c0, ldk);
+  adj_setup_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a);
+  transpose(k + c0, ldk, a.kc, n_r, n_r, Cp, s);
+  SM_TRY_CUDA(cudaMemsetAsync(a.g, 0, sizeof(double) * (size_t)Cp * n_cot * n_r, s));
   SM_TRY_CUDA(cudaGetLastError());
   SM_TRY_CUDA(cudaMemcpyAsync(st->h_counters, dd.counters, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
   SM_TRY_CUDA(cudaStreamSynchronize(s));
-  st->launches += 1;
+  st->launches += 2;
   *Kmax = st->h_counters[3];
   *Nmax = st->h_counters[1];
   *dd_out = dd;
@@ -2415,6 +2550,49 @@ sm_status adj_count_bad(sm_state* st, int64_t* bad) {
   SM_TRY_CUDA(cudaMemcpyAsync(st->h_counters, st->d.counters, 4 * sizeof(int), cudaMemcpyDeviceToHost, st->s));
   SM_TRY_CUDA(cudaStreamSynchronize(st->s));
   *bad += st->h_counters[2];
+  return SM_OK;
+}
+
+// CTAs per cell of the replays' FP64 refresh: with few cells one CTA each left
+// most SMs idle for the 10 M cycles of a 470-species factorisation, nearly all
+// of them FP64 FMAs of the trailing updates.  The most CTAs (six at most: a
+// 349-column tail has six columns of tiles) for which every cell's cluster is
+// resident at once.
+int replay_cluster(const sm_state* st, int64_t C) {
+  for (int S = 6; S > 1; --S) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)S);
+    cfg.blockDim = dim3(kRefreshThreads);
+    cfg.dynamicSmemBytes = st->plan.bytes;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)S;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, refresh_kernel<double>, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    if (n >= C) return S;
+  }
+  return 1;
+}
+
+sm_status launch_replay_refresh(sm_state* st, const Dev& d, int S, const double* k, int64_t ldk) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(S > 1 ? S * d.C : st->refresh_ctas));
+  cfg.blockDim = dim3(kRefreshThreads);
+  cfg.dynamicSmemBytes = st->plan.bytes;
+  cfg.stream = st->s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)S;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = S > 1 ? 1 : 0;
+  SM_TRY_CUDA(cudaLaunchKernelEx(&cfg, refresh_kernel<double>, d, k, ldk, st->plan, S));
   return SM_OK;
 }
 
@@ -2437,19 +2615,25 @@ sm_status adjoint_pass(sm_state* st, int64_t c0, int64_t Cp, int64_t lda, const 
     x.lu = a.slots + (int64_t)j * Cp * dd.lu_stride;
     return x;
   };
+  const int S = replay_cluster(st, Cp);
+  // few cells: their cotangents over several blocks, a warp per scheduler
+  int groups = 1;
+  if (warps > 4 && Cp * ((n_cot + 3) / 4) <= 2 * 152) {
+    groups = (n_cot + 3) / 4;
+    warps = 4;
+  }
   auto refresh_at = [&](int j, int need_flag) -> sm_status {
     SM_TRY_CUDA(cudaMemsetAsync(dd.counters, 0, sizeof(int), s));
     adj_list_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, j, need_flag);
-    refresh_kernel<double><<<st->refresh_ctas, kRefreshThreads, st->plan.bytes, s>>>(slot_dev(j), kp, ldk, st->plan);
     st->launches += 2;
-    return SM_OK;
+    return launch_replay_refresh(st, slot_dev(j), S, kp, ldk);
   };
   const size_t solve_smem = sizeof(double) * (size_t)kSolveWarps * ((dd.n + 3) / 4 * 4);
   for (int rs = 0; rs < Kmax; ++rs) {
     seg_restore_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, rs);
     st->launches += 1;
     for (int j = 0; j < kCkpt; ++j) {
-      rpredict_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, j, 1);
+      rpredict_kernel<<<blocks(Cp, 32), 32 * kCoopWarps, 0, s>>>(dd, a, j, 1);
       st->launches += 1;
       // Newton matrix: the factors at y_{m-1} (slot j - 1), or, for the cells
       // flagged F_REFRESH, fresh ones at the predictor in slot j (replaced by
@@ -2473,21 +2657,23 @@ sm_status adjoint_pass(sm_state* st, int64_t c0, int64_t Cp, int64_t lda, const 
           st->launches += 3;
         }
       }
-      rcommit_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, j, 1);
+      rcommit_kernel<<<blocks(Cp, 32), 32 * kCoopWarps, 0, s>>>(dd, a, j, 1);
       st->launches += 1;
       if ((r = refresh_at(j, 0)) != SM_OK) return r;
     }
     for (int j = kCkpt - 1; j >= 0; --j) {
-      adj_step_kernel<<<(unsigned)Cp, 32 * warps, smem, s>>>(dd, a, j);
+      adj_step_kernel<<<dim3((unsigned)Cp, (unsigned)groups), 32 * warps, smem, s>>>(dd, a, j);
       st->launches += 1;
     }
     SM_TRY_CUDA(cudaGetLastError());
   }
   SM_TRY_CUDA(cudaMemsetAsync(dd.counters + 2, 0, sizeof(int), s));
-  adj_out_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, grad + c0, ldk, astat ? astat + c0 : nullptr);
-  st->launches += 1;
+  transpose(a.g, (int64_t)n_cot * dd.n_r, grad + c0, ldk, Cp, (int64_t)n_cot * dd.n_r, s);
+  adj_out_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, astat ? astat + c0 : nullptr);
+  st->launches += 2;
   if (grad_y0) {
-    adj_y0_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, grad_y0 + c0, ldk);
+    const dim3 grid((unsigned)((Cp + 31) / 32), (unsigned)((dd.n + 7) / 8), (unsigned)n_cot);
+    adj_y0_kernel<<<grid, 256, 0, s>>>(dd, a, grad_y0 + c0, ldk);
     st->launches += 1;
   }
   SM_TRY_CUDA(cudaGetLastError());
@@ -2510,10 +2696,11 @@ sm_status replay_pass(sm_state* st, int64_t c0, int64_t Cp, int64_t lda, const d
   const double* kp = k + c0;
   double* scratch = st->scratch.as<double>() + c0;
   const size_t solve_smem = sizeof(double) * (size_t)kSolveWarps * ((dd.n + 3) / 4 * 4);
+  const int S = replay_cluster(st, Cp);
   seg_restore_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, -1);
   st->launches += 1;
   for (int j = 0; j < Nmax; ++j) {
-    rpredict_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, j, 0);
+    rpredict_kernel<<<blocks(Cp, 32), 32 * kCoopWarps, 0, s>>>(dd, a, j, 0);
     st->launches += 1;
     for (int attempt = 0; attempt < 2; ++attempt) {
       if (attempt == 1) {
@@ -2522,7 +2709,7 @@ sm_status replay_pass(sm_state* st, int64_t c0, int64_t Cp, int64_t lda, const d
       }
       SM_TRY_CUDA(cudaMemsetAsync(dd.counters, 0, sizeof(int), s));
       adj_list_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, j, F_NEWTON | F_REFRESH);
-      refresh_kernel<double><<<st->refresh_ctas, kRefreshThreads, st->plan.bytes, s>>>(dd, kp, ldk, st->plan);
+      if ((r = launch_replay_refresh(st, dd, S, kp, ldk)) != SM_OK) return r;
       st->launches += 2;
       for (int it = 0; it < kReplayIters; ++it) {
         r = launch_rhs_masked(net, Cp, kp, ldk, dd.y, dd.f, dd.ld, scratch, dd.ld, dd.flags, F_NEWTON, nullptr, s);
@@ -2531,7 +2718,7 @@ sm_status replay_pass(sm_state* st, int64_t c0, int64_t Cp, int64_t lda, const d
         st->launches += 3;
       }
     }
-    rcommit_kernel<<<blocks(Cp, 128), 128, 0, s>>>(dd, a, j, 0);
+    rcommit_kernel<<<blocks(Cp, 32), 32 * kCoopWarps, 0, s>>>(dd, a, j, 0);
     st->launches += 1;
     SM_TRY_CUDA(cudaGetLastError());
   }
