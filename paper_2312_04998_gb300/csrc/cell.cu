@@ -361,14 +361,21 @@ __device__ __forceinline__ T diag_forward(T xi, const T* dg, int lane, int w) {
 }
 template <class T>
 __device__ __forceinline__ T diag_backward(T xi, const T* dg, int lane, int w) {
+  // a product, a shuffle and an FMA a step: every lane forms its own entry's
+  // product with its inverse pivot, the shuffle takes lane k's; a finished
+  // lane's result is kept aside, what it computes after that is not used
+  const T inv = lane < w ? dg[lane * 32 + lane] : T(0);
+  T out = T(0);
+  if (lane >= w) xi = T(0);   // (past w: padding)
 #pragma unroll 8
   for (int k = 31; k >= 0; --k) {
-    const T u = lane <= k ? dg[k * 32 + lane] : T(0);
-    const T t = xi * u;   // the solved entry in lane k (inverse pivots)
+    const T u = lane < k && k < w ? dg[k * 32 + lane] : T(0);
+    const T t = xi * inv;
     const T xk = __shfl_sync(kFull, t, k);
-    if (k < w) xi = lane == k ? t : (lane < k ? xi - u * xk : xi);   // (past w: padding)
+    out = lane == k ? t : out;
+    xi -= u * xk;
   }
-  return xi;
+  return out;
 }
 
 // One row block of the tail in a warp's registers: its entry per lane and the
@@ -479,6 +486,7 @@ __device__ __forceinline__ void cell_solve() {
     if (K + 1 == ra) {
       a.x = diag_forward(a.x, dg + ra * 1024, lane, min(32, nt - 32 * ra));
       xt[32 * ra + lane] = ina ? a.x : T(0);
+      if (ra < nb - 1) a.load(D + (32 * (nb - 1)) * ldd + 32 * ra + lane, ldd, nt - 32 * (nb - 1));   // the way back's first
     } else if (K + 1 >= nw && (K + 1) % nw == ra) {
       __syncwarp();
       far_solve(K + 1, true);
@@ -487,7 +495,6 @@ __device__ __forceinline__ void cell_solve() {
   __syncthreads();
   // tail, backward (inverse pivots on the diagonal)
   auto col = [&](int K) { return D + (32 * K) * ldd + 32 * ra + lane; };
-  if (ra < nb - 1) a.load(col(nb - 1), ldd, nt - 32 * (nb - 1));
   for (int K = nb; K > 0; --K) {
     if (K < nb) {
       __syncthreads();
