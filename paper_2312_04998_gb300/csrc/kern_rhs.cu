@@ -2,9 +2,9 @@
 //
 // Four traversals of S, the GPU counterparts of the paper's Listings 1-4:
 //  * CRS  (Listing 3): rows gathered; the nonzeros of S are cut into equal
-//    chunks (one per half-warp) so the long hub rows (H: ~2000 nonzeros) are
-//    shared; rows split across chunks are summed in chunk order through shared
-//    memory, so results are deterministic.
+//    chunks (a warp or half-warp each) so the long hub rows (H: ~2000
+//    nonzeros) are shared; rows split across chunks are summed in chunk order
+//    through shared memory, so results are deterministic.
 //  * COO  (Listing 1): each nonzero adds coef * R_col into f_row (two indirect
 //    indices, FP64 atomics in L2).
 //  * CCS  (Listing 2): each reaction's rate is formed once in registers and
@@ -13,6 +13,7 @@
 //    the slice column-major, pads included.
 // In every traversal a lane owns one cell: index loads are warp-uniform
 // broadcasts and abundance / rate loads are 128-byte coalesced rows.
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -26,24 +27,6 @@ constexpr int kChunks = 32;       // CRS nonzero chunks per CTA (two per warp)
 constexpr int kRThreads = 128;
 constexpr int kRChunk = 64;
 
-__device__ __forceinline__ int upper_bound_i32(const int* __restrict__ a, int n, int v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (__ldg(a + mid) <= v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-__device__ __forceinline__ int lower_bound_i32(const int* __restrict__ a, int n, int v) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (__ldg(a + mid) < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
 __device__ __forceinline__ double neg_if(double v, bool neg) {
   return neg ? __longlong_as_double(__double_as_longlong(v) ^ (1ll << 63)) : v;
 }
@@ -52,15 +35,15 @@ __device__ __forceinline__ double neg_if(double v, bool neg) {
 __global__ void __launch_bounds__(kRThreads)
 reaction_rate_kernel(int n_r, int64_t C, const int2* __restrict__ reac, const double* __restrict__ k,
                      int64_t ldk, const double* __restrict__ y, int64_t ldy, double* __restrict__ r,
-                     int64_t ldr, const int* __restrict__ mask, int bit, const int* __restrict__ cact) {
+                     int64_t ldr, int chunk, const int* __restrict__ mask, int bit, const int* __restrict__ cact) {
   if (cact && (int64_t)blockIdx.x * kRThreads >= *cact) return;   // no running cell in this block
   const int64_t c = (int64_t)blockIdx.x * kRThreads + threadIdx.x;
   const bool act = c < C && (!mask || (mask[c] & bit));
   if (mask && !__syncthreads_or(act)) return;
   if (!act) return;
-  const int j1 = min(n_r, (int)(blockIdx.y + 1) * kRChunk);
+  const int j1 = min(n_r, (int)(blockIdx.y + 1) * chunk);
 #pragma unroll 4
-  for (int j = blockIdx.y * kRChunk; j < j1; ++j) {
+  for (int j = blockIdx.y * chunk; j < j1; ++j) {
     const int2 a = __ldg(reac + j);
     double v = k[(int64_t)j * ldk + c] * y[(int64_t)a.x * ldy + c];
     if (a.y >= 0) v *= y[(int64_t)a.y * ldy + c];
@@ -68,13 +51,37 @@ reaction_rate_kernel(int n_r, int64_t C, const int2* __restrict__ reac, const do
   }
 }
 
-// sum over entries [b, e) of coef * r[col]: four independent partial sums so
-// that four rate loads are in flight per thread (the FP64 gather is bound by
-// their latency, not by the FP64 pipe)
+// Reactions per thread of that kernel: kRChunk, fewer where that leaves less
+// than 16 warps per SM (37 cells of 180 reactions: the kernel's latency is one
+// round of loads, not 16).
+int rate_chunk(int64_t n_r, int64_t C) {
+  constexpr int kSms = 152;
+  const int64_t fit = n_r * ((C + 31) / 32) / (16 * kSms);
+  return (int)std::min<int64_t>(kRChunk, std::max<int64_t>(4, fit));
+}
+
+// sum over entries [b, e) of coef * r[col]: four independent partial sums, eight
+// entries' loads in flight (index words, then rates: the gather waits for
+// memory, not for the FP64 unit)
 __device__ __forceinline__ double dot_range(const uint32_t* __restrict__ ent, int b, int e,
                                             const double* __restrict__ r, int64_t ldr, int64_t c) {
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
   int p = b;
+  for (; p + 7 < e; p += 8) {
+    uint32_t w[8];
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) w[u] = __ldg(ent + p + u);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = r[(int64_t)(w[u] & 0xFFFFFFu) * ldr + c];
+#pragma unroll
+    for (int u = 0; u < 8; u += 4) {
+      s0 = fma(c_coef[w[u] >> 24], v[u], s0);
+      s1 = fma(c_coef[w[u + 1] >> 24], v[u + 1], s1);
+      s2 = fma(c_coef[w[u + 2] >> 24], v[u + 2], s2);
+      s3 = fma(c_coef[w[u + 3] >> 24], v[u + 3], s3);
+    }
+  }
   for (; p + 3 < e; p += 4) {
     const uint32_t w0 = __ldg(ent + p), w1 = __ldg(ent + p + 1), w2 = __ldg(ent + p + 2), w3 = __ldg(ent + p + 3);
     const double r0 = r[(int64_t)(w0 & 0xFFFFFFu) * ldr + c], r1 = r[(int64_t)(w1 & 0xFFFFFFu) * ldr + c];
@@ -98,7 +105,7 @@ __device__ __forceinline__ double dot_range(const uint32_t* __restrict__ ent, in
 template <int KC, int KCH>
 __global__ void __launch_bounds__(KC * KCH)
 rhs_crs_kernel(int n_s, int64_t C, const int* __restrict__ row_ptr, const uint32_t* __restrict__ ent,
-               const int* __restrict__ row_id, const int* __restrict__ chunk_nz,
+               const int* __restrict__ row_id, const int4* __restrict__ chunk,
                const double* __restrict__ r, int64_t ldr, double* __restrict__ f, int64_t ld,
                const int* __restrict__ mask, int bit, const int* __restrict__ cact) {
   static_assert(KC * KCH == kCells * kChunks && 32 % KC == 0, "block shape");
@@ -111,32 +118,33 @@ rhs_crs_kernel(int n_s, int64_t C, const int* __restrict__ row_ptr, const uint32
   const bool live = c0 < C && (!mask || (mask[c0] & bit));
   if (mask && !__syncthreads_or(live)) return;
   const int64_t c = live ? c0 : 0;  // dead lanes read cell 0 and store nothing
-  const int z0 = __ldg(chunk_nz + ch), z1 = __ldg(chunk_nz + ch + 1);
-  // carry-in row: contains position z0 but starts before it
-  const int rc = upper_bound_i32(row_ptr, n_s + 1, z0) - 1;
-  double carry = 0.0;
-  bool has_carry = false;
-  if (z0 < z1 && rc < n_s && __ldg(row_ptr + rc) < z0) {
-    has_carry = true;
-    carry = dot_range(ent, z0, min(__ldg(row_ptr + rc + 1), z1), r, ldr, c);
-  }
+  // per chunk {end, row that it goes on with (-1: none), first and end of the
+  // rows that begin in it}; its first nonzero is the end of the chunk before
+  const int4 ci = __ldg(chunk + ch);
+  const int z0 = ch > 0 ? __ldg(&chunk[ch - 1].x) : 0, z1 = ci.x, rc = ci.y;
+  const double carry = rc >= 0 ? dot_range(ent, z0, min(__ldg(row_ptr + rc + 1), z1), r, ldr, c) : 0.0;
   // -2 marks an empty chunk (possible when nnz < KCH): fix-ups skip it
-  if (cl == 0) carry_row[ch] = z0 == z1 ? -2 : (has_carry ? rc : -1);
+  if (cl == 0) carry_row[ch] = z0 == z1 ? -2 : rc;
   part[ch][0][cl] = carry;
-  // rows owned by this chunk: row_ptr[row] in [z0, z1) (all rows for the last)
-  const int r_first = lower_bound_i32(row_ptr, n_s, z0);
-  const int r_end = (ch == KCH - 1) ? n_s : lower_bound_i32(row_ptr, n_s, z1);
+  const int r_first = ci.z, r_end = ci.w;
   double tail = 0.0;
   int tail_row = -1;
+  // (the next row's end and place are read ahead)
+  int b = r_first < r_end ? __ldg(row_ptr + r_first) : 0, e = r_first < r_end ? __ldg(row_ptr + r_first + 1) : 0;
+  int id = r_first < r_end ? __ldg(row_id + r_first) : 0;
   for (int row = r_first; row < r_end; ++row) {
-    const int b = __ldg(row_ptr + row), e = __ldg(row_ptr + row + 1);
+    const bool more = row + 1 < r_end;
+    const int e2 = more ? __ldg(row_ptr + row + 2) : 0, id2 = more ? __ldg(row_id + row + 1) : 0;
     const double s = dot_range(ent, b, min(e, z1), r, ldr, c);
     if (e <= z1) {
-      if (live) f[(int64_t)__ldg(row_id + row) * ld + c] = s;
+      if (live) f[(int64_t)id * ld + c] = s;
     } else {
       tail = s;
       tail_row = row;
     }
+    b = e;
+    e = e2;
+    id = id2;
   }
   part[ch][1][cl] = tail;
   __syncthreads();
@@ -149,6 +157,76 @@ rhs_crs_kernel(int n_s, int64_t C, const int* __restrict__ row_ptr, const uint32
     }
     if (live) f[(int64_t)__ldg(row_id + tail_row) * ld + c] = tot;
   }
+}
+
+// The same sums for every cell (rhs_eval): a warp per chunk and 32 cells, the 32
+// chunks of a group over a cluster of eight CTAs, which pass the parts of split
+// rows through distributed shared memory.  With 16 cells per chunk the two
+// halves of a warp walked rows of different lengths in turns; and a CTA of all
+// chunks left 4096 cells as 256 CTAs, 2 on some SMs and 1 on others (1024 small
+// ones: 7 or 6).  470 species, rates and gather, L2 flushed, one CTA per 16 cells
+// / this: 199 / 112 us for 33 cells, 218 / 137 for 1024, 435 / 346 for 4096, 834 /
+// 610 for 8192; the smaller networks tried (120, 32 species) gain at every size
+// too.  4096 cells: FP64 arithmetic takes 255 us.
+constexpr int kClChunks = 4, kCl = kChunks / kClChunks;
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t remote(const void* p, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(32 * kClChunks)
+rhs_crs_cluster_kernel(int64_t C, const int* __restrict__ row_ptr, const uint32_t* __restrict__ ent,
+                       const int* __restrict__ row_id, const int4* __restrict__ chunk, const double* __restrict__ r,
+                       int64_t ldr, double* __restrict__ f, int64_t ld) {
+  __shared__ double part[kClChunks][32];   // the part of the row that the chunk goes on with
+  __shared__ int carry_row[kClChunks];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ch = (blockIdx.x % kCl) * kClChunks + warp;
+  const int64_t c0 = (int64_t)(blockIdx.x / kCl) * 32 + lane;
+  const bool live = c0 < C;
+  const int64_t c = live ? c0 : 0;  // dead lanes read cell 0 and store nothing
+  const int4 ci = __ldg(chunk + ch);
+  const int z0 = ch > 0 ? __ldg(&chunk[ch - 1].x) : 0, z1 = ci.x, rc = ci.y;
+  part[warp][lane] = rc >= 0 ? dot_range(ent, z0, min(__ldg(row_ptr + rc + 1), z1), r, ldr, c) : 0.0;
+  if (lane == 0) carry_row[warp] = z0 == z1 ? -2 : rc;   // -2: empty chunk
+  double tail = 0.0;
+  int tail_row = -1, tail_id = 0;
+  int b = ci.z < ci.w ? __ldg(row_ptr + ci.z) : 0, e = ci.z < ci.w ? __ldg(row_ptr + ci.z + 1) : 0;
+  int id = ci.z < ci.w ? __ldg(row_id + ci.z) : 0;
+  for (int row = ci.z; row < ci.w; ++row) {   // (the next row's end and place are read ahead)
+    const bool more = row + 1 < ci.w;
+    const int e2 = more ? __ldg(row_ptr + row + 2) : 0, id2 = more ? __ldg(row_id + row + 1) : 0;
+    const double s = dot_range(ent, b, min(e, z1), r, ldr, c);
+    if (e <= z1) {
+      if (live) f[(int64_t)id * ld + c] = s;
+    } else {
+      tail = s;
+      tail_row = row;
+      tail_id = id;
+    }
+    b = e;
+    e = e2;
+    id = id2;
+  }
+  cluster_sync();
+  if (tail_row >= 0) {
+    for (int w = ch + 1; w < kChunks; ++w) {
+      int from;
+      double v;
+      asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(from) : "r"(remote(&carry_row[w % kClChunks], w / kClChunks)));
+      if (from == -2) continue;
+      if (from != tail_row) break;
+      asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(remote(&part[w % kClChunks][lane], w / kClChunks)));
+      tail += v;
+    }
+    if (live) f[(int64_t)tail_id * ld + c] = tail;
+  }
+  cluster_sync();   // the parts stay until everyone has read them
 }
 
 // COO: nonzeros in column-major order; ent = row | coef, col[] = reaction.
@@ -193,6 +271,8 @@ rhs_ccs_kernel(int n_r, int64_t C, const int* __restrict__ col_ptr, const uint32
 }
 
 // SELL-C-sigma: block = kCells cells x C slice rows, one slice per blockIdx.y.
+// Bound by the chain of the longest row: 1501 cells of 470 species took 727 us
+// with each entry's loads waiting for the one before, 285 us with them ahead.
 __global__ void rhs_sell_kernel(int64_t C, int slice_h, const int* __restrict__ slice_ptr,
                                 const uint32_t* __restrict__ ent, const int* __restrict__ row_id,
                                 const double* __restrict__ r, int64_t ldr, double* __restrict__ f,
@@ -203,9 +283,43 @@ __global__ void rhs_sell_kernel(int64_t C, int slice_h, const int* __restrict__ 
   const int i = __ldg(row_id + (int64_t)s * slice_h + rr);
   const int b = __ldg(slice_ptr + s);
   const int L = (__ldg(slice_ptr + s + 1) - b) / slice_h;
+  // a row is one chain of FMAs (2000 in the hub rows): while eight entries are
+  // added, the rates of the next eight and the index words of those after are
+  // on their way
   double acc = 0.0;
-  for (int kk = 0; kk < L; ++kk) {
-    const uint32_t w = __ldg(ent + b + kk * slice_h + rr);
+  constexpr int U = 8;
+  const uint32_t* q = ent + b + rr;
+  auto words = [&](int kk, uint32_t (&w)[U]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) w[u] = kk + U <= L ? __ldg(q + (kk + u) * slice_h) : 0;
+  };
+  auto rates = [&](int kk, const uint32_t (&w)[U], double (&v)[U]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = kk + U <= L ? r[(int64_t)(w[u] & 0xFFFFFFu) * ldr + c] : 0.0;
+  };
+  uint32_t w0[U], w1[U];
+  double v0[U];
+  words(0, w0);
+  words(U, w1);
+  rates(0, w0, v0);
+  int kk = 0;
+  for (; kk + U <= L; kk += U) {
+    uint32_t w2[U];
+    double v1[U];
+    rates(kk + U, w1, v1);
+    words(kk + 2 * U, w2);
+#pragma unroll
+    for (int u = 0; u < U; ++u) acc = fma(c_coef[w0[u] >> 24], v0[u], acc);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      w0[u] = w1[u];
+      w1[u] = w2[u];
+      v0[u] = v1[u];
+    }
+  }
+#pragma unroll 1
+  for (; kk < L; ++kk) {
+    const uint32_t w = __ldg(q + kk * slice_h);
     acc = fma(c_coef[w >> 24], r[(int64_t)(w & 0xFFFFFFu) * ldr + c], acc);
   }
   if (i >= 0) f[(int64_t)i * ld + c] = acc;
@@ -259,18 +373,17 @@ sm_status launch_rhs(const sm_net* net, int64_t C, const double* k, const double
     return SM_OK;
   }
   {
-    dim3 grid(groups_r, (unsigned)((net->n_r + kRChunk - 1) / kRChunk));
+    const int chunk = rate_chunk(net->n_r, C);
+    dim3 grid(groups_r, (unsigned)((net->n_r + chunk - 1) / chunk));
     reaction_rate_kernel<<<grid, kRThreads, 0, s>>>(net->n_r, C, net->d_reac.as<int2>(), k, ld, y, ld,
-                                                    scratch, ldr, nullptr, 0, nullptr);
+                                                    scratch, ldr, chunk, nullptr, 0, nullptr);
     SM_TRY_CUDA(cudaGetLastError());
   }
   const unsigned groups = (unsigned)((C + kCells - 1) / kCells);
   if (F.fmt == SM_FMT_CRS) {
     if ((int)F.chunk_nz.size() != kChunks + 1) return SM_EINVAL;
-    rhs_crs_kernel<kCells, kChunks><<<groups, kCells * kChunks, 0, s>>>(net->n_s, C, F.d_ptr.as<int>(),
-                                                       F.d_packed.as<uint32_t>(), F.d_aux.as<int>(),
-                                                       F.d_chunk.as<int>(), scratch, ldr, f, ld,
-                                                       nullptr, 0, nullptr);
+    rhs_crs_cluster_kernel<<<(unsigned)((C + 31) / 32) * kCl, 32 * kClChunks, 0, s>>>(
+        C, F.d_ptr.as<int>(), F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), F.d_chunk.as<int4>(), scratch, ldr, f, ld);
   } else if (F.fmt == SM_FMT_COO) {
     SM_TRY_CUDA(cudaMemsetAsync(f, 0, sizeof(double) * (size_t)net->n_s * ld, s));
     const int nnz = (int)F.idx.size();
@@ -295,21 +408,22 @@ sm_status launch_rhs_masked(const sm_net* net, int64_t C, const double* k, int64
   if (st != SM_OK) return st;
   const Format& F = net->integ_fmt[net->integ_order];
   if (F.packed.empty()) return SM_EINVAL;
-  dim3 grid((unsigned)((C + kRThreads - 1) / kRThreads), (unsigned)((net->n_r + kRChunk - 1) / kRChunk));
+  const int chunk = rate_chunk(net->n_r, C);
+  dim3 grid((unsigned)((C + kRThreads - 1) / kRThreads), (unsigned)((net->n_r + chunk - 1) / chunk));
   reaction_rate_kernel<<<grid, kRThreads, 0, s>>>(net->n_r, C, net->d_reac.as<int2>(), k, ldk, y, ld,
-                                                  scratch, ldr, mask, bit, cact);
+                                                  scratch, ldr, chunk, mask, bit, cact);
   SM_TRY_CUDA(cudaGetLastError());
   const int kc = net->integ_kc;
   const unsigned nb = (unsigned)((C + kc - 1) / kc);
   if (kc == 8) {
     rhs_crs_kernel<8, 64><<<nb, kCells * kChunks, 0, s>>>(net->n_s, C, F.d_ptr.as<int>(),
-        F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), F.d_chunk64.as<int>(), scratch, ldr, f, ld, mask, bit, cact);
+        F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), F.d_chunk64.as<int4>(), scratch, ldr, f, ld, mask, bit, cact);
   } else if (kc == 32) {
     rhs_crs_kernel<32, 16><<<nb, kCells * kChunks, 0, s>>>(net->n_s, C, F.d_ptr.as<int>(),
-        F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), F.d_chunk16.as<int>(), scratch, ldr, f, ld, mask, bit, cact);
+        F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), F.d_chunk16.as<int4>(), scratch, ldr, f, ld, mask, bit, cact);
   } else {
     rhs_crs_kernel<16, 32><<<nb, kCells * kChunks, 0, s>>>(net->n_s, C, F.d_ptr.as<int>(),
-        F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), F.d_chunk.as<int>(), scratch, ldr, f, ld, mask, bit, cact);
+        F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), F.d_chunk.as<int4>(), scratch, ldr, f, ld, mask, bit, cact);
   }
   SM_TRY_CUDA(cudaGetLastError());
   return SM_OK;

@@ -686,11 +686,22 @@ sm_status build_format(const sm_net* net, int32_t fmt, int32_t order, int32_t C,
   if (!g.ptr.empty() && (st = g.d_ptr.upload(g.ptr.data(), g.ptr.size() * 4)) != SM_OK) return st;
   if ((st = g.d_packed.upload(g.packed.data(), g.packed.size() * 4)) != SM_OK) return st;
   if (!g.aux.empty() && (st = g.d_aux.upload(g.aux.data(), g.aux.size() * 4)) != SM_OK) return st;
-  if (!g.chunk_nz.empty() && (st = g.d_chunk.upload(g.chunk_nz.data(), g.chunk_nz.size() * 4)) != SM_OK)
-    return st;
-  if (!g.chunk_nz64.empty() && (st = g.d_chunk64.upload(g.chunk_nz64.data(), g.chunk_nz64.size() * 4)) != SM_OK)
-    return st;
-  if (!g.chunk_nz16.empty() && (st = g.d_chunk16.upload(g.chunk_nz16.data(), g.chunk_nz16.size() * 4)) != SM_OK)
+  // the kernels' view of a partition: per chunk {end, row it goes on with (-1:
+  // none), first and end of the rows that begin in it}
+  auto chunks = [&](const std::vector<int32_t>& nz, DevArray& dst) -> sm_status {
+    if (nz.empty()) return SM_OK;
+    const int32_t n_ch = (int32_t)nz.size() - 1, n_row = (int32_t)g.ptr.size() - 1;
+    std::vector<int32_t> v;
+    for (int32_t c = 0; c < n_ch; ++c) {
+      const int32_t z0 = nz[c], z1 = nz[c + 1];
+      const int32_t rc = (int32_t)(std::upper_bound(g.ptr.begin(), g.ptr.end(), z0) - g.ptr.begin()) - 1;
+      auto first = [&](int32_t z) { return (int32_t)(std::lower_bound(g.ptr.begin(), g.ptr.end() - 1, z) - g.ptr.begin()); };
+      v.insert(v.end(), {z1, z0 < z1 && rc < n_row && g.ptr[rc] < z0 ? rc : -1, first(z0), c + 1 == n_ch ? n_row : first(z1)});
+    }
+    return dst.upload(v.data(), v.size() * 4);
+  };
+  if ((st = chunks(g.chunk_nz, g.d_chunk)) != SM_OK || (st = chunks(g.chunk_nz64, g.d_chunk64)) != SM_OK ||
+      (st = chunks(g.chunk_nz16, g.d_chunk16)) != SM_OK)
     return st;
   return SM_OK;
 }
