@@ -247,12 +247,10 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
         lr[base + l] = rc[lng[t + l]];
       }
     }
-    for (int32_t q = 0; q < ng; ++q) {
-      for (size_t l = 0; l < lng.size(); ++l)
-        if (grp[lng[l]] == q) {
-          de.push_back(dst[lng[l]]);
-          de.push_back(at[l]);
-        }
+    std::vector<std::vector<int32_t>> by(ng);
+    for (size_t l = 0; l < lng.size(); ++l) by[grp[lng[l]]].insert(by[grp[lng[l]]].end(), {dst[lng[l]], at[l]});
+    for (const auto& v : by) {
+      de.insert(de.end(), v.begin(), v.end());
       dg.push_back((int32_t)de.size() / 2);
     }
     p.n_jsl = s.slices();
@@ -285,32 +283,40 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
   }
   // Schur targets by panel
   {
-    std::vector<std::vector<int32_t>> tgt((size_t)nt * nt);
-    for (int32_t k = 0; k < h; ++k)
-      for (int32_t a = lu.lptr[k]; a < lu.lptr[k + 1]; ++a) {
-        const int32_t i = lu.lidx[a];
-        if (i < h) continue;
-        for (int32_t b = lu.uptr[k]; b < lu.uptr[k + 1]; ++b) {
-          const int32_t j = lu.uidx[b];
-          if (j >= h)
-            tgt[(size_t)(j - h) * nt + (i - h)].push_back(hpos[(size_t)i * n + k] | (hpos[(size_t)k * n + j] << 16));
+    // every target's terms, in pivot order (counted, then filled)
+    std::vector<int32_t> at((size_t)nt * nt + 1, 0), term;
+    auto each = [&](auto f) {
+      for (int32_t k = 0; k < h; ++k)
+        for (int32_t a = lu.lptr[k]; a < lu.lptr[k + 1]; ++a) {
+          const int32_t i = lu.lidx[a];
+          if (i < h) continue;
+          const int32_t l = hpos[(size_t)i * n + k];
+          for (int32_t b = lu.uptr[k]; b < lu.uptr[k + 1]; ++b)
+            if (lu.uidx[b] >= h) f((size_t)(lu.uidx[b] - h) * nt + (i - h), l, k, lu.uidx[b]);
         }
-      }
-    std::vector<int32_t> g(1, 0), ent;
+    };
+    each([&](size_t q, int32_t, int32_t, int32_t) { ++at[q + 1]; });
+    for (size_t q = 0; q < (size_t)nt * nt; ++q) at[q + 1] += at[q];
+    term.resize(at[(size_t)nt * nt]);
+    std::vector<int32_t> fill(at.begin(), at.end() - 1);
+    each([&](size_t q, int32_t l, int32_t k, int32_t j) { term[fill[q]++] = l | (hpos[(size_t)k * n + j] << 16); });
+    std::vector<int32_t> g(1, 0), ent, o;
     const int32_t pad = lu.p_d | (lu.p_d << 16);
+    auto size = [&](int32_t q) { return at[q + 1] - at[q]; };
     for (int32_t J = 0; J * kGroup < nt; ++J) {
-      const int32_t lo = kGroup * J * nt, hi = std::min(kGroup * (J + 1), nt) * nt;
-      std::vector<int32_t> o = by_length(tgt, lo, hi);
-      while (!o.empty() && tgt[o.back()].empty()) o.pop_back();
+      o.clear();
+      for (int32_t q = kGroup * J * nt; q < std::min(kGroup * (J + 1), nt) * nt; ++q)
+        if (size(q) > 0) o.push_back(q);
+      std::stable_sort(o.begin(), o.end(), [&](int32_t x, int32_t y) { return size(x) > size(y); });
       for (size_t b = 0; b < o.size(); b += 32) {
-        const size_t len = tgt[o[b]].size(), base = ent.size();
-        ent.resize(base + 32 * (len + 1), pad);
+        const int32_t len = size(o[b]);
+        const size_t base = ent.size();
+        ent.resize(base + 32 * ((size_t)len + 1), pad);
         for (size_t l = 0; l < 32; ++l) {
           const bool in = b + l < o.size();
           const int32_t q = in ? o[b + l] : 0;
-          ent[base + l] = (in ? tail_pos(h + q % nt, h + q / nt) : 0xFFFF) | (int32_t)(len << 16);
-          if (in)
-            for (size_t e = 0; e < tgt[q].size(); ++e) ent[base + 32 * (e + 1) + l] = tgt[q][e];
+          ent[base + l] = (in ? tail_pos(h + q % nt, h + q / nt) : 0xFFFF) | (len << 16);
+          for (int32_t e = 0; in && e < size(q); ++e) ent[base + 32 * ((size_t)e + 1) + l] = term[at[q] + e];
         }
       }
       g.push_back((int32_t)(ent.size() / 32));
