@@ -11,19 +11,25 @@
 // (substitution) busy at once, since different cells are in different phases.
 //
 // Work split inside an attempt (n species, n_r reactions, tail of nt columns):
-//   rates, S R    a thread per reaction, then the rows of S in pieces of at
-//                 most 32 entries, a piece per lane (CellProg); bound by the
-//                 FP64 pipe (2 lanes a clock per SM)
+//   rates, S R    a thread per reaction, then the rows of S in chains, a chain
+//                 per lane (CellProg); bound by the FP64 pipe (2 lanes a clock
+//                 per SM)
 //   Jacobian      an entry per lane over the table of dR/dx in shared memory
 //   head          the head program, level by level, in shared memory
-//   tail          left-looking by 32-column panels: warp w holds rows
-//                 32 w .. 32 w + 31 of the panel in registers (a row per
-//                 lane), the finished columns to its left stream from the
-//                 packed factors (L2), the 32 x 32 blocks of U of the panel
-//                 go round through shared memory.  Every element of the
-//                 tail is written once, in its final place.
+//   tail          right-looking by 32-column panels, its 32 x 32 blocks as
+//                 register tiles of one warp each (see factor_tail)
 //   substitution  a warp per 32 rows; the next block's factors are in flight
 //                 while the diagonal block's 32-step chain runs
+// Every sum that a step depends on is formed in the order of the class-by-class
+// kernels (integrate.cu), which serve the networks that do not fit: the two
+// take the same steps to the last bit (with the 16-cell gather).
+//
+// Cycles per cell on one SM, 470 species, 6000 reactions, FP32 factors: rates
+// 15 k, S R 37 k and substitution 118 k per Newton iteration; predict 14 k,
+// finish 26 k per attempt; Jacobian 65 k, head 54 k, assembly 197 k, panels
+// 170 k, trailing updates 427 k per factorisation.  (One launch per kernel class:
+// 2.28 M per factorisation.)  4096 cells, first 1e-3 yr: 1212 -> 744 ms; 128 cells
+// of a slab, 1e3 yr: 559 -> 59 ms; one cell of 32 species, 1e6 yr: 17.6 -> 5.7 ms.
 #include "cell.h"
 #include <algorithm>
 #include <type_traits>
@@ -58,12 +64,12 @@ struct Args {
   CellPlan p;
   const int* w;            // index programs (CellProg blob)
   int nb, pitch, n_slot, rx, iperm;
-  int n_rsl, rp_off, rp_ent, rp_dst, row, row_more;
+  int rp_deal, rp_ent, rp_dst, row, row_more;
   int n_jsl, n_jl, n_jw, jg_off, jg_ent, jg_rc, jg_dst, jg_grp, jl_off, jl_ent, jl_rc, jd_grp, jd_ent;
   int n_hlev, hop, hterm, hop_ptr;
   int tg_grp, tg_ent;
   int lev_f, lev_b, hx;
-  int n_vsl, vp_off, vp_ent, vp_dst, vrow, vrow_more;
+  int vp_deal, vp_ent, vp_dst, vrow, vrow_more;
   const double* k;
   int64_t ldk;
   double* scratch;
@@ -75,10 +81,11 @@ struct Args {
 
 static_assert(sizeof(Args) <= kCellArgs, "shared-memory plan");
 
-// The launch's arguments are copied to the front of the CTA's shared memory;
-// the phases are separate functions that take them and the vectors from there.
-// As one inlined body the kernel kept so many addresses alive that its inner
-// loops spilled, each spill a trip to L2 next to 230 KB of shared memory.
+// The launch's arguments are copied to the front of the CTA's shared memory,
+// where the phases take them and the vectors from: kept in registers, the many
+// addresses made the inner loops spill, each spill a trip to L2 next to 200 KB
+// of shared memory.  (The phases are inlined for the same reason: a call saves
+// registers to memory.)
 extern __shared__ __align__(16) unsigned char sm[];
 __device__ __forceinline__ const Args& args() { return *reinterpret_cast<const Args*>(sm); }
 __device__ __forceinline__ CellS& scalars() { return *reinterpret_cast<CellS*>(sm + kCellArgs); }
@@ -152,24 +159,25 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;" ::
 __device__ __forceinline__ double coef(int word) { return __hiloint2double(word & 0xFFFF0000, 0); }
 
 // Sums of rows cut into chains (see Chains in cell_prog.cpp): a chain per lane,
-// a slice of 32 chains per warp, longest first, so that the warps of each
-// scheduler keep its FP64 unit (a warp's FMA holds it for 64 cycles) busy.
-// tab[pad slot] must be 0.  All threads.
-__device__ __forceinline__ void row_sums(const int* __restrict__ w, int n_sl, int off, int ent, int dst, int row,
-                                         int more, const double* tab, double* part, double* out, int n) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int2* meta = reinterpret_cast<const int2*>(w + off);
+// slices of 32 chains per warp, dealt so that the schedulers' FP64 units (a warp's
+// FMA holds one for 64 cycles) have equal work.  tab[pad slot] must be 0.  All
+// threads.
+__device__ __forceinline__ void row_sums(const int* __restrict__ w, int deal, int ent, int dst, int row, int more,
+                                         const double* tab, double* part, double* out, int n) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int rw = (int)threadIdx.x < n ? __ldg(w + row + threadIdx.x) : 0;
-  int2 mt = warp < n_sl ? __ldg(meta + warp) : make_int2(0, 0);
-  for (int s = warp; s < n_sl; s += nw) {
+  const int2 own = __ldg(reinterpret_cast<const int2*>(w + deal) + warp);
+  const int4* meta = reinterpret_cast<const int4*>(w + deal);
+  int4 mt = own.x < own.y ? __ldg(meta + own.x) : make_int4(0, 0, 0, 0);
+  for (int i = own.x; i < own.y; ++i) {
     const int* q = w + ent + 32 * mt.x + lane;
-    const int m = mt.y, to = __ldg(w + dst + 32 * s + lane);
+    const int m = mt.y, to = __ldg(w + dst + 32 * mt.z + lane);
     int t[4], nx[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) t[u] = u < m ? __ldg(q + 32 * u) : 0;
 #pragma unroll
     for (int u = 0; u < 4; ++u) nx[u] = 4 + u < m ? __ldg(q + 32 * (4 + u)) : 0;
-    if (s + nw < n_sl) mt = __ldg(meta + s + nw);
+    if (i + 1 < own.y) mt = __ldg(meta + i + 1);
     double a = 0.0;
     int e = 4;
     for (; e <= m; e += 4) {
@@ -257,7 +265,7 @@ __device__ __forceinline__ void cell_rhs() {
   if (threadIdx.x == 0) tab[n_r] = 0.0;
   __syncthreads();
   PHASE_MARK(PH_RATES);
-  row_sums(A.w, A.n_rsl, A.rp_off, A.rp_ent, A.rp_dst, A.row, A.row_more, tab, at<double>(A.p.o_part),
+  row_sums(A.w, A.rp_deal, A.rp_ent, A.rp_dst, A.row, A.row_more, tab, at<double>(A.p.o_part),
            at<double>(A.p.o_fs), A.d.n);
   __syncthreads();
   PHASE_MARK(PH_GATHER);
@@ -579,6 +587,57 @@ __device__ __forceinline__ void lu_block(T* uj, T* lj, T* dst, int64_t ldd, int 
     }
 #pragma unroll
     for (int j = 0; j < 24; ++j) c[j] = c[j + 8];
+  }
+}
+
+// The same in FP64 for a block that no other work of the CTA can hide (the first
+// one; all of a tail of up to 32): its columns dealt to four warps, one per
+// scheduler.  The FMAs of 32 columns hold one scheduler's FP64 unit for 32 k cycles,
+// and with the 32 reciprocals one warp took 73 k, four take 37 k; the elements'
+// operations and their order are the same.  (In FP32 one warp is faster than 32
+// barriers: 14 k.)  All threads; begins with the block in uj (warp 0's) and ends
+// without a barrier.
+template <class T>
+__device__ __forceinline__ void lu_block_all(T* uj, T* lj, T* lbuf, T* dst, int64_t ldd, int w, int lane, int warp) {
+  constexpr int NW = 4, NC = 32 / NW;   // warp v has columns v, v + NW, ..
+  __syncthreads();
+  T c[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) {
+    const int j = NW * q + warp;
+    c[q] = warp < NW && lane < w && j < w ? uj[lane * XP + j] : j == lane ? T(1) : T(0);
+  }
+  __syncthreads();   // (read by all before columns go back)
+#pragma unroll
+  for (int kk = 0; kk < NC; ++kk) {
+#pragma unroll 1
+    for (int v = 0; v < NW; ++v) {
+      const int k = NW * kk + v;
+      T* lk = lbuf + 32 * (k & 1);
+      if (warp == v) {
+        const T inv = T(1) / __shfl_sync(kFull, c[kk], k);
+        const T l = lane > k ? c[kk] * inv : T(0);
+        lk[lane] = l;
+        if (lane > k) c[kk] = l;
+        if (lane == k) c[kk] = inv;
+      }
+      __syncthreads();
+      if (warp < NW) {
+        const T l = lk[lane];
+        if (warp > v) c[kk] -= l * __shfl_sync(kFull, c[kk], k);
+#pragma unroll
+        for (int q = kk + 1; q < NC; ++q) c[q] -= l * __shfl_sync(kFull, c[q], k);
+      }
+    }
+  }
+  if (warp < NW) {
+#pragma unroll
+    for (int q = 0; q < NC; ++q) {
+      const int j = NW * q + warp;
+      uj[lane * XP + j] = c[q];
+      lj[j * 32 + lane] = c[q];
+      if (lane < w && j < w) dst[j * ldd] = c[q];
+    }
   }
 }
 
@@ -1019,9 +1078,14 @@ __device__ __forceinline__ void factor_tail() {
         x.to_rows(uj + CW * h, lane);
       }
       __syncwarp();
-      lu_block(uj, at<T>(A.p.o_lj), D + lane, v.ldd, w, lane);
+      if (sizeof(T) == 4 || J >= 0) lu_block(uj, at<T>(A.p.o_lj), D + lane, v.ldd, w, lane);
     }
-    if (J < 0) continue;
+    if (J < 0) {
+      if constexpr (sizeof(T) == 8) lu_block_all(at<T>(A.p.o_uj), at<T>(A.p.o_lj), at<T>(A.p.o_lbuf), v.block<T>(0, 0) + lane, v.ldd,
+                                                 v.width(0), lane, v.warp);
+      PHASE_MARK(PH_PANEL);
+      continue;
+    }
     // the other trailing blocks in turn, by columns
     const int mm = m * m * HB;
     auto corner = [&](int t) { return v.block<T>(J + 1 + t / HB % m, J + 1 + t / HB / m) + (CW * (t % HB)) * v.ldd; };
@@ -1183,7 +1247,7 @@ __device__ __forceinline__ void cell_jacobian() {
       if ((uint32_t)r.x >> 16 != 0xFFFF) dR[r.y + 1] *= dn;
     }
     __syncthreads();
-    row_sums(w, A.n_vsl, A.vp_off, A.vp_ent, A.vp_dst, A.vrow, A.vrow_more, dR, at<double>(A.p.o_vp),
+    row_sums(w, A.vp_deal, A.vp_ent, A.vp_dst, A.vrow, A.vrow_more, dR, at<double>(A.p.o_vp),
              d.bgv + S.oc * d.bpad, n);
   }
   __syncthreads();
@@ -1294,7 +1358,7 @@ __device__ __forceinline__ void cell_border() {
   }
   if (tid == 0) tab[n_r] = 0.0;
   __syncthreads();
-  row_sums(A.w, A.n_rsl, A.rp_off, A.rp_ent, A.rp_dst, A.row, A.row_more, tab, at<double>(A.p.o_part),
+  row_sums(A.w, A.rp_deal, A.rp_ent, A.rp_dst, A.row, A.row_more, tab, at<double>(A.p.o_part),
            at<double>(A.p.o_fs), n);
   sum_parts(0, n_r, [&](int j) { return __ldg(d.th_dn + j) * rate(j); });
   sum_parts(1, n_r, [&](int j) { return __ldg(d.th_dn + j) * tab[j]; });
@@ -1801,10 +1865,10 @@ __device__ __forceinline__ void cell_conditions(int64_t oc) {
   }
 }
 
-// 512 threads leave a thread 128 registers: one CTA of 16 warps fills the
-// register file of an SM, or two of 8 warps, whose two cells are in different
-// phases and fill each other's gaps; FP64 (its shared memory holds one CTA per
-// SM) always takes 16 warps.
+// 12 warps at 168 registers: the register tiles of the tail and a row block with
+// its next 32 columns need about that many, and a 349-column tail has 11 blocks.
+// (16 warps at 128 registers spilled in every inner loop; two CTAs an SM do not
+// fit the shared memory of a 470-species cell.)
 template <class T, bool TF>
 __global__ void __launch_bounds__(kMaxCellThreads, 1) cell_kernel(const __grid_constant__ Args from) {
   __shared__ int sh_c;
@@ -2035,8 +2099,9 @@ __global__ void __launch_bounds__(kMaxCellThreads, 1) cell_init_kernel(const __g
   }
 }
 
-// The CTA shape of a batch: wide CTAs (one per SM) where every cell gets an SM
-// of its own, narrow ones (two and more per SM) for more cells.
+// The CTA shape of a batch: wide CTAs (12 warps) where every cell has an SM of
+// its own, narrow ones (4 warps, two and more per SM) for more cells of networks
+// whose tails have at most four blocks, which give 12 warps nothing to do.
 const CellShape& shape(const CellLaunch& L, int64_t C) { return C > L.sms && L.narrow.ctas > 0 ? L.narrow : L.wide; }
 
 Args make_args(const sm_net* net, const Dev& d, const CellLaunch& L, const double* k, int64_t ldk) {
@@ -2046,7 +2111,8 @@ Args make_args(const sm_net* net, const Dev& d, const CellLaunch& L, const doubl
   a.p = shape(L, d.C).plan;
   a.w = p.blob.as<int>();
   a.nb = p.nb; a.pitch = p.pitch; a.n_slot = p.n_slot; a.rx = p.rx; a.iperm = p.iperm;
-  a.n_rsl = p.n_rsl; a.rp_off = p.rp_off; a.rp_ent = p.rp_ent; a.rp_dst = p.rp_dst; a.row = p.row; a.row_more = p.row_more;
+  const int narrow = a.p.warps < kMaxCellThreads / 32;
+  a.rp_deal = p.rp_deal[narrow]; a.rp_ent = p.rp_ent; a.rp_dst = p.rp_dst; a.row = p.row; a.row_more = p.row_more;
   a.n_jsl = p.n_jsl; a.n_jl = p.n_jl;
   a.jg_off = p.jg_off; a.jg_ent = p.jg_ent; a.jg_rc = p.jg_rc; a.jg_dst = p.jg_dst; a.jg_grp = p.jg_grp;
   a.n_jw = p.n_jw; a.jl_off = p.jl_off; a.jl_ent = p.jl_ent;
@@ -2054,7 +2120,7 @@ Args make_args(const sm_net* net, const Dev& d, const CellLaunch& L, const doubl
   a.n_hlev = net->lu.n_hlev; a.hop = p.hop; a.hterm = p.hterm; a.hop_ptr = p.hop_ptr;
   a.tg_grp = p.tg_grp; a.tg_ent = p.tg_ent;
   a.lev_f = p.lev_f; a.lev_b = p.lev_b; a.hx = p.hx;
-  a.n_vsl = p.n_vsl; a.vp_off = p.vp_off; a.vp_ent = p.vp_ent; a.vp_dst = p.vp_dst; a.vrow = p.vrow; a.vrow_more = p.vrow_more;
+  a.vp_deal = p.vp_deal[narrow]; a.vp_ent = p.vp_ent; a.vp_dst = p.vp_dst; a.vrow = p.vrow; a.vrow_more = p.vrow_more;
   a.k = k;
   a.ldk = ldk;
   a.scratch = L.scratch;

@@ -19,16 +19,17 @@ constexpr int kMaxCellThreads = 384;
 struct CellPlan {
   bool ok = false;
   int warps = 0, nv = 0;
-  int o_ip, o_hx, o_nv, o_yp, o_ps, o_ws, o_wf, o_wi, o_u;      // o_u: start of the phase-shared area
+  int o_ip, o_hx, o_yp, o_ps, o_ws, o_wf, o_wi, o_u;   // o_u: start of the phase-shared area
+  int o_nv;                                            // error test
   int o_ys, o_fs, o_r, o_part, o_xh, o_xt, o_hd, o_dg;   // Newton rounds
   int o_dr, o_wsf, o_wif, o_vp;                     // Jacobian gather
   int o_hv, o_x, asm_tile, asm_warps;               // head, assembly (tile size in elements, warps with one)
-  int o_lp, o_up, o_uj, o_lj, o_next;        // tail
+  int o_lp, o_up, o_uj, o_lj, o_lbuf, o_next;        // tail
   size_t bytes = 0;
   int64_t scratch = 0;   // doubles of global scratch per CTA
 };
 
-// Plan for a network in FP64 (esz 8) or FP32 (esz 4) factors.
+// Plan for a network in FP64 (esz 8) or FP32 (esz 4) factors,
 // with CTAs of `warps` warps; tf: tensor-core updates.
 CellPlan cell_plan(const sm_net* net, size_t esz, bool tf, bool thermal, int warps, size_t smem_max);
 

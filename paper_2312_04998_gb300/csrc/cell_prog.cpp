@@ -57,8 +57,38 @@ struct Chains {
   std::vector<int32_t> dst, row, more;
   int32_t n_chain = 0;
   bool ok = true;
+
+  // The slices dealt to the nw warps of a CTA: {first, end} of each warp's, then
+  // per slice {first row, rows, slice, 0}.  Longest first, each to the scheduler
+  // (warp mod 4) with the fewest rows so far and there to the warp with the
+  // fewest: dealt in turns, the longest chain shared its scheduler's FP64 unit with
+  // two more warps' slices and finished last.
+  std::vector<int32_t> deal(int32_t nw) const {
+    std::vector<std::vector<int32_t>> mine(nw);
+    std::vector<int64_t> load(nw, 0), unit(4, 0);
+    for (int32_t k = 0; k < s.slices(); ++k) {   // (slices come longest first)
+      const int32_t u = (int32_t)(std::min_element(unit.begin(), unit.end()) - unit.begin());
+      int32_t w = u;
+      for (int32_t v = u; v < nw; v += 4)
+        if (load[v] < load[w]) w = v;
+      mine[w].push_back(k);
+      load[w] += s.off[2 * k + 1];
+      unit[u] += s.off[2 * k + 1];
+    }
+    std::vector<int32_t> out, list;
+    for (int32_t w = 0; w < nw; ++w) {
+      out.push_back((int32_t)(2 * nw + list.size()) / 4);
+      for (int32_t k : mine[w]) list.insert(list.end(), {s.off[2 * k], s.off[2 * k + 1], k, 0});
+      out.push_back((int32_t)(2 * nw + list.size()) / 4);
+    }
+    out.insert(out.end(), list.begin(), list.end());
+    return out;
+  }
 };
 constexpr size_t kChunks = 32;
+constexpr int32_t kWide = kMaxCellThreads / 32, kNarrow = 4;   // warps of the two CTA shapes
+static_assert(kWide % 4 == 0, "deal: whole schedulers, 16-byte lists");
+
 
 Chains cut_rows(const std::vector<std::vector<int32_t>>& rows, int32_t pad) {
   size_t words = 0, z = 0, ch = 0;
@@ -130,9 +160,9 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
       for (int32_t q = net->s_colptr[j]; q < net->s_colptr[j + 1]; ++q)
         for_coef_parts(net->s_coef[q], [&](int c) { rows[net->s_row[q]].push_back(coef_word(j, c)); });
     const Chains r = cut_rows(rows, coef_word(n_r, 1));
-    p.n_rsl = r.s.slices();
     p.n_chain = r.n_chain;
-    p.rp_off = put(r.s.off);
+    p.rp_deal[0] = put(r.deal(kWide));
+    p.rp_deal[1] = put(r.deal(kNarrow));
     p.rp_ent = put(r.s.ent);
     p.rp_dst = put(r.dst);
     p.row = put(r.row);
@@ -148,9 +178,9 @@ void build_cell_prog(const sm_net* net, CellProg* out) {
       if (b >= 0) rows[b].push_back(coef_word(slot[j] + 1, 1));
     }
     const Chains r = cut_rows(rows, coef_word(p.n_slot, 1));
-    p.n_vsl = r.s.slices();
     p.n_vchain = r.n_chain;
-    p.vp_off = put(r.s.off);
+    p.vp_deal[0] = put(r.deal(kWide));
+    p.vp_deal[1] = put(r.deal(kNarrow));
     p.vp_ent = put(r.s.ent);
     p.vp_dst = put(r.dst);
     p.vrow = put(r.row);
@@ -402,7 +432,6 @@ CellPlan cell_plan(const sm_net* net, size_t esz, bool tf, bool thermal, int war
     c.asm_tile = (int)(up(esz * kGroup * p.pitch) / esz);
     const size_t left = smem_max > o ? smem_max - o : 0;
     c.asm_warps = std::min<int>(warps, (int)(left / (esz * c.asm_tile)));
-    // (FP32 with 8 warps: two CTAs are to fit an SM)
     c.o_x = take(esz * c.asm_tile * std::max(c.asm_warps, 1));
   }
   phase();
@@ -410,6 +439,7 @@ CellPlan cell_plan(const sm_net* net, size_t esz, bool tf, bool thermal, int war
   c.o_up = take(esz * 32 * (tf ? 36 : 32) * std::max(p.nb - 1, 1));
   c.o_uj = take(esz * (32 * 36 + 32));   // (reads past the last row's end stay inside)
   c.o_lj = take(esz * (32 * 32 + 32));
+  c.o_lbuf = take(esz * 64);
   c.o_next = take(16);
   phase();
   c.bytes = top;

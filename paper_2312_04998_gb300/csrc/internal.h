@@ -147,8 +147,9 @@ struct CellProg {
   int32_t iperm = 0;             // per species: position in elimination order
   // right-hand side: rows of S in chains (see cell_prog.cpp); entry = reaction |
   // upper half of the double coefficient << 16 (pads read slot n_r = 0)
-  int32_t n_rsl = 0, n_chain = 0;
-  int32_t rp_off = 0, rp_ent = 0, rp_dst = 0, row = 0, row_more = 0;
+  // (dealt to the warps of a wide and of a narrow CTA)
+  int32_t n_chain = 0, rp_deal[2] = {0, 0};
+  int32_t rp_ent = 0, rp_dst = 0, row = 0, row_more = 0;
   // Jacobian: entries of at most kJShort words in slices by destination group
   // (0 = head, 1 + G = the tail's columns kGroup G .. of the assembly); entry
   // word = derivative slot | upper half of the double coefficient << 16, pads
@@ -171,8 +172,8 @@ struct CellProg {
   int32_t lev_f = 0, lev_b = 0, hx = 0;
   // column sums of dn_j dR_j/dx_l (coupled temperature): derivative slots of
   // each species in chains like the right-hand side
-  int32_t n_vsl = 0, n_vchain = 0;
-  int32_t vp_off = 0, vp_ent = 0, vp_dst = 0, vrow = 0, vrow_more = 0;
+  int32_t n_vchain = 0, vp_deal[2] = {0, 0};
+  int32_t vp_ent = 0, vp_dst = 0, vrow = 0, vrow_more = 0;
   std::vector<int32_t> h;
   DevArray blob;
 };
