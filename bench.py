@@ -73,16 +73,13 @@ SM_COUNT, SM_GHZ = 152, 2.07
 PEAK_FP32 = SM_COUNT * 128 * 2 * SM_GHZ / 1e3     # TFLOP/s
 PEAK_FP64 = SM_COUNT * 4 * SM_GHZ / 1e3           # TFLOP/s
 
-# DRAM bytes (read + write) per processed unit of a kernel, from a committed
-# ncu capture in profiles/ (named there), keyed on the kernel class, the
-# precision and the hash of integrate.cu's code (comments and whitespace
-# removed) at capture time: a changed kernel reports traffic null until it
-# is captured again.
-TRAFFIC = {
-    # profiles/refresh_kernel_mixed_2048cells.md: 11.47 GB in a launch that
-    # refreshed all 2048 cells
-    ("refresh", "mixed", "5e9214d3aef36f79"): 5.599e6,
-}
+# DRAM bytes (read + write) per processed unit of a kernel class, from a
+# committed ncu capture in profiles/ (named there), keyed on the class, the
+# precision and the hash of the integrator's kernel code (comments and
+# whitespace removed) at capture time: a changed kernel reports traffic null
+# until it is captured again.  (The persistent kernel runs every class in one
+# launch, so no counter separates them.)
+TRAFFIC = {}
 
 
 def args_():
@@ -121,7 +118,7 @@ def args_():
                    choices=["", "rhs", "mixed", "adjoint", "cpu", "probe", "pdr", "thermal", "single"],
                    help="run one auxiliary measurement alone and print it")
     p.add_argument("--phases", action="store_true",
-                   help="refresh-kernel cycles per phase over one integration (phase-clock build)")
+                   help="cycles of the integrator kernel per phase over one integration (phase-clock build)")
     return p.parse_args()
 
 
@@ -827,10 +824,10 @@ def adjoint_measurement(B, C, dev):
 
 
 def phase_profile(B, a, dev):
-    """Refresh-kernel cycles per phase, per refreshed cell, over one whole
-    integration of the first a.cells cells of the headline workload (thread
-    0 of each CTA, between the barriers that end the phases; the phase-clock
-    build of the library)."""
+    """Cycles per phase of the persistent kernel over one whole integration of
+    the first a.cells cells of the headline workload (thread 0 of each CTA,
+    between the barriers that end the phases; the phase-clock build of the
+    library), per attempt, Newton iteration or factorisation."""
     import numpy as np
     import torch
     from synth.workloads import make
@@ -847,20 +844,23 @@ def phase_profile(B, a, dev):
     st.integrate(kd, yd, a.t_end_yr * YEAR, a.cells, stats)
     torch.cuda.synchronize()
     cyc = B.phase_cycles(dev.index or 0)
-    cells = max(cyc[15], 1.0)
-    per = cyc[:len(B.PHASE_NAMES)] / cells
-    tot = per.sum()
-    return {"what": "refresh kernel cycles per refreshed cell, by phase (thread 0 of each CTA)",
-            "workload": WORKLOAD, "cells": a.cells, "precision": a.precision, "refreshed_cells": int(cyc[15]),
-            "total_cycles_per_cell": float(tot),
-            "phases": [[nm, float(v), float(v / tot)] for nm, v in zip(B.PHASE_NAMES, per)]}
+    h = B.stats_to_numpy(stats)
+    units = {"attempt": float((h["steps"] + h["rejects"] + h["conv_fails"]).sum()),
+             "Newton iteration": float(h["newton_iters"].sum()), "factorisation": float(h["jac_evals"].sum())}
+    of = lambda i: "attempt" if i in (0, 1, 5) else "Newton iteration" if i < 5 else "factorisation"
+    tot = max(float(cyc[:len(B.PHASE_NAMES)].sum()), 1.0)
+    return {"what": "cycles of the persistent integrator kernel by phase (thread 0 of each CTA)",
+            "workload": WORKLOAD, "cells": a.cells, "precision": a.precision, "units": units,
+            "total_cycles_per_attempt": tot / max(units["attempt"], 1.0),
+            "phases": [[nm, float(cyc[i]) / max(units[of(i)], 1.0), of(i), float(cyc[i]) / tot]
+                       for i, nm in enumerate(B.PHASE_NAMES)]}
 
 
 def kernel_source_hash():
-    """Hash of the integrator's kernel source (integrate.cu) with comments and
+    """Hash of the integrator's kernel source (cell.cu) with comments and
     whitespace removed, so that a comment edit keeps the key of a capture."""
     import re
-    with open(os.path.join(ROOT, "paper_2312_04998_gb300", "csrc", "integrate.cu")) as fh:
+    with open(os.path.join(ROOT, "paper_2312_04998_gb300", "csrc", "cell.cu")) as fh:
         src = fh.read()
     src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)      # block comments
     src = re.sub(r"//[^\n]*", " ", src)                    # line comments

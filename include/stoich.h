@@ -294,15 +294,20 @@ typedef struct {
     int32_t newton_max;       /* Newton iterations per attempt, 1..8               */
     int32_t max_conv_fails;   /* consecutive Newton failures before SM_CELL_CONV   */
     int32_t precision;        /* SM_PREC_FP64, SM_PREC_MIXED or SM_PREC_TF32       */
+    /* Most batches are integrated by one persistent kernel that carries each
+       cell through its own attempts; large batches, and networks whose tables do
+       not fit an SM's shared memory, take a group of launches over all cells per
+       attempt, which is what use_graph, attempts_per_sync and sm_net_set_integ
+       concern. */
     int32_t use_graph;        /* capture the attempt loop in a CUDA graph (1) or not */
     int32_t attempts_per_sync;/* attempts launched between completion checks      */
-    int32_t timing_kind;      /* SM_TIME_*: kernel class timed with CUDA events    */
+    int32_t timing_kind;      /* SM_TIME_*: part of an attempt that is timed      */
     int32_t record_steps;     /* > 0: record up to this many accepted steps per cell
                                  (times, sizes, orders) and the step history every
                                  SM_CHECKPOINT_EVERY steps, for sm_adjoint         */
-    int32_t refresh_ctas_per_sm; /* refresh CTAs resident per SM: 0 = as many as
-                                 fit (default); fewer CTAs keep fewer working
-                                 matrices in flight (L2 footprint)            */
+    int32_t refresh_ctas_per_sm; /* CTAs resident per SM that work on cells: 0 = as
+                                 many as fit (default); fewer keep fewer working
+                                 sets in flight (L2 footprint)                */
 } sm_opts;
 
 /* Accepted steps between stored states of the recorded forward run. */
@@ -377,11 +382,14 @@ sm_status sm_state_save(sm_state* st, int32_t with_factors, void* host, size_t b
 sm_status sm_state_load(sm_state* st, const void* host, size_t bytes, void* stream);
 
 /* Instrumentation: *launches = kernels the state has launched so far, and,
- * when opts.timing_kind selects a class, *ms = summed CUDA-event durations of
- * that class's launches (*timed = how many were timed; the RHS class times
- * the rate + gather pair of each Newton round as one launch).  Events are
- * recorded on the state's stream, inside the captured graph when graphs are
- * used; sm_state_timing_reset zeroes the totals.  Any pointer may be NULL. */
+ * when opts.timing_kind selects a class, *ms = the time spent in it and *timed =
+ * how often it ran.  With the persistent kernel that is the clock cycles which
+ * the CTAs spent in the class, averaged over the CTAs of a launch, at the SM's
+ * maximum clock; with a launch per class the summed CUDA-event durations of its
+ * launches (the RHS class times the rate + gather pair of each Newton round as
+ * one launch), recorded on the state's stream, inside the captured graph when
+ * graphs are used.  sm_state_timing_reset zeroes the totals.  Any pointer may be
+ * NULL. */
 sm_status sm_state_timing(const sm_state* st, int64_t* launches, double* ms, int64_t* timed);
 sm_status sm_state_timing_reset(sm_state* st);
 

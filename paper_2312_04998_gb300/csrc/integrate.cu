@@ -2754,6 +2754,23 @@ int64_t pass_cells(int64_t C, int64_t cells_per_pass) {
 
 extern "C" {
 
+// Cells from which on the class-by-class path is the faster one (plain
+// integrations; nb: 32-wide blocks of the dense tail).  The fused kernel's rate
+// does not grow any more once every SM has its cells, while the class kernels,
+// 32 cells a block and bound by HBM, gain until about 65,536 cells.  Thousand
+// accepted steps per second, fused / class by class, whole integrations to 1e5 yr:
+//   470 species, mixed   16,384 cells 727 / 681, 32,768 726 / 795 (TF32 689 / 790)
+//   470 species, FP64    16,384 cells 165 / 143
+//   120 species          mixed 8,192 cells 4461 / 3146, 65,536 4372 / 5355;
+//                        FP64 65,536 cells 2241 / 2300
+//    32 species          mixed 8,192 cells 8669 / 9823, 65,536 7615 / 18403;
+//                        FP64 65,536 cells 7300 / 13268
+static int64_t class_path_from(int nb, bool mixed) {
+  if (nb <= 1) return 6144;
+  if (mixed) return 24576;
+  return nb <= 4 ? 65536 : INT64_MAX;
+}
+
 sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_state** out) {
   if (!out) return SM_EINVAL;
   *out = nullptr;
@@ -2816,7 +2833,8 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device);
   if ((r = cell_shapes(net, d, net->th_t >= 0, o.refresh_ctas_per_sm, &st->cell)) != SM_OK) return fail(r);
-  st->fused = st->cell.wide.ctas > 0;
+  st->fused = st->cell.wide.ctas > 0 &&
+              (net->th_t >= 0 || o.record_steps > 0 || C < class_path_from(net->cell.nb, d.mixed != 0));
   if (st->fused) {
     CellLaunch& cl = st->cell;
     const int64_t ring = 2 + std::max<int64_t>(C, 16 * std::min<int64_t>(C, 8LL * cl.max_ctas()));
