@@ -81,6 +81,20 @@ def test_integrator_batches(torch, B, size, precision):
     assert np.all(np.abs(y[:, 7] - ref) <= 1e-6 * np.abs(ref) + 1e-16)
 
 
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_integrator_paths_agree(torch, B, precision):
+    """A batch that goes through one launch per kernel class, and some of its
+    cells through the persistent kernel: the same sums in the same order."""
+    C = 6150
+    d, k, y0 = workload(32, 180, 64)
+    k, y0 = np.tile(k, (1, 97))[:, :C], np.tile(y0, (1, 97))[:, :C]
+    few = [0, 5, 63]
+    many = integrate(torch, B, d, k, y0, 1e3, precision=precision)
+    alone = integrate(torch, B, d, k[:, few], y0[:, few], 1e3, precision=precision)
+    assert np.array_equal(alone, many[:, few])
+    assert np.array_equal(many[:, 64 * 95 + 5], many[:, 5])
+
+
 def test_rates_outside_the_ordinary_range(torch, B):
     """Zero exponents, underflow and overflow, coefficients and conditions that
     the fixed-point form does not take."""
