@@ -376,11 +376,11 @@ template <class T> __device__ __forceinline__ T from_rank0(const T* p) {   // ra
   return v;
 }
 
-template <class T>
+template <class T, bool kCluster>
 __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, const double* __restrict__ k,
-                                                                 int64_t ldk, RefreshPlan plan, int S) {
+                                                                 int64_t ldk, RefreshPlan plan, int ctas) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int rank = S > 1 ? blockIdx.x % S : 0;
+  const int S = kCluster ? ctas : 1, rank = kCluster ? blockIdx.x % S : 0;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
   const int n = d.n, n_r = d.n_r, ldm = d.ldm, h = d.head, nt = n - h, pitch = plan.pitch;
@@ -2303,7 +2303,7 @@ sm_status enqueue_attempt(sm_state* st, const double* k, int64_t ldk, cudaStream
     th_rates_kernel<<<th_grid, 128, 0, s>>>(d, d.ypred + (int64_t)d.t_idx * d.ld, 0);
     st->launches += 1;
   }
-  refresh_kernel<T><<<st->refresh_ctas, kRefreshThreads, st->plan.bytes, s>>>(d, k, ldk, st->plan, 1);
+  refresh_kernel<T, false><<<st->refresh_ctas, kRefreshThreads, st->plan.bytes, s>>>(d, k, ldk, st->plan, 1);
   if (d.therm) {
     const unsigned nb = (unsigned)std::min<int64_t>(blocks(d.C, kBorderWarps), 152LL * 16);
     th_border_kernel<T><<<nb, 32 * kBorderWarps, st->border_smem, s>>>(d);
@@ -2571,7 +2571,7 @@ int replay_cluster(const sm_state* st, int64_t C) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, refresh_kernel<double>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, refresh_kernel<double, true>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -2592,7 +2592,8 @@ sm_status launch_replay_refresh(sm_state* st, const Dev& d, int S, const double*
   at.val.clusterDim.y = at.val.clusterDim.z = 1;
   cfg.attrs = &at;
   cfg.numAttrs = S > 1 ? 1 : 0;
-  SM_TRY_CUDA(cudaLaunchKernelEx(&cfg, refresh_kernel<double>, d, k, ldk, st->plan, S));
+  SM_TRY_CUDA(cudaLaunchKernelEx(&cfg, S > 1 ? refresh_kernel<double, true> : refresh_kernel<double, false>, d, k, ldk,
+                                 st->plan, S));
   return SM_OK;
 }
 
@@ -2965,15 +2966,16 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   // device limit so that a later state with a smaller plan cannot lower it
   // below what an earlier state launches with
   if (d.mixed) {
-    SM_TRY_CUDA(cudaFuncSetAttribute(refresh_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
+    SM_TRY_CUDA(cudaFuncSetAttribute(refresh_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
   } else {
-    SM_TRY_CUDA(cudaFuncSetAttribute(refresh_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
+    SM_TRY_CUDA(cudaFuncSetAttribute(refresh_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
+    SM_TRY_CUDA(cudaFuncSetAttribute(refresh_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
   }
   int per_sm = 0;
   if (d.mixed) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, refresh_kernel<float>, kRefreshThreads, rsm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, refresh_kernel<float, false>, kRefreshThreads, rsm);
   } else {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, refresh_kernel<double>, kRefreshThreads, rsm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, refresh_kernel<double, false>, kRefreshThreads, rsm);
   }
   if (o.refresh_ctas_per_sm > 0) per_sm = std::min(per_sm, (int)o.refresh_ctas_per_sm);
   st->refresh_ctas = (sms > 0 ? sms : 1) * (per_sm > 0 ? per_sm : 1);
