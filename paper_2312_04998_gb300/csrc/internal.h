@@ -51,6 +51,7 @@ struct DevArray {
 struct Format {
   int32_t fmt = SM_FMT_CRS, order = SM_ORDER_NONE, C = 1, sigma = 1;
   std::vector<int32_t> ptr, idx, idx2, len;
+  int32_t longest = 0;                    // SELL: the largest of len
   std::vector<double> val;
   // Device-only companion indices: CRS row ids, CCS column ids, COO column
   // per nonzero, SELL row ids (-1 = padding row).

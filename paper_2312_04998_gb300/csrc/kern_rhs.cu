@@ -61,6 +61,17 @@ int rate_chunk(int64_t n_r, int64_t C) {
   return (int)std::min<int64_t>(kRChunk, std::max<int64_t>(4, fit));
 }
 
+// Whether the SELL kernel reads ahead.  A row of the longest slice is a chain of
+// L entries, the batch's entries (pads included) fill the device's threads
+// `rounds` times for as long; ahead / not, over 32, 120 and 470 species, slice
+// heights 8 to 32 and 37 to 65,536 cells: 0.26 to 0.89 at up to 0.8 rounds, 0.92
+// to 1.01 at 1.3 to 2.1, 0.99 to 1.11 from 2.4 on.
+bool sell_ahead(const Format& F, int64_t C) {
+  constexpr double kThreads = 152 * 2048.0;
+  const double rounds = (double)F.packed.size() * (double)C / (kThreads * std::max(F.longest, 1));
+  return rounds < 2.25;
+}
+
 // sum over entries [b, e) of coef * r[col]: four independent partial sums, U
 // entries' loads in flight (index words, then rates: the gather waits for
 // memory, not for the FP64 unit).  Eight for a warp per chunk; the half-warps of
@@ -261,8 +272,12 @@ rhs_ccs_kernel(int n_r, int64_t C, const int* __restrict__ col_ptr, const uint32
 }
 
 // SELL-C-sigma: block = kCells cells x C slice rows, one slice per blockIdx.y.
-// Bound by the chain of the longest row: 1501 cells of 470 species took 727 us
-// with each entry's loads waiting for the one before, 285 us with them ahead.
+// Bound by the chain of the longest row while a batch is small: 1501 cells of 470
+// species took 727 us with each entry's loads waiting for the one before, 285 us
+// with them ahead (kAhead).  That takes 72 registers; once there are entries
+// enough to keep an SM's 2048 threads busy, the plain loop with its 32 is the
+// faster one (see sell_ahead).
+template <bool kAhead>
 __global__ void rhs_sell_kernel(int64_t C, int slice_h, const int* __restrict__ slice_ptr,
                                 const uint32_t* __restrict__ ent, const int* __restrict__ row_id,
                                 const double* __restrict__ r, int64_t ldr, double* __restrict__ f,
@@ -273,44 +288,49 @@ __global__ void rhs_sell_kernel(int64_t C, int slice_h, const int* __restrict__ 
   const int i = __ldg(row_id + (int64_t)s * slice_h + rr);
   const int b = __ldg(slice_ptr + s);
   const int L = (__ldg(slice_ptr + s + 1) - b) / slice_h;
-  // a row is one chain of FMAs (2000 in the hub rows): while eight entries are
-  // added, the rates of the next eight and the index words of those after are
-  // on their way
   double acc = 0.0;
-  constexpr int U = 8;
   const uint32_t* q = ent + b + rr;
-  auto words = [&](int kk, uint32_t (&w)[U]) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) w[u] = kk + U <= L ? __ldg(q + (kk + u) * slice_h) : 0;
-  };
-  auto rates = [&](int kk, const uint32_t (&w)[U], double (&v)[U]) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) v[u] = kk + U <= L ? r[(int64_t)(w[u] & 0xFFFFFFu) * ldr + c] : 0.0;
-  };
-  uint32_t w0[U], w1[U];
-  double v0[U];
-  words(0, w0);
-  words(U, w1);
-  rates(0, w0, v0);
-  int kk = 0;
-  for (; kk + U <= L; kk += U) {
-    uint32_t w2[U];
-    double v1[U];
-    rates(kk + U, w1, v1);
-    words(kk + 2 * U, w2);
-#pragma unroll
-    for (int u = 0; u < U; ++u) acc = fma(c_coef[w0[u] >> 24], v0[u], acc);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      w0[u] = w1[u];
-      w1[u] = w2[u];
-      v0[u] = v1[u];
-    }
-  }
-#pragma unroll 1
-  for (; kk < L; ++kk) {
-    const uint32_t w = __ldg(q + kk * slice_h);
+  auto entry = [&](int k) {
+    const uint32_t w = __ldg(q + k * slice_h);
     acc = fma(c_coef[w >> 24], r[(int64_t)(w & 0xFFFFFFu) * ldr + c], acc);
+  };
+  if constexpr (kAhead) {
+    // a row is one chain of FMAs (2000 in the hub rows): while eight entries are
+    // added, the rates of the next eight and the index words of those after are
+    // on their way
+    constexpr int U = 8;
+    auto words = [&](int k, uint32_t (&w)[U]) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) w[u] = k + U <= L ? __ldg(q + (k + u) * slice_h) : 0;
+    };
+    auto rates = [&](int k, const uint32_t (&w)[U], double (&v)[U]) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = k + U <= L ? r[(int64_t)(w[u] & 0xFFFFFFu) * ldr + c] : 0.0;
+    };
+    uint32_t w0[U], w1[U];
+    double v0[U];
+    words(0, w0);
+    words(U, w1);
+    rates(0, w0, v0);
+    int k = 0;
+    for (; k + U <= L; k += U) {
+      uint32_t w2[U];
+      double v1[U];
+      rates(k + U, w1, v1);
+      words(k + 2 * U, w2);
+#pragma unroll
+      for (int u = 0; u < U; ++u) acc = fma(c_coef[w0[u] >> 24], v0[u], acc);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        w0[u] = w1[u];
+        w1[u] = w2[u];
+        v0[u] = v1[u];
+      }
+    }
+#pragma unroll 1
+    for (; k < L; ++k) entry(k);
+  } else {
+    for (int k = 0; k < L; ++k) entry(k);
   }
   if (i >= 0) f[(int64_t)i * ld + c] = acc;
 }
@@ -383,8 +403,9 @@ sm_status launch_rhs(const sm_net* net, int64_t C, const double* k, const double
   } else {
     dim3 block(kCells, F.C);
     dim3 grid(groups, (unsigned)F.len.size());
-    rhs_sell_kernel<<<grid, block, 0, s>>>(C, F.C, F.d_ptr.as<int>(), F.d_packed.as<uint32_t>(),
-                                           F.d_aux.as<int>(), scratch, ldr, f, ld);
+    const auto kernel = sell_ahead(F, C) ? rhs_sell_kernel<true> : rhs_sell_kernel<false>;
+    kernel<<<grid, block, 0, s>>>(C, F.C, F.d_ptr.as<int>(), F.d_packed.as<uint32_t>(), F.d_aux.as<int>(), scratch, ldr,
+                                  f, ld);
   }
   SM_TRY_CUDA(cudaGetLastError());
   return SM_OK;

@@ -644,6 +644,7 @@ sm_status build_format(const sm_net* net, int32_t fmt, int32_t order, int32_t C,
         if (i >= 0) L = std::max(L, (int32_t)rows[i].size());
       }
       f.len.push_back(L);
+      f.longest = std::max(f.longest, L);
       for (int32_t k = 0; k < L; ++k)
         for (int32_t r = 0; r < C; ++r) {
           int32_t i = f.idx2[(size_t)s * C + r];

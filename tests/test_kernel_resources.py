@@ -38,3 +38,10 @@ def test_fp32_refresh_has_the_registers_it_needs(usage):
     f32 = [r for r in rows if "refresh_kernelIf" in r[0]]
     assert len(f32) == 1   # one CTA a cell: no cluster form
     assert f32[0][1] <= 128 and f32[0][2] <= 16 and f32[0][3] <= 16, f32
+
+
+def test_sell_gather_has_a_form_for_full_sms(usage):
+    """32 registers: 2048 threads on an SM.  (With 72 alone, batches that fill the
+    device took up to 11 % longer.)"""
+    rows = [r for r in usage("kern_rhs.cu") if "rhs_sell_kernel" in r[0]]
+    assert min(r[1] for r in rows) <= 32 and all(r[2] == r[3] == 0 for r in rows), rows
