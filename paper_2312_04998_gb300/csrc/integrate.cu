@@ -2772,18 +2772,9 @@ static int64_t class_path_from(int nb, bool mixed) {
   return nb <= 4 ? 65536 : INT64_MAX;
 }
 
-sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_state** out) {
-  if (!out) return SM_EINVAL;
-  *out = nullptr;
-  if (!net || net->device < 0 || C < 1) return SM_EINVAL;
-  sm_opts o;
-  sm_opts_default(&o);
-  if (opts) o = *opts;
-  if (!opts_ok(o)) return SM_EINVAL;
-  Scope scope(net->device);
-  if (!scope.ok) return SM_ECUDA;
-  sm_state* st = new (std::nothrow) sm_state();
-  if (!st) return SM_ENOMEM;
+// Allocates and fills in a new state; what a failure leaves behind is the
+// caller's to free.
+static sm_status build_state(const sm_net* net, int64_t C, const sm_opts& o, sm_state* st) {
   st->net = net;
   st->opts = o;
   st->cap = C;
@@ -2812,43 +2803,45 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   d.max_conv_fails = o.max_conv_fails;
   d.ldm = lu.ld;
   d.head = lu.head;
+  SM_TRY_CUDA(cudaStreamCreateWithFlags(&st->s, cudaStreamNonBlocking));
+  SM_TRY_CUDA(cudaEventCreateWithFlags(&st->ev_in, cudaEventDisableTiming));
+  SM_TRY_CUDA(cudaEventCreateWithFlags(&st->ev_out, cudaEventDisableTiming));
+  SM_TRY_CUDA(cudaStreamCreateWithFlags(&st->s2, cudaStreamNonBlocking));
+  SM_TRY_CUDA(cudaEventCreateWithFlags(&st->ev_fork, cudaEventDisableTiming));
+  SM_TRY_CUDA(cudaEventCreateWithFlags(&st->ev_join, cudaEventDisableTiming));
+  SM_TRY_CUDA(cudaMallocHost(&st->h_counters, kCounters * sizeof(int)));
   sm_status r = SM_OK;
-  auto fail = [&](sm_status e) {
-    free_state(st);
-    delete st;
-    return e;
-  };
   const int n_dscal = 6 + 2 * (QMAX + 1);   // t h gam gam_J crate dprev | tn[6] alpha[6]
   const int n_iscal = 15;                   // q nh n_at_q j_age flags crej ccf status m_it steps rejects
                                             // conv_fails newton_iters jac_evals slot_cell
   const int n_vec = (QMAX + 1) + 8;         // Y[6] ypred y psi f f0 eprev w wf
-  if ((r = st->scal_d.ensure(sizeof(double) * n_dscal * ld)) != SM_OK) return fail(r);
-  if ((r = st->scal_i.ensure(sizeof(int) * n_iscal * ld)) != SM_OK) return fail(r);
-  if ((r = st->vec.ensure(sizeof(double) * (size_t)n_vec * n * ld)) != SM_OK) return fail(r);
+  if ((r = st->scal_d.ensure(sizeof(double) * n_dscal * ld)) != SM_OK) return r;
+  if ((r = st->scal_i.ensure(sizeof(int) * n_iscal * ld)) != SM_OK) return r;
+  if ((r = st->vec.ensure(sizeof(double) * (size_t)n_vec * n * ld)) != SM_OK) return r;
   const size_t esz = d.mixed ? sizeof(float) : sizeof(double);
   d.lu_stride = (int64_t)n * lu.ld;
   d.lup_stride = lu.p_size;
-  if ((r = st->lup.ensure(esz * (size_t)d.lup_stride * C)) != SM_OK) return fail(r);
-  if ((r = st->list.ensure(sizeof(int) * ld)) != SM_OK) return fail(r);
-  if ((r = st->counters.ensure(sizeof(int) * kCounters)) != SM_OK) return fail(r);
+  if ((r = st->lup.ensure(esz * (size_t)d.lup_stride * C)) != SM_OK) return r;
+  if ((r = st->list.ensure(sizeof(int) * ld)) != SM_OK) return r;
+  if ((r = st->counters.ensure(sizeof(int) * kCounters)) != SM_OK) return r;
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device);
-  if ((r = cell_shapes(net, d, net->th_t >= 0, o.refresh_ctas_per_sm, &st->cell)) != SM_OK) return fail(r);
+  if ((r = cell_shapes(net, d, net->th_t >= 0, o.refresh_ctas_per_sm, &st->cell)) != SM_OK) return r;
   st->fused = st->cell.wide.ctas > 0 &&
               (net->th_t >= 0 || o.record_steps > 0 || C < class_path_from(net->cell.nb, d.mixed != 0));
   if (st->fused) {
     CellLaunch& cl = st->cell;
     const int64_t ring = 2 + std::max<int64_t>(C, 16 * std::min<int64_t>(C, 8LL * cl.max_ctas()));
     const int64_t nc = std::min<int64_t>(C, cl.max_ctas());
-    if ((r = st->cell_scratch.ensure(sizeof(double) * (size_t)(cl.wide.plan.scratch * nc))) != SM_OK) return fail(r);
-    if ((r = st->ring.ensure(sizeof(int) * (size_t)(ring + ld))) != SM_OK) return fail(r);
+    if ((r = st->cell_scratch.ensure(sizeof(double) * (size_t)(cl.wide.plan.scratch * nc))) != SM_OK) return r;
+    if ((r = st->ring.ensure(sizeof(int) * (size_t)(ring + ld))) != SM_OK) return r;
     cl.scratch = st->cell_scratch.as<double>();
     cl.ring = st->ring.as<int>();
     cl.done = cl.ring + ring;
     cl.timing_kind = o.timing_kind;
     if (o.timing_kind != SM_TIME_NONE) {
-      if ((r = st->cell_time.ensure(2 * sizeof(double))) != SM_OK) return fail(r);
-      SM_TRY_CUDA(cudaMemset(st->cell_time.p, 0, 2 * sizeof(double)));
+      if ((r = st->cell_time.ensure(2 * sizeof(double))) != SM_OK) return r;
+      SM_TRY_CUDA(cudaMemsetAsync(st->cell_time.p, 0, 2 * sizeof(double), st->s));
       cl.timing = st->cell_time.as<double>();
     }
   }
@@ -2858,14 +2851,14 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   // slot-ordered rate coefficients: with compaction, and always with a
   // coupled temperature (its k'(T) is rewritten before every right-hand side)
   if (d.compact || (net->th_t >= 0 && !st->fused)) {
-    if ((r = st->kslot.ensure(sizeof(double) * (size_t)net->n_r * ld)) != SM_OK) return fail(r);
+    if ((r = st->kslot.ensure(sizeof(double) * (size_t)net->n_r * ld)) != SM_OK) return r;
   }
   if (d.compact) {
-    if ((r = st->cpt.ensure(sizeof(int) * 2 * (size_t)ld)) != SM_OK) return fail(r);
+    if ((r = st->cpt.ensure(sizeof(int) * 2 * (size_t)ld)) != SM_OK) return r;
   }
   if ((!st->fused || o.record_steps > 0) &&
       (r = st->scratch.ensure(sizeof(double) * (size_t)net->n_r * ld)) != SM_OK)
-    return fail(r);
+    return r;
   double* ds = st->scal_d.as<double>();
   d.t = ds; d.h = ds + ld; d.gam = ds + 2 * ld; d.gam_J = ds + 3 * ld; d.crate = ds + 4 * ld;
   d.dprev = ds + 5 * ld; d.tn = ds + 6 * ld; d.alpha = ds + (6 + QMAX + 1) * ld;
@@ -2910,8 +2903,8 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
     const int64_t R = d.record, K = R / kCkpt + 1;
     if ((r = st->rec_d.ensure(sizeof(double) * (size_t)(2 * R * ld + K * (QMAX + 1) * (int64_t)n * ld +
                                                         K * (QMAX + 1) * ld))) != SM_OK)
-      return fail(r);
-    if ((r = st->rec_i.ensure(sizeof(int) * (size_t)(R * ld + K * ld))) != SM_OK) return fail(r);
+      return r;
+    if ((r = st->rec_i.ensure(sizeof(int) * (size_t)(R * ld + K * ld))) != SM_OK) return r;
     double* rd = st->rec_d.as<double>();
     d.log_t = rd;
     d.log_h = rd + R * ld;
@@ -2921,13 +2914,6 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
     d.log_q = ri;
     d.ck_nh = ri + R * ld;
   }
-  if (cudaStreamCreateWithFlags(&st->s, cudaStreamNonBlocking) != cudaSuccess) return fail(SM_ECUDA);
-  if (cudaEventCreateWithFlags(&st->ev_in, cudaEventDisableTiming) != cudaSuccess) return fail(SM_ECUDA);
-  if (cudaEventCreateWithFlags(&st->ev_out, cudaEventDisableTiming) != cudaSuccess) return fail(SM_ECUDA);
-  if (cudaStreamCreateWithFlags(&st->s2, cudaStreamNonBlocking) != cudaSuccess) return fail(SM_ECUDA);
-  if (cudaEventCreateWithFlags(&st->ev_fork, cudaEventDisableTiming) != cudaSuccess) return fail(SM_ECUDA);
-  if (cudaEventCreateWithFlags(&st->ev_join, cudaEventDisableTiming) != cudaSuccess) return fail(SM_ECUDA);
-  if (cudaMallocHost(&st->h_counters, kCounters * sizeof(int)) != cudaSuccess) return fail(SM_ENOMEM);
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, net->device);
   {
@@ -2961,7 +2947,7 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
 
   // (a fused state without recorded steps never launches it)
   const bool classes = !st->fused || d.record;
-  if (classes && (int64_t)rsm > smem_max) return fail(SM_ENOTSUP);
+  if (classes && (int64_t)rsm > smem_max) return SM_ENOTSUP;
   // the attribute is a per-kernel cap shared by every state: set it to the
   // device limit so that a later state with a smaller plan cannot lower it
   // below what an earlier state launches with
@@ -2983,7 +2969,7 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
   // recording states, whose replays keep dense factors per cell
   d.lu_cta = d.record ? 0 : 1;
   if (classes && (r = st->lu.ensure(esz * (size_t)d.lu_stride * (d.lu_cta ? st->refresh_ctas : C))) != SM_OK)
-    return fail(r);
+    return r;
   d.lu = st->lu.p;
   // coupled temperature: a copy of the network's setting
   d.therm = 0;
@@ -3009,19 +2995,19 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
       for (int q = 0; q < 4; ++q) dn += net->prod[4 * j + q] >= 0 ? 1 : 0;
       par[2 * n + j] = dn;
     }
-    if ((r = st->th_par.upload(par.data(), par.size() * sizeof(double))) != SM_OK) return fail(r);
+    if ((r = st->th_par.upload(par.data(), par.size() * sizeof(double))) != SM_OK) return r;
     d.th_L = st->th_par.as<double>();
     d.th_E = d.th_L + n;
     d.th_dn = d.th_L + 2 * n;
     d.n_cool = (int)cool.size();
-    if (!cool.empty() && (r = st->th_cool.upload(cool.data(), cool.size() * sizeof(int))) != SM_OK) return fail(r);
+    if (!cool.empty() && (r = st->th_cool.upload(cool.data(), cool.size() * sizeof(int))) != SM_OK) return r;
     d.th_cool = st->th_cool.as<int>();
-    if ((r = st->cond.ensure(sizeof(double) * 3 * (size_t)ld)) != SM_OK) return fail(r);
+    if ((r = st->cond.ensure(sizeof(double) * 3 * (size_t)ld)) != SM_OK) return r;
     d.c_nH = st->cond.as<double>();
     d.c_Av = d.c_nH + ld;
     d.c_chi = d.c_nH + 2 * ld;
     d.bpad = (n + 3) / 4 * 4;
-    if ((r = st->bord.ensure(sizeof(double) * (2 * (size_t)d.bpad + 1) * ld)) != SM_OK) return fail(r);
+    if ((r = st->bord.ensure(sizeof(double) * (2 * (size_t)d.bpad + 1) * ld)) != SM_OK) return r;
     d.bz = st->bord.as<double>();
     d.bgv = d.bz + (int64_t)d.bpad * ld;
     d.bs = d.bgv + (int64_t)d.bpad * ld;
@@ -3033,10 +3019,31 @@ sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_
                                          (int)st->border_smem)
                   : cudaFuncSetAttribute(th_border_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)st->border_smem);
-      if (e != cudaSuccess) return fail(SM_ECUDA);
+      SM_TRY_CUDA(e);
     }
   }
-  SM_TRY_CUDA(cudaMemset(st->scal_i.p, 0, st->scal_i.bytes));
+  SM_TRY_CUDA(cudaMemsetAsync(st->scal_i.p, 0, st->scal_i.bytes, st->s));
+  return SM_OK;
+}
+
+sm_status sm_state_create(const sm_net* net, int64_t C, const sm_opts* opts, sm_state** out) {
+  if (!out) return SM_EINVAL;
+  *out = nullptr;
+  if (!net || net->device < 0 || C < 1) return SM_EINVAL;
+  sm_opts o;
+  sm_opts_default(&o);
+  if (opts) o = *opts;
+  if (!opts_ok(o)) return SM_EINVAL;
+  Scope scope(net->device);
+  if (!scope.ok) return SM_ECUDA;
+  sm_state* st = new (std::nothrow) sm_state();
+  if (!st) return SM_ENOMEM;
+  const sm_status r = build_state(net, C, o, st);
+  if (r != SM_OK) {
+    free_state(st);
+    delete st;
+    return r;
+  }
   *out = st;
   return SM_OK;
 }
