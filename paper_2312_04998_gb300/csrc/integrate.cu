@@ -2945,9 +2945,8 @@ static sm_status build_state(const sm_net* net, int64_t C, const sm_opts& o, sm_
   }
   const size_t rsm = st->plan.bytes;
 
-  // (a fused state without recorded steps never launches it)
-  const bool classes = !st->fused || d.record;
-  if (classes && (int64_t)rsm > smem_max) return SM_ENOTSUP;
+  if ((int64_t)rsm > smem_max) return SM_ENOTSUP;   // one limit for every state, whichever kernels it runs
+  const bool classes = !st->fused || d.record;      // (a fused state without recorded steps never launches the refresh)
   // the attribute is a per-kernel cap shared by every state: set it to the
   // device limit so that a later state with a smaller plan cannot lower it
   // below what an earlier state launches with
