@@ -823,11 +823,33 @@ def adjoint_measurement(B, C, dev):
     return out
 
 
+def phase_table(B, refresh, cell, stats):
+    """Cycles per phase from the counters of the two kernels that may have run:
+    per refreshed cell of the refresh kernel (launch per class), or per attempt,
+    Newton iteration or factorisation of the persistent kernel."""
+    if refresh[15] > 0:
+        per = refresh[:len(B.PHASE_NAMES)] / refresh[15]
+        tot = per.sum()
+        return {"what": "refresh kernel cycles per refreshed cell, by phase (thread 0 of each CTA)",
+                "refreshed_cells": int(refresh[15]), "total_cycles_per_cell": float(tot),
+                "phases": [[nm, float(v), float(v / tot)] for nm, v in zip(B.PHASE_NAMES, per)]}
+    tot = float(cell[:len(B.CELL_PHASE_NAMES)].sum())
+    if not tot > 0.0:
+        raise RuntimeError("no kernel with phase counters ran (is this the phase-clock build?)")
+    units = {"attempt": float((stats["steps"] + stats["rejects"] + stats["conv_fails"]).sum()),
+             "Newton iteration": float(stats["newton_iters"].sum()), "factorisation": float(stats["jac_evals"].sum())}
+    of = lambda i: "attempt" if i in (0, 1, 5) else "Newton iteration" if i < 5 else "factorisation"
+    return {"what": "cycles of the persistent integrator kernel by phase (thread 0 of each CTA)", "units": units,
+            "total_cycles_per_attempt": tot / max(units["attempt"], 1.0),
+            "phases": [[nm, float(cell[i]) / max(units[of(i)], 1.0), of(i), float(cell[i]) / tot]
+                       for i, nm in enumerate(B.CELL_PHASE_NAMES)]}
+
+
 def phase_profile(B, a, dev):
-    """Cycles per phase of the persistent kernel over one whole integration of
-    the first a.cells cells of the headline workload (thread 0 of each CTA,
-    between the barriers that end the phases; the phase-clock build of the
-    library), per attempt, Newton iteration or factorisation."""
+    """Cycles per phase of the kernel that integrates the batch (see
+    phase_table), over one whole integration of the first a.cells cells of the
+    headline workload; thread 0 of each CTA, between the barriers that end the
+    phases, in the phase-clock build of the library."""
     import numpy as np
     import torch
     from synth.workloads import make
@@ -840,20 +862,13 @@ def phase_profile(B, a, dev):
     st.step(kd, 8)
     torch.cuda.synchronize()
     B.phase_cycles(dev.index or 0, reset=True)
+    B.cell_phase_cycles(dev.index or 0, reset=True)
     yd = y0d.clone()
     st.integrate(kd, yd, a.t_end_yr * YEAR, a.cells, stats)
     torch.cuda.synchronize()
-    cyc = B.phase_cycles(dev.index or 0)
-    h = B.stats_to_numpy(stats)
-    units = {"attempt": float((h["steps"] + h["rejects"] + h["conv_fails"]).sum()),
-             "Newton iteration": float(h["newton_iters"].sum()), "factorisation": float(h["jac_evals"].sum())}
-    of = lambda i: "attempt" if i in (0, 1, 5) else "Newton iteration" if i < 5 else "factorisation"
-    tot = max(float(cyc[:len(B.PHASE_NAMES)].sum()), 1.0)
-    return {"what": "cycles of the persistent integrator kernel by phase (thread 0 of each CTA)",
-            "workload": WORKLOAD, "cells": a.cells, "precision": a.precision, "units": units,
-            "total_cycles_per_attempt": tot / max(units["attempt"], 1.0),
-            "phases": [[nm, float(cyc[i]) / max(units[of(i)], 1.0), of(i), float(cyc[i]) / tot]
-                       for i, nm in enumerate(B.PHASE_NAMES)]}
+    return {"workload": WORKLOAD, "cells": a.cells, "precision": a.precision,
+            **phase_table(B, B.phase_cycles(dev.index or 0), B.cell_phase_cycles(dev.index or 0),
+                          B.stats_to_numpy(stats))}
 
 
 def kernel_source_hash():

@@ -113,6 +113,7 @@ _SIGS = [
     ("sm_sync", ct.c_int32, [ct.c_void_p, ct.c_void_p]),
     ("sm_probe_fma", ct.c_int32, [ct.c_int32, ct.c_int32, ct.POINTER(ct.c_double)]),
     ("sm_phase_cycles", ct.c_int32, [ct.c_int32, ct.c_void_p, ct.c_int32]),
+    ("sm_cell_phase_cycles", ct.c_int32, [ct.c_int32, ct.c_void_p, ct.c_int32]),
     ("sm_opts_default", None, [ct.POINTER(Opts_c)]),
     ("sm_state_create", ct.c_int32, [ct.c_void_p, ct.c_int64, ct.POINTER(Opts_c), ct.POINTER(ct.c_void_p)]),
     ("sm_state_free", ct.c_int32, [ct.c_void_p]),
@@ -506,8 +507,12 @@ def probe_fma(device: int, fp64: bool) -> float:
     return v.value
 
 
-PHASE_NAMES = ["state load / store", "predict", "reaction rates", "S R gather", "residual + substitution + update",
-               "finish", "dR/dx + Jacobian gather", "head program", "panel assembly", "panel updates", "panel LU"]
+PHASE_NAMES = ["zero + dR + weights", "Jacobian gather + M", "sparse head (A11, L21, U12)",
+               "head Schur complement", "head packing", "panel loads", "panel LU", "U block load",
+               "U block solve", "trailing update", "epilogue"]
+CELL_PHASE_NAMES = ["state load / store", "predict", "reaction rates", "S R gather",
+                    "residual + substitution + update", "finish", "dR/dx + Jacobian gather", "head program",
+                    "panel assembly", "panel updates", "panel LU"]
 
 
 def use_phase_build():
@@ -524,6 +529,14 @@ def phase_cycles(device: int, reset: bool = False) -> np.ndarray:
     needs the phase-clock build (STOICH_PHASES=1)."""
     out = np.zeros(16)
     _check(lib().sm_phase_cycles(int(device), out.ctypes.data, int(bool(reset))), "sm_phase_cycles")
+    return out
+
+
+def cell_phase_cycles(device: int, reset: bool = False) -> np.ndarray:
+    """The persistent kernel's cycles per phase (16 slots, see
+    sm_cell_phase_cycles); needs the phase-clock build."""
+    out = np.zeros(16)
+    _check(lib().sm_cell_phase_cycles(int(device), out.ctypes.data, int(bool(reset))), "sm_cell_phase_cycles")
     return out
 
 

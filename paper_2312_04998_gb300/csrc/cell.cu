@@ -2210,7 +2210,7 @@ sm_status launch_cell_attempts(const sm_net* net, const Dev& d, const CellLaunch
   return SM_OK;
 }
 
-extern "C" sm_status sm_phase_cycles(int32_t device, double* h_out, int32_t reset) {
+extern "C" sm_status sm_cell_phase_cycles(int32_t device, double* h_out, int32_t reset) {
 #ifdef SM_PHASE_CLOCKS
   if (!h_out || device < 0) return SM_EINVAL;
   int prev = -1;

@@ -237,6 +237,28 @@ __global__ void __launch_bounds__(32 * kCoopWarps) predict_kernel(Dev d) {
 //     update is a register-tiled GEMM.
 // Inverse pivots replace the diagonal.
 // ---------------------------------------------------------------------------
+// Optional per-phase cycle counters of the refresh kernel (build option
+// SM_PHASE_CLOCKS, see build.py): thread 0 of every CTA (of a cluster's first)
+// adds the clock64() cycles between consecutive phase marks (taken right after
+// the CTA-wide barriers that end the phases) to g_phase_cycles[phase]; slot 15
+// counts the refreshed cells.  Compiled out otherwise.
+constexpr int kPhaseSlots = 16;
+#ifdef SM_PHASE_CLOCKS
+__device__ unsigned long long g_phase_cycles[kPhaseSlots];
+#define PHASE_START() long long ph_t = clock64()
+#define PHASE_MARK(k)                                                                         \
+  do {                                                                                        \
+    if (threadIdx.x == 0 && rank == 0) {                                                      \
+      const long long ph_now = clock64();                                                     \
+      atomicAdd(&g_phase_cycles[(k)], (unsigned long long)(ph_now - ph_t));                   \
+      ph_t = ph_now;                                                                          \
+    }                                                                                         \
+  } while (0)
+#else
+#define PHASE_START() do {} while (0)
+#define PHASE_MARK(k) do {} while (0)
+#endif
+
 constexpr int kRefreshThreads = 256;
 constexpr int kNB = 32;
 constexpr int kTM = 4, kTN = 4;
@@ -406,6 +428,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
     T* A = static_cast<T*>(d.lu) + (d.lu_cta ? (int64_t)blockIdx.x : c) * d.lu_stride;
     T* P = d.lup ? static_cast<T*>(d.lup) + (int64_t)d.slot_cell[c] * d.lup_stride : nullptr;
     T* D = P ? P + d.p_d : nullptr;   // packed tail block, column-major
+    PHASE_START();
     const double gamma = d.gam[c];
     if (rank == 0) {
       // zero the dense trailing block and the head's pattern entries
@@ -436,6 +459,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           wif[s] = (float)(1.0 / wv);
         }
       __syncthreads();
+      PHASE_MARK(0);   // zero the working matrix, dR/dx, weights
       // M_ij = delta_ij - gamma sum_terms coef dR, stored in elimination order
       // (W M W^-1 with this step's error weights, scaled in FP32, when mixed)
       auto store_m = [&](const int4 ds, double acc) {
@@ -488,6 +512,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
       }
     }
     __syncthreads();
+    PHASE_MARK(1);   // Jacobian gather, M = I - gamma J
     // ---- phase B: sparse head.  The head program (see LUSymbolic) computes
     // every head factor entry in the packed layout, in shared memory: level
     // by level, first the level's pivots (stored inverted), then the U rows
@@ -521,6 +546,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           __syncthreads();
         }
       }
+      PHASE_MARK(2);   // head program
       if (S > 1) {
         cluster_sync();   // M and the head are complete
         if (rank > 0)
@@ -610,6 +636,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         __syncthreads();
       }
     }
+    PHASE_MARK(3);   // head Schur complement (or the pivot-by-pivot head)
     // the head's factors are final.  Packed output: copy them out (from H, or
     // from the dense matrix after the pivot-by-pivot head); dense output: put
     // H's values back at their dense positions
@@ -642,6 +669,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         for (int q = lane; q < cnt; q += 32) P[d.p_l21 + o + q] = Ai[__ldg(d.lridx + p0 + q)];
       }
     }
+    PHASE_MARK(4);   // packed head factors
     if (S > 1) cluster_sync();   // the Schur complement is complete, rank 0's head has been read
     // ---- phase C: dense trailing block, blocked right-looking LU
     for (int pb = 0; pb * kNB < nt; ++pb) {
@@ -656,6 +684,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
       for (int a = m + tid; a < pitch; a += nthr)
         for (int b = 0; b < w; ++b) Pt[b * pitch + a] = T(0);
       __syncthreads();
+      PHASE_MARK(5);   // panel loads
       if (rank > 0) {
         // (rank 0's)
       } else if (sizeof(T) == 4 && w == kNB) {
@@ -715,6 +744,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
         }
         __syncthreads();
       }
+      PHASE_MARK(6);   // panel LU
       if (D) {
         // the panel's columns (diagonal block and L below it) are final
         for (int b = warp; b < w; b += nwarps)
@@ -734,6 +764,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
           for (int b = lane; b < rp; b += 32)
             if (mine(b)) U[a * upitch + b] = b < r ? A[(int64_t)(p0 + a) * ldm + p0 + w + b] : T(0);
         __syncthreads();
+        PHASE_MARK(7);   // panel stored, U block loaded
         // U12 = L11^-1 A12, one thread per column
         if (w == kNB) {
           for (int b = tid; b < r; b += nthr) {
@@ -756,6 +787,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
             }
         }
         __syncthreads();
+        PHASE_MARK(8);   // U block solved
         if (D) {
           // the panel's U rows are final: column b of the block, rows p0..p0+w
           for (int e = tid; e < r * 32; e += nthr) {
@@ -822,6 +854,7 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
       }
       __syncthreads();
       if (S > 1 && r > 0) cluster_sync();   // the trailing block is up to date
+      PHASE_MARK(9);   // trailing update
     }
     if (tid == 0 && rank == 0) {
       d.gam_J[c] = gamma;
@@ -831,6 +864,10 @@ __global__ void __launch_bounds__(kRefreshThreads, 2) refresh_kernel(Dev d, cons
       d.jac_evals[c] += 1;
     }
     __syncthreads();
+#ifdef SM_PHASE_CLOCKS
+    if (tid == 0 && rank == 0) atomicAdd(&g_phase_cycles[kPhaseSlots - 1], 1ull);
+#endif
+    PHASE_MARK(10);  // epilogue
   }
 }
 
@@ -3436,4 +3473,25 @@ extern "C" sm_status sm_state_timing_reset(sm_state* st) {
     SM_TRY_CUDA(cudaMemsetAsync(st->cell.timing, 0, 2 * sizeof(double), st->s));
   }
   return SM_OK;
+}
+
+extern "C" sm_status sm_phase_cycles(int32_t device, double* h_out, int32_t reset) {
+#ifdef SM_PHASE_CLOCKS
+  if (!h_out || device < 0) return SM_EINVAL;
+  Scope scope(device);
+  if (!scope.ok) return SM_ECUDA;
+  unsigned long long v[kPhaseSlots];
+  SM_TRY_CUDA(cudaMemcpyFromSymbol(v, g_phase_cycles, sizeof(v)));
+  for (int i = 0; i < kPhaseSlots; ++i) h_out[i] = (double)v[i];
+  if (reset) {
+    const unsigned long long z[kPhaseSlots] = {0};
+    SM_TRY_CUDA(cudaMemcpyToSymbol(g_phase_cycles, z, sizeof(z)));
+  }
+  return SM_OK;
+#else
+  (void)device;
+  (void)h_out;
+  (void)reset;
+  return SM_ENOTSUP;
+#endif
 }
