@@ -75,10 +75,11 @@ PEAK_FP64 = SM_COUNT * 4 * SM_GHZ / 1e3           # TFLOP/s
 
 # DRAM bytes (read + write) per processed unit of a kernel class, from a
 # committed ncu capture in profiles/ (named there), keyed on the class, the
-# precision and the hash of the integrator's kernel code (comments and
+# precision and the hash of the launch-per-class kernels' sources (comments and
 # whitespace removed) at capture time: a changed kernel reports traffic null
-# until it is captured again.  (The persistent kernel runs every class in one
-# launch, so no counter separates them.)
+# until it is captured again.  (Batches that the persistent kernel integrates
+# report null too: it runs every class in one launch, so no counter separates
+# them.)
 TRAFFIC = {}
 
 
@@ -871,20 +872,26 @@ def phase_profile(B, a, dev):
                           B.stats_to_numpy(stats))}
 
 
+CLASS_SOURCES = ("integrate.cu", "integ.h", "kern_rhs.cu")   # the launch-per-class kernels
+
+
 def kernel_source_hash():
-    """Hash of the integrator's kernel source (cell.cu) with comments and
-    whitespace removed, so that a comment edit keeps the key of a capture."""
+    """Hash of the launch-per-class kernels' sources with comments and whitespace
+    removed, so that a comment edit keeps the key of a capture."""
     import re
-    with open(os.path.join(ROOT, "paper_2312_04998_gb300", "csrc", "cell.cu")) as fh:
-        src = fh.read()
-    src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)      # block comments
-    src = re.sub(r"//[^\n]*", " ", src)                    # line comments
-    src = re.sub(r"\s+", " ", src).strip()
-    return hashlib.sha256(src.encode()).hexdigest()[:16]
+    h = hashlib.sha256()
+    for name in CLASS_SOURCES:
+        with open(os.path.join(ROOT, "paper_2312_04998_gb300", "csrc", name)) as fh:
+            src = fh.read()
+        src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)      # block comments
+        src = re.sub(r"//[^\n]*", " ", src)                    # line comments
+        h.update(re.sub(r"\s+", " ", src).strip().encode())
+    return h.hexdigest()[:16]
 
 
-def roofline(info, s, kind, precision, kern_ms, kern_n, peaks):
-    """Roofline of the timed kernel class over the timed integration."""
+def roofline(info, s, kind, precision, kern_ms, kern_n, peaks, by_class=True):
+    """Roofline of the timed kernel class over the timed integration; by_class:
+    it ran as launches of its own, not inside the persistent kernel."""
     if not kern_n:
         return None
     refreshes = float(s["jac_evals"].sum())
@@ -904,7 +911,7 @@ def roofline(info, s, kind, precision, kern_ms, kern_n, peaks):
         units = newton
         per_launch_units = units / kern_n
         ach = unit * per_launch_units / (kern_ms * 1e-3 / kern_n) / 1e9
-        tr = TRAFFIC.get((kind, precision, kernel_source_hash()))
+        tr = TRAFFIC.get((kind, precision, kernel_source_hash())) if by_class else None
         return {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": ach / peaks["hbm_gbs"], "traffic": None if tr is None else tr * per_launch_units,
                 "kernel": "solve (packed factors, warp per cell)", "avg_launch_ms": kern_ms / kern_n,
@@ -916,7 +923,7 @@ def roofline(info, s, kind, precision, kern_ms, kern_n, peaks):
     avg_s = kern_ms * 1e-3 / kern_n
     ach = unit * per_launch_units / avg_s / 1e12
     pk = peaks["fp32_tflops"] if fp32 else peaks["fp64_tflops"]
-    tr = TRAFFIC.get((kind, precision, kernel_source_hash()))
+    tr = TRAFFIC.get((kind, precision, kernel_source_hash())) if by_class else None
     return {"bound": "alu", "achieved": ach, "peak": pk, "unit": "TFLOP/s", "frac": ach / pk,
             "traffic": None if tr is None else tr * per_launch_units,
             "kernel": f"{kind} ({'FP32' if fp32 else 'FP64'} pipe)", "avg_launch_ms": kern_ms / kern_n,
@@ -1089,7 +1096,9 @@ def main():
             return {"error": f"{type(exc).__name__}: {exc}"}
 
     peaks = aux(peaks_, B, dev)
-    roof = roofline(info, s, a.time_kernel, a.precision, kern_ms, kern_n, peaks)
+    # (a launch per class is a dozen launches an attempt, the persistent kernel
+    # many attempts a launch)
+    roof = roofline(info, s, a.time_kernel, a.precision, kern_ms, kern_n, peaks, by_class=l_after - l_before > attempts)
     if roof is not None:
         roof["peak_kind"] = "derived (unit counts x max clock), timed inside a long step"
     mixed = aux(fp64_vs_mixed, B, a.mixed_cells, dev) if a.mixed_cells > 0 else None
