@@ -73,7 +73,6 @@ struct LUSymbolic {
   std::vector<int32_t> lptr, lidx;        // per pivot: rows below it (positions)
   std::vector<int32_t> uptr, uidx;        // per pivot: columns right of it
   std::vector<int32_t> lrptr, lridx;      // per row: columns of L left of the diagonal
-  std::vector<int32_t> ucptr, ucidx;      // per tail column j >= head: head rows k with U(k, j) != 0
   std::vector<int32_t> jrc;               // per J pattern entry: (row position << 16) | column position
   std::vector<int32_t> lrhead;            // per tail row: entries of its L row in head columns
   std::vector<int32_t> lrhoff;            // exclusive prefix sum of lrhead (n - head + 1 entries)
@@ -82,7 +81,6 @@ struct LUSymbolic {
   std::vector<int32_t> srow;              // tail rows with L21 entries, longest first
   std::vector<int32_t> uoff;              // per head row k: [n_panels + 1] offsets into its U list where
                                           // the tail columns of each 32-wide panel start
-  std::vector<int32_t> jpos;              // per J pattern entry: dense offset p*ld+q
   // Packed factor layout read by the substitution (per cell, values only,
   // in the precision of the factors), segment offsets in elements:
   //   [p_l11, +lrptr[head])   L11: head rows' L entries, order of lrptr/lridx

@@ -276,20 +276,6 @@ void build_lu_symbolic(sm_net& net) {
       break;
     }
   }
-  // column-wise view of the U entries of head rows in tail columns
-  {
-    const int32_t h = lu.head;
-    std::vector<std::vector<int32_t>> cols(n);
-    for (int32_t k = 0; k < h; ++k)
-      for (int32_t p = lu.uptr[k]; p < lu.uptr[k + 1]; ++p)
-        if (lu.uidx[p] >= h) cols[lu.uidx[p]].push_back(k);
-    lu.ucptr.assign(1, 0);
-    lu.ucidx.clear();
-    for (int32_t j = h; j < n; ++j) {
-      lu.ucidx.insert(lu.ucidx.end(), cols[j].begin(), cols[j].end());
-      lu.ucptr.push_back((int32_t)lu.ucidx.size());
-    }
-  }
   // per head row: where each 32-wide tail panel's columns start in its U list
   {
     const int32_t h = lu.head, np = (n - h + 31) / 32;
@@ -440,14 +426,10 @@ void build_lu_symbolic(sm_net& net) {
       lu.hop_ptr.push_back((int32_t)lu.hop_piv.size());
     }
   }
-  lu.jpos.resize(net.jp_col.size());
   lu.jrc.resize(net.jp_col.size());
   for (int32_t i = 0; i < n; ++i)
     for (int32_t p = net.jp_ptr[i]; p < net.jp_ptr[i + 1]; ++p)
-    {
-      lu.jpos[p] = lu.iperm[i] * lu.ld + lu.iperm[net.jp_col[p]];
       lu.jrc[p] = (lu.iperm[i] << 16) | lu.iperm[net.jp_col[p]];
-    }
 }
 
 }  // namespace
