@@ -2792,21 +2792,46 @@ int64_t pass_cells(int64_t C, int64_t cells_per_pass) {
 
 extern "C" {
 
-// Cells from which on the class-by-class path is the faster one (plain
-// integrations; nb: 32-wide blocks of the dense tail).  The fused kernel's rate
+// Cells from which on a state takes the class-by-class path (nt: rows of the dense
+// tail; plain: no coupled temperature, no recorded steps).  The fused kernel's rate
 // does not grow any more once every SM has its cells, while the class kernels,
-// 32 cells a block and bound by HBM, gain until about 65,536 cells.  Thousand
-// accepted steps per second, fused / class by class, whole integrations to 1e5 yr:
-//   470 species, mixed   16,384 cells 727 / 681, 32,768 726 / 795 (TF32 689 / 790)
-//   470 species, FP64    16,384 cells 165 / 143
-//   120 species          mixed 8,192 cells 4461 / 3146, 65,536 4372 / 5355;
-//                        FP64 65,536 cells 2241 / 2300
-//    32 species          mixed 8,192 cells 8669 / 9823, 65,536 7615 / 18403;
-//                        FP64 65,536 cells 7300 / 13268
-static int64_t class_path_from(int nb, bool mixed) {
-  if (nb <= 1) return 6144;
-  if (mixed) return 24576;
-  return nb <= 4 ? 65536 : INT64_MAX;
+// 32 cells a block and bound by HBM, gain until about 65,536 cells, the sooner the
+// smaller the network and the emptier the tail's last 32-wide block (which the
+// fused kernel works through in full).  Where cells are alike, all of them running
+// until the end, the class path overtakes early; where some need many times the
+// attempts of others it idles over their last ones, most of all where it does not
+// compact the running cells (recorded steps).  The line lies about where what the
+// former lose equals what the latter gain.  Time fused / class by class, like cells
+// (a PDR slab over 1e-2 yr) | unlike ones (T 10 to 1000 K, n_H 1e2 to 1e8, whole
+// integrations; coupled temperature and recorded: 1 yr):
+//   rows                    4096 cells    8192          16,384        65,536
+//    21 FP32 plain          1.09 | 0.80   1.40 | 1.17   1.59          2.05 | 2.42
+//            recorded       1.09 | 0.65   1.41 | 0.83   1.60 | 0.96   2.06 | 1.56
+//            temperature    1.01 | 0.52   1.48 | 0.84   1.77 | 1.23   2.17
+//       FP64 plain          0.77 | 0.69   0.92 | 0.93   1.02          1.32 | 1.82
+//            recorded       0.77 | 0.56   0.92 | 0.69   1.03 | 0.79   1.31 | 1.24
+//            temperature    0.82 | 0.48   1.12 | 0.75   1.31 | 1.05   1.62
+//    40 FP32 plain          1.13 | 0.64   1.25 | 0.86   1.36 | 1.11   1.40
+//            recorded       1.10 | 0.49   1.24 | 0.59   1.35 | 0.77   1.37 | 1.19
+//            temperature    1.13 | 0.38   1.28 | 0.62   1.39 | 0.87   1.40
+//       FP64 plain          1.03 | 0.63   1.11 | 0.84   1.16 | 1.02   1.11
+//            recorded       1.02 | 0.54   1.10 | 0.68   1.15 | 0.83   1.11 | 1.07
+//            temperature    1.08 | 0.44   1.18 | 0.68   1.24 | 0.89   1.18
+//    62 FP32 all three      0.81 - 0.86   0.94 - 0.96   1.04 - 1.10   1.16 - 1.22
+//       FP64 all three      0.75 - 0.76   0.82 - 0.85   0.89 - 0.92   0.91 - 0.95
+//    83 FP32 plain          0.86 | 0.52   0.93 | 0.69   0.98 | 0.86   1.00 | 1.22
+//            the other two  0.80 - 0.84   0.90 - 0.92   0.94 - 0.96   0.95 - 0.98
+//       FP64 all three      0.99 - 1.00   1.03 - 1.05   1.06          1.04 - 1.06
+//   127 FP32, FP64          0.78 - 0.87   0.82 - 0.93   0.82 - 0.98   0.82 - 0.96
+//   349 FP32 plain          0.89 | 0.63   | 0.78        0.93 | 0.94   | 1.10 (32,768)
+static int64_t class_path_from(int nt, bool mixed, bool plain) {
+  const int nb = (nt + 31) / 32;
+  const bool padded = 10 * nt < 9 * 32 * nb;   // more than a tenth of the blocks is padding
+  if (nb <= 1) return mixed ? (plain ? 4608 : 6144) : plain ? 6144 : 12288;
+  if (nb == 2 && padded) return mixed && plain ? 7168 : 12288;
+  if (nb == 2 && mixed) return 16384;
+  if (mixed) return plain ? 24576 : INT64_MAX;
+  return nb <= 4 && (plain || padded) ? 65536 : INT64_MAX;
 }
 
 // Allocates and fills in a new state; what a failure leaves behind is the
@@ -2865,7 +2890,7 @@ static sm_status build_state(const sm_net* net, int64_t C, const sm_opts& o, sm_
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, net->device);
   if ((r = cell_shapes(net, d, net->th_t >= 0, o.refresh_ctas_per_sm, &st->cell)) != SM_OK) return r;
   st->fused = st->cell.wide.ctas > 0 &&
-              (net->th_t >= 0 || o.record_steps > 0 || C < class_path_from(net->cell.nb, d.mixed != 0));
+              C < class_path_from(n - lu.head, d.mixed != 0, net->th_t < 0 && o.record_steps == 0);
   if (st->fused) {
     CellLaunch& cl = st->cell;
     const int64_t ring = 2 + std::max<int64_t>(C, 16 * std::min<int64_t>(C, 8LL * cl.max_ctas()));
