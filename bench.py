@@ -80,7 +80,11 @@ PEAK_FP64 = SM_COUNT * 4 * SM_GHZ / 1e3           # TFLOP/s
 # until it is captured again.  (Batches that the persistent kernel integrates
 # report null too: it runs every class in one launch, so no counter separates
 # them.)
-TRAFFIC = {}
+TRAFFIC = {
+    # profiles/refresh_kernel_mixed_24576cells.md: 140.9 GB in a launch that
+    # refreshed all 24,576 cells
+    ("refresh", "mixed", "d020121fd3ea2f16"): 5.733e6,
+}
 
 
 def args_():

@@ -295,10 +295,11 @@ typedef struct {
     int32_t max_conv_fails;   /* consecutive Newton failures before SM_CELL_CONV   */
     int32_t precision;        /* SM_PREC_FP64, SM_PREC_MIXED or SM_PREC_TF32       */
     /* Most batches are integrated by one persistent kernel that carries each
-       cell through its own attempts; large batches, and networks whose tables do
-       not fit an SM's shared memory, take a group of launches over all cells per
-       attempt, which is what use_graph, attempts_per_sync and sm_net_set_integ
-       concern. */
+       cell through its own attempts; states of large capacity (from 4,608 cells
+       for the smallest networks, 24,576 for large ones in mixed precision), and
+       networks whose tables do not fit an SM's shared memory, take a group of
+       launches over all cells per attempt, which is what use_graph,
+       attempts_per_sync and sm_net_set_integ concern. */
     int32_t use_graph;        /* capture the attempt loop in a CUDA graph (1) or not */
     int32_t attempts_per_sync;/* attempts launched between completion checks      */
     int32_t timing_kind;      /* SM_TIME_*: part of an attempt that is timed      */

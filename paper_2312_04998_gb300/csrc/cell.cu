@@ -21,15 +21,15 @@
 //   substitution  a warp per 32 rows; the next block's factors are in flight
 //                 while the diagonal block's 32-step chain runs
 // Every sum that a step depends on is formed in the order of the class-by-class
-// kernels (integrate.cu), which serve the networks that do not fit: the two
-// take the same steps to the last bit (with the 16-cell gather).
+// kernels (integrate.cu), which serve large batches and the networks that do not
+// fit: the two take the same steps to the last bit (with the 16-cell gather).
 //
 // Cycles per cell on one SM, 470 species, 6000 reactions, FP32 factors: rates
-// 15 k, S R 37 k and substitution 118 k per Newton iteration; predict 14 k,
-// finish 26 k per attempt; Jacobian 65 k, head 54 k, assembly 197 k, panels
-// 170 k, trailing updates 427 k per factorisation.  (One launch per kernel class:
-// 2.28 M per factorisation.)  4096 cells, first 1e-3 yr: 1212 -> 744 ms; 128 cells
-// of a slab, 1e3 yr: 559 -> 59 ms; one cell of 32 species, 1e6 yr: 17.6 -> 5.7 ms.
+// 15 k, S R 29 k and substitution 118 k per Newton iteration; predict 14 k,
+// finish 26 k per attempt; Jacobian 69 k, head 54 k, assembly 197 k, panels
+// 171 k, trailing updates 428 k per factorisation.  (One launch per kernel class:
+// 2.28 M per factorisation.)  4096 cells, first 1e-3 yr: 1203 -> 723 ms; 128 cells
+// of a slab, 1e3 yr: 562 -> 57 ms; one cell of 32 species, 1e6 yr: 17.0 -> 4.9 ms.
 #include "cell.h"
 #include <algorithm>
 #include <type_traits>
@@ -1409,7 +1409,7 @@ __device__ __forceinline__ void cell_border() {
   __syncthreads();
 }
 
-// One BDF attempt of the cell; returns false when the cell stopped before it.
+// The clock cycles of the timed class (sm_opts.timing_kind), by thread 0.
 __device__ __forceinline__ void class_begin(int kind) {
   if (args().timing_kind == kind && threadIdx.x == 0) scalars().t0 = clock64();
 }

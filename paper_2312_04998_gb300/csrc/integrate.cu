@@ -2,7 +2,12 @@
 // (the stiff-solver role of DLSODES in Section 3), one independent state
 // machine per cell.
 //
-// One "attempt" advances every unfinished cell by one trial step:
+// This file holds the host side of every state and the kernels that work class
+// by class over all cells: large batches and networks whose tables do not fit an
+// SM take these (see class_path_from); the others one persistent kernel that
+// carries each cell through its own attempts (cell.cu).
+//
+// Class by class, one "attempt" advances every unfinished cell by one trial step:
 //   predict   32 cells per CTA, the species split over 8 warps: Lagrange
 //             predictor, BDF coefficients, weights, and the decision whether
 //             the Newton matrix must be refreshed;
@@ -21,8 +26,8 @@
 // right-hand side, the temperature row follows each gather, and T is
 // eliminated last in the Newton solve (th_* kernels below).
 // The host enqueues attempts in groups (captured once in a CUDA graph) and
-// reads back only the number of running cells between groups.  The same file
-// holds the step recording and the discrete adjoint of the frozen-step map
+// reads back only the number of running cells between groups.  Here are also
+// the step recording and the discrete adjoint of the frozen-step map
 // (sm_state_steps, sm_adjoint, sm_replay) and checkpoint / resume
 // (sm_state_save, sm_state_load).
 #include <algorithm>
